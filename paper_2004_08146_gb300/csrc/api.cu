@@ -463,12 +463,13 @@ void sap_smooth(qcd_ctx* ctx, int prec, int op, int nrhs, const void* b, void* x
                 double tol, const int* act = nullptr) {
     ensure_sap(ctx);
     const size_t n = ctx->nfine();
-    void* r = ctx->buf("sap.r", n * nrhs * esz(prec));
+    const bool fused = sap_forms_residual(ctx->sap.B);
+    void* r = fused ? nullptr : ctx->buf("sap.r", n * nrhs * esz(prec));
     void* scr = ctx->buf("sap.scratch", sap_scratch_bytes(ctx->sap, prec, nrhs, ctx->p.sap_block_iters));
     for (int s = 0; s < sweeps; ++s) {
         for (int colour = 0; colour < 2; ++colour) {
-            residual_op(ctx->f, prec, op, nrhs, b, x, r, tau, ctx->st, act);
-            sap_blocks(ctx->f, ctx->sap, colour, prec, op, nrhs, r, x, tau, ctx->p.sap_block_iters, tol, scr, ctx->st,
+            if (!fused) residual_op(ctx->f, prec, op, nrhs, b, x, r, tau, ctx->st, act);
+            sap_blocks(ctx->f, ctx->sap, colour, prec, op, nrhs, fused ? b : r, x, tau, ctx->p.sap_block_iters, tol, scr, ctx->st,
                        act, ctx->p.sap_half != 0);
         }
     }
@@ -2037,8 +2038,9 @@ extern "C" int qcd_sap_static(qcd_ctx* ctx, int op, int prec, int nrhs, const vo
                                                                       plan.blocks_of_colour[1]);
     for (int s = 0; s < sweeps; ++s) {
         for (int colour = 0; colour < 2; ++colour) {
-            residual_op(ctx->f, prec, op, nrhs, b, x, r, tau, ctx->st);
-            sap_blocks(ctx->f, plan, colour, prec, op, nrhs, r, x, tau, ctx->p.sap_block_iters, block_tol, scr,
+            const bool fused = sap_forms_residual(B);
+            if (!fused) residual_op(ctx->f, prec, op, nrhs, b, x, r, tau, ctx->st);
+            sap_blocks(ctx->f, plan, colour, prec, op, nrhs, fused ? b : r, x, tau, ctx->p.sap_block_iters, block_tol, scr,
                        ctx->st);
         }
     }

@@ -42,6 +42,26 @@ template <typename Z> QCD_HD Z conj(Z a) { a.y = -a.y; return a; }
 template <typename Z> QCD_HD Z cmulc(Z a, Z b) {
     Z r; r.x = a.x * b.x + a.y * b.y; r.y = a.x * b.y - a.y * b.x; return r;
 }
+// acc += a b, acc += conj(a) b, acc -= a b as two fused multiply-adds per
+// component: `acc += a * b` would take a multiply, a fused multiply-add and an
+// add, because the product's own rounding may not be contracted away.
+template <typename Z> QCD_HD void cmac(Z& c, Z a, Z b) {
+    c.x = fma(-a.y, b.y, fma(a.x, b.x, c.x));
+    c.y = fma(a.y, b.x, fma(a.x, b.y, c.y));
+}
+template <typename Z> QCD_HD void cmacc(Z& c, Z a, Z b) {
+    c.x = fma(a.y, b.y, fma(a.x, b.x, c.x));
+    c.y = fma(-a.y, b.x, fma(a.x, b.y, c.y));
+}
+template <typename Z> QCD_HD void cmsub(Z& c, Z a, Z b) {
+    c.x = fma(a.y, b.y, fma(-a.x, b.x, c.x));
+    c.y = fma(-a.y, b.x, fma(-a.x, b.y, c.y));
+}
+// (re, im) += conj(a) b for scalars kept apart
+template <typename R, typename Z> QCD_HD void cdot(R& re, R& im, Z a, Z b) {
+    re = fma(a.y, b.y, fma(a.x, b.x, re));
+    im = fma(-a.y, b.x, fma(a.x, b.y, im));
+}
 // a * i^k (k = 0..3)
 template <typename Z> QCD_HD Z mul_ipow(Z a, int k) {
     Z r;

@@ -187,6 +187,9 @@ struct SapPlan {
     int* blocks_of_colour[2] = {nullptr, nullptr};  // device lists of block ids
     int ncol[2] = {0, 0};
 };
+// Whether sap_blocks forms the residual itself (2^4 blocks): its r argument is
+// then the right-hand side b of the sweep, not the residual field.
+bool sap_forms_residual(const Blocking& B);
 // x += block solves of op(tau) on the blocks of `colour`, rhs r (full fields)
 // half: FP32 solves on 16-site blocks keep the block Krylov basis in FP16
 void sap_blocks(const FineOp& f, const SapPlan& sp, int colour, int prec, int op, int nrhs,

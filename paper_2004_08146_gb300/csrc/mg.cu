@@ -1266,6 +1266,13 @@ __device__ __forceinline__ void bstore(float2* p, float2 v) { *p = v; }
 __device__ __forceinline__ void bstore(double2* p, double2 v) { *p = v; }
 __device__ __forceinline__ void bstore(__half2* p, float2 v) { *p = __float22half2_rn(v); }
 
+// the value a stored entry reads back as
+template <typename BT> __device__ __forceinline__ float2 bround(float2 v) {
+    if constexpr (sizeof(BT) == 4) return __half22float2(__float22half2_rn(v));
+    else return v;
+}
+template <typename BT> __device__ __forceinline__ double2 bround(double2 v) { return v; }
+
 // Copy N 16-byte words from global to shared memory with all N loads in
 // flight before the first store (staging without a round trip per word).
 template <int N>
@@ -1515,6 +1522,8 @@ __global__ void __launch_bounds__(128) sap_chi_kernel(Geom g, Blocking B, const 
     for (int k = 0; k < 6; ++k) x[(size_t)y * 12 + 6 * chi + k] = e[k];
 }
 
+#include "sap_cube.cuh"
+
 inline int grid_for(size_t n, int th = 256) {
     size_t gsz = (n + th - 1) / th;
     return (int)(gsz > 1048576 ? 1048576 : (gsz == 0 ? 1 : gsz));
@@ -1664,6 +1673,28 @@ void coarse_apply(const Coarse& c, int prec, int op, int nrhs, const void* x, vo
     }
 }
 
+bool sap_forms_residual(const Blocking& B) { return B.b[0] == 2 && B.b[1] == 2 && B.b[2] == 2 && B.b[3] == 2; }
+
+// Launch of sap_cube_kernel: rw right-hand sides (warps) share a CTA and its
+// staged links, as few CTAs per block as hold at most four, evenly filled
+// (5 right-hand sides: 3 + 2), fewer when the bases of many steps do not fit.
+template <typename R, typename BT>
+static void launch_cube(const FineOp& f, const SapPlan& sp, int colour, int op, int nrhs, const void* b, void* x,
+                        const Shifts& sh, int iters, double tol, cudaStream_t st, const int* act) {
+    int rw = (nrhs + 3) / 4;
+    rw = (nrhs + rw - 1) / rw;
+    while (rw > 1 && cube_layout<R, BT>(iters, rw).total > 226 * 1024) --rw;
+    const size_t sm = cube_layout<R, BT>(iters, rw).total;
+    if (sm + 1024 > 48 * 1024)
+        cudaFuncSetAttribute(sap_cube_kernel<R, BT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    const dim3 grid(sp.ncol[colour], (nrhs + rw - 1) / rw);
+    const bool dp = sizeof(R) == 8;
+    sap_cube_kernel<R, BT><<<grid, 32 * rw, sm, st>>>(f.g, sp.B, dp ? (const cplx<R>*)f.U64 : (const cplx<R>*)f.U32,
+                                                      dp ? (const R*)f.A64 : (const R*)f.A32,
+                                                      sp.blocks_of_colour[colour], op, sh, (const cplx<R>*)b,
+                                                      (cplx<R>*)x, iters, tol, act, nrhs);
+}
+
 bool sap_needs_scratch(const Blocking& B) { return B.bs != 16 && B.bs != 32; }
 
 void sap_work_reset() {
@@ -1705,6 +1736,18 @@ void sap_blocks(const FineOp& f, const SapPlan& sp, int colour, int prec, int op
     const int bs = sp.B.bs;
     const double rs = prec == QCD_FP64 ? 8.0 : 4.0;
     const double sites = (double)sp.ncol[colour] * bs;
+    if (sap_forms_residual(sp.B)) {
+        // b, x in and out, x of the other colour, links of both colours, clover
+        KTimer kt(prec == QCD_FP64 ? "sap_block_f64" : (half ? "sap_block_f32h" : "sap_block_f32"),
+                  rs * sites * (nrhs * 96.0 + 216.0), 1824.0 * sites * nrhs * (iters + 1), st);
+        if (prec == QCD_FP64)
+            launch_cube<double, double2>(f, sp, colour, op, nrhs, r, x, sh, iters, tol, st, act);
+        else if (half)
+            launch_cube<float, __half2>(f, sp, colour, op, nrhs, r, x, sh, iters, tol, st, act);
+        else
+            launch_cube<float, float2>(f, sp, colour, op, nrhs, r, x, sh, iters, tol, st, act);
+        return;
+    }
     KTimer kt(prec == QCD_FP64 ? "sap_block_f64" : (half && bs == 16 ? "sap_block_f32h" : "sap_block_f32"),
               rs * sites * (nrhs * 72.0 + 144.0),
               1824.0 * sites * nrhs * iters, st);
