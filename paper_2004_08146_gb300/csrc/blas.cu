@@ -46,9 +46,7 @@ __global__ void multidot_partial_kernel(const Z* __restrict__ X, size_t xstride_
     using Rt = decltype(Z{}.x);
     Rt ret = 0, imt = 0;
     for (size_t k = lo + threadIdx.x; k < hi; k += blockDim.x) {
-        Z a = x[k], b = y[k];
-        ret += a.x * b.x + a.y * b.y;
-        imt += a.x * b.y - a.y * b.x;
+        cdot(ret, imt, x[k], y[k]);
     }
     __shared__ double sre[32], sim[32];
     double re = (double)warp_sum(ret);
@@ -112,7 +110,7 @@ __global__ void multiaxpy_kernel(const Z* __restrict__ X, int nvec, size_t xstri
             if (staged) ci = cs[i * nrhs + j];
             else { ci.x = (R)c[i * nrhs + j].x; ci.y = (R)c[i * nrhs + j].y; }
             if (ci.x == R(0) && ci.y == R(0)) continue;   // unused basis slots may hold stale data
-            acc += ci * X[(size_t)i * xstride_vec + (size_t)j * n + k];
+            cmac(acc, ci, X[(size_t)i * xstride_vec + (size_t)j * n + k]);
         }
         Z o = w[t];
         const R sg = (R)sign;

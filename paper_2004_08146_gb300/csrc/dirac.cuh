@@ -49,8 +49,9 @@ __device__ __forceinline__ void su3_mul_half(const Link<R>& u, const cplx<R> h[6
             cplx<R> acc = czero<R>();
 #pragma unroll
             for (int b = 0; b < 3; ++b) {
-                if (dag) acc += cmulc(u.e[b * 3 + a], h[s * 3 + b]);
-                else     acc += u.e[a * 3 + b] * h[s * 3 + b];
+                if (b == 0) acc = dag ? cmulc(u.e[a], h[s * 3]) : u.e[a * 3] * h[s * 3];
+                else if (dag) cmacc(acc, u.e[b * 3 + a], h[s * 3 + b]);
+                else cmac(acc, u.e[a * 3 + b], h[s * 3 + b]);
             }
             o[s * 3 + a] = acc;
         }
@@ -122,7 +123,7 @@ __device__ __forceinline__ void hop_accumulate_dir(const Spinor<R>& psi, const L
         for (int a = 0; a < 3; ++a) {
             cplx<R> accv = czero<R>();
 #pragma unroll
-            for (int b = 0; b < 3; ++b) accv += e[a * 3 + b] * h[s * 3 + b];
+            for (int b = 0; b < 3; ++b) cmac(accv, e[a * 3 + b], h[s * 3 + b]);
             o[s * 3 + a] = accv;
         }
     }
@@ -138,67 +139,62 @@ __device__ __forceinline__ void hop_accumulate_dir(const Spinor<R>& psi, const L
     }
 }
 
-// y = A x for the two packed Hermitian 6x6 chirality blocks (diagonal reals,
-// then the upper triangle as (re, im) pairs in herm_off order)
+// y = (off-diagonal part of A) x for one packed Hermitian 6x6 block (diagonal
+// reals, then the upper triangle as (re, im) pairs in herm_off order).  The
+// diagonal term, the largest of a row, is added last (clover_diag), so that the
+// partial sums before it are small and round less.
+template <typename R>
+__device__ __forceinline__ void herm_off_apply(const R* a, const cplx<R>* xs, cplx<R>* ys) {
+#pragma unroll
+    for (int i = 0; i < 6; ++i) {
+#pragma unroll
+        for (int j = i + 1; j < 6; ++j) {
+            const int o = herm_off(i, j);
+            const cplx<R> aij = mk<R>(a[o], a[o + 1]);
+            if (i == 0 && j == 1) ys[0] = aij * xs[1];
+            else cmac(ys[i], aij, xs[j]);
+            if (i == 0) ys[j] = cmulc(aij, xs[0]);
+            else cmacc(ys[j], aij, xs[i]);
+        }
+    }
+}
+
+// y = A x for the two packed blocks of a site
 template <typename R>
 __device__ __forceinline__ void clover_apply_regs(const R* a0, const Spinor<R>& x, Spinor<R>& y) {
 #pragma unroll
     for (int chi = 0; chi < 2; ++chi) {
-        const R* a = a0 + 36 * chi;
-        const cplx<R>* xs = x.c + 6 * chi;
-        cplx<R>* ys = y.c + 6 * chi;
-#pragma unroll
-        for (int i = 0; i < 6; ++i) ys[i] = a[i] * xs[i];
+        herm_off_apply<R>(a0 + 36 * chi, x.c + 6 * chi, y.c + 6 * chi);
 #pragma unroll
         for (int i = 0; i < 6; ++i) {
-#pragma unroll
-            for (int j = i + 1; j < 6; ++j) {
-                const int o = herm_off(i, j);
-                cplx<R> aij = mk<R>(a[o], a[o + 1]);
-                ys[i] += aij * xs[j];
-                ys[j] += cmulc(aij, xs[i]);
-            }
+            const R d = a0[36 * chi + i];
+            cplx<R>& v = y.c[6 * chi + i];
+            v.x = fma(d, x.c[6 * chi + i].x, v.x);
+            v.y = fma(d, x.c[6 * chi + i].y, v.y);
         }
     }
 }
 
 template <typename R>
 __device__ __forceinline__ void clover_apply(const R* __restrict__ A, const Spinor<R>& x, Spinor<R>& y) {
-    // the 72 reals of the site (288 B in FP32, 576 B in FP64; 16-byte aligned)
-    // in 16-byte loads
+    // the 72 reals of the site in 16-byte loads (288 B in FP32, 576 B in FP64)
+    R ar[72];
     if constexpr (sizeof(R) == 4) {
-        R ar[72];
         const float4* q = reinterpret_cast<const float4*>(A);
 #pragma unroll
         for (int k = 0; k < 18; ++k) {
             const float4 v = __ldg(q + k);
             ar[4 * k] = v.x; ar[4 * k + 1] = v.y; ar[4 * k + 2] = v.z; ar[4 * k + 3] = v.w;
         }
-        clover_apply_regs<R>(ar, x, y);
     } else {
-        // FP64: (re, im) pairs on demand (all pairs start at even offsets)
+        const double2* q = reinterpret_cast<const double2*>(A);
 #pragma unroll
-        for (int chi = 0; chi < 2; ++chi) {
-            const double2* q = reinterpret_cast<const double2*>(A + 36 * chi);
-            const cplx<R>* xs = x.c + 6 * chi;
-            cplx<R>* ys = y.c + 6 * chi;
-#pragma unroll
-            for (int i = 0; i < 3; ++i) {
-                const double2 d = __ldg(q + i);
-                ys[2 * i] = d.x * xs[2 * i];
-                ys[2 * i + 1] = d.y * xs[2 * i + 1];
-            }
-#pragma unroll
-            for (int i = 0; i < 6; ++i) {
-#pragma unroll
-                for (int j = i + 1; j < 6; ++j) {
-                    const double2 aij = __ldg(q + herm_off(i, j) / 2);
-                    ys[i] += aij * xs[j];
-                    ys[j] += cmulc(aij, xs[i]);
-                }
-            }
+        for (int k = 0; k < 36; ++k) {
+            const double2 v = __ldg(q + k);
+            ar[2 * k] = v.x; ar[2 * k + 1] = v.y;
         }
     }
+    clover_apply_regs<R>(ar, x, y);
 }
 
 // Same product with the packed blocks in shared memory.

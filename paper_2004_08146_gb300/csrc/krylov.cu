@@ -171,7 +171,7 @@ __device__ __forceinline__ void coarse_row(const CoarseArgs<Z, R>& a, const Z* x
         }
         const Z* am = a.A + (((size_t)s * 9 + d) * a.nc) * a.nc + r;
         const Z* xs = xj + (size_t)sn * a.nc;
-        for (int col = 0; col < a.nc; ++col) acc += am[(size_t)col * a.nc] * xs[col];
+        for (int col = 0; col < a.nc; ++col) cmac(acc, am[(size_t)col * a.nc], xs[col]);
     }
     const R sg = r < a.nc / 2 ? R(1) : R(-1);
     Z xv = xj[(size_t)s * a.nc + r];
@@ -285,8 +285,7 @@ __global__ void __launch_bounds__(256) coarse_gmres_kernel(CoarseArgs<Z, R> a) {
                 const Z* ya = Y + (size_t)j * E;
                 for (int e = lane; e < len; e += 32) {
                     Z u = xa[e], v = ya[e];
-                    re[q] += u.x * v.x + u.y * v.y;
-                    im[q] += u.x * v.y - u.y * v.x;
+                    cdot(re[q], im[q], u, v);
                 }
                 slot[q] = p < ni * nrhs ? p : (maxit + 1) * nrhs + j;
             }
@@ -310,7 +309,7 @@ __global__ void __launch_bounds__(256) coarse_gmres_kernel(CoarseArgs<Z, R> a) {
             const int j = t / len, e = t % len;
             if (!live[j]) continue;
             Z acc = ws[(size_t)j * E + e];
-            for (int i = 0; i < ni; ++i) acc -= hr[i * nrhs + j] * VS(i, j)[e];
+            for (int i = 0; i < ni; ++i) cmsub(acc, hr[i * nrhs + j], VS(i, j)[e]);
             ws[(size_t)j * E + e] = acc;
         }
     };
@@ -379,7 +378,7 @@ __global__ void __launch_bounds__(256) coarse_gmres_kernel(CoarseArgs<Z, R> a) {
                     const Z* am = As + (size_t)sl * 9 * nc * nc + r;
                     const Z* xs = xn + ((size_t)j * nsl + sl) * 9 * nc;
                     const int d0 = sub * span, d1 = min(9 * nc, d0 + span);
-                    for (int dc = d0; dc < d1; ++dc) acc += am[(size_t)dc * nc] * xs[dc];
+                    for (int dc = d0; dc < d1; ++dc) cmac(acc, am[(size_t)dc * nc], xs[dc]);
                 }
                 for (int o = tpr / 2; o > 0; o >>= 1) {
                     acc.x += __shfl_xor_sync(0xffffffffu, acc.x, o);
@@ -519,7 +518,7 @@ __global__ void __launch_bounds__(256) coarse_gmres_kernel(CoarseArgs<Z, R> a) {
         const int k = kd[j];
         const Z* y = reinterpret_cast<const Z*>(a.yv) + (size_t)j * maxit;
         Z o; o.x = 0; o.y = 0;
-        for (int i = 0; i < k; ++i) o += y[i] * VS(i, j)[e];
+        for (int i = 0; i < k; ++i) cmac(o, y[i], VS(i, j)[e]);
         a.x[(size_t)j * nco + lo + e] = o;
     }
 }

@@ -80,7 +80,7 @@ __global__ void build_P_kernel(Geom g, Blocking B, int nv, const double2* __rest
                 double2 h = make_double2(0, 0);
                 for (int d = threadIdx.x; d < nloc; d += blockDim.x) h += cmulc(pj[d], pi[d]);
                 h = block_sum2(h, red);
-                for (int d = threadIdx.x; d < nloc; d += blockDim.x) pi[d] -= h * pj[d];
+                for (int d = threadIdx.x; d < nloc; d += blockDim.x) cmsub(pi[d], h, pj[d]);
                 __syncthreads();
             }
             double2 nn = make_double2(0, 0);
@@ -125,8 +125,7 @@ __global__ void restrict_kernel(Geom g, Blocking B, int nv, const Z* __restrict_
                     const int j = j0 + q;
                     if (j >= nrhs || (act != nullptr && !act[j])) continue;
                     const Z b = r[(size_t)j * fstride + off];
-                    re[q] += a.x * b.x + a.y * b.y;
-                    im[q] += a.x * b.y - a.y * b.x;
+                    cdot(re[q], im[q], a, b);
                 }
             }
 #pragma unroll
@@ -185,8 +184,7 @@ __global__ void __launch_bounds__(256) restrict_agg_kernel(Geom g, Blocking B, i
 #pragma unroll
             for (int q = 0; q < RC; ++q) {
                 const Z b = rs[(size_t)q * nloc + d];
-                re[q] += a.x * b.x + a.y * b.y;
-                im[q] += a.x * b.y - a.y * b.x;
+                cdot(re[q], im[q], a, b);
             }
         }
 #pragma unroll
@@ -235,7 +233,7 @@ __global__ void prolong_kernel(Geom g, Blocking B, int nv, const Z* __restrict__
                 const Z pi = p[(size_t)i * nloc];
 #pragma unroll
                 for (int q = 0; q < kProlongRC; ++q)
-                    if (j0 + q < nrhs) acc[q] += pi * c0[(size_t)(j0 + q) * cstride + i];
+                    if (j0 + q < nrhs) cmac(acc[q], pi, c0[(size_t)(j0 + q) * cstride + i]);
             }
 #pragma unroll
             for (int q = 0; q < kProlongRC; ++q) {
@@ -363,8 +361,7 @@ __global__ void __launch_bounds__(256) build_coarse_kernel(Geom g, Blocking B, i
             for (int q = lane; q < na * 6; q += 32) {
                 const int a = q / 6, sc = q % 6;
                 const cplx<R> pv = pr[lst[a] * 6 + sc], hv = h[a * 12 + sc];
-                re += pv.x * hv.x + pv.y * hv.y;
-                im += pv.x * hv.y - pv.y * hv.x;
+                cdot(re, im, pv, hv);
             }
             re = warp_sum(re);
             im = warp_sum(im);
@@ -447,7 +444,7 @@ __global__ void coarse_apply_mrhs_kernel(Geom gc, int nc, const Z* __restrict__ 
             const Z a = __ldg(Ad + (size_t)col * nc);
             const Z* xv = xd + (size_t)col * rc;
 #pragma unroll
-            for (int k = 0; k < kCoarseRPT; ++k) acc[k] += a * xv[k];
+            for (int k = 0; k < kCoarseRPT; ++k) cmac(acc[k], a, xv[k]);
         }
     }
     const R sg = r < nc / 2 ? R(1) : R(-1);
@@ -926,7 +923,7 @@ __global__ void sap_block_kernel(Geom g, Blocking B, const cplx<R>* __restrict__
             h = block_sum2(h, red);
             const cplx<R> hr = mk<R>((R)h.x, (R)h.y);
 #pragma unroll
-            for (int k = 0; k < 12; ++k) w.c[k] -= hr * vi[k];
+            for (int k = 0; k < 12; ++k) cmsub(w.c[k], hr, vi[k]);
             if (l == 0) H[i * iters + jj] = h;
         }
         double2 hn2 = make_double2(0, 0);
@@ -988,7 +985,7 @@ __global__ void sap_block_kernel(Geom g, Blocking B, const cplx<R>* __restrict__
         const cplx<R> yi = mk<R>((R)yv[i].x, (R)yv[i].y);
         const cplx<R>* vi = kv + (size_t)i * bs * 12 + (size_t)l * 12;
 #pragma unroll
-        for (int k = 0; k < 12; ++k) e.c[k] += yi * vi[k];
+        for (int k = 0; k < 12; ++k) cmac(e.c[k], yi, vi[k]);
     }
     store_spinor<R>(x + (size_t)y * 12, e);
 }
@@ -1183,15 +1180,13 @@ __global__ void __launch_bounds__(32) sap_warp_kernel(Geom g, Blocking B, const 
             R hr = 0, hi = 0;
 #pragma unroll
             for (int k = 0; k < 12; ++k) {
-                cplx<R> a = vi[k];
-                hr += a.x * acc.c[k].x + a.y * acc.c[k].y;
-                hi += a.x * acc.c[k].y - a.y * acc.c[k].x;
+                cdot(hr, hi, vi[k], acc.c[k]);
             }
             hr = seg_sum<BS>(hr);
             hi = seg_sum<BS>(hi);
             const cplx<R> h = mk<R>(hr, hi);
 #pragma unroll
-            for (int k = 0; k < 12; ++k) acc.c[k] -= h * vi[k];
+            for (int k = 0; k < 12; ++k) cmsub(acc.c[k], h, vi[k]);
             if (l == 0 && active) H[i * iters + jj] = mk<R>(hr, hi);
         }
         R hn2 = 0;
@@ -1250,7 +1245,7 @@ __global__ void __launch_bounds__(32) sap_warp_kernel(Geom g, Blocking B, const 
         const cplx<R> yi = yv[i];
         const cplx<R>* vi = basis + (size_t)i * BS * 12 + l * 12;
 #pragma unroll
-        for (int k = 0; k < 12; ++k) e.c[k] += yi * vi[k];
+        for (int k = 0; k < 12; ++k) cmac(e.c[k], yi, vi[k]);
     }
     store_spinor<R>(x + (size_t)y * 12, e);
 }
@@ -1382,8 +1377,8 @@ __global__ void __launch_bounds__(128) sap_chi_kernel(Geom g, Blocking B, const 
                 for (int jc = i + 1; jc < 6; ++jc) {
                     const int oo = herm_off(i, jc);
                     const cplx<R> aij = mk<R>(a[oo], a[oo + 1]);
-                    acc[i] += aij * psi[jc];
-                    acc[jc] += cmulc(aij, psi[i]);
+                    cmac(acc[i], aij, psi[jc]);
+                    cmacc(acc[jc], aij, psi[i]);
                 }
             }
         }
@@ -1411,7 +1406,7 @@ __global__ void __launch_bounds__(128) sap_chi_kernel(Geom g, Blocking B, const 
                 for (int a = 0; a < 3; ++a) {
                     cplx<R> v = czero<R>();
 #pragma unroll
-                    for (int b = 0; b < 3; ++b) v += (fw ? lk[a * 3 + b] : conj(lk[b * 3 + a])) * h[b];
+                    for (int b = 0; b < 3; ++b) cmac(v, fw ? lk[a * 3 + b] : conj(lk[b * 3 + a]), h[b]);
                     os[a] = has ? v : czero<R>();
                 }
                 cplx<R> ot[3];
@@ -1448,15 +1443,13 @@ __global__ void __launch_bounds__(128) sap_chi_kernel(Geom g, Blocking B, const 
             R hr = 0, hi = 0;
 #pragma unroll
             for (int k = 0; k < 6; ++k) {
-                const cplx<R> a = bload(vi + k);
-                hr += a.x * acc[k].x + a.y * acc[k].y;
-                hi += a.x * acc[k].y - a.y * acc[k].x;
+                cdot(hr, hi, bload(vi + k), acc[k]);
             }
             hr = warp_sum(hr);
             hi = warp_sum(hi);
             const cplx<R> h = mk<R>(hr, hi);
 #pragma unroll
-            for (int k = 0; k < 6; ++k) acc[k] -= h * bload(vi + k);
+            for (int k = 0; k < 6; ++k) cmsub(acc[k], h, bload(vi + k));
             if (lane == 0) H[i * iters + jj] = h;
         }
         R hn2 = 0;
@@ -1516,7 +1509,7 @@ __global__ void __launch_bounds__(128) sap_chi_kernel(Geom g, Blocking B, const 
         const cplx<R> yi = yv[i];
         const BT* vi = basis + (size_t)i * BS * 12 + l * 12 + 6 * chi;
 #pragma unroll
-        for (int k = 0; k < 6; ++k) e[k] += yi * bload(vi + k);
+        for (int k = 0; k < 6; ++k) cmac(e[k], yi, bload(vi + k));
     }
 #pragma unroll
     for (int k = 0; k < 6; ++k) x[(size_t)y * 12 + 6 * chi + k] = e[k];
