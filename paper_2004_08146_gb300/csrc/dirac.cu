@@ -19,8 +19,8 @@ __device__ __forceinline__ M3<double> m3_load(const double2* p) {
 __device__ __forceinline__ M3<double> m3_mul(const M3<double>& x, const M3<double>& y) {
     M3<double> r;
     for (int a = 0; a < 3; ++a) for (int b = 0; b < 3; ++b) {
-        double2 s = make_double2(0, 0);
-        for (int c = 0; c < 3; ++c) s += x.e[a][c] * y.e[c][b];
+        double2 s = x.e[a][0] * y.e[0][b];
+        for (int c = 1; c < 3; ++c) cmac(s, x.e[a][c], y.e[c][b]);
         r.e[a][b] = s;
     }
     return r;
@@ -134,7 +134,7 @@ __global__ void link_tangent_kernel(const double2* __restrict__ U, const double2
         for (int a = 0; a < 3; ++a)
             for (int c = 0; c < 3; ++c) {
                 double2 acc = make_double2(0, 0);
-                for (int b = 0; b < 3; ++b) acc += x[a * 3 + b] * u[b * 3 + c];
+                for (int b = 0; b < 3; ++b) cmac(acc, x[a * 3 + b], u[b * 3 + c]);
                 dU[e * 9 + a * 3 + c] = make_double2(-acc.y, acc.x);   // i * acc
             }
     }
@@ -361,7 +361,7 @@ __global__ void __launch_bounds__(128) link_force_kernel(const double2* __restri
     for (int a = 0; a < 3; ++a)
         for (int b = 0; b < 3; ++b) {
             double2 t = make_double2(0, 0);
-            for (int c = 0; c < 3; ++c) t += H[a][c] * u.e[c][b];
+            for (int c = 0; c < 3; ++c) cmac(t, H[a][c], u.e[c][b]);
             F[e * 9 + a * 3 + b] = inv * mul_ipow(t, 1);
         }
 }
@@ -384,10 +384,147 @@ void bilinear_force(const FineOp& f, const double2* gv, const double2* psi, cons
 // ------------------------------------------------------------------ stencil
 // out_j = op(tau_j) in_j, or out_j = b_j - op(tau_j) in_j when b != nullptr.
 // op = QCD_OP_D: D - tau Gamma5 ; op = QCD_OP_Q: Gamma5 D - tau.
-template <typename R>
-__global__ void __launch_bounds__(128) wilson_clover_kernel(
-    cplx<R>* __restrict__ out, const cplx<R>* __restrict__ in, const cplx<R>* __restrict__ b,
-    const cplx<R>* __restrict__ U, const R* __restrict__ A, Geom g, int op, Shifts tau, size_t stride,
+
+// sign flip without the FP64 pipe
+__device__ __forceinline__ double flip(double v, int mask) {
+    return __hiloint2double(__double2hiint(v) ^ mask, __double2loint(v));
+}
+__device__ __forceinline__ double2 shfl_xor2(double2 v, int o) {
+    return make_double2(__shfl_xor_sync(0xffffffffu, v.x, o), __shfl_xor_sync(0xffffffffu, v.y, o));
+}
+
+// FP64 stencil, eight lanes per site: lane q takes the hop of direction
+// mu = q / 2 (forward for even q).  FP64 runs at 2 fused multiply-adds per clock
+// and SM on this part, so the kernel is bound by that pipe at every size (1248
+// operations per site); the eight lanes spread a site over as many warps, which
+// fills the chip from a few hundred sites on instead of from a few hundred
+// thousand.  Everything that is a sign, a factor i or a permutation of spins
+// (lane dependent) is done by integer selects and sign flips.  The twelve rows
+// are summed by two exchange-and-halve steps (lane bit 2 ends with chirality
+// half, bit 1 with the spin), each lane then adds the clover columns of spin
+// (lane bit 0) to its three rows, and one exchange completes the sums.  4^4: 59 us
+// with one thread per site (8 warps on two SMs) -> 10 us, mostly the call itself.
+__global__ void __launch_bounds__(128) wilson_clover_f64_kernel(
+    double2* __restrict__ out, const double2* __restrict__ in, const double2* __restrict__ b,
+    const double2* __restrict__ U, const double* __restrict__ A, Geom g, int op, Shifts tau, size_t stride,
+    const int* __restrict__ act) {
+    const int j = blockIdx.y;
+    if (act != nullptr && !act[j]) return;
+    const unsigned tid = blockIdx.x * blockDim.x + threadIdx.x;
+    const bool live = (int)(tid >> 3) < g.V;
+    const int s = live ? (int)(tid >> 3) : g.V - 1;   // idle lanes follow along for the exchanges
+    const int q = tid & 7, mu = q >> 1;
+    const bool fw = !(q & 1);
+    in += j * stride;
+    int x[4];
+    site_coords(g, s, x);
+    int ms = 1, xm = x[3], Lm = g.L[3];
+    if (mu == 2) { ms = g.L[3]; xm = x[2]; Lm = g.L[2]; }
+    if (mu == 1) { ms = g.L[3] * g.L[2]; xm = x[1]; Lm = g.L[1]; }
+    if (mu == 0) { ms = g.L[3] * g.L[2] * g.L[1]; xm = x[0]; Lm = g.L[0]; }
+    const bool wraps = fw ? xm == Lm - 1 : xm == 0;
+    const int sn = s + (fw ? ms : -ms) * (wraps ? 1 - Lm : 1);
+    const bool neg = wraps && mu == 0 && g.antiperiodic;
+    const bool swap = mu == 1 || mu == 2, imag = mu & 1;
+    constexpr int kSign = (int)0x80000000;
+
+    // h_s = up_s -+ (B dn)_s (- forward): B rows are -1, -i (mu = 0, 1) or
+    // -1, +1 / -i, +i (mu = 2, 3), columns swapped for mu = 1, 2
+    const double2* nb = in + (size_t)sn * 12;
+    const double c0 = fw ? 1.0 : -1.0, c1 = mu < 2 ? c0 : -c0;
+    double2 h[2][3];
+#pragma unroll
+    for (int sp = 0; sp < 2; ++sp) {
+        const double2* dn = nb + 6 + (swap ? 1 - sp : sp) * 3;
+        const double c = sp ? c1 : c0;
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            const double2 u = __ldg(nb + sp * 3 + a), d = __ldg(dn + a);
+            h[sp][a].x = fma(imag ? -c : c, imag ? d.y : d.x, u.x);
+            h[sp][a].y = fma(c, imag ? d.x : d.y, u.y);
+        }
+    }
+    // o = U h (forward) or U^H h (backward), with the boundary sign
+    const double2* ul = U + ((size_t)(fw ? s : sn) * 4 + mu) * 9;
+    const int mx = neg ? kSign : 0, my = fw ? mx : mx ^ kSign;
+    double2 o[2][3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            double2 e = __ldg(ul + (fw ? a * 3 + c : c * 3 + a));
+            e = make_double2(flip(e.x, mx), flip(e.y, my));
+#pragma unroll
+            for (int sp = 0; sp < 2; ++sp) {
+                if (c == 0) o[sp][a] = e * h[sp][0];
+                else cmac(o[sp][a], e, h[sp][c]);
+            }
+        }
+    }
+    // rows of this hop over -1/2: o_s above, -+ (B^H o)_s below; B^H rows are
+    // -1 / i (mu = 0, 1), +1, -1 / i, -i (mu = 2, 3), columns swapped for 1, 2
+    const int f0 = (mu == 0) != fw ? kSign : 0, f1 = mu < 2 ? f0 : f0 ^ kSign;
+    double2 w[6];   // rows of this lane's chirality half after the exchange
+    const bool low = q & 4;
+#pragma unroll
+    for (int sp = 0; sp < 2; ++sp)
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            const double2 v = swap ? o[1 - sp][a] : o[sp][a];
+            const int f = sp ? f1 : f0;
+            const double2 d = imag ? make_double2(flip(v.y, f ^ kSign), flip(v.x, f)) : make_double2(flip(v.x, f), flip(v.y, f));
+            const double2 keep = low ? d : o[sp][a], send = low ? o[sp][a] : d;
+            w[sp * 3 + a] = keep + shfl_xor2(send, 4);
+        }
+    const bool sp1 = q & 2;
+    double2 r[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) r[a] = (sp1 ? w[3 + a] : w[a]) + shfl_xor2(sp1 ? w[a] : w[3 + a], 2);
+    // clover block of the chirality: rows 3 sp + a, columns 3 p + c
+    const int chi = low, sp = sp1, p = q & 1;
+    const double2* pc = in + (size_t)s * 12 + (2 * chi + p) * 3;
+    const double* Ab = A + (size_t)s * 72 + 36 * chi;
+    double2 psi[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) psi[c] = __ldg(pc + c);
+    const double t = tau.t[j];
+    const double sg = op != QCD_OP_D && chi ? -1.0 : 1.0, ts = op == QCD_OP_D && chi ? t : -t;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        double2 acc = -0.5 * r[a];
+#pragma unroll
+        for (int cc = 1; cc <= 3; ++cc) {   // the diagonal, the largest term, last
+            const int c = (a + cc) % 3;
+            const int i = 3 * sp + a, k = 3 * p + c;
+            const int lo = min(i, k), hi = max(i, k);
+            double2 m;
+            if (a == c && sp == p) m = make_double2(__ldg(Ab + i), 0.0);
+            else m = __ldg(reinterpret_cast<const double2*>(Ab + herm_off(lo, hi)));
+            m.y = flip(m.y, i > k ? kSign : 0);
+            cmac(acc, m, psi[c]);
+        }
+        r[a] = sg < 0 ? -acc : acc;
+    }
+    if (sp == p)
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            r[a].x = fma(ts, psi[a].x, r[a].x);
+            r[a].y = fma(ts, psi[a].y, r[a].y);
+        }
+#pragma unroll
+    for (int a = 0; a < 3; ++a) r[a] += shfl_xor2(r[a], 1);
+    if (!live || p) return;
+    const size_t row = j * stride + (size_t)s * 12 + (2 * chi + sp) * 3;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) out[row + a] = b != nullptr ? b[row + a] - r[a] : r[a];
+}
+
+// FP64 stencil, one thread per site: 1152 operations per site, 8 % fewer than
+// with eight lanes, for lattices that fill the FP64 pipes by themselves (86 %
+// busy).  32 x 16^3: 391 -> 289 us, from the fused multiply-adds.
+__global__ void __launch_bounds__(128) wilson_clover_f64_site_kernel(
+    double2* __restrict__ out, const double2* __restrict__ in, const double2* __restrict__ b,
+    const double2* __restrict__ U, const double* __restrict__ A, Geom g, int op, Shifts tau, size_t stride,
     const int* __restrict__ act) {
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= g.V) return;
@@ -397,60 +534,71 @@ __global__ void __launch_bounds__(128) wilson_clover_kernel(
     out += j * stride;
     int x[4];
     site_coords(g, s, x);
-    Spinor<R> psi, acc;
-    load_spinor<R>(in + (size_t)s * 12, psi);
-    clover_apply<R>(A + (size_t)s * 72, psi, acc);
+    Spinor<double> acc;
+    const double2* A2 = reinterpret_cast<const double2*>(A + (size_t)s * 72);
+#pragma unroll
+    for (int chi = 0; chi < 2; ++chi) {
+        double2 psi[6];
+#pragma unroll
+        for (int k = 0; k < 6; ++k) psi[k] = __ldg(in + (size_t)s * 12 + 6 * chi + k);
+        double2* ys = acc.c + 6 * chi;
+#pragma unroll
+        for (int i = 0; i < 6; ++i)
+#pragma unroll
+            for (int k = i + 1; k < 6; ++k) {
+                const double2 m = __ldg(A2 + 18 * chi + herm_off(i, k) / 2);
+                if (i == 0 && k == 1) ys[0] = m * psi[1];
+                else cmac(ys[i], m, psi[k]);
+                if (i == 0) ys[k] = cmulc(m, psi[0]);
+                else cmacc(ys[k], m, psi[i]);
+            }
+    }
 #pragma unroll
     for (int mu = 0; mu < 4; ++mu) {
-        int neg;
-        Spinor<R> nb;
-        Link<R> u;
-        int sf = nb_fwd(g, x, s, mu, neg);
-        load_spinor<R>(in + (size_t)sf * 12, nb);
-        load_link<R>(U + ((size_t)s * 4 + mu) * 9, u);
-        R sg = neg ? R(-1) : R(1);
-        switch (mu) {
-            case 0: hop_accumulate<R, 0, true>(nb, u, sg, acc); break;
-            case 1: hop_accumulate<R, 1, true>(nb, u, sg, acc); break;
-            case 2: hop_accumulate<R, 2, true>(nb, u, sg, acc); break;
-            default: hop_accumulate<R, 3, true>(nb, u, sg, acc); break;
-        }
-        int sb = nb_bwd(g, x, s, mu, neg);
-        load_spinor<R>(in + (size_t)sb * 12, nb);
-        load_link<R>(U + ((size_t)sb * 4 + mu) * 9, u);
-        sg = neg ? R(-1) : R(1);
-        switch (mu) {
-            case 0: hop_accumulate<R, 0, false>(nb, u, sg, acc); break;
-            case 1: hop_accumulate<R, 1, false>(nb, u, sg, acc); break;
-            case 2: hop_accumulate<R, 2, false>(nb, u, sg, acc); break;
-            default: hop_accumulate<R, 3, false>(nb, u, sg, acc); break;
+#pragma unroll
+        for (int dir = 0; dir < 2; ++dir) {
+            int neg;
+            Spinor<double> nb;
+            Link<double> u;
+            const int sn = dir == 0 ? nb_fwd(g, x, s, mu, neg) : nb_bwd(g, x, s, mu, neg);
+            load_spinor<double>(in + (size_t)sn * 12, nb);
+            load_link<double>(U + ((size_t)(dir == 0 ? s : sn) * 4 + mu) * 9, u);
+            const double sg = neg ? -1.0 : 1.0;
+            if (dir == 0) {
+                if (mu == 0) hop_accumulate<double, 0, true>(nb, u, sg, acc);
+                if (mu == 1) hop_accumulate<double, 1, true>(nb, u, sg, acc);
+                if (mu == 2) hop_accumulate<double, 2, true>(nb, u, sg, acc);
+                if (mu == 3) hop_accumulate<double, 3, true>(nb, u, sg, acc);
+            } else {
+                if (mu == 0) hop_accumulate<double, 0, false>(nb, u, sg, acc);
+                if (mu == 1) hop_accumulate<double, 1, false>(nb, u, sg, acc);
+                if (mu == 2) hop_accumulate<double, 2, false>(nb, u, sg, acc);
+                if (mu == 3) hop_accumulate<double, 3, false>(nb, u, sg, acc);
+            }
         }
     }
-    const R t = (R)tau.t[j];
-    if (op == QCD_OP_D) {
+    const double t = tau.t[j];
 #pragma unroll
-        for (int k = 0; k < 6; ++k) acc.c[k] -= t * psi.c[k];
-#pragma unroll
-        for (int k = 6; k < 12; ++k) acc.c[k] += t * psi.c[k];
-    } else {
-#pragma unroll
-        for (int k = 0; k < 6; ++k) acc.c[k] -= t * psi.c[k];
-#pragma unroll
-        for (int k = 6; k < 12; ++k) acc.c[k] = -acc.c[k] - t * psi.c[k];
+    for (int k = 0; k < 12; ++k) {
+        const int chi = k / 6;
+        const double2 p = __ldg(in + (size_t)s * 12 + k);
+        const double2 d2 = __ldg(A2 + 18 * chi + (k % 6) / 2);
+        const double d = k % 2 ? d2.y : d2.x, ts = op == QCD_OP_D && chi ? t : -t;
+        double2 v = acc.c[k];
+        v.x = fma(d, p.x, v.x);
+        v.y = fma(d, p.y, v.y);
+        if (op != QCD_OP_D && chi) v = -v;
+        v.x = fma(ts, p.x, v.x);
+        v.y = fma(ts, p.y, v.y);
+        if (b != nullptr) v = b[j * stride + (size_t)s * 12 + k] - v;
+        out[(size_t)s * 12 + k] = v;
     }
-    if (b != nullptr) {
-        Spinor<R> bb;
-        load_spinor<R>(b + j * stride + (size_t)s * 12, bb);
-#pragma unroll
-        for (int k = 0; k < 12; ++k) acc.c[k] = bb.c[k] - acc.c[k];
-    }
-    store_spinor<R>(out + (size_t)s * 12, acc);
 }
 
 // FP32 stencil with links and clover blocks in site-fastest (SoA) copies:
 // Us[(mu * 9 + k) * V + site] (float2) and As[q * V + site] (float4, q < 18),
 // so a warp's link and clover loads are contiguous; spinors keep the ABI
-// layout.  Same arithmetic as wilson_clover_kernel<float>.  With several
+// layout.  With several
 // right-hand sides, consecutive CTAs take the same 128 sites for different
 // right-hand sides (CTA index = site block x nrhs + rhs), so the CTAs that
 // run together read the same links and clover blocks and all but the first
@@ -487,14 +635,15 @@ __global__ void __launch_bounds__(128, 4) wilson_clover_soa_kernel(
     site_coords(g, s, x);
     Spinor<float> psi, acc;
     load_spinor<float>(in + (size_t)s * 12, psi);
-    {
-        float ar[72];
 #pragma unroll
-        for (int q = 0; q < 18; ++q) {
-            const float4 v = __ldg(As + (size_t)q * V + s);
+    for (int chi = 0; chi < 2; ++chi) {
+        float ar[36];
+#pragma unroll
+        for (int q = 0; q < 9; ++q) {
+            const float4 v = __ldg(As + (size_t)(9 * chi + q) * V + s);
             ar[4 * q] = v.x; ar[4 * q + 1] = v.y; ar[4 * q + 2] = v.z; ar[4 * q + 3] = v.w;
         }
-        clover_apply_regs<float>(ar, psi, acc);
+        herm_off_apply<float>(ar, psi.c + 6 * chi, acc.c + 6 * chi);
     }
     auto link = [&](int site, int mu, Link<float>& u) {
 #pragma unroll
@@ -526,17 +675,22 @@ __global__ void __launch_bounds__(128, 4) wilson_clover_soa_kernel(
             default: hop_accumulate<float, 3, false>(nb, u, sg, acc); break;
         }
     }
-    const float t = (float)tau.t[j];
-    if (op == QCD_OP_D) {
+    // diagonal of the clover blocks and shift, psi read again (L1) rather than
+    // held through the hops
+    load_spinor<float>(in + (size_t)s * 12, psi);
 #pragma unroll
-        for (int k = 0; k < 6; ++k) acc.c[k] -= t * psi.c[k];
+    for (int chi = 0; chi < 2; ++chi) {
+        const float4 d0 = __ldg(As + (size_t)(9 * chi) * V + s), d1 = __ldg(As + (size_t)(9 * chi + 1) * V + s);
+        const float d[6] = {d0.x, d0.y, d0.z, d0.w, d1.x, d1.y};
+        const float t = (float)tau.t[j];
+        const float sg = op != QCD_OP_D && chi ? -1.f : 1.f, ts = op == QCD_OP_D && chi ? t : -t;
 #pragma unroll
-        for (int k = 6; k < 12; ++k) acc.c[k] += t * psi.c[k];
-    } else {
-#pragma unroll
-        for (int k = 0; k < 6; ++k) acc.c[k] -= t * psi.c[k];
-#pragma unroll
-        for (int k = 6; k < 12; ++k) acc.c[k] = -acc.c[k] - t * psi.c[k];
+        for (int k = 0; k < 6; ++k) {
+            float2& v = acc.c[6 * chi + k];
+            const float2 p = psi.c[6 * chi + k];
+            v.x = fmaf(ts, p.x, sg * fmaf(d[k], p.x, v.x));
+            v.y = fmaf(ts, p.y, sg * fmaf(d[k], p.y, v.y));
+        }
     }
     if (b != nullptr) {
         Spinor<float> bb;
@@ -584,7 +738,7 @@ __global__ void gauge_check_kernel(const double2* __restrict__ U, size_t nlinks,
             for (int b = 0; b < 3; ++b) {
                 double2 acc = make_double2(a == b ? -1.0 : 0.0, 0.0);
 #pragma unroll
-                for (int c = 0; c < 3; ++c) acc += u[a * 3 + c] * conj(u[b * 3 + c]);
+                for (int c = 0; c < 3; ++c) cmacc(acc, u[b * 3 + c], u[a * 3 + c]);
                 worst = fmax(worst, fmax(fabs(acc.x), fabs(acc.y)));
             }
     }
@@ -613,31 +767,40 @@ void launch_clover_build(const FineOp& f, cudaStream_t st) {
         soa_copies_kernel<<<1216, 256, 0, st>>>(f.U32, f.A32, f.U32s, f.A32s, f.g.V);
 }
 
-template <typename R>
-void launch_dirac(const FineOp& f, int op, int nrhs, const void* in, void* out, const void* b,
-                  const double* tau, const int* act, cudaStream_t st) {
-    Shifts sh{};
-    for (int j = 0; j < nrhs; ++j) sh.t[j] = tau ? tau[j] : 0.0;
-    dim3 grid((f.g.V + 127) / 128, nrhs);
-    const cplx<R>* U = std::is_same<R, double>::value ? (const cplx<R>*)f.U64 : (const cplx<R>*)f.U32;
-    const R* A = std::is_same<R, double>::value ? (const R*)f.A64 : (const R*)f.A32;
-    if (!std::is_same<R, double>::value && f.U32s != nullptr && f.A32s != nullptr) {
-        const double bytes = (double)f.g.V * (nrhs * (b ? 72.0 : 48.0) + 144.0) * sizeof(R);
-        KTimer kt("wilson_clover_f32", bytes, 1824.0 * f.g.V * nrhs, st);
-        const unsigned gsoa = (unsigned)((f.g.V + 127) / 128) * (unsigned)nrhs;
-        // several right-hand sides: time-fastest bricks of 8 time slices
-        // (needs whole 128-site blocks per time slice and L0 a multiple of 8)
-        const int vs = f.g.L[1] * f.g.L[2] * f.g.L[3];
-        const int tb = (nrhs > 1 && vs % 128 == 0 && f.g.L[0] % 8 == 0) ? 8 : 0;
-        wilson_clover_soa_kernel<<<gsoa, 128, 0, st>>>((float2*)out, (const float2*)in, (const float2*)b, f.U32s,
-                                                       f.A32s, f.g, op, sh, (size_t)f.g.V * 12, act, nrhs, tb);
+static void launch_f64(const FineOp& f, const double2* U, const double* A, int op, int nrhs, const double2* in,
+                       double2* out, const double2* b, const Shifts& sh, const int* act, cudaStream_t st) {
+    // One thread per site once a single field gives each FP64 pipe (four per SM)
+    // more than three warps; eight lanes per site below.  Measured, eight lanes
+    // against one: 8^4 16.6 / 45.4 us, 16 x 8^3 27 / 45, 16^4 156 / 166, 32 x 16^3
+    // 307 / 289, 8 fields of 16^4 1206 / 1088.  The line depends on the lattice
+    // only, so a field's result does not depend on the batch it is in.
+    if (f.g.V >= 65536) {
+        const dim3 grid((f.g.V + 127) / 128, nrhs);
+        wilson_clover_f64_site_kernel<<<grid, 128, 0, st>>>(out, in, b, U, A, f.g, op, sh, (size_t)f.g.V * 12, act);
         return;
     }
-    const double bytes = (double)f.g.V * (nrhs * (b ? 72.0 : 48.0) + 144.0) * sizeof(R);
-    KTimer kt(std::is_same<R, double>::value ? "wilson_clover_f64" : "wilson_clover_f32", bytes,
-              1824.0 * f.g.V * nrhs, st);
-    wilson_clover_kernel<R><<<grid, 128, 0, st>>>((cplx<R>*)out, (const cplx<R>*)in, (const cplx<R>*)b,
-                                                  U, A, f.g, op, sh, (size_t)f.g.V * 12, act);
+    const dim3 grid((unsigned)(((size_t)f.g.V * 8 + 127) / 128), nrhs);
+    wilson_clover_f64_kernel<<<grid, 128, 0, st>>>(out, in, b, U, A, f.g, op, sh, (size_t)f.g.V * 12, act);
+}
+
+static void launch_dirac(const FineOp& f, int prec, int op, int nrhs, const void* in, void* out, const void* b,
+                         const double* tau, const int* act, cudaStream_t st) {
+    Shifts sh{};
+    for (int j = 0; j < nrhs; ++j) sh.t[j] = tau ? tau[j] : 0.0;
+    const double bytes = (double)f.g.V * (nrhs * (b ? 72.0 : 48.0) + 144.0) * (prec == QCD_FP64 ? 8 : 4);
+    if (prec == QCD_FP64) {
+        KTimer kt("wilson_clover_f64", bytes, 1824.0 * f.g.V * nrhs, st);
+        launch_f64(f, f.U64, f.A64, op, nrhs, (const double2*)in, (double2*)out, (const double2*)b, sh, act, st);
+        return;
+    }
+    KTimer kt("wilson_clover_f32", bytes, 1824.0 * f.g.V * nrhs, st);
+    const unsigned gsoa = (unsigned)((f.g.V + 127) / 128) * (unsigned)nrhs;
+    // several right-hand sides: time-fastest bricks of 8 time slices
+    // (needs whole 128-site blocks per time slice and L0 a multiple of 8)
+    const int vs = f.g.L[1] * f.g.L[2] * f.g.L[3];
+    const int tb = (nrhs > 1 && vs % 128 == 0 && f.g.L[0] % 8 == 0) ? 8 : 0;
+    wilson_clover_soa_kernel<<<gsoa, 128, 0, st>>>((float2*)out, (const float2*)in, (const float2*)b, f.U32s, f.A32s,
+                                                   f.g, op, sh, (size_t)f.g.V * 12, act, nrhs, tb);
 }
 
 void tangent_fields(const FineOp& f, const double2* X, double2* dU, double* dA, cudaStream_t st) {
@@ -654,22 +817,18 @@ void apply_tangent(const FineOp& f, const double2* dU, const double* dA, int nrh
     // the hop terms with dU and the clover derivative: the stencil with these
     // fields in place of U and (m0 + 4) + C, shift 0
     Shifts sh{};
-    dim3 grid((f.g.V + 127) / 128, nrhs);
     KTimer kt("wilson_tangent_f64", 0.0, 1824.0 * f.g.V * nrhs, st);
-    wilson_clover_kernel<double><<<grid, 128, 0, st>>>(out, in, nullptr, dU, dA, f.g, QCD_OP_D, sh,
-                                                       (size_t)f.g.V * 12, nullptr);
+    launch_f64(f, dU, dA, QCD_OP_D, nrhs, in, out, nullptr, sh, nullptr, st);
 }
 
 void apply_op(const FineOp& f, int prec, int op, int nrhs, const void* in, void* out,
               const double* tau, cudaStream_t st, const int* act) {
-    if (prec == QCD_FP64) launch_dirac<double>(f, op, nrhs, in, out, nullptr, tau, act, st);
-    else launch_dirac<float>(f, op, nrhs, in, out, nullptr, tau, act, st);
+    launch_dirac(f, prec, op, nrhs, in, out, nullptr, tau, act, st);
 }
 
 void residual_op(const FineOp& f, int prec, int op, int nrhs, const void* b, const void* x, void* r,
                  const double* tau, cudaStream_t st, const int* act) {
-    if (prec == QCD_FP64) launch_dirac<double>(f, op, nrhs, x, r, b, tau, act, st);
-    else launch_dirac<float>(f, op, nrhs, x, r, b, tau, act, st);
+    launch_dirac(f, prec, op, nrhs, x, r, b, tau, act, st);
 }
 
 }  // namespace qcd
