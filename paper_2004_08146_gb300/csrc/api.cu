@@ -605,7 +605,7 @@ void mg_cycle_impl(qcd_ctx* ctx, int prec, int op, int nrhs, const void* b, void
         };
         const int kmax = std::min(ctx->p.coarse_maxiter, kMaxKry);
         gmres_dev(ctx, prec, nco, nrhs, A1, &M1, rc, xc, ctx->p.coarse_tol, kmax, "kc1", act, 4);
-        mg_prolong(ctx->f, c, prec, nrhs, xc, x, false, ctx->st, act);
+        mg_prolong(ctx->f, c, prec, nrhs, xc, x, ctx->st, act);
         smooth(ctx, prec, op, nrhs, b, x, tau, act);
         check_launch("mg k-cycle");
         return;
@@ -640,7 +640,7 @@ void mg_cycle_impl(qcd_ctx* ctx, int prec, int op, int nrhs, const void* b, void
         };
         gmres_batched(ctx, prec, nco, nrhs, Ac, nullptr, rc, xc, ctx->p.coarse_tol, ctx->p.coarse_maxiter, "coarse");
     }
-    mg_prolong(ctx->f, c, prec, nrhs, xc, x, false, ctx->st, act);
+    mg_prolong(ctx->f, c, prec, nrhs, xc, x, ctx->st, act);
     smooth(ctx, prec, op, nrhs, b, x, tau, act);
     check_launch("mg cycle");
 }
@@ -1721,7 +1721,7 @@ int qcd_mg_prolong(qcd_ctx* ctx, int prec, int nrhs, const void* xc, void* x) {
     return guarded(ctx, [&]() {
         require_mg(ctx);
         if (nrhs < 1 || nrhs > kMaxRhs || !x || !xc) throw QcdError(QCD_EINVAL, "bad arguments");
-        mg_prolong(ctx->f, ctx->c, prec, nrhs, xc, x, false, ctx->st);
+        mg_prolong(ctx->f, ctx->c, prec, nrhs, xc, x, ctx->st);
         check_launch("prolong");
         return QCD_OK;
     });

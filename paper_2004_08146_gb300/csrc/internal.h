@@ -163,8 +163,8 @@ void mg_build_P(const FineOp& f, Coarse& c, const double2* vecs, int nvec, cudaS
 void mg_build_coarse(const FineOp& f, Coarse& c, cudaStream_t st, bool fp32_only = false);
 void mg_restrict(const FineOp& f, const Coarse& c, int prec, int nrhs, const void* r, void* xc, cudaStream_t st,
                  const int* act = nullptr);
-void mg_prolong(const FineOp& f, const Coarse& c, int prec, int nrhs, const void* xc, void* x, bool accumulate,
-                cudaStream_t st, const int* act = nullptr);
+void mg_prolong(const FineOp& f, const Coarse& c, int prec, int nrhs, const void* xc, void* x, cudaStream_t st,
+                const int* act = nullptr);
 // tensor: FP32 applies with 2 Nv a multiple of 8 run on the tensor cores
 // (3xTF32); otherwise, and for FP64, on the CUDA cores
 void coarse_apply(const Coarse& c, int prec, int op, int nrhs, const void* x, void* y, const double* tau,

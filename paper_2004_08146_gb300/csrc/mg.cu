@@ -96,153 +96,255 @@ __global__ void build_P_kernel(Geom g, Blocking B, int nv, const double2* __rest
 }
 
 // ------------------------------------------------------------------ restrict / prolong
-// One warp per (coarse site, chirality, vector i): <P_i, r_j> over the
-// aggregate for a chunk of up to kRestrictRC right-hand sides at a time, so
-// each entry of P is read once per chunk instead of once per right-hand side.
-constexpr int kRestrictRC = 8;
-template <typename Z, typename R>
-__global__ void restrict_kernel(Geom g, Blocking B, int nv, const Z* __restrict__ P, const Z* __restrict__ r,
-                                Z* __restrict__ xc, int nrhs, const int* __restrict__ act) {
-    const int nc = 2 * nv;
-    const int nloc = B.bs * 6;
-    const long total = (long)B.nb * nc;
-    const int lane = threadIdx.x & 31;
-    const size_t fstride = (size_t)g.V * 12;
-    for (long w = (blockIdx.x * (long)blockDim.x + threadIdx.x) >> 5; w < total; w += ((long)gridDim.x * blockDim.x) >> 5) {
-        const int blk = (int)(w / nc), ci = (int)(w % nc);
-        const int chi = ci / nv, i = ci % nv;
-        const Z* p = P + (((size_t)blk * 2 + chi) * nv + i) * nloc;
-        for (int j0 = 0; j0 < nrhs; j0 += kRestrictRC) {
-            R re[kRestrictRC], im[kRestrictRC];
+// E consecutive complex numbers loaded at once: two complex64 (16-byte aligned
+// fields), one complex64 (fields aligned to 8 bytes only) or one complex128
+template <typename R, int E> struct Piece;
+template <> struct Piece<float, 2> {
+    float4 v;
+    __device__ __forceinline__ float2 at(int k) const { return k ? make_float2(v.z, v.w) : make_float2(v.x, v.y); }
+};
+template <> struct Piece<float, 1> {
+    float2 v;
+    __device__ __forceinline__ float2 at(int) const { return v; }
+};
+template <> struct Piece<double, 1> {
+    double2 v;
+    __device__ __forceinline__ double2 at(int) const { return v; }
+};
+template <typename R, int E> __device__ __forceinline__ Piece<R, E> load_piece(const cplx<R>* p) {
+    Piece<R, E> o;
+    o.v = __ldg(reinterpret_cast<const decltype(o.v)*>(p));
+    return o;
+}
+
+// copy of one piece to shared memory behind the loads of other stages; take =
+// false writes zeros
+template <typename R, int E> __device__ __forceinline__ void async_piece(Piece<R, E>* dst, const cplx<R>* src, bool take) {
+    const uint32_t d = static_cast<uint32_t>(__cvta_generic_to_shared(dst));
+    constexpr int n = sizeof(Piece<R, E>);
+    const int bytes = take ? n : 0;
+    if constexpr (n == 16)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(bytes) : "memory");
+    else
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(d), "l"(src), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N> __device__ __forceinline__ void async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+
+// Sum of N values per lane over the warp, halving what a lane holds at each
+// step: afterwards v[0 .. max(N / 32, 1)) are the sums of the values from
+// `base` on.
+template <int N, int O, typename R>
+__device__ __forceinline__ void scatter_sum(R* v, int lane, int& base) {
+    if constexpr (O > 0) {
+        constexpr int n = N > 1 ? N / 2 : 1;
+        if constexpr (N > 1) {
+            const bool up = lane & O;
 #pragma unroll
-            for (int q = 0; q < kRestrictRC; ++q) { re[q] = 0; im[q] = 0; }
-            for (int d = lane; d < nloc; d += 32) {
-                const int l = d / 6, sc = d % 6;
-                const size_t off = (size_t)block_fine_site(g, B, blk, l) * 12 + 6 * chi + sc;
-                const Z a = p[d];
-#pragma unroll
-                for (int q = 0; q < kRestrictRC; ++q) {
-                    const int j = j0 + q;
-                    if (j >= nrhs || (act != nullptr && !act[j])) continue;
-                    const Z b = r[(size_t)j * fstride + off];
-                    cdot(re[q], im[q], a, b);
-                }
+            for (int k = 0; k < n; ++k) {
+                const R send = up ? v[k] : v[k + n], keep = up ? v[k + n] : v[k];
+                v[k] = keep + __shfl_xor_sync(0xffffffffu, send, O);
             }
-#pragma unroll
-            for (int q = 0; q < kRestrictRC; ++q) {
-                re[q] = warp_sum(re[q]);
-                im[q] = warp_sum(im[q]);
-            }
-            if (lane == 0)
-#pragma unroll
-                for (int q = 0; q < kRestrictRC; ++q) {
-                    const int j = j0 + q;
-                    if (j >= nrhs || (act != nullptr && !act[j])) continue;
-                    Z o; o.x = re[q]; o.y = im[q];
-                    xc[(size_t)j * B.nb * nc + (size_t)blk * nc + ci] = o;
-                }
+            if (up) base += n;
+        } else {
+            v[0] += __shfl_xor_sync(0xffffffffu, v[0], O);
         }
+        scatter_sum<n, O / 2>(v, lane, base);
     }
 }
 
-// One CTA per (aggregate, chirality, chunk of RC right-hand sides): the
-// aggregate's half of each fine vector (nloc = 6 x block sites entries) is
-// gathered into shared memory once ([rhs][d], conflict-free for consecutive
-// d), then the warps take the nv vectors P_i in turn, so every fine entry is
-// read from memory once and every entry of P once per chunk.
-template <typename Z, typename R, int RC>
-__global__ void __launch_bounds__(256) restrict_agg_kernel(Geom g, Blocking B, int nv, const Z* __restrict__ P,
-                                                           const Z* __restrict__ r, Z* __restrict__ xc, int nrhs,
-                                                           const int* __restrict__ act) {
+// x_c = P^H r: per (aggregate, chirality) the product of the nv x nloc rows of P
+// with the nloc x nrhs fine entries (nloc = 6 x aggregate sites).  A warp owns a
+// 4 x TJ tile of results, its lanes run along nloc in pieces of E entries (P rows
+// and the 48 bytes of a site's chirality half are contiguous), so 4 + TJ loads
+// feed 4 TJ products per entry, and the lanes are summed once at the end.  The
+// warps of a CTA cover all tiles of the aggregate and up to kTransferRhs
+// right-hand sides: P and r come from memory once, kStage pieces of every row per
+// stage, through a ring of kRing stages of asynchronous copies (loading into
+// registers kept one stage, 18 KB per SM, in flight and ran at 1.6 TB/s).
+// 32 x 16^3, 4^4 aggregates, nv 20, 16 right-hand sides: 786 us with
+// one chunk of 8 per pass and one warp per vector -> 143 us (3.2 TB/s, 47 % of the
+// FMA pipe; prologue of a single resident CTA per SM not hidden).
+template <typename R> constexpr int kTransferRhs = sizeof(R) == 4 ? 16 : 8;
+constexpr int kRestrictTI = 4;
+constexpr int kRing = 4, kStage = 64;
+constexpr int kSiteTable = 1024;   // aggregates up to this size look their entries up
+template <typename R, int E, int TJ>
+__global__ void __launch_bounds__(TJ == 4 ? 640 : 512) restrict_tile_kernel(
+    Geom g, Blocking B, int nv, const cplx<R>* __restrict__ P, const cplx<R>* __restrict__ r, cplx<R>* __restrict__ xc,
+    int nrhs, int ring, const int* __restrict__ act) {
+    constexpr int TI = kRestrictTI;
+    using Pc = Piece<R, E>;
     extern __shared__ __align__(16) unsigned char rsm[];
-    Z* rs = reinterpret_cast<Z*>(rsm);   // [RC][nloc]
-    const int nc = 2 * nv;
-    const int nloc = B.bs * 6;
+    const int nc = 2 * nv, nloc = B.bs * 6, np = nloc / E;
+    const bool table = B.bs <= kSiteTable;
     const int blk = blockIdx.x >> 1, chi = blockIdx.x & 1;
-    const int j0 = blockIdx.y * RC;
+    const int jc = blockIdx.y * kTransferRhs<R>, nr = min(nrhs - jc, kTransferRhs<R>), rows = nv + nr;
+    Pc* stage = reinterpret_cast<Pc*>(rsm);                                       // [ring][rows][kStage]
+    int* entry = reinterpret_cast<int*>(stage + (size_t)ring * rows * kStage);    // fine entry of a piece
+    auto entry_of = [&](int e) { return block_fine_site(g, B, blk, e * E / 6) * 12 + e * E % 6 + 6 * chi; };
+    if (table) {
+        for (int e = threadIdx.x; e < np; e += blockDim.x) entry[e] = entry_of(e);
+        __syncthreads();
+    }
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     const size_t fstride = (size_t)g.V * 12;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarp = blockDim.x >> 5;
-    for (int e = tid; e < nloc * RC; e += blockDim.x) {
-        const int q = e / nloc, d = e % nloc, j = j0 + q;
-        Z v;
-        v.x = 0;
-        v.y = 0;
-        if (j < nrhs && (act == nullptr || act[j])) {
-            const int l = d / 6, sc = d % 6;
-            v = r[(size_t)j * fstride + (size_t)block_fine_site(g, B, blk, l) * 12 + 6 * chi + sc];
+    const cplx<R>* Pb = P + ((size_t)blk * 2 + chi) * nv * nloc;
+    const cplx<R>* rb = r + (size_t)jc * fstride;
+    const int nst = (np + kStage - 1) / kStage, slots = rows * kStage;
+    auto fill = [&](int st, int at) {   // one commit group per stage, empty past the last
+        if (st < nst) {
+#pragma unroll
+            for (int h = 0; h < kStage; h += 32) {
+                const int e = st * kStage + h + lane;
+                const bool in = e < np;
+                const int ee = in ? e : 0;
+                Pc* dst = stage + at + h + lane;
+                const cplx<R>* ps = Pb + ee * E;
+                const cplx<R>* rs = rb + (table ? entry[ee] : entry_of(ee));
+                int q = warp;
+                for (; q < nv; q += nw) async_piece<R, E>(dst + q * kStage, ps + (size_t)q * nloc, in);
+                for (; q < rows; q += nw) async_piece<R, E>(dst + q * kStage, rs + (size_t)(q - nv) * fstride, in);
+            }
         }
-        rs[(size_t)q * nloc + d] = v;
+        async_commit();
+    };
+#pragma unroll
+    for (int st = 0; st < kRing - 1; ++st) fill(st, st * slots);
+    const int nit = (nv + TI - 1) / TI;
+    const int i0 = (warp % nit) * TI, j0 = (warp / nit) * TJ;
+    R acc[TI * TJ * 2];
+#pragma unroll
+    for (int q = 0; q < TI * TJ * 2; ++q) acc[q] = R(0);
+    // rows past the last are read like the last and not written
+    int ra[TI], ru[TJ];
+#pragma unroll
+    for (int q = 0; q < TI; ++q) ra[q] = min(i0 + q, nv - 1) * kStage + lane;
+#pragma unroll
+    for (int u = 0; u < TJ; ++u) ru[u] = (nv + min(j0 + u, nr - 1)) * kStage + lane;
+    int cur = 0, next = (kRing - 1) * slots;
+    for (int st = 0; st < nst; ++st) {
+        async_wait<kRing - 2>();
+        __syncthreads();   // stage st has arrived for all, stage st - 1 is read
+        fill(st + kRing - 1, next);
+        next = cur;
+        const Pc* sp = stage + cur;
+        cur = cur + slots == kRing * slots ? 0 : cur + slots;
+#pragma unroll
+        for (int h = 0; h < kStage; h += 32) {
+            Pc a[TI];
+#pragma unroll
+            for (int q = 0; q < TI; ++q) a[q] = sp[ra[q] + h];
+#pragma unroll
+            for (int u = 0; u < TJ; ++u) {
+                const Pc b = sp[ru[u] + h];
+#pragma unroll
+                for (int k = 0; k < E; ++k)
+#pragma unroll
+                    for (int q = 0; q < TI; ++q)
+                        cdot(acc[(q * TJ + u) * 2], acc[(q * TJ + u) * 2 + 1], a[q].at(k), b.at(k));
+            }
+        }
+    }
+    constexpr int N = TI * TJ * 2, keep = N / 32 > 1 ? N / 32 : 1, dup = N < 32 ? 32 / N : 1;
+    int base = 0;
+    scatter_sum<N, 16>(acc, lane, base);
+    if (lane % dup) return;
+    R* out = reinterpret_cast<R*>(xc);
+#pragma unroll
+    for (int k = 0; k < keep; ++k) {
+        const int e = base + k, i = i0 + e / 2 / TJ, u = j0 + e / 2 % TJ, j = jc + u;
+        if (i < nv && u < nr && (act == nullptr || act[j]))
+            out[((size_t)j * B.nb * nc + (size_t)blk * nc + chi * nv + i) * 2 + e % 2] = acc[k];
+    }
+}
+
+// x = P x_c: a thread takes two pieces of E entries of an aggregate's fine
+// entries (a warp's pieces are whole sites) and TJ right-hand sides, whose
+// coarse entries are broadcast from shared memory ([chirality][i][rhs], the two
+// halves in different banks).  A broadcast costs as much shared-memory bandwidth
+// as any other load of its width, so the tile is 2 E x TJ instead of E x 2 TJ;
+// the CTAs of the other right-hand sides follow in launch order and find P in
+// L2.  P comes by asynchronous copies kAhead rows ahead into a ring that each
+// thread fills and reads for itself (no barrier).
+// 32 x 16^3, 4^4 aggregates, nv 20, 16 right-hand sides: 339 us ->
+// 145 us (3.1 TB/s, 46 % of the FMA pipe).
+constexpr int kAhead = 8;
+constexpr int kProlongT = 96;   // whole warps and whole sites: both pieces lie at the same place of a site
+template <typename R, int E, int TJ>
+__global__ void __launch_bounds__(kProlongT) prolong_tile_kernel(Geom g, Blocking B, int nv,
+                                                                 const cplx<R>* __restrict__ P,
+                                                                 const cplx<R>* __restrict__ xc, cplx<R>* __restrict__ x,
+                                                                 int nrhs, int parts, const int* __restrict__ act) {
+    constexpr int kPer = 12 / E, T = kProlongT, kStep = T / kPer;   // pieces per site, sites between the two pieces
+    static_assert(T % kPer == 0 && T % 32 == 0, "CTA of whole warps and whole sites");
+    using Pc = Piece<R, E>;
+    extern __shared__ __align__(16) unsigned char psm[];
+    Pc* ring = reinterpret_cast<Pc*>(psm) + threadIdx.x;   // [kAhead][2][T]
+    cplx<R>* cs = reinterpret_cast<cplx<R>*>(psm + sizeof(Pc) * kAhead * 2 * T);
+    const int nc = 2 * nv, nloc = B.bs * 6, half = nv * TJ + 2;
+    const int groups = (nrhs + TJ - 1) / TJ;
+    const int j0 = (blockIdx.x % groups) * TJ, part = (blockIdx.x / groups) % parts, blk = blockIdx.x / groups / parts;
+    const int l = 2 * part * kStep + threadIdx.x / kPer, w = threadIdx.x % kPer;
+    const int chi = w / (kPer / 2), s = (w % (kPer / 2)) * E;
+    const bool two = B.bs > kStep;   // otherwise the second piece repeats the first and is not stored
+    const cplx<R>* p = P + ((size_t)blk * 2 + chi) * nv * nloc + s;
+    auto fill = [&](int i) {
+        if (i < nv)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int lh = l + h * kStep;
+                const bool in = lh < B.bs;
+                if (h == 0 || two)
+                    async_piece<R, E>(ring + ((i % kAhead) * 2 + h) * T, p + (size_t)i * nloc + (in ? lh * 6 : 0), in);
+            }
+        async_commit();
+    };
+#pragma unroll
+    for (int i = 0; i < kAhead - 1; ++i) fill(i);
+    for (int e = threadIdx.x; e < nc * TJ; e += T) {
+        const int i = e % nc, u = e / nc;
+        cplx<R> v = czero<R>();
+        if (j0 + u < nrhs) v = xc[(size_t)(j0 + u) * B.nb * nc + (size_t)blk * nc + i];
+        cs[(i / nv) * half + (i % nv) * TJ + u] = v;
     }
     __syncthreads();
-    for (int i = warp; i < nv; i += nwarp) {
-        const Z* p = P + (((size_t)blk * 2 + chi) * nv + i) * nloc;
-        R re[RC], im[RC];
+    const cplx<R>* c = cs + chi * half;
+    cplx<R> acc[2][TJ][E];
 #pragma unroll
-        for (int q = 0; q < RC; ++q) { re[q] = 0; im[q] = 0; }
-        for (int d = lane; d < nloc; d += 32) {
-            const Z a = p[d];
+    for (int h = 0; h < 2; ++h)
 #pragma unroll
-            for (int q = 0; q < RC; ++q) {
-                const Z b = rs[(size_t)q * nloc + d];
-                cdot(re[q], im[q], a, b);
-            }
-        }
+        for (int u = 0; u < TJ; ++u)
 #pragma unroll
-        for (int q = 0; q < RC; ++q) {
-            re[q] = warp_sum(re[q]);
-            im[q] = warp_sum(im[q]);
-        }
-        if (lane == 0) {
+            for (int k = 0; k < E; ++k) acc[h][u][k] = czero<R>();
+    for (int i = 0; i < nv; ++i) {
+        async_wait<kAhead - 2>();
+        const Pc a0 = ring[(i % kAhead) * 2 * T], a1 = ring[((i % kAhead) * 2 + (two ? 1 : 0)) * T];
+        fill(i + kAhead - 1);
 #pragma unroll
-            for (int q = 0; q < RC; ++q) {
-                const int j = j0 + q;
-                if (j >= nrhs || (act != nullptr && !act[j])) continue;
-                Z o;
-                o.x = re[q];
-                o.y = im[q];
-                xc[(size_t)j * B.nb * nc + (size_t)blk * nc + chi * nv + i] = o;
+        for (int u = 0; u < TJ; ++u) {
+            const cplx<R> v = c[i * TJ + u];
+#pragma unroll
+            for (int k = 0; k < E; ++k) {
+                cmac(acc[0][u][k], a0.at(k), v);
+                cmac(acc[1][u][k], a1.at(k), v);
             }
         }
     }
-}
-
-// One thread per fine degree of freedom of an aggregate (coarse site,
-// chirality, local index d); the nv entries P_i[d] are read once per chunk of
-// kProlongRC right-hand sides.
-constexpr int kProlongRC = 4;
-template <typename Z>
-__global__ void prolong_kernel(Geom g, Blocking B, int nv, const Z* __restrict__ P, const Z* __restrict__ xc,
-                               Z* __restrict__ x, int nrhs, bool accumulate, const int* __restrict__ act) {
-    const int nc = 2 * nv;
-    const int nloc = B.bs * 6;
-    const size_t total = (size_t)B.nb * 2 * nloc;
-    const size_t fstride = (size_t)g.V * 12, cstride = (size_t)B.nb * nc;
-    for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < total; t += (size_t)gridDim.x * blockDim.x) {
-        const int blk = (int)(t / (2 * nloc));
-        const int chi = (int)((t / nloc) % 2);
-        const int d = (int)(t % nloc);
-        const Z* p = P + ((size_t)blk * 2 + chi) * nv * nloc + d;
-        const int l = d / 6, sc = d % 6;
-        const size_t idx = (size_t)block_fine_site(g, B, blk, l) * 12 + 6 * chi + sc;
-        const Z* c0 = xc + (size_t)blk * nc + chi * nv;
-        for (int j0 = 0; j0 < nrhs; j0 += kProlongRC) {
-            Z acc[kProlongRC];
 #pragma unroll
-            for (int q = 0; q < kProlongRC; ++q) { acc[q].x = 0; acc[q].y = 0; }
-            for (int i = 0; i < nv; ++i) {
-                const Z pi = p[(size_t)i * nloc];
+    for (int h = 0; h < 2; ++h) {
+        const int lh = l + h * kStep;
+        if (lh >= B.bs) continue;
+        cplx<R>* o = x + (size_t)block_fine_site(g, B, blk, lh) * 12 + 6 * chi + s;
 #pragma unroll
-                for (int q = 0; q < kProlongRC; ++q)
-                    if (j0 + q < nrhs) cmac(acc[q], pi, c0[(size_t)(j0 + q) * cstride + i]);
-            }
-#pragma unroll
-            for (int q = 0; q < kProlongRC; ++q) {
-                const int j = j0 + q;
-                if (j >= nrhs || (act != nullptr && !act[j])) continue;
-                Z o = acc[q];
-                if (accumulate) o += x[(size_t)j * fstride + idx];
-                x[(size_t)j * fstride + idx] = o;
-            }
+        for (int u = 0; u < TJ; ++u) {
+            const int j = j0 + u;
+            if (j >= nrhs || (act != nullptr && !act[j])) continue;
+            cplx<R>* q = o + (size_t)j * g.V * 12;
+            if constexpr (E == 2)
+                *reinterpret_cast<float4*>(q) = make_float4(acc[h][u][0].x, acc[h][u][0].y, acc[h][u][1].x, acc[h][u][1].y);
+            else
+                *q = acc[h][u][0];
         }
     }
 }
@@ -1558,58 +1660,70 @@ void mg_build_coarse(const FineOp& f, Coarse& c, cudaStream_t st, bool fp32_only
     c.a64_stale = false;
 }
 
-void mg_restrict(const FineOp& f, const Coarse& c, int prec, int nrhs, const void* r, void* xc, cudaStream_t st,
-                 const int* act) {
-    size_t warps = (size_t)c.B.nb * c.nc;
-    int grid = grid_for(warps * 32);
-    const double es = prec == QCD_FP64 ? 16.0 : 8.0;
-    const double nfine = (double)f.g.V * 12;
-    const double chunks = (nrhs + (prec == QCD_FP64 ? 3 : 7)) / (prec == QCD_FP64 ? 4 : 8);
-    KTimer kt(prec == QCD_FP64 ? "restrict_f64" : "restrict_f32",
-              es * (nfine * c.nv * chunks + nrhs * (nfine + (double)c.gc.V * c.nc)), 8.0 * nfine * c.nv * nrhs, st);
-    // aggregate kernel while one chunk of the gathered fine vectors fits
-    // in shared memory (8 FP32 / 4 FP64 right-hand sides per chunk)
-    const int nloc = c.B.bs * 6;
-    const size_t sm = (size_t)nloc * 8 * sizeof(float2);
-    if (sm <= 160 * 1024) {
-        const int rcs = prec == QCD_FP64 ? 4 : 8;
-        const dim3 ag(c.B.nb * 2, (nrhs + rcs - 1) / rcs);
-        if (prec == QCD_FP64) {
-            if (sm + 1024 > 48 * 1024)
-                cudaFuncSetAttribute(restrict_agg_kernel<double2, double, 4>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-            restrict_agg_kernel<double2, double, 4><<<ag, 256, sm, st>>>(f.g, c.B, c.nv, c.P64, (const double2*)r,
-                                                                        (double2*)xc, nrhs, act);
-        } else {
-            if (sm + 1024 > 48 * 1024)
-                cudaFuncSetAttribute(restrict_agg_kernel<float2, float, 8>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-            restrict_agg_kernel<float2, float, 8><<<ag, 256, sm, st>>>(f.g, c.B, c.nv, c.P32, (const float2*)r,
-                                                                      (float2*)xc, nrhs, act);
-        }
-        return;
-    }
-    if (prec == QCD_FP64)
-        restrict_kernel<double2, double><<<grid, 256, 0, st>>>(f.g, c.B, c.nv, c.P64, (const double2*)r, (double2*)xc, nrhs, act);
-    else
-        restrict_kernel<float2, float><<<grid, 256, 0, st>>>(f.g, c.B, c.nv, c.P32, (const float2*)r, (float2*)xc, nrhs, act);
+template <typename R, int E, int TJ>
+static void launch_restrict(const FineOp& f, const Coarse& c, int nrhs, const cplx<R>* P, const void* r, void* xc,
+                            cudaStream_t st, const int* act) {
+    const int chunk = std::min(nrhs, kTransferRhs<R>);
+    const int warps = (c.nv + kRestrictTI - 1) / kRestrictTI * ((chunk + TJ - 1) / TJ);
+    const dim3 grid(c.B.nb * 2, (nrhs + kTransferRhs<R> - 1) / kTransferRhs<R>);
+    const int ring = std::min(kRing, (c.B.bs * 6 / E + kStage - 1) / kStage);   // no more stages than there are
+    const size_t sm = (size_t)ring * (c.nv + chunk) * kStage * sizeof(Piece<R, E>) +
+                      (c.B.bs <= kSiteTable ? c.B.bs * 6 / E * sizeof(int) : 0);
+    if (sm > 48 * 1024)
+        cudaFuncSetAttribute(restrict_tile_kernel<R, E, TJ>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    restrict_tile_kernel<R, E, TJ><<<grid, 32 * warps, sm, st>>>(f.g, c.B, c.nv, P, (const cplx<R>*)r, (cplx<R>*)xc, nrhs,
+                                                                 ring, act);
+}
+template <typename R, int E, int TJ>
+static void launch_prolong(const FineOp& f, const Coarse& c, int nrhs, const cplx<R>* P, const void* xc, void* x,
+                           cudaStream_t st, const int* act) {
+    const int parts = (c.B.bs * 12 / E + 2 * kProlongT - 1) / (2 * kProlongT);
+    const unsigned grid = (unsigned)c.B.nb * parts * ((nrhs + TJ - 1) / TJ);
+    const size_t sm = sizeof(Piece<R, E>) * kAhead * 2 * kProlongT + 2 * (size_t)(c.nv * TJ + 2) * sizeof(cplx<R>);
+    prolong_tile_kernel<R, E, TJ><<<grid, kProlongT, sm, st>>>(f.g, c.B, c.nv, P, (const cplx<R>*)xc, (cplx<R>*)x, nrhs,
+                                                               parts, act);
 }
 
-void mg_prolong(const FineOp& f, const Coarse& c, int prec, int nrhs, const void* xc, void* x, bool accumulate,
-                cudaStream_t st, const int* act) {
-    size_t n = (size_t)c.B.nb * 2 * c.B.bs * 6;
+// tiles as wide as the right-hand sides fill, at most TJ
+template <typename R, int E, int TJ>
+static void restrict_width(const FineOp& f, const Coarse& c, int nrhs, const cplx<R>* P, const void* r, void* xc,
+                           cudaStream_t st, const int* act) {
+    if constexpr (TJ > 1)
+        if (2 * nrhs <= TJ || (TJ == 8 && c.nv <= 20)) return restrict_width<R, E, TJ / 2>(f, c, nrhs, P, r, xc, st, act);
+    launch_restrict<R, E, TJ>(f, c, nrhs, P, r, xc, st, act);
+}
+template <typename R, int E, int TJ>
+static void prolong_width(const FineOp& f, const Coarse& c, int nrhs, const cplx<R>* P, const void* xc, void* x,
+                          cudaStream_t st, const int* act) {
+    if constexpr (TJ > 1)
+        if (2 * nrhs <= TJ) return prolong_width<R, E, TJ / 2>(f, c, nrhs, P, xc, x, st, act);
+    launch_prolong<R, E, TJ>(f, c, nrhs, P, xc, x, st, act);
+}
+
+void mg_restrict(const FineOp& f, const Coarse& c, int prec, int nrhs, const void* r, void* xc, cudaStream_t st,
+                 const int* act) {
     const double es = prec == QCD_FP64 ? 16.0 : 8.0;
     const double nfine = (double)f.g.V * 12;
-    const double chunks = (nrhs + kProlongRC - 1) / kProlongRC;
-    KTimer kt(prec == QCD_FP64 ? "prolong_f64" : "prolong_f32",
-              es * (nfine * c.nv * chunks + nrhs * (nfine * (accumulate ? 2 : 1) + (double)c.gc.V * c.nc)),
+    const int per = prec == QCD_FP64 ? kTransferRhs<double> : kTransferRhs<float>;
+    KTimer kt(prec == QCD_FP64 ? "restrict_f64" : "restrict_f32",
+              es * (nfine * c.nv * ((nrhs + per - 1) / per) + nrhs * (nfine + (double)c.gc.V * c.nc)),
               8.0 * nfine * c.nv * nrhs, st);
-    if (prec == QCD_FP64)
-        prolong_kernel<double2><<<grid_for(n), 256, 0, st>>>(f.g, c.B, c.nv, c.P64, (const double2*)xc, (double2*)x, nrhs,
-                                                             accumulate, act);
-    else
-        prolong_kernel<float2><<<grid_for(n), 256, 0, st>>>(f.g, c.B, c.nv, c.P32, (const float2*)xc, (float2*)x, nrhs,
-                                                            accumulate, act);
+    if (prec == QCD_FP64) restrict_width<double, 1, 4>(f, c, nrhs, c.P64, r, xc, st, act);
+    else if ((uintptr_t)r & 15) restrict_width<float, 1, 8>(f, c, nrhs, c.P32, r, xc, st, act);
+    else restrict_width<float, 2, 8>(f, c, nrhs, c.P32, r, xc, st, act);
+}
+
+void mg_prolong(const FineOp& f, const Coarse& c, int prec, int nrhs, const void* xc, void* x, cudaStream_t st,
+                const int* act) {
+    const double es = prec == QCD_FP64 ? 16.0 : 8.0;
+    const double nfine = (double)f.g.V * 12;
+    const int per = prec == QCD_FP64 ? kTransferRhs<double> : kTransferRhs<float>;
+    KTimer kt(prec == QCD_FP64 ? "prolong_f64" : "prolong_f32",
+              es * (nfine * c.nv * ((nrhs + per - 1) / per) + nrhs * (nfine + (double)c.gc.V * c.nc)),
+              8.0 * nfine * c.nv * nrhs, st);
+    if (prec == QCD_FP64) prolong_width<double, 1, 4>(f, c, nrhs, c.P64, xc, x, st, act);
+    else if ((uintptr_t)x & 15) prolong_width<float, 1, 8>(f, c, nrhs, c.P32, xc, x, st, act);
+    else prolong_width<float, 2, 8>(f, c, nrhs, c.P32, xc, x, st, act);
 }
 
 void coarse_apply(const Coarse& c, int prec, int op, int nrhs, const void* x, void* y, const double* tau,
