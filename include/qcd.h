@@ -298,6 +298,13 @@ int qcd_eig_force(qcd_ctx* ctx, int nvec, const void* V, void* F);
  * pointers, grad not 0 or 1; nvec = 0 does nothing. */
 int qcd_bilinear_force(qcd_ctx* ctx, int nvec, const void* G, const void* Psi, int grad, void* F);
 
+/* The sum over k < nvec of the fields qcd_bilinear_force would give (one link
+ * field F, DEVICE complex128 [site][mu][3][3]): the link gradient of a batch.
+ * The field is linear in the outer products of psi_k and g_k, which are summed
+ * first, so the cost is close to that of one field.  nvec = 0 leaves F alone;
+ * otherwise as qcd_bilinear_force. */
+int qcd_bilinear_force_sum(qcd_ctx* ctx, int nvec, const void* G, const void* Psi, int grad, void* F);
+
 /* Local coherence lc(v) = ||Pi v|| / ||v|| (Sec. 3, the local coherence
  * measure) of nvec FP64 fine vectors V (DEVICE, complex128 [nvec][V*12],
  * 16-byte aligned) with respect to the current interpolation P; Pi = P P^H is

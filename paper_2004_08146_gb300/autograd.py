@@ -4,7 +4,7 @@ differentiable in the spinor fields and in the gauge links.
 Forward and backward run in the library: ``qcd_apply`` (Q - tau on a batch
 of fields) forwards; the spinor adjoint is the same operator (Q = Gamma5 D is
 Hermitian, Sec. 2, and tau is real), and the link adjoint is
-``qcd_bilinear_force``.  For a real loss L with cotangent g of the output,
+``qcd_bilinear_force_sum``.  For a real loss L with cotangent g of the output,
 dL = Re <g, (dQ) psi> along link moves U -> exp(i eps X) U (X traceless
 Hermitian); the links' gradient is the tangent field i F U with F the force
 of that bilinear form, summed over the batch, so that Re tr(grad^H dU)
@@ -52,9 +52,12 @@ class ShiftedQ(torch.autograd.Function):
             ctx.qctx.qcd_apply(qcd.QCD_OP_Q, qcd.QCD_FP64, ctx.nrhs, grad, g_psi, [ctx.tau] * ctx.nrhs)
         if ctx.links_shape is not None and ctx.needs_input_grad[1]:
             shape, device, dtype = ctx.links_shape
-            F = torch.empty(ctx.nrhs * ctx.V * 36, dtype=torch.complex128, device=grad.device)
-            ctx.qctx.qcd_bilinear_force(ctx.nrhs, grad, psi, 1, F)
-            g_links = F.view(ctx.nrhs, -1).sum(dim=0).view(shape).to(device=device, dtype=dtype)
+            # the library sums the batch before its plaquette products; a
+            # stand-in context without that call gives the fields one by one
+            summed = getattr(ctx.qctx, "qcd_bilinear_force_sum", None)
+            F = torch.empty((1 if summed else ctx.nrhs) * ctx.V * 36, dtype=torch.complex128, device=grad.device)
+            (summed or ctx.qctx.qcd_bilinear_force)(ctx.nrhs, grad, psi, 1, F)
+            g_links = (F if summed else F.view(ctx.nrhs, -1).sum(dim=0)).view(shape).to(device=device, dtype=dtype)
         return g_psi, g_links, None, None, None
 
 

@@ -1684,20 +1684,21 @@ int qcd_eig_force(qcd_ctx* ctx, int nvec, const void* V, void* F) {
         check_align(F, "F");
         const FineOp& f = ctx->f;
         const size_t n = ctx->nfine(), nl = (size_t)f.g.V * 36;
-        double2* Bt = (double2*)ctx->buf("force.Bt", (size_t)f.g.V * 54 * sizeof(double2));
+        void* scratch = ctx->buf("force", force_scratch(f));
         double2* nrm = (double2*)ctx->buf("force.nrm", sizeof(double2));
         double2* part = (double2*)ctx->buf("force.part", (size_t)64 * sizeof(double2));
         for (int j = 0; j < nvec; ++j) {
             const double2* v = (const double2*)V + (size_t)j * n;
             blas_multidot(QCD_FP64, v, 1, n, v, 1, n, nrm, part, ctx->dot_counters(1), ctx->st);
-            eig_force(f, v, nrm, Bt, (double2*)F + (size_t)j * nl, ctx->st);
+            bilinear_force(f, 1, v, v, nrm, 0, scratch, (double2*)F + (size_t)j * nl, ctx->st);
         }
         check_launch("eig force");
         return QCD_OK;
     });
 }
 
-int qcd_bilinear_force(qcd_ctx* ctx, int nvec, const void* G, const void* Psi, int grad, void* F) {
+// the nvec forces one by one (F has nvec link fields), or their sum (one)
+static int bilinear_force_call(qcd_ctx* ctx, int nvec, const void* G, const void* Psi, int grad, void* F, bool sum) {
     return guarded(ctx, [&]() {
         require_gauge(ctx);
         if (nvec < 0 || (nvec > 0 && (!G || !Psi || !F)) || (grad != 0 && grad != 1))
@@ -1708,13 +1709,21 @@ int qcd_bilinear_force(qcd_ctx* ctx, int nvec, const void* G, const void* Psi, i
         check_align(F, "F");
         const FineOp& f = ctx->f;
         const size_t n = ctx->nfine(), nl = (size_t)f.g.V * 36;
-        double2* Bt = (double2*)ctx->buf("force.Bt", (size_t)f.g.V * 54 * sizeof(double2));
-        for (int j = 0; j < nvec; ++j)
-            bilinear_force(f, (const double2*)G + (size_t)j * n, (const double2*)Psi + (size_t)j * n, nullptr, grad, Bt,
-                           (double2*)F + (size_t)j * nl, ctx->st);
+        void* scratch = ctx->buf("force", force_scratch(f));
+        for (int j = 0; j < (sum ? 1 : nvec); ++j)
+            bilinear_force(f, sum ? nvec : 1, (const double2*)G + (size_t)j * n, (const double2*)Psi + (size_t)j * n,
+                           nullptr, grad, scratch, (double2*)F + (size_t)j * nl, ctx->st);
         check_launch("bilinear force");
         return QCD_OK;
     });
+}
+
+int qcd_bilinear_force(qcd_ctx* ctx, int nvec, const void* G, const void* Psi, int grad, void* F) {
+    return bilinear_force_call(ctx, nvec, G, Psi, grad, F, false);
+}
+
+int qcd_bilinear_force_sum(qcd_ctx* ctx, int nvec, const void* G, const void* Psi, int grad, void* F) {
+    return bilinear_force_call(ctx, nvec, G, Psi, grad, F, true);
 }
 
 int qcd_mg_prolong(qcd_ctx* ctx, int prec, int nrhs, const void* xc, void* x) {

@@ -207,47 +207,81 @@ __global__ void clover_tangent_kernel(const double2* __restrict__ U, const doubl
 }
 
 // ------------------------------------------------------------------ force: the derivative per link
-// F_rho(y) traceless Hermitian with d lambda / d eps = sum tr(X_rho(y) F_rho(y))
-// for every direction field X (links moving as exp(i eps X) U).  With w =
-// Gamma5 v, the hop terms give K = -i U A with the colour outer product
-// A = sum_s ((1 - gamma_rho) v(y + rho))_s w_s(y)^H (the backward hop is its
-// complex conjugate), and the clover term gives, per plane (rho, nu),
-// (c_sw / 16) (below - above): the plaquettes above and below the link with the
-// insertion Bt = B + B^H, B = sum_st sigma_{rho nu, st} v_t w_s^H, placed at
-// each corner.  F is the traceless Hermitian part of K over v^H v.
+// F_rho(y) traceless Hermitian with d/d eps sum_k Re <g_k, Q psi_k> = sum
+// tr(X_rho(y) F_rho(y)) (links moving as exp(i eps X) U); for g = psi = v that is
+// the eigenvalue force times v^H v.  Q' is Hermitian, so the hop terms give
+// K = -i U A with the colour outer products A = sum_k (A(psi_k, g_k) +
+// A(g_k, psi_k)) / 2, A(a, b) = sum_s ((1 - gamma_rho) a(y + rho))_s (Gamma5
+// b)_s(y)^H, and the clover term gives, per plane (rho, nu), (c_sw / 16) (below -
+// above): the plaquettes above and below the link with the insertion Bt = B +
+// B^H, B = sum_k sum_st sigma_{rho nu, st} psi_t (Gamma5 g)_s^H, placed at each
+// corner.  F is the traceless Hermitian part of K.  Both outer products are
+// linear in the fields, so a sum over fields needs the plaquette products, 98 %
+// of the arithmetic, once.  Everything here is bound by the FP64 pipe (2 fused
+// multiply-adds per clock and SM): the kernels are written for the fewest
+// operations.  16^4, 8 fields: 8 x (6.54 + 0.82) ms with one thread per link and
+// field -> 2.8 ms (plaquettes 1.50, hops 0.80, insertions 0.37, links 0.16).
 
 __device__ __forceinline__ int plane_index(int mu, int nu) {   // mu < nu
     return mu == 0 ? nu - 1 : (mu == 1 ? nu + 1 : 5);
 }
+__device__ __forceinline__ double2 shfl2(double2 v, int o) {
+    return make_double2(__shfl_xor_sync(0xffffffffu, v.x, o), __shfl_xor_sync(0xffffffffu, v.y, o));
+}
 
-// Bt_{mu nu}(x) = B + B^H for the six planes mu < nu: [site][plane][3][3],
-// B = sum_{st} sigma_st psi_t(x) (Gamma5 gv)_s(x)^H.  sigma is block diagonal
-// in chirality and Gamma5 gv = +gv (spins 0, 1), -gv (spins 2, 3).
-__global__ void clover_insertion_kernel(const double2* __restrict__ psi, const double2* __restrict__ gv, Geom g,
-                                        double2* __restrict__ Bt) {
-    const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= g.V) return;
-    double2 p[12], q[12];
-    for (int k = 0; k < 12; ++k) {
-        p[k] = psi[(size_t)s * 12 + k];
-        q[k] = gv[(size_t)s * 12 + k];
+// Bt of the six planes mu < nu: [site][plane][3][3].  Eight lanes per site: lane
+// (chi, i, j) sums M = psi_j g_i^H of spins 2 chi + j, 2 chi + i over the fields.
+// With T_k = sum_ij (sigma_k)_ij M_ij per chirality, sigma^chi_{0k} = +-sigma_k
+// and sigma^chi_{jk} = -eps_jkl sigma_l, and Gamma5 g changes sign with chi, so
+// plane (0, k) is T^0_k + T^1_k and plane (j, k) is -eps_jkl (T^0_l - T^1_l): sums
+// and differences between lanes.
+__global__ void __launch_bounds__(128) clover_insertion_kernel(const double2* __restrict__ psi,
+                                                               const double2* __restrict__ gv, int nvec, Geom g,
+                                                               double2* __restrict__ Bt) {
+    const unsigned tid = blockIdx.x * blockDim.x + threadIdx.x;
+    const bool live = (int)(tid >> 3) < g.V;
+    const int s = live ? (int)(tid >> 3) : g.V - 1;
+    const int chi = (tid >> 2) & 1, i = (tid >> 1) & 1, j = tid & 1;
+    const size_t n = (size_t)g.V * 12;
+    const double2* p = psi + (size_t)s * 12 + (2 * chi + j) * 3;
+    const double2* q = gv + (size_t)s * 12 + (2 * chi + i) * 3;
+    double2 M[9];
+#pragma unroll
+    for (int k = 0; k < 9; ++k) M[k] = make_double2(0, 0);
+    for (int f = 0; f < nvec; ++f) {
+        double2 pv[3], qv[3];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            pv[c] = __ldg(p + f * n + c);
+            qv[c] = __ldg(q + f * n + c);
+        }
+#pragma unroll
+        for (int a = 0; a < 3; ++a)
+#pragma unroll
+            for (int b = 0; b < 3; ++b) cmacc(M[a * 3 + b], qv[b], pv[a]);
     }
-    for (int mu = 0; mu < 4; ++mu)
-        for (int nu = mu + 1; nu < 4; ++nu) {
-            double2 B[3][3];
-            for (int a = 0; a < 3; ++a) for (int b = 0; b < 3; ++b) B[a][b] = make_double2(0, 0);
-            for (int chi = 0; chi < 2; ++chi) {
-                double2 S[2][2];
-                sigma_block(mu, nu, chi, S);
-                const double sg = chi == 0 ? 1.0 : -1.0;
-                for (int i = 0; i < 2; ++i) for (int j = 0; j < 2; ++j) {
-                    const double2 c = sg * S[i][j];
-                    for (int a = 0; a < 3; ++a) for (int b = 0; b < 3; ++b)
-                        B[a][b] += c * (p[(2 * chi + j) * 3 + a] * conj(q[(2 * chi + i) * 3 + b]));
-                }
-            }
-            double2* o = Bt + ((size_t)s * 6 + plane_index(mu, nu)) * 9;
-            for (int a = 0; a < 3; ++a) for (int b = 0; b < 3; ++b) o[a * 3 + b] = B[a][b] + conj(B[b][a]);
+    // lanes (0,0): T_3 = M_00 - M_11; (0,1): T_1 = M_01 + M_10; (1,0): T_2 = -i M_01 + i M_10
+    // then over chi: lane chi = 0 the sum (plane 0 k), chi = 1 the difference (spatial plane)
+    const int k = i == j ? 3 : (j ? 1 : 2);
+#pragma unroll
+    for (int e = 0; e < 9; ++e) {
+        const double2 o = shfl2(M[e], 3);
+        if (k == 1) M[e] = M[e] + o;
+        else M[e] = M[e] - o;                               // (1,0): M_10 - M_01
+        if (k == 2) M[e] = make_double2(-M[e].y, M[e].x);   // times i
+        const double2 t = shfl2(M[e], 4);
+        M[e] = chi ? t - M[e] : M[e] + t;
+    }
+    if (!live || (i && j)) return;
+    const int plane = chi ? 6 - k : k - 1;
+    const bool minus = chi && k != 2;   // -eps: planes (1,2), (2,3) minus, (1,3) plus
+    double2* o = Bt + ((size_t)s * 6 + plane) * 9;
+#pragma unroll
+    for (int a = 0; a < 3; ++a)
+#pragma unroll
+        for (int b = 0; b < 3; ++b) {
+            const double2 v = M[a * 3 + b] + conj(M[b * 3 + a]);
+            o[a * 3 + b] = minus ? -v : v;
         }
 }
 
@@ -256,129 +290,230 @@ __device__ __forceinline__ M3<double> m3_add(const M3<double>& x, const M3<doubl
     for (int a = 0; a < 3; ++a) for (int b = 0; b < 3; ++b) r.e[a][b] = x.e[a][b] + y.e[a][b];
     return r;
 }
-
-// Forward-hop colour outer product A(a, b) = sum_{st} (I - gamma_rho)_{st}
-// a_t(x + rho) (Gamma5 b)_s(x)^H: h = up - B dn of the projected neighbour,
-// lower half -B^H h; A = sum_i h_i b_i^H + (B^H h)_i b_{2+i}^H (Gamma5 b
-// flips the lower sign).  sg: boundary phase of the hop.
-__device__ __forceinline__ M3<double> hop_outer(const double2* __restrict__ an, const double2* __restrict__ bs,
-                                                int rho, double sg) {
-    const SpinMono Bm = kB(rho), BHm = kBH(rho);
-    double2 h[2][3], q[2][3];
-    for (int i = 0; i < 2; ++i) for (int a = 0; a < 3; ++a)
-        h[i][a] = sg * (an[i * 3 + a] - mul_ipow(an[(2 + Bm.perm[i]) * 3 + a], Bm.ph[i]));
-    for (int i = 0; i < 2; ++i) for (int a = 0; a < 3; ++a) q[i][a] = mul_ipow(h[BHm.perm[i]][a], BHm.ph[i]);
-    M3<double> A;
-    for (int a = 0; a < 3; ++a) for (int b = 0; b < 3; ++b) {
-        double2 t = make_double2(0, 0);
-        for (int i = 0; i < 2; ++i) t += h[i][a] * conj(bs[i * 3 + b]) + q[i][a] * conj(bs[(2 + i) * 3 + b]);
-        A.e[a][b] = t;
-    }
-    return A;
+// z += x y
+__device__ __forceinline__ void m3_mac(M3<double>& z, const M3<double>& x, const M3<double>& y) {
+#pragma unroll
+    for (int a = 0; a < 3; ++a)
+#pragma unroll
+        for (int b = 0; b < 3; ++b)
+#pragma unroll
+            for (int c = 0; c < 3; ++c) cmac(z.e[a][b], x.e[a][c], y.e[c][b]);
+}
+__device__ __forceinline__ void m3_store(double2* p, const M3<double>& m) {
+#pragma unroll
+    for (int a = 0; a < 3; ++a)
+#pragma unroll
+        for (int b = 0; b < 3; ++b) p[a * 3 + b] = m.e[a][b];
 }
 
-// One thread per link (site, rho): the force of Re <gv, Q' psi> (for
-// psi = gv = v the eigenvalue force times v^H v).  Hop terms: Q' is
-// Hermitian, so the real part is carried by the two forward terms
-// -i/2 U (A(psi, gv) + A(gv, psi)); clover term through the insertions Bt.
-// nrm: device v^H v dividing the result, or null.  grad = 1 writes the link
-// gradient i F U instead of F.
-__global__ void __launch_bounds__(128) link_force_kernel(const double2* __restrict__ U, const double2* __restrict__ psi,
-                                                         const double2* __restrict__ gv, const double2* __restrict__ Bt,
-                                                         const double2* __restrict__ nrm, Geom g, double csw, int grad,
-                                                         double2* __restrict__ F) {
+// A += A(a, b) of direction rho: h = up - B dn of a(y + rho) (times the boundary
+// sign) against c_k = b_k + (B b_low)_k of b(y): the two halves of Gamma5 b meet
+// the same h, so they are added before the product.
+template <int rho>
+__device__ __forceinline__ void hop_outer(const double2* __restrict__ an, const double2* __restrict__ bs, double sg,
+                                          double2 (&A)[9]) {
+    constexpr SpinMono Bm = kB(rho), BHm = kBH(rho);
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        double2 h[3], c[3];
+        const int lo = BHm.perm[i];   // spin 2 + lo reads h_i with phase i^ph[lo]
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            h[a] = __ldg(an + i * 3 + a) - mul_ipow(__ldg(an + (2 + Bm.perm[i]) * 3 + a), Bm.ph[i]);
+            if (sg < 0) h[a] = -h[a];
+            c[a] = __ldg(bs + i * 3 + a) + mul_ipow(__ldg(bs + (2 + lo) * 3 + a), 4 - BHm.ph[lo]);
+        }
+#pragma unroll
+        for (int a = 0; a < 3; ++a)
+#pragma unroll
+            for (int b = 0; b < 3; ++b) cmacc(A[a * 3 + b], c[b], h[a]);
+    }
+}
+
+// Hop part K = -i U A of every link, summed over the fields; blockIdx.y = rho.
+template <int rho>
+__device__ __forceinline__ void hop_force(const double2* __restrict__ U, const double2* __restrict__ psi,
+                                          const double2* __restrict__ gv, int nvec, const Geom& g, int s,
+                                          double2* __restrict__ K) {
+    int x[4], neg;
+    site_coords(g, s, x);
+    const int sf = nb_fwd(g, x, s, rho, neg);
+    const double sg = neg ? -1.0 : 1.0;
+    const size_t n = (size_t)g.V * 12;
+    double2 A[9];
+#pragma unroll
+    for (int k = 0; k < 9; ++k) A[k] = make_double2(0, 0);
+    for (int f = 0; f < nvec; ++f) {
+        const double2 *p = psi + f * n, *q = gv + f * n;
+        hop_outer<rho>(p + (size_t)sf * 12, q + (size_t)s * 12, sg, A);
+        if (psi != gv) hop_outer<rho>(q + (size_t)sf * 12, p + (size_t)s * 12, sg, A);
+    }
+    const double c = psi != gv ? 0.5 : 1.0;
+    const size_t e = (size_t)s * 4 + rho;
+    M3<double> u = m3_load(U + e * 9), Am;
+    for (int a = 0; a < 3; ++a) for (int b = 0; b < 3; ++b) Am.e[a][b] = c * A[a * 3 + b];
+    const M3<double> UA = m3_mul(u, Am);
+    for (int a = 0; a < 3; ++a) for (int b = 0; b < 3; ++b) K[e * 9 + a * 3 + b] = mul_ipow(UA.e[a][b], 3);   // -i U A
+}
+__global__ void __launch_bounds__(128) hop_force_kernel(const double2* __restrict__ U, const double2* __restrict__ psi,
+                                                        const double2* __restrict__ gv, int nvec, Geom g,
+                                                        double2* __restrict__ K) {
+    const int s = blockIdx.x * blockDim.x + threadIdx.x;
+    if (s >= g.V) return;
+    switch (blockIdx.y) {
+        case 0: hop_force<0>(U, psi, gv, nvec, g, s, K); break;
+        case 1: hop_force<1>(U, psi, gv, nvec, g, s, K); break;
+        case 2: hop_force<2>(U, psi, gv, nvec, g, s, K); break;
+        default: hop_force<3>(U, psi, gv, nvec, g, s, K); break;
+    }
+}
+
+// One thread per plaquette (x; mu < nu) = a b (d c)^H with corners 0..3 at x,
+// x + mu, x + mu + nu, x + nu: the clover force on its four links.  With the
+// inserted half paths X = a B1 b and Y = d B3 c and the sums over the three
+// other insertions S1 = B2 W + Y^H + W B0 (W = (d c)^H), S2 = B0 E + X + E B2
+// (E = a b), every link's term closes with one or two products more, because
+// the Hermitian B make the sums of the reversed paths S1^H and S2^H:
+//   above a = X W + E S1           below c = (B3 d^H E + d^H S2) c^H
+//   above d = Y E^H + D S2^H       below b = (B1 a^H D + a^H S1^H) b^H
+// 20 products instead of the 36 of one thread per link.  W4: [plane][a, b, c,
+// d][site][3][3].
+__global__ void __launch_bounds__(128) plaquette_force_kernel(const double2* __restrict__ U,
+                                                              const double2* __restrict__ Bt, Geom g, int plane0,
+                                                              double2* __restrict__ W4) {
+    const int s = blockIdx.x * blockDim.x + threadIdx.x;
+    if (s >= g.V) return;
+    const int pl = plane0 + blockIdx.y;
+    const int mu = pl < 3 ? 0 : (pl < 5 ? 1 : 2), nu = pl < 3 ? pl + 1 : (pl < 5 ? pl - 1 : 3);
+    int x[4];
+    site_coords(g, s, x);
+    const int s1 = shifted(g, x, mu, 1, nu, 0), s3 = shifted(g, x, mu, 0, nu, 1), s2 = shifted(g, x, mu, 1, nu, 1);
+    auto link = [&](int site, int d) { return m3_load(U + ((size_t)site * 4 + d) * 9); };
+    auto ins = [&](int site) { return m3_load(Bt + ((size_t)site * 6 + pl) * 9); };
+    double2* out = W4 + (size_t)blockIdx.y * 4 * g.V * 9 + (size_t)s * 9;
+    const size_t step = (size_t)g.V * 9;
+    M3<double> E, D, X, Y;
+    M3<double> aB1, dB3;
+    {
+        const M3<double> a = link(s, mu), b = link(s1, nu);
+        E = m3_mul(a, b);
+        aB1 = m3_mul(a, ins(s1));
+        X = m3_mul(aB1, b);
+    }
+    {
+        const M3<double> d = link(s, nu), c = link(s3, mu);
+        D = m3_mul(d, c);
+        dB3 = m3_mul(d, ins(s3));
+        Y = m3_mul(dB3, c);
+    }
+    {
+        const M3<double> W = m3_dag(D);
+        M3<double> S1 = m3_dag(Y);
+        m3_mac(S1, ins(s2), W);
+        m3_mac(S1, W, ins(s));
+        M3<double> r = m3_mul(X, W);
+        m3_mac(r, E, S1);
+        m3_store(out, r);                                   // above a
+        M3<double> t = m3_mul(m3_dag(aB1), D);
+        m3_mac(t, m3_dag(link(s, mu)), m3_dag(S1));
+        m3_store(out + step, m3_mul(t, m3_dag(link(s1, nu))));        // below b
+    }
+    {
+        M3<double> S2 = X;
+        m3_mac(S2, ins(s), E);
+        m3_mac(S2, E, ins(s2));
+        M3<double> r = m3_mul(Y, m3_dag(E));
+        m3_mac(r, D, m3_dag(S2));
+        m3_store(out + 3 * step, r);                        // above d
+        M3<double> t = m3_mul(m3_dag(dB3), E);
+        m3_mac(t, m3_dag(link(s, nu)), S2);
+        m3_store(out + 2 * step, m3_mul(t, m3_dag(link(s3, mu))));    // below c
+    }
+}
+
+// One thread per link: adds the plaquette terms of planes plane0 .. plane0 +
+// nplanes - 1 to K (in F) and, with `last`, leaves F = traceless Hermitian part
+// (over nrm, device v^H v, unless null) or, with grad, the link gradient i F U.
+__global__ void __launch_bounds__(128) link_force_kernel(const double2* __restrict__ U, const double2* __restrict__ W4,
+                                                         const double2* __restrict__ nrm, Geom g, double csw, int plane0,
+                                                         int nplanes, int last, int grad, double2* __restrict__ F) {
     const size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
     if (e >= (size_t)g.V * 4) return;
     const int s = (int)(e >> 2), rho = (int)(e & 3);
     int x[4];
     site_coords(g, s, x);
-    auto L = [&](int site, int d) { return m3_load(U + ((size_t)site * 4 + d) * 9); };
-    const M3<double> u = L(s, rho);
-    M3<double> K;
-    {
-        int neg;
-        const int sf = nb_fwd(g, x, s, rho, neg);
-        const double sg = neg ? -1.0 : 1.0;
-        M3<double> A = hop_outer(psi + (size_t)sf * 12, gv + (size_t)s * 12, rho, sg);
-        if (psi != gv) {
-            const M3<double> A2 = hop_outer(gv + (size_t)sf * 12, psi + (size_t)s * 12, rho, sg);
-            for (int a = 0; a < 3; ++a) for (int b = 0; b < 3; ++b) A.e[a][b] = 0.5 * (A.e[a][b] + A2.e[a][b]);
+    M3<double> K = m3_load(F + e * 9);
+    const size_t step = (size_t)g.V * 9;
+    for (int o = 0; o < 4; ++o) {
+        if (o == rho || nplanes == 0) continue;
+        const int pl = (rho < o ? plane_index(rho, o) : plane_index(o, rho)) - plane0;
+        if (pl < 0 || pl >= nplanes) continue;
+        // the link is a of the plaquette above and c of the one below in planes
+        // (rho, o), d and b in planes (o, rho), where the insertion changes sign
+        const double c = (rho < o ? 1.0 : -1.0) * csw / 16.0;
+        const double2* up = W4 + (size_t)pl * 4 * step + (rho < o ? 0 : 3) * step + (size_t)s * 9;
+        const double2* dn = W4 + (size_t)pl * 4 * step + (rho < o ? 2 : 1) * step +
+                            (size_t)shifted(g, x, rho, 0, o, -1) * 9;
+#pragma unroll
+        for (int k = 0; k < 9; ++k) {
+            const double2 u = up[k], d = dn[k];
+            K.e[k / 3][k % 3] += c * (d - u);
         }
-        const M3<double> UA = m3_mul(u, A);
-        for (int a = 0; a < 3; ++a) for (int b = 0; b < 3; ++b) K.e[a][b] = mul_ipow(UA.e[a][b], 3);   // -i U A
     }
-    if (csw != 0.0) {
-        const double c = csw / 16.0;
-        for (int nu = 0; nu < 4; ++nu) {
-            if (nu == rho) continue;
-            const int pl = rho < nu ? plane_index(rho, nu) : plane_index(nu, rho);
-            const double sg = rho < nu ? c : -c;   // Bt_{rho nu} = -Bt_{nu rho}
-            auto Bx = [&](int site) { return m3_load(Bt + ((size_t)site * 6 + pl) * 9); };
-            // plaquette above: a b c d from y, corners y, y+rho, y+rho+nu, y+nu
-            M3<double> above;
-            {
-                const M3<double> b = L(shifted(g, x, rho, 1, nu, 0), nu);
-                const M3<double> cm = m3_dag(L(shifted(g, x, rho, 0, nu, 1), rho));
-                const M3<double> d = m3_dag(L(s, nu));
-                const M3<double> cd = m3_mul(cm, d);
-                const M3<double> t1 = m3_add(m3_mul(Bx(shifted(g, x, rho, 0, nu, 1)), d), m3_mul(d, Bx(s)));
-                const M3<double> t2 = m3_add(m3_mul(Bx(shifted(g, x, rho, 1, nu, 1)), cd), m3_mul(cm, t1));
-                const M3<double> t3 = m3_add(m3_mul(Bx(shifted(g, x, rho, 1, nu, 0)), m3_mul(b, cd)), m3_mul(b, t2));
-                above = m3_mul(u, t3);
-            }
-            // plaquette below: path y -> y-nu -> y-nu+rho -> y+rho, then U_rho(y)^H
-            M3<double> below;
-            {
-                const M3<double> dp = m3_dag(L(shifted(g, x, rho, 0, nu, -1), nu));
-                const M3<double> ap = L(shifted(g, x, rho, 0, nu, -1), rho);
-                const M3<double> bp = L(shifted(g, x, rho, 1, nu, -1), nu);
-                const M3<double> apbp = m3_mul(ap, bp);
-                const M3<double> t1 = m3_add(m3_mul(Bx(shifted(g, x, rho, 1, nu, -1)), bp),
-                                             m3_mul(bp, Bx(shifted(g, x, rho, 1, nu, 0))));
-                const M3<double> t2 = m3_add(m3_mul(Bx(shifted(g, x, rho, 0, nu, -1)), apbp), m3_mul(ap, t1));
-                const M3<double> pre = m3_add(m3_mul(Bx(s), m3_mul(dp, apbp)), m3_mul(dp, t2));
-                below = m3_mul(pre, m3_dag(u));
-            }
-            for (int a = 0; a < 3; ++a) for (int b = 0; b < 3; ++b)
-                K.e[a][b] += sg * (below.e[a][b] - above.e[a][b]);
-        }
+    if (!last) {
+        m3_store(F + e * 9, K);
+        return;
     }
     double inv = 1.0;
     if (nrm != nullptr) {
         const double n = nrm[0].x;
         inv = n > 0 ? 1.0 / n : 0.0;
     }
-    double2 H[3][3];
-    for (int a = 0; a < 3; ++a) for (int b = 0; b < 3; ++b) H[a][b] = 0.5 * (K.e[a][b] + conj(K.e[b][a]));
-    const double tr = (H[0][0].x + H[1][1].x + H[2][2].x) / 3.0;
-    for (int a = 0; a < 3; ++a) H[a][a].x -= tr;
-    if (!grad) {
-        for (int a = 0; a < 3; ++a) for (int b = 0; b < 3; ++b) F[e * 9 + a * 3 + b] = inv * H[a][b];
+    M3<double> H;
+    for (int a = 0; a < 3; ++a) for (int b = 0; b < 3; ++b) H.e[a][b] = 0.5 * (K.e[a][b] + conj(K.e[b][a]));
+    const double tr = (H.e[0][0].x + H.e[1][1].x + H.e[2][2].x) / 3.0;
+    for (int a = 0; a < 3; ++a) H.e[a][a].x -= tr;
+    // link gradient i F U: the tangent vector whose real inner product with any
+    // dU = i X U is tr(X F)
+    if (grad) H = m3_mul(H, m3_load(U + e * 9));
+    for (int a = 0; a < 3; ++a)
+        for (int b = 0; b < 3; ++b) F[e * 9 + a * 3 + b] = inv * (grad ? mul_ipow(H.e[a][b], 1) : H.e[a][b]);
+}
+
+// planes handled per launch: all six while their terms (3456 bytes per site)
+// stay below 1 GB, one at a time on larger lattices
+static int force_planes(const FineOp& f) { return f.csw == 0.0 ? 0 : (f.g.V <= 300000 ? 6 : 1); }
+size_t force_scratch(const FineOp& f) {
+    return f.csw == 0.0 ? 0 : ((size_t)54 + 36 * force_planes(f)) * f.g.V * sizeof(double2);
+}
+
+void bilinear_force(const FineOp& f, int nvec, const double2* gv, const double2* psi, const double2* nrm, int grad,
+                    void* scratch, double2* F, cudaStream_t st) {
+    double2* Bt = (double2*)scratch;
+    double2* W4 = Bt + (size_t)f.g.V * 54;
+    const unsigned sites = (f.g.V + 127) / 128, links = (unsigned)(((size_t)f.g.V * 4 + 127) / 128);
+    {
+        KTimer kt("hop_force", 0.0, 0.0, st);
+        hop_force_kernel<<<dim3(sites, 4), 128, 0, st>>>(f.U64, psi, gv, nvec, f.g, F);
+    }
+    const int np = force_planes(f);
+    if (np == 0) {
+        KTimer kt("link_force", 0.0, 0.0, st);
+        link_force_kernel<<<links, 128, 0, st>>>(f.U64, nullptr, nrm, f.g, 0.0, 0, 0, 1, grad, F);
         return;
     }
-    // link gradient i F U: the tangent vector whose real inner product with
-    // any dU = i X U is tr(X F)
-    for (int a = 0; a < 3; ++a)
-        for (int b = 0; b < 3; ++b) {
-            double2 t = make_double2(0, 0);
-            for (int c = 0; c < 3; ++c) cmac(t, H[a][c], u.e[c][b]);
-            F[e * 9 + a * 3 + b] = inv * mul_ipow(t, 1);
-        }
-}
-
-void eig_force(const FineOp& f, const double2* v, const double2* nrm, double2* Bt, double2* F, cudaStream_t st) {
-    bilinear_force(f, v, v, nrm, 0, Bt, F, st);
-}
-
-void bilinear_force(const FineOp& f, const double2* gv, const double2* psi, const double2* nrm, int grad, double2* Bt,
-                    double2* F, cudaStream_t st) {
     {
         KTimer kt("clover_insertion", 0.0, 0.0, st);
-        clover_insertion_kernel<<<(f.g.V + 127) / 128, 128, 0, st>>>(psi, gv, f.g, Bt);
+        clover_insertion_kernel<<<(unsigned)(((size_t)f.g.V * 8 + 127) / 128), 128, 0, st>>>(psi, gv, nvec, f.g, Bt);
     }
-    KTimer kt("link_force", 0.0, 0.0, st);
-    const size_t nl = (size_t)f.g.V * 4;
-    link_force_kernel<<<(unsigned)((nl + 127) / 128), 128, 0, st>>>(f.U64, psi, gv, Bt, nrm, f.g, f.csw, grad, F);
+    for (int p0 = 0; p0 < 6; p0 += np) {
+        {
+            KTimer kt("plaquette_force", 0.0, 0.0, st);
+            plaquette_force_kernel<<<dim3(sites, np), 128, 0, st>>>(f.U64, Bt, f.g, p0, W4);
+        }
+        KTimer kt("link_force", 0.0, 0.0, st);
+        link_force_kernel<<<links, 128, 0, st>>>(f.U64, W4, nrm, f.g, f.csw, p0, np, p0 + np >= 6, grad, F);
+    }
 }
 
 // ------------------------------------------------------------------ stencil
@@ -388,9 +523,6 @@ void bilinear_force(const FineOp& f, const double2* gv, const double2* psi, cons
 // sign flip without the FP64 pipe
 __device__ __forceinline__ double flip(double v, int mask) {
     return __hiloint2double(__double2hiint(v) ^ mask, __double2loint(v));
-}
-__device__ __forceinline__ double2 shfl_xor2(double2 v, int o) {
-    return make_double2(__shfl_xor_sync(0xffffffffu, v.x, o), __shfl_xor_sync(0xffffffffu, v.y, o));
 }
 
 // FP64 stencil, eight lanes per site: lane q takes the hop of direction
@@ -474,12 +606,12 @@ __global__ void __launch_bounds__(128) wilson_clover_f64_kernel(
             const int f = sp ? f1 : f0;
             const double2 d = imag ? make_double2(flip(v.y, f ^ kSign), flip(v.x, f)) : make_double2(flip(v.x, f), flip(v.y, f));
             const double2 keep = low ? d : o[sp][a], send = low ? o[sp][a] : d;
-            w[sp * 3 + a] = keep + shfl_xor2(send, 4);
+            w[sp * 3 + a] = keep + shfl2(send, 4);
         }
     const bool sp1 = q & 2;
     double2 r[3];
 #pragma unroll
-    for (int a = 0; a < 3; ++a) r[a] = (sp1 ? w[3 + a] : w[a]) + shfl_xor2(sp1 ? w[a] : w[3 + a], 2);
+    for (int a = 0; a < 3; ++a) r[a] = (sp1 ? w[3 + a] : w[a]) + shfl2(sp1 ? w[a] : w[3 + a], 2);
     // clover block of the chirality: rows 3 sp + a, columns 3 p + c
     const int chi = low, sp = sp1, p = q & 1;
     const double2* pc = in + (size_t)s * 12 + (2 * chi + p) * 3;
@@ -512,7 +644,7 @@ __global__ void __launch_bounds__(128) wilson_clover_f64_kernel(
             r[a].y = fma(ts, psi[a].y, r[a].y);
         }
 #pragma unroll
-    for (int a = 0; a < 3; ++a) r[a] += shfl_xor2(r[a], 1);
+    for (int a = 0; a < 3; ++a) r[a] += shfl2(r[a], 1);
     if (!live || p) return;
     const size_t row = j * stride + (size_t)s * 12 + (2 * chi + sp) * 3;
 #pragma unroll

@@ -102,13 +102,12 @@ double gauge_unitarity_deviation(const double2* U, size_t nlinks, unsigned long 
 void tangent_fields(const FineOp& f, const double2* X, double2* dU, double* dA, cudaStream_t st);
 void apply_tangent(const FineOp& f, const double2* dU, const double* dA, int nrhs, const double2* in, double2* out,
                    cudaStream_t st);
-// Per-link force of the eigenvalue v^H Q v / v^H v: insertion fields Bt
-// ([V][6][9]) then F ([V][4][9], traceless Hermitian); nrm: device v^H v.
-void eig_force(const FineOp& f, const double2* v, const double2* nrm, double2* Bt, double2* F, cudaStream_t st);
-// Force of Re <gv, Q' psi> per link (F [V][4][9], traceless Hermitian), or
-// with grad = 1 the link gradient i F U; nrm (device, may be null) divides.
-void bilinear_force(const FineOp& f, const double2* gv, const double2* psi, const double2* nrm, int grad, double2* Bt,
-                    double2* F, cudaStream_t st);
+// Force of sum_k Re <gv_k, Q' psi_k> per link (F [V][4][9], traceless
+// Hermitian; nvec consecutive fields each), or with grad = 1 the link gradient
+// i F U; nrm (device, may be null) divides.  scratch: force_scratch bytes.
+size_t force_scratch(const FineOp& f);
+void bilinear_force(const FineOp& f, int nvec, const double2* gv, const double2* psi, const double2* nrm, int grad,
+                    void* scratch, double2* F, cudaStream_t st);
 void apply_op(const FineOp& f, int prec, int op, int nrhs, const void* in, void* out,
               const double* tau, cudaStream_t st, const int* act = nullptr);
 void residual_op(const FineOp& f, int prec, int op, int nrhs, const void* b, const void* x, void* r,

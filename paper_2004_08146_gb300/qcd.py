@@ -112,6 +112,7 @@ _SIGS = {
     "qcd_eig_derivative": (_I, [_P, _DP, _I, _P, _DP]),
     "qcd_eig_force": (_I, [_P, _I, _P, _P]),
     "qcd_bilinear_force": (_I, [_P, _I, _P, _P, _I, _P]),
+    "qcd_bilinear_force_sum": (_I, [_P, _I, _P, _P, _I, _P]),
     "qcd_coarse_apply": (_I, [_P, _I, _I, _I, _P, _P, _DP]),
     "qcd_mg_get_P": (_I, [_P, _DP]),
     "qcd_mg_get_coarse": (_I, [_P, _DP]),
@@ -305,6 +306,9 @@ class Context:
 
     def qcd_bilinear_force(self, nvec, G, Psi, grad, F):
         return self._check(_lib.qcd_bilinear_force(self.h, int(nvec), _ptr(G), _ptr(Psi), int(grad), _ptr(F)))
+
+    def qcd_bilinear_force_sum(self, nvec, G, Psi, grad, F):
+        return self._check(_lib.qcd_bilinear_force_sum(self.h, int(nvec), _ptr(G), _ptr(Psi), int(grad), _ptr(F)))
 
     def qcd_local_coherence(self, nvec, V):
         out = np.zeros(int(nvec), dtype=np.float64)
