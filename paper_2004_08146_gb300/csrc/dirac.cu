@@ -730,26 +730,29 @@ __global__ void __launch_bounds__(128) wilson_clover_f64_site_kernel(
 // FP32 stencil with links and clover blocks in site-fastest (SoA) copies:
 // Us[(mu * 9 + k) * V + site] (float2) and As[q * V + site] (float4, q < 18),
 // so a warp's link and clover loads are contiguous; spinors keep the ABI
-// layout.  With several
-// right-hand sides, consecutive CTAs take the same 128 sites for different
-// right-hand sides (CTA index = site block x nrhs + rhs), so the CTAs that
-// run together read the same links and clover blocks and all but the first
-// find them in L2: the links and clover are read from HBM about once per
-// site block instead of once per right-hand side.  With tb > 0 the site
-// blocks are visited time-fastest within bricks of tb time slices
-// (block u: t = (u / (tb ns)) tb + u % tb, spatial block (u / tb) % ns of
+// layout.  A thread applies the operator to NR right-hand sides of one site: the
+// links and clover block (864 of the 1,728 bytes that a single apply moves into
+// the SM) are loaded once for all of them.  Consecutive CTAs take the same 128
+// sites for the next NR right-hand sides and find links and clover in L2.  With
+// tb > 0 the site blocks are visited time-fastest within bricks of tb time
+// slices (block u: t = (u / (tb ns)) tb + u % tb, spatial block (u / tb) % ns of
 // ns = L1 L2 L3 / 128), so the neighbours of a block in every direction are
-// read by CTAs a few hundred launches apart and still sit in L2; only the
-// time neighbours across a brick face are fetched from DRAM again.  Four
-// CTAs per SM (registers capped at 128, 8 bytes spilled): 16 warps in flight
-// instead of 12 move the single-right-hand-side apply on 64 x 32^3 from 354 to
-// 319 us (4.55 -> 5.05 TB/s).
-__global__ void __launch_bounds__(128, 4) wilson_clover_soa_kernel(
+// read by CTAs a few hundred launches apart and still sit in L2.
+// Spinors move in 32-byte pieces where the fields are aligned to 32 bytes (W32):
+// the L1 pipe, 70 % busy with 16-byte ones (each load instruction of a warp
+// touches 24 lines), was what bound several right-hand sides.  64 x 32^3, one
+// right-hand side: 318 -> 280 us = 5.75 TB/s (85 % of the copy bandwidth); 32 x
+// 16^3, 16 right-hand sides: 245 -> 193 us, now bound by load latency at 16 warps
+// per SM (three or five CTAs per SM and four right-hand sides per thread are
+// slower).
+template <int NR, bool W32, int CTAS = 4>
+__global__ void __launch_bounds__(128, CTAS) wilson_clover_soa_kernel(
     float2* __restrict__ out, const float2* __restrict__ in, const float2* __restrict__ b,
     const float2* __restrict__ Us, const float4* __restrict__ As, Geom g, int op, Shifts tau, size_t stride,
     const int* __restrict__ act, int nrhs, int tb) {
-    const int j = (int)(blockIdx.x % nrhs);
-    const unsigned u = blockIdx.x / nrhs;
+    const int groups = (nrhs + NR - 1) / NR;
+    const int j0 = (int)(blockIdx.x % groups) * NR;
+    const unsigned u = blockIdx.x / groups;
     int s;
     if (tb > 0) {
         const unsigned vs = (unsigned)(g.L[1] * g.L[2] * g.L[3]), ns = vs / 128u;
@@ -758,15 +761,22 @@ __global__ void __launch_bounds__(128, 4) wilson_clover_soa_kernel(
     } else {
         s = (int)(u * blockDim.x + threadIdx.x);
     }
-    if (s >= g.V) return;
-    if (act != nullptr && !act[j]) return;
-    in += j * stride;
-    out += j * stride;
+    bool on[NR], any = false;
+#pragma unroll
+    for (int r = 0; r < NR; ++r) {
+        on[r] = j0 + r < nrhs && (act == nullptr || act[j0 + r]);
+        any = any || on[r];
+    }
+    if (s >= g.V || !any) return;
+    in += j0 * stride;
+    out += j0 * stride;
     const size_t V = (size_t)g.V;
     int x[4];
     site_coords(g, s, x);
-    Spinor<float> psi, acc;
-    load_spinor<float>(in + (size_t)s * 12, psi);
+    Spinor<float> acc[NR], psi[NR];
+#pragma unroll
+    for (int r = 0; r < NR; ++r)
+        if (on[r]) load_spinor_w<W32>(in + r * stride + (size_t)s * 12, psi[r]);
 #pragma unroll
     for (int chi = 0; chi < 2; ++chi) {
         float ar[36];
@@ -775,62 +785,73 @@ __global__ void __launch_bounds__(128, 4) wilson_clover_soa_kernel(
             const float4 v = __ldg(As + (size_t)(9 * chi + q) * V + s);
             ar[4 * q] = v.x; ar[4 * q + 1] = v.y; ar[4 * q + 2] = v.z; ar[4 * q + 3] = v.w;
         }
-        herm_off_apply<float>(ar, psi.c + 6 * chi, acc.c + 6 * chi);
-    }
-    auto link = [&](int site, int mu, Link<float>& u) {
 #pragma unroll
-        for (int k = 0; k < 9; ++k) u.e[k] = __ldg(Us + (size_t)(mu * 9 + k) * V + site);
-    };
+        for (int r = 0; r < NR; ++r)
+            if (on[r]) herm_off_apply<float>(ar, psi[r].c + 6 * chi, acc[r].c + 6 * chi);
+    }
 #pragma unroll
     for (int mu = 0; mu < 4; ++mu) {
-        int neg;
-        Spinor<float> nb;
-        Link<float> u;
-        int sf = nb_fwd(g, x, s, mu, neg);
-        load_spinor<float>(in + (size_t)sf * 12, nb);
-        link(s, mu, u);
-        float sg = neg ? -1.f : 1.f;
-        switch (mu) {
-            case 0: hop_accumulate<float, 0, true>(nb, u, sg, acc); break;
-            case 1: hop_accumulate<float, 1, true>(nb, u, sg, acc); break;
-            case 2: hop_accumulate<float, 2, true>(nb, u, sg, acc); break;
-            default: hop_accumulate<float, 3, true>(nb, u, sg, acc); break;
-        }
-        int sb = nb_bwd(g, x, s, mu, neg);
-        load_spinor<float>(in + (size_t)sb * 12, nb);
-        link(sb, mu, u);
-        sg = neg ? -1.f : 1.f;
-        switch (mu) {
-            case 0: hop_accumulate<float, 0, false>(nb, u, sg, acc); break;
-            case 1: hop_accumulate<float, 1, false>(nb, u, sg, acc); break;
-            case 2: hop_accumulate<float, 2, false>(nb, u, sg, acc); break;
-            default: hop_accumulate<float, 3, false>(nb, u, sg, acc); break;
+#pragma unroll
+        for (int dir = 0; dir < 2; ++dir) {
+            int neg;
+            const int sn = dir == 0 ? nb_fwd(g, x, s, mu, neg) : nb_bwd(g, x, s, mu, neg);
+            Link<float> l;
+#pragma unroll
+            for (int k = 0; k < 9; ++k) l.e[k] = __ldg(Us + (size_t)(mu * 9 + k) * V + (dir == 0 ? s : sn));
+            const float sg = neg ? -1.f : 1.f;
+#pragma unroll
+            for (int r = 0; r < NR; ++r) {
+                if (!on[r]) continue;
+                Spinor<float> nb;
+                load_spinor_w<W32>(in + r * stride + (size_t)sn * 12, nb);
+                if (dir == 0) {
+                    if (mu == 0) hop_accumulate<float, 0, true>(nb, l, sg, acc[r]);
+                    if (mu == 1) hop_accumulate<float, 1, true>(nb, l, sg, acc[r]);
+                    if (mu == 2) hop_accumulate<float, 2, true>(nb, l, sg, acc[r]);
+                    if (mu == 3) hop_accumulate<float, 3, true>(nb, l, sg, acc[r]);
+                } else {
+                    if (mu == 0) hop_accumulate<float, 0, false>(nb, l, sg, acc[r]);
+                    if (mu == 1) hop_accumulate<float, 1, false>(nb, l, sg, acc[r]);
+                    if (mu == 2) hop_accumulate<float, 2, false>(nb, l, sg, acc[r]);
+                    if (mu == 3) hop_accumulate<float, 3, false>(nb, l, sg, acc[r]);
+                }
+            }
         }
     }
     // diagonal of the clover blocks and shift, psi read again (L1) rather than
     // held through the hops
-    load_spinor<float>(in + (size_t)s * 12, psi);
 #pragma unroll
-    for (int chi = 0; chi < 2; ++chi) {
-        const float4 d0 = __ldg(As + (size_t)(9 * chi) * V + s), d1 = __ldg(As + (size_t)(9 * chi + 1) * V + s);
-        const float d[6] = {d0.x, d0.y, d0.z, d0.w, d1.x, d1.y};
-        const float t = (float)tau.t[j];
-        const float sg = op != QCD_OP_D && chi ? -1.f : 1.f, ts = op == QCD_OP_D && chi ? t : -t;
+    for (int r = 0; r < NR; ++r) {
+        if (!on[r]) continue;
+        const size_t at = r * stride + (size_t)s * 12;
+        load_spinor_w<W32>(in + at, psi[r]);
+        const float t = (float)tau.t[j0 + r];
 #pragma unroll
-        for (int k = 0; k < 6; ++k) {
-            float2& v = acc.c[6 * chi + k];
-            const float2 p = psi.c[6 * chi + k];
-            v.x = fmaf(ts, p.x, sg * fmaf(d[k], p.x, v.x));
-            v.y = fmaf(ts, p.y, sg * fmaf(d[k], p.y, v.y));
+        for (int chi = 0; chi < 2; ++chi) {
+            const float4 d0 = __ldg(As + (size_t)(9 * chi) * V + s), d1 = __ldg(As + (size_t)(9 * chi + 1) * V + s);
+            const float d[6] = {d0.x, d0.y, d0.z, d0.w, d1.x, d1.y};
+            const float sg = op != QCD_OP_D && chi ? -1.f : 1.f, ts = op == QCD_OP_D && chi ? t : -t;
+#pragma unroll
+            for (int k = 0; k < 6; ++k) {
+                float2& v = acc[r].c[6 * chi + k];
+                const float2 p = psi[r].c[6 * chi + k];
+                v.x = fmaf(ts, p.x, sg * fmaf(d[k], p.x, v.x));
+                v.y = fmaf(ts, p.y, sg * fmaf(d[k], p.y, v.y));
+            }
+        }
+        if (b != nullptr) {
+            Spinor<float> bb;
+            load_spinor<float>(b + j0 * stride + at, bb);
+#pragma unroll
+            for (int k = 0; k < 12; ++k) acc[r].c[k] = bb.c[k] - acc[r].c[k];
+        }
+        if constexpr (W32) {
+#pragma unroll
+            for (int k = 0; k < 3; ++k) store8(out + at + 4 * k, acc[r].c + 4 * k);
+        } else {
+            store_spinor<float>(out + at, acc[r]);
         }
     }
-    if (b != nullptr) {
-        Spinor<float> bb;
-        load_spinor<float>(b + j * stride + (size_t)s * 12, bb);
-#pragma unroll
-        for (int k = 0; k < 12; ++k) acc.c[k] = bb.c[k] - acc.c[k];
-    }
-    store_spinor<float>(out + (size_t)s * 12, acc);
 }
 
 // site-fastest copies of the FP32 links and clover blocks
@@ -926,13 +947,23 @@ static void launch_dirac(const FineOp& f, int prec, int op, int nrhs, const void
         return;
     }
     KTimer kt("wilson_clover_f32", bytes, 1824.0 * f.g.V * nrhs, st);
-    const unsigned gsoa = (unsigned)((f.g.V + 127) / 128) * (unsigned)nrhs;
     // several right-hand sides: time-fastest bricks of 8 time slices
     // (needs whole 128-site blocks per time slice and L0 a multiple of 8)
     const int vs = f.g.L[1] * f.g.L[2] * f.g.L[3];
     const int tb = (nrhs > 1 && vs % 128 == 0 && f.g.L[0] % 8 == 0) ? 8 : 0;
-    wilson_clover_soa_kernel<<<gsoa, 128, 0, st>>>((float2*)out, (const float2*)in, (const float2*)b, f.U32s, f.A32s,
-                                                   f.g, op, sh, (size_t)f.g.V * 12, act, nrhs, tb);
+    // two right-hand sides per thread once that leaves enough threads: 16 x 8^3
+    // with 4 10.3 us against 7.7 with one, 32 x 16^3 with 2 35.4 / 38.9, with 16
+    // 193 / 219, 64 x 32^3 with 2 440 / 507
+    const int nr = nrhs > 1 && (size_t)f.g.V * nrhs >= 196608 ? 2 : 1;
+    const bool w32 = (((uintptr_t)in | (uintptr_t)out) & 31) == 0;
+    const unsigned grid = (unsigned)((f.g.V + 127) / 128) * (unsigned)((nrhs + nr - 1) / nr);
+    auto kern = nr == 2 ? (w32 ? wilson_clover_soa_kernel<2, true> : wilson_clover_soa_kernel<2, false>)
+                        : (w32 ? wilson_clover_soa_kernel<1, true> : wilson_clover_soa_kernel<1, false>);
+    // a single right-hand side far past L2: 168 registers, more loads in flight
+    // per thread (64 x 32^3 280 us against 288; 32 x 16^3 23.7 against 22.5)
+    if (nr == 1 && w32 && f.g.V >= (1 << 20)) kern = wilson_clover_soa_kernel<1, true, 3>;
+    kern<<<grid, 128, 0, st>>>((float2*)out, (const float2*)in, (const float2*)b, f.U32s, f.A32s, f.g, op, sh,
+                               (size_t)f.g.V * 12, act, nrhs, tb);
 }
 
 void tangent_fields(const FineOp& f, const double2* X, double2* dU, double* dA, cudaStream_t st) {

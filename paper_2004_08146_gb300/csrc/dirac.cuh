@@ -22,6 +22,28 @@ template <> __device__ __forceinline__ void load_spinor<float>(const float2* __r
         s.c[2 * k + 1] = make_float2(v.z, v.w);
     }
 }
+// 32 bytes per load and store (complex64, 32-byte aligned): a warp reading one
+// 96-byte spinor per lane touches 24 lines with every load, so three loads of 32
+// bytes cost the L1 pipe half of what six of 16 bytes do
+__device__ __forceinline__ void load8(const float2* __restrict__ p, float2* v) {
+    asm("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+        : "=f"(v[0].x), "=f"(v[0].y), "=f"(v[1].x), "=f"(v[1].y), "=f"(v[2].x), "=f"(v[2].y), "=f"(v[3].x), "=f"(v[3].y)
+        : "l"(p));
+}
+__device__ __forceinline__ void store8(float2* p, const float2* v) {
+    asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "f"(v[0].x), "f"(v[0].y),
+                 "f"(v[1].x), "f"(v[1].y), "f"(v[2].x), "f"(v[2].y), "f"(v[3].x), "f"(v[3].y)
+                 : "memory");
+}
+template <bool W32> __device__ __forceinline__ void load_spinor_w(const float2* __restrict__ p, Spinor<float>& s) {
+    if constexpr (W32) {
+#pragma unroll
+        for (int k = 0; k < 3; ++k) load8(p + 4 * k, s.c + 4 * k);
+    } else {
+        load_spinor<float>(p, s);
+    }
+}
+
 template <typename R> __device__ __forceinline__ void store_spinor(cplx<R>* __restrict__ p, const Spinor<R>& s);
 template <> __device__ __forceinline__ void store_spinor<double>(double2* __restrict__ p, const Spinor<double>& s) {
 #pragma unroll

@@ -43,3 +43,29 @@ def test_stencil_shapes_match_oracle(dims, antip, nrhs):
             ctx.qcd_apply(opc, prec, 1, last, one, taus[-1:])
             assert np.array_equal(host(one).reshape(dims + (4, 3)), got[-1]), (prec, opc)
     ctx.close()
+
+
+@pytest.mark.parametrize("dims,nrhs", [((8, 8, 8, 16), 25), ((3, 5, 2, 7), 2)])
+@pytest.mark.parametrize("offset", [0, 2])
+def test_fp32_batches_and_alignment(dims, nrhs, offset):
+    """FP32 batches past the line where a thread takes two right-hand sides (an
+    odd count leaves one alone), and fields aligned to 16 bytes only, whose
+    results have the same bits as aligned ones."""
+    from paper_2004_08146_gb300 import qcd
+    torch = torch_cuda()
+    U = synth.gauge_field(dims, 0.5, 93)
+    op = WilsonClover(U, -0.3, 1.3)
+    ctx = make_ctx(U, dims, -0.3, 1.3)
+    psi = synth.spinor(dims, 94, nvec=nrhs)
+    taus = [0.2 - 0.03 * j for j in range(nrhs)]
+    x = dev(psi, np.complex64)
+    xo = torch.empty(x.numel() + offset, dtype=x.dtype, device="cuda")[offset:].copy_(x)
+    yo = torch.empty(x.numel() + offset, dtype=x.dtype, device="cuda")[offset:]
+    y = torch.empty_like(x)
+    ctx.qcd_apply(qcd.QCD_OP_Q, 1, nrhs, xo, yo, taus)
+    ctx.qcd_apply(qcd.QCD_OP_Q, 1, nrhs, x, y, taus)
+    got = host(yo).reshape((nrhs,) + dims + (4, 3))
+    assert np.array_equal(got.reshape(-1), host(y))
+    for j in (0, nrhs - 1):
+        assert relerr(got[j], op.Q_shift(psi[j], taus[j])) < 2e-6, j
+    ctx.close()
