@@ -878,17 +878,6 @@ double shifted_solve_impl(qcd_ctx* ctx, int nrhs, const double2* b, double2* x, 
 }
 
 // ------------------------------------------------------------------ GD-lambda-AMG
-// G[i][m] = d1[i], G[m][i] = conj d1[i]; Hm[i][m] = d2[i]; Hm[m][i] = conj d2[i]  (ld = column stride).
-// H = W^H V = V^H Q V is Hermitian because Q is (Sec. 2), so its new row
-// is the conjugate of its new column.
-__global__ void gram_update_kernel(double2* G, double2* Hm, int ld, int m, const double2* d1, const double2* d2) {
-    int i = threadIdx.x;
-    if (i > m) return;
-    G[(size_t)m * ld + i] = d1[i];
-    G[(size_t)i * ld + m] = conj(d1[i]);
-    Hm[(size_t)m * ld + i] = d2[i];
-    Hm[(size_t)i * ld + m] = conj(d2[i]);
-}
 __global__ void gather_columns_kernel(const double2* S, int m, const int* idx, int p, double2* out) {
     for (int e = threadIdx.x; e < m * p; e += blockDim.x) out[e] = S[(size_t)idx[e / m] * m + e % m];
 }
@@ -957,9 +946,9 @@ struct GD {
     qcd_ctx* ctx;
     size_t n;
     int mcap, kcap;
-    // V, W = Q V, X and u, Qu, r are stored double-float (QCD_FF, 16 bytes per
+    // V, W = Q V, X and u, Qu are stored double-float (QCD_FF, 16 bytes per
     // complex number); R, T and tmp, tmp2 are FP64
-    double2 *V, *W, *X, *G, *Hm, *Gt, *Hmt, *S, *work, *C, *dots, *part, *u, *Qu, *rff, *R, *T, *tmp, *tmp2;
+    double2 *V, *W, *X, *G, *Hm, *Gt, *Hmt, *S, *work, *C, *dots, *part, *u, *Qu, *R, *T, *tmp, *tmp2;
     double2 *ffc, *ffw;   // double-float copies of transform / reflector coefficients
     double* mu;
     double* mu_ref;   // refined eigenvalues of the targets
@@ -983,8 +972,8 @@ struct GD {
         Gt = B("Gt", (size_t)mcap * mcap); Hmt = B("Hmt", (size_t)mcap * mcap);
         S = B("S", (size_t)mcap * mcap); work = B("work", (size_t)(6 + block) * mcap * mcap); C = B("C", (size_t)mcap * mcap);
         dots = B("dots", (size_t)4 * (mcap + kcap + 8));
-        part = B("part", (size_t)(mcap + kcap + 8) * 64);
-        u = B("u", n); Qu = B("Qu", n); rff = B("rff", n); R = B("R", (size_t)block * n); T = B("T", (size_t)block * n);
+        part = B("part", (size_t)(2 * mcap + kcap + 8) * kFFParts);
+        u = B("u", n); Qu = B("Qu", n); R = B("R", (size_t)block * n); T = B("T", (size_t)block * n);
         tmp = B("tmp", n); tmp2 = B("tmp2", n);
         ffc = B("ffc", (size_t)mcap * mcap); ffw = B("ffw", (size_t)mcap + 1);
         mu = (double*)ctx->buf("gd.mu", mcap * sizeof(double));
@@ -1016,11 +1005,10 @@ struct GD {
         cudaStream_t st = ctx->st;
         double2* v = V + (size_t)m * n;
         double2* dx = dots + m + 1;
+        unsigned* cnt = ctx->dot_counters(mcap + kcap);
         blas_convert(QCD_FP64, t, QCD_FF, v, n, st);
-        blas_multidot(QCD_FF, V, m + 1, n, v, 1, n, dots, part, ctx->dot_counters(m + 1), st);
-        if (nlock > 0) blas_multidot(QCD_FF, X, nlock, n, v, 1, n, dx, part, ctx->dot_counters(nlock), st);
-        if (m > 0) blas_multiaxpy(QCD_FF, V, m, n, dots, -1.0, v, 1, n, st);
-        if (nlock > 0) blas_multiaxpy(QCD_FF, X, nlock, n, dx, -1.0, v, 1, n, st);
+        ff_dots(V, m + 1, X, nlock, n, v, dots, part, cnt, st);
+        ff_project(V, m, dots, X, nlock, dx, v, n, st);
         const double2* h = ctx->fetch(dots, m + 1 + nlock);
         const double t0 = h[m].x;
         double c2 = 0.0;
@@ -1028,29 +1016,20 @@ struct GD {
             if (i != m) c2 += h[i].x * h[i].x + h[i].y * h[i].y;
         double nt2 = t0 - c2;
         if (!(nt2 >= 0.5 * t0)) {
-            if (m > 0) {
-                blas_multidot(QCD_FF, V, m, n, v, 1, n, dots, part, ctx->dot_counters(m), st);
-                blas_multiaxpy(QCD_FF, V, m, n, dots, -1.0, v, 1, n, st);
-            }
-            if (nlock > 0) {
-                blas_multidot(QCD_FF, X, nlock, n, v, 1, n, dots, part, ctx->dot_counters(nlock), st);
-                blas_multiaxpy(QCD_FF, X, nlock, n, dots, -1.0, v, 1, n, st);
-            }
-            blas_multidot(QCD_FF, v, 1, n, v, 1, n, dots, part, ctx->dot_counters(1), st);
+            ff_dots(V, m, X, nlock, n, v, dots, part, cnt, st);
+            ff_project(V, m, dots, X, nlock, dots + m, v, n, st);
+            ff_dots(v, 1, nullptr, 0, n, v, dots, part, cnt, st);
             nt2 = ctx->fetch(dots, 1)[0].x;
         }
         const double nt = std::sqrt(std::max(nt2, 0.0));
         if (!(nt > 1e-12) || !std::isfinite(nt)) return false;
-        blas_axpby(QCD_FF, make_double2(0, 0), v, make_double2(1.0 / nt, 0), v, n, st);
         // W[m] = Q v in FP64 (v and W are stored double-float)
-        blas_convert(QCD_FF, v, QCD_FP64, tmp, n, st);
+        ff_scale_out(v, 1.0 / nt, tmp, n, st);
         applyQ(tmp, tmp2);
         blas_convert(QCD_FP64, tmp2, QCD_FF, W + (size_t)m * n, n, st);
-        // new Gram column / row
-        blas_multidot(QCD_FF, W, m + 1, n, W + (size_t)m * n, 1, n, dots, part, ctx->dot_counters(m + 1), st);
-        blas_multidot(QCD_FF, W, m + 1, n, v, 1, n, dots + mcap, part, ctx->dot_counters(m + 1), st);
-        KTimer kt("gram_update", 0.0, 0.0, st);
-        gram_update_kernel<<<1, kMaxBasis + 1, 0, st>>>(G, Hm, mcap, m, dots, dots + mcap);
+        // H = W^H V = V^H Q V is Hermitian because Q is (Sec. 2), so its new row
+        // is the conjugate of its new column
+        ff_gram_column(W, m, n, W + (size_t)m * n, v, dots, G, Hm, mcap, part, cnt, st);
         check_launch("add_vector");
         ++m;
         return true;
@@ -1226,25 +1205,12 @@ int eigs_impl(qcd_ctx* ctx, int k, double tol, double* lambda, double2* Vout, qc
             int nr = 0;
             for (int ti : tg) {
                 const double2* s = gd.S + (size_t)col[ti] * gd.m;   // column of S (ld = m)
-                blas_zero(QCD_FF, gd.u, n, st);
-                blas_zero(QCD_FF, gd.Qu, n, st);
-                blas_multiaxpy(QCD_FF, gd.V, gd.m, n, s, 1.0, gd.u, 1, n, st);
-                blas_multiaxpy(QCD_FF, gd.W, gd.m, n, s, 1.0, gd.Qu, 1, n, st);
-                blas_multidot(QCD_FF, gd.u, 1, n, gd.u, 1, n, gd.dots, gd.part, gd.ctx->dot_counters(1), st);
-                blas_multidot(QCD_FF, gd.u, 1, n, gd.Qu, 1, n, gd.dots + 1, gd.part, gd.ctx->dot_counters(1), st);
-                const double2* h = ctx->fetch(gd.dots, 2);
-                const double uu = h[0].x;
-                const double rho = h[1].x / uu;
-                const double iu = 1.0 / std::sqrt(uu);
-                double2* rj = gd.R + (size_t)nr * n;
-                // r = (Qu - rho u)/||u|| ; u <- u/||u||
-                blas_copy(QCD_FF, gd.Qu, gd.rff, n, st);
-                blas_axpby(QCD_FF, make_double2(-rho * iu, 0), gd.u, make_double2(iu, 0), gd.rff, n, st);
-                blas_axpby(QCD_FF, make_double2(0, 0), gd.u, make_double2(iu, 0), gd.u, n, st);
-                blas_multidot(QCD_FF, gd.rff, 1, n, gd.rff, 1, n, gd.dots, gd.part, gd.ctx->dot_counters(1), st);
-                blas_convert(QCD_FF, gd.rff, QCD_FP64, rj, n, st);
-                const double2* hr = ctx->fetch(gd.dots, 1);
-                const double rn = std::sqrt(std::max(hr[0].x, 0.0));
+                // r = (Qu - rho u)/||u||, u <- u/||u||
+                ff_ritz(gd.V, gd.W, gd.m, n, s, gd.u, gd.Qu, gd.R + (size_t)nr * n, gd.dots, gd.part,
+                        ctx->dot_counters(1), st);
+                const double2* h = ctx->fetch(gd.dots, 3);
+                const double rho = h[1].x / h[0].x;
+                const double rn = std::sqrt(std::max(h[2].x, 0.0));
                 if (rn <= tol) {
                     if (gd.nlock < gd.kcap) {
                         gd.lock_vector(gd.u);

@@ -10,6 +10,8 @@
 // On this part FP32 FMA throughput is about 60x the FP64 rate, so these
 // operations run at HBM speed where the FP64 forms were bound by the FP64
 // pipe.  Results of inner products are returned in FP64.
+#include <algorithm>
+
 #include "internal.h"
 
 namespace qcd {
@@ -93,175 +95,354 @@ __global__ void ff_from_fp32_kernel(const float2* __restrict__ x, float4* __rest
     }
 }
 
-// dots[v] = <X_i, w_j> (v = i * nrhs + j), same split-reduction scheme as the
-// FP64 kernel: per-thread double-float sums, FP64 across the CTA and across
-// CTAs (the last CTA of each dot adds the partials in a fixed order).
-// blockIdx.x runs over the dots so that CTAs reading the same chunk of w
-// are scheduled together.
-__global__ void ff_multidot_kernel(const float4* __restrict__ X, size_t xstride_vec, const float4* __restrict__ w,
-                                   int nrhs, size_t n, int nsplit, double2* __restrict__ partial,
-                                   unsigned* __restrict__ counters, double2* __restrict__ dots,
-                                   const int* __restrict__ act) {
-    const int v = blockIdx.x;
-    const int i = v / nrhs, j = v % nrhs;
-    if (act != nullptr && !act[j]) return;
-    const float4* x = X + (size_t)i * xstride_vec + (size_t)j * n;
-    const float4* y = w + (size_t)j * n;
-    const size_t chunk = (n + nsplit - 1) / nsplit;
-    const size_t lo = (size_t)blockIdx.y * chunk;
-    const size_t hi = lo + chunk < n ? lo + chunk : n;
-    // two independent accumulator pairs (even / odd strides): twice the
-    // loads in flight and two interleaved error-free chains per thread
-    acc_t re, im, re1, im1;
-    const size_t bd = blockDim.x;
-    size_t k = lo + threadIdx.x;
-    for (; k + bd < hi; k += 2 * bd) {
-        const float4 a = x[k], b = y[k], a1 = x[k + bd], b1 = y[k + bd];
-        // conj(a) b: re = ar br + ai bi, im = ar bi - ai br
+// (re, im) accumulators of conj(a) b and of c a
+struct acc2_t {
+    acc_t re, im;
+    __device__ __forceinline__ void dot(const float4& a, const float4& b) {
         re.mac(a.x, a.z, b.x, b.z);
-        re1.mac(a1.x, a1.z, b1.x, b1.z);
         im.mac(a.x, a.z, b.y, b.w);
-        im1.mac(a1.x, a1.z, b1.y, b1.w);
         re.mac(a.y, a.w, b.y, b.w);
-        re1.mac(a1.y, a1.w, b1.y, b1.w);
-        im.msub(a.y, a.w, b.x, b.z);
-        im1.msub(a1.y, a1.w, b1.x, b1.z);
-    }
-    if (k < hi) {
-        const float4 a = x[k], b = y[k];
-        re.mac(a.x, a.z, b.x, b.z);
-        re.mac(a.y, a.w, b.y, b.w);
-        im.mac(a.x, a.z, b.y, b.w);
         im.msub(a.y, a.w, b.x, b.z);
     }
-    double dr = join(re.get()) + join(re1.get()), di = join(im.get()) + join(im1.get());
-    dr = warp_sum(dr);
-    di = warp_sum(di);
-    __shared__ double sre[32], sim[32];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    if (lane == 0) { sre[wid] = dr; sim[wid] = di; }
-    __syncthreads();
-    if (wid == 0) {
-        const int nw = blockDim.x >> 5;
-        dr = lane < nw ? sre[lane] : 0.0;
-        di = lane < nw ? sim[lane] : 0.0;
-        dr = warp_sum(dr);
-        di = warp_sum(di);
-        if (lane == 0) partial[(size_t)v * nsplit + blockIdx.y] = make_double2(dr, di);
+    __device__ __forceinline__ void axpy(const float4& c, const float4& a) {
+        re.mac(c.x, c.z, a.x, a.z);
+        re.msub(c.y, c.w, a.y, a.w);
+        im.mac(c.x, c.z, a.y, a.w);
+        im.mac(c.y, c.w, a.x, a.z);
     }
-    __shared__ bool last;
-    if (threadIdx.x == 0) {
-        __threadfence();
-        last = atomicAdd(&counters[v], 1u) == (unsigned)nsplit - 1;
+};
+
+__device__ __forceinline__ ffr ff_warp_sum(ffr v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const ffr w{__shfl_xor_sync(0xffffffffu, v.h, o), __shfl_xor_sync(0xffffffffu, v.l, o)};
+        v = ff_add(v, w);
     }
-    __syncthreads();
-    if (!last || wid != 0) return;
-    __threadfence();
-    double sr = 0.0, si = 0.0;
-    for (int k = lane; k < nsplit; k += 32) {
-        const double2 q = __ldcg(&partial[(size_t)v * nsplit + k]);
-        sr += q.x;
-        si += q.y;
+    return v;
+}
+// Sum of many double-floats: three floats that are exact sums of one another's
+// rounding errors, so the total is good to FP64 roundoff without the FP64 pipe
+// (2 additions per clock and SM).
+struct sum3_t {
+    float a = 0.f, b = 0.f, c = 0.f;
+    __device__ __forceinline__ void add(float h, float l) {
+        const ffr s = two_sum(a, h), t = two_sum(b, l), u = two_sum(t.h, s.l);
+        a = s.h;
+        b = u.h;
+        c += t.l + u.l;
     }
-    sr = warp_sum(sr);
-    si = warp_sum(si);
-    if (lane == 0) {
-        dots[v] = make_double2(sr, si);
-        counters[v] = 0u;
+    __device__ __forceinline__ void add_lane(int o) {
+        const float h = __shfl_xor_sync(0xffffffffu, a, o), l = __shfl_xor_sync(0xffffffffu, b, o),
+                    m = __shfl_xor_sync(0xffffffffu, c, o);
+        add(h, l);
+        c += m;
     }
+    __device__ __forceinline__ ffr get() const {
+        const ffr s = two_sum(a, b);
+        return fast_two_sum(s.h, s.l + c);
+    }
+    __device__ __forceinline__ double warp_sum() {   // the same in all lanes
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) add_lane(o);
+        return (double)a + ((double)b + (double)c);
+    }
+};
+// both sums of a complex number, (re, im) in lanes 0 and 16: the halves of the warp
+// share them first
+__device__ __forceinline__ ffr ff_warp_sum2(ffr re, ffr im, int lane) {
+    const bool up = lane & 16;
+    const ffr k = up ? im : re, s = up ? re : im;
+    sum3_t t;
+    t.a = k.h;
+    t.b = k.l;
+    t.add(__shfl_xor_sync(0xffffffffu, s.h, 16), __shfl_xor_sync(0xffffffffu, s.l, 16));
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) t.add_lane(o);
+    return t.get();
 }
 
-constexpr int kFFCoef = 2048;   // coefficients staged per CTA (nvec * nrhs)
+// Dot products of up to two vectors y with the na vectors of set A and the nb of
+// set B (Gram-Schmidt against [V X]; the Gram columns W^H W_m, W^H V_m).  A warp
+// owns Q vectors over a part of the entries, so every y entry it reads serves Q
+// products and 2 Q + 2 loads are in flight; the eight warps of a CTA take
+// neighbouring parts for the same vectors and leave one partial, and the CTA that
+// finishes a set of vectors last adds them, one sum per warp.  Products
+// are 16 FP32 operations each, so warps in flight count: four CTAs per SM with Q = 4
+// (Q = 2 for two vectors y), one wave.  16 x 8^3, about 40 vectors: 31 us with idle
+// warps in the last set and three CTAs, 21 us now (two y: 40 with Q = 4 and two CTAs,
+// 30 now).
+struct GramOut {
+    double2 *G, *H;   // null: dots only
+    int ld, m;
+};
+template <int Q, int NY>
+__global__ void __launch_bounds__(256, 4) ff_dots_kernel(const float4* __restrict__ A, int na, const float4* __restrict__ B,
+                                                      int nb, size_t n, const float4* __restrict__ y0,
+                                                      const float4* __restrict__ y1,
+                                                      float2* __restrict__ partial, unsigned* __restrict__ counters,
+                                                      double2* __restrict__ d0, double2* __restrict__ d1, GramOut go) {
+    __shared__ float2 red[8][2 * NY * Q];   // re and im of each sum
+    __shared__ bool last;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nv = na + nb, v0 = blockIdx.y * Q;
+    const int part = blockIdx.x * 8 + warp, parts = gridDim.x * 8;
+    const size_t lo = n * part / parts, hi = n * (part + 1) / parts;
+    const float4* x[Q];
+#pragma unroll
+    for (int q = 0; q < Q; ++q) {
+        const int v = min(v0 + q, nv - 1);   // past the last: read like the last, not kept
+        x[q] = v < na ? A + (size_t)v * n : B + (size_t)(v - na) * n;
+    }
+    acc2_t acc[NY][Q];
+    size_t e = lo + lane;
+    for (; e + 32 < hi; e += 64) {
+        float4 a[Q], b[Q], y[2][NY];
+#pragma unroll
+        for (int q = 0; q < Q; ++q) {
+            a[q] = __ldg(x[q] + e);
+            b[q] = __ldg(x[q] + e + 32);
+        }
+        y[0][0] = __ldg(y0 + e);
+        y[1][0] = __ldg(y0 + e + 32);
+        if constexpr (NY == 2) {
+            y[0][1] = __ldg(y1 + e);
+            y[1][1] = __ldg(y1 + e + 32);
+        }
+#pragma unroll
+        for (int k = 0; k < NY; ++k)
+#pragma unroll
+            for (int q = 0; q < Q; ++q) {
+                acc[k][q].dot(a[q], y[0][k]);
+                acc[k][q].dot(b[q], y[1][k]);
+            }
+    }
+    if (e < hi) {
+        float4 y[NY];
+        y[0] = __ldg(y0 + e);
+        if constexpr (NY == 2) y[1] = __ldg(y1 + e);
+#pragma unroll
+        for (int q = 0; q < Q; ++q) {
+            const float4 a = __ldg(x[q] + e);
+#pragma unroll
+            for (int k = 0; k < NY; ++k) {
+                acc[k][q].dot(a, y[k]);
+            }
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < NY; ++k)
+#pragma unroll
+        for (int q = 0; q < Q; ++q) {
+            const ffr r = ff_warp_sum2(acc[k][q].re.get(), acc[k][q].im.get(), lane);
+            if ((lane & 15) == 0) red[warp][2 * (k * Q + q) + (lane >> 4)] = make_float2(r.h, r.l);
+        }
+    __syncthreads();
+    if (warp == 0) {
+        if (lane < 2 * NY * Q) {
+            sum3_t t;
+#pragma unroll
+            for (int w = 0; w < 8; ++w) t.add(red[w][lane].x, red[w][lane].y);
+            const ffr r = t.get();
+            partial[((size_t)blockIdx.y * 2 * NY * Q + lane) * gridDim.x + blockIdx.x] = make_float2(r.h, r.l);
+            __threadfence();
+        }
+        __syncwarp();
+        if (lane == 0) last = atomicAdd(&counters[blockIdx.y], 1u) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    const int k = warp / Q, v = v0 + warp % Q;
+    if (warp < NY * Q && v < nv) {
+        sum3_t re, im;
+        for (unsigned t = lane; t < gridDim.x; t += 32) {
+            const float2* p = partial + ((size_t)blockIdx.y * 2 * NY * Q + 2 * warp) * gridDim.x + t;
+            const float2 x = __ldcg(p), y = __ldcg(p + gridDim.x);
+            re.add(x.x, x.y);
+            im.add(y.x, y.y);
+        }
+        const double2 d = make_double2(re.warp_sum(), im.warp_sum());
+        if (lane == 0) {
+            (k == 0 ? d0 : d1)[v] = d;
+            // new column and row of G = W^H W and H = W^H V (Hermitian)
+            if (NY == 2 && go.G != nullptr) {
+                double2* M = k == 0 ? go.G : go.H;
+                M[(size_t)go.m * go.ld + v] = d;
+                M[(size_t)v * go.ld + go.m] = conj(d);
+            }
+        }
+    }
+    if (threadIdx.x == 0) counters[blockIdx.y] = 0u;
+}
 
-// w[j] += sign * sum_i c[i * nrhs + j] X[i][j] (coefficients FP64, split once per CTA)
-__global__ void ff_multiaxpy_kernel(const float4* __restrict__ X, int nvec, size_t xstride_vec,
-                                    const double2* __restrict__ c, double sign, float4* __restrict__ w, int nrhs,
-                                    size_t n, const int* __restrict__ act) {
-    __shared__ float4 cs[kFFCoef];
-    const int nco = nvec * nrhs;
-    const bool staged = nco <= kFFCoef;
-    if (staged)
-        for (int e = threadIdx.x; e < nco; e += blockDim.x) {
-            const double2 v = c[e];
+constexpr int kFFCoef = 512;   // coefficients staged at a time, a multiple of 8
+
+// acc += sign * sum_i c_i X_i[k]; eight loads in flight; a zero coefficient leaves
+// its vector unread (unused basis slots may hold anything).  All threads of the CTA
+// take part, in = false without an entry.
+__device__ __forceinline__ void ff_accumulate(acc2_t& acc, const float4* __restrict__ X, int nv, size_t n,
+                                              const double2* __restrict__ c, double sign, size_t k, bool in,
+                                              float4* cs) {
+    for (int i0 = 0; i0 < nv; i0 += kFFCoef) {
+        const int cnt = min(kFFCoef, nv - i0), pad = (cnt + 7) & ~7;
+        __syncthreads();
+        for (int e = threadIdx.x; e < pad; e += blockDim.x) {
+            const double2 v = e < cnt ? c[i0 + e] : make_double2(0.0, 0.0);
             cs[e] = pack(split(sign * v.x), split(sign * v.y));
         }
-    __syncthreads();
-    const size_t total = n * nrhs;
-    for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < total; t += (size_t)gridDim.x * blockDim.x) {
-        const int j = (int)(t / n);
-        if (act != nullptr && !act[j]) continue;
-        const size_t k = t - (size_t)j * n;
-        const float4 w0 = w[t];
-        acc_t re, im;
-        re.h = w0.x; re.l = w0.z;
-        im.h = w0.y; im.l = w0.w;
-        for (int i = 0; i < nvec; ++i) {
-            float4 ci;
-            if (staged) ci = cs[i * nrhs + j];
-            else {
-                const double2 v = c[i * nrhs + j];
-                ci = pack(split(sign * v.x), split(sign * v.y));
+        __syncthreads();
+        if (!in) continue;
+        const float4* x = X + (size_t)i0 * n + k;
+        for (int i = 0; i < cnt; i += 8) {
+            float4 a[8];
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                a[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (cs[i + q].x != 0.f || cs[i + q].y != 0.f) a[q] = __ldg(x + (size_t)(i + q) * n);
             }
-            if (ci.x == 0.f && ci.y == 0.f) continue;   // unused basis slots may hold stale data
-            const float4 a = X[(size_t)i * xstride_vec + (size_t)j * n + k];
-            // c a: re = cr ar - ci ai, im = cr ai + ci ar
-            re.mac(ci.x, ci.z, a.x, a.z);
-            re.msub(ci.y, ci.w, a.y, a.w);
-            im.mac(ci.x, ci.z, a.y, a.w);
-            im.mac(ci.y, ci.w, a.x, a.z);
+#pragma unroll
+            for (int q = 0; q < 8; ++q) acc.axpy(cs[i + q], a[q]);
         }
-        w[t] = pack(re.get(), im.get());
     }
 }
 
-// y[j] = alpha_j x[j] (+ y[j]); alpha FP64 on the device
-__global__ void ff_scale_kernel(const float4* __restrict__ x, float4* __restrict__ y, const double2* __restrict__ alpha,
-                                int nrhs, size_t n, bool accumulate, const int* __restrict__ act) {
-    const size_t total = n * nrhs;
-    for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < total; t += (size_t)gridDim.x * blockDim.x) {
-        const int j = (int)(t / n);
-        if (act != nullptr && !act[j]) continue;
-        const double2 a = alpha[j];
-        const ffr ar = split(a.x), ai = split(a.y);
-        const float4 v = x[t];
-        acc_t re, im;
-        if (accumulate) {
-            const float4 o = y[t];
-            re.h = o.x; re.l = o.z;
-            im.h = o.y; im.l = o.w;
-        }
-        re.mac(ar.h, ar.l, v.x, v.z);
-        re.msub(ai.h, ai.l, v.y, v.w);
-        im.mac(ar.h, ar.l, v.y, v.w);
-        im.mac(ai.h, ai.l, v.x, v.z);
-        y[t] = pack(re.get(), im.get());
+// w -= sum_i ca_i A_i + sum_i cb_i B_i.  One thread per entry: the vectors are read
+// once and w once, where a chain of updates would pass over w for each.  Six CTAs
+// per SM keep 24 warps of eight loads in flight; four quarter sums per entry (32
+// warps) gained nothing: 27.6 against 25.0 us.  16 x 8^3, about 50 vectors: 34 -> 25 us.
+__global__ void __launch_bounds__(128, 6) ff_project_kernel(const float4* __restrict__ A, int na,
+                                                            const double2* __restrict__ ca,
+                                                            const float4* __restrict__ B, int nb,
+                                                            const double2* __restrict__ cb, float4* __restrict__ w,
+                                                            size_t n) {
+    __shared__ float4 cs[kFFCoef];
+    const size_t k = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
+    const bool in = k < n;
+    acc2_t acc;
+    if (in) {
+        const float4 w0 = w[k];
+        acc.re.h = w0.x; acc.re.l = w0.z;
+        acc.im.h = w0.y; acc.im.l = w0.w;
     }
+    ff_accumulate(acc, A, na, n, ca, -1.0, k, in, cs);
+    ff_accumulate(acc, B, nb, n, cb, -1.0, k, in, cs);
+    if (in) w[k] = pack(acc.re.get(), acc.im.get());
 }
 
-// y = a x + b y (host scalars)
-__global__ void ff_axpby_kernel(double2 a, const float4* __restrict__ x, double2 b, float4* __restrict__ y, size_t n) {
-    const ffr ar = split(a.x), ai = split(a.y), br = split(b.x), bi = split(b.y);
+// Double-float sums of NV values over all threads of the grid, NV <= 2: one
+// partial per CTA, the last CTA adds them; FP64 results in out[v].x.
+template <int NV>
+__device__ __forceinline__ void ff_grid_sum(ffr (&v)[NV], float2* partial, unsigned* counter, double2* out) {
+    __shared__ float2 red[NV][32];
+    __shared__ bool last;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+#pragma unroll
+    for (int q = 0; q < NV; ++q) {
+        const ffr r = ff_warp_sum(v[q]);
+        if (lane == 0) red[q][warp] = make_float2(r.h, r.l);
+    }
+    __syncthreads();
+    if (warp == 0) {
+#pragma unroll
+        for (int q = 0; q < NV; ++q) {
+            const float2 r = lane < nw ? red[q][lane] : make_float2(0.f, 0.f);
+            const ffr s = ff_warp_sum(ffr{r.x, r.y});
+            if (lane == 0) partial[(size_t)q * gridDim.x + blockIdx.x] = make_float2(s.h, s.l);
+        }
+    }
+    if (threadIdx.x == 0) {
+        __threadfence();
+        last = atomicAdd(counter, 1u) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+#pragma unroll
+    for (int q = 0; q < NV; ++q) {
+        if (warp != q) continue;   // NV <= warps of the CTA
+        sum3_t a;
+        for (unsigned t = lane; t < gridDim.x; t += 32) {
+            const float2 r = __ldcg(&partial[(size_t)q * gridDim.x + t]);
+            a.add(r.x, r.y);
+        }
+        const double s = a.warp_sum();
+        if (lane == 0) out[q] = make_double2(s, 0.0);
+    }
+    if (threadIdx.x == 0) *counter = 0u;
+}
+
+// u = V s, Qu = W s (m vectors each) and d = (u^H u, Re u^H Qu) in one pass; bound
+// by the reads of V and W at 24 warps per SM (see above).  16 x 8^3: 56 -> 42 us.
+__global__ void __launch_bounds__(128, 6) ff_ritz_kernel(const float4* __restrict__ V, const float4* __restrict__ W,
+                                                         int m, size_t n, const double2* __restrict__ s,
+                                                         float4* __restrict__ u, float4* __restrict__ Qu,
+                                                         float2* __restrict__ partial, unsigned* __restrict__ counter,
+                                                         double2* __restrict__ d) {
+    __shared__ float4 cs[kFFCoef];
+    acc_t uu, uq;
+    const size_t step = (size_t)gridDim.x * blockDim.x;
+    for (size_t k0 = blockIdx.x * (size_t)blockDim.x; k0 < n; k0 += step) {
+        const size_t k = k0 + threadIdx.x;
+        const bool in = k < n;
+        acc2_t a, b;
+        ff_accumulate(a, V, m, n, s, 1.0, k, in, cs);
+        ff_accumulate(b, W, m, n, s, 1.0, k, in, cs);
+        if (!in) continue;
+        const float4 x = pack(a.re.get(), a.im.get()), y = pack(b.re.get(), b.im.get());
+        u[k] = x;
+        Qu[k] = y;
+        uu.mac(x.x, x.z, x.x, x.z);
+        uu.mac(x.y, x.w, x.y, x.w);
+        uq.mac(x.x, x.z, y.x, y.z);
+        uq.mac(x.y, x.w, y.y, y.w);
+    }
+    ffr v[2] = {uu.get(), uq.get()};
+    ff_grid_sum<2>(v, partial, counter, d);
+}
+
+// With d = (u^H u, Re u^H Qu) of the kernel above: r = (Qu - rho u) / ||u|| in
+// FP64 (rho the Rayleigh quotient), u <- u / ||u||, and rr = r^H r.
+__global__ void __launch_bounds__(256) ff_residual_kernel(float4* __restrict__ u, const float4* __restrict__ Qu,
+                                                          const double2* __restrict__ d, size_t n,
+                                                          double2* __restrict__ r, float2* __restrict__ partial,
+                                                          unsigned* __restrict__ counter, double2* __restrict__ rr) {
+    __shared__ float4 cf;   // iu and -rho iu
+    if (threadIdx.x == 0) {
+        const double uu = d[0].x, rho = d[1].x / uu, iu = 1.0 / sqrt(uu);
+        cf = pack(split(iu), split(-rho * iu));
+    }
+    __syncthreads();
+    const float4 c = cf;
+    acc_t sum;
+    for (size_t k = blockIdx.x * (size_t)blockDim.x + threadIdx.x; k < n; k += (size_t)gridDim.x * blockDim.x) {
+        const float4 x = u[k], y = Qu[k];
+        acc_t re, im, ur, ui;
+        re.mac(c.y, c.w, x.x, x.z);
+        re.mac(c.x, c.z, y.x, y.z);
+        im.mac(c.y, c.w, x.y, x.w);
+        im.mac(c.x, c.z, y.y, y.w);
+        const ffr a = re.get(), b = im.get();
+        r[k] = make_double2(join(a), join(b));
+        sum.mac(a.h, a.l, a.h, a.l);
+        sum.mac(b.h, b.l, b.h, b.l);
+        ur.mac(c.x, c.z, x.x, x.z);
+        ui.mac(c.x, c.z, x.y, x.w);
+        u[k] = pack(ur.get(), ui.get());
+    }
+    ffr v[1] = {sum.get()};
+    ff_grid_sum<1>(v, partial, counter, rr);
+}
+
+// v <- a v (double-float) and y = v in FP64
+__global__ void ff_scale_out_kernel(float4* __restrict__ v, double a, double2* __restrict__ y, size_t n) {
+    const ffr s = split(a);
     for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < n; t += (size_t)gridDim.x * blockDim.x) {
-        const float4 v = x[t], u = y[t];
+        const float4 x = v[t];
         acc_t re, im;
-        re.mac(ar.h, ar.l, v.x, v.z);
-        re.msub(ai.h, ai.l, v.y, v.w);
-        im.mac(ar.h, ar.l, v.y, v.w);
-        im.mac(ai.h, ai.l, v.x, v.z);
-        re.mac(br.h, br.l, u.x, u.z);
-        re.msub(bi.h, bi.l, u.y, u.w);
-        im.mac(br.h, br.l, u.y, u.w);
-        im.mac(bi.h, bi.l, u.x, u.z);
-        y[t] = pack(re.get(), im.get());
-    }
-}
-
-__global__ void ff_gamma5_kernel(const float4* __restrict__ x, float4* __restrict__ y, size_t nsites) {
-    const size_t total = nsites * 12;
-    for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < total; t += (size_t)gridDim.x * blockDim.x) {
-        float4 v = x[t];
-        if ((t % 12) >= 6) { v.x = -v.x; v.y = -v.y; v.z = -v.z; v.w = -v.w; }
-        y[t] = v;
+        re.mac(s.h, s.l, x.x, x.z);
+        im.mac(s.h, s.l, x.y, x.w);
+        const ffr a0 = re.get(), b0 = im.get();
+        v[t] = pack(a0, b0);
+        y[t] = make_double2(join(a0), join(b0));
     }
 }
 
@@ -377,45 +558,62 @@ void ff_convert(int prec_in, const void* x, int prec_out, void* y, size_t n, cud
         ff_from_fp32_kernel<<<grid_for(n), kThreads, 0, st>>>((const float2*)x, (float4*)y, n);
 }
 
-void ff_multidot(const void* X, int nvec, size_t xstride_vec, const void* w, int nrhs, size_t n, double2* dots,
-                 double2* partial, unsigned* counters, cudaStream_t st, const int* act) {
-    if (nvec <= 0) return;
-    int nsplit = 4 * sm_count() / (nvec * nrhs);
-    if (nsplit > 64) nsplit = 64;
-    if ((size_t)nsplit * 2048 > n) nsplit = (int)(n / 2048);
-    if (nsplit < 1) nsplit = 1;
-    dim3 grid(nvec * nrhs, nsplit);
-    KTimer kt("multidot_ff", (double)(nvec + 1) * nrhs * n * 16, 8.0 * nvec * nrhs * n, st);
-    ff_multidot_kernel<<<grid, kThreads, 0, st>>>((const float4*)X, xstride_vec, (const float4*)w, nrhs, n, nsplit,
-                                                  partial, counters, dots, act);
+// CTAs: one wave over all sets of vectors, at least 64 entries per warp
+template <int Q, int NY>
+static void launch_dots(const void* A, int na, const void* B, int nb, size_t n, const void* y0, const void* y1,
+                        double2* d0, double2* d1, void* partial, unsigned* counters, GramOut go, cudaStream_t st) {
+    static_assert(Q * NY <= 8, "one warp per sum");
+    const int sets = (na + nb + Q - 1) / Q;
+    size_t gx = std::max(1, 4 * sm_count() / sets);
+    gx = std::min({gx, std::max<size_t>(1, n / 512), (size_t)kFFParts});
+    ff_dots_kernel<Q, NY><<<dim3((unsigned)gx, sets), 256, 0, st>>>(
+        (const float4*)A, na, (const float4*)B, nb, n, (const float4*)y0, (const float4*)y1, (float2*)partial,
+        counters, d0, d1, go);
 }
 
-void ff_multiaxpy(const void* X, int nvec, size_t xstride_vec, const double2* c, double sign, void* w, int nrhs,
-                  size_t n, cudaStream_t st, const int* act) {
-    if (nvec <= 0) return;
-    const size_t total = n * nrhs;
-    KTimer kt("multiaxpy_ff", (double)(nvec + 2) * nrhs * n * 16, 8.0 * nvec * nrhs * n, st);
-    ff_multiaxpy_kernel<<<grid_for(total), kThreads, 0, st>>>((const float4*)X, nvec, xstride_vec, c, sign,
-                                                              (float4*)w, nrhs, n, act);
+void ff_dots(const void* A, int na, const void* B, int nb, size_t n, const void* y, double2* dots, void* partial,
+             unsigned* counters, cudaStream_t st) {
+    const int nv = na + nb;
+    if (nv <= 0) return;
+    KTimer kt("dots_ff", (double)(nv + 1) * n * 16, 8.0 * nv * n, st);
+    const GramOut go{};
+    if (nv <= 8) launch_dots<1, 1>(A, na, B, nb, n, y, nullptr, dots, nullptr, partial, counters, go, st);
+    else if (nv <= 16) launch_dots<2, 1>(A, na, B, nb, n, y, nullptr, dots, nullptr, partial, counters, go, st);
+    else launch_dots<4, 1>(A, na, B, nb, n, y, nullptr, dots, nullptr, partial, counters, go, st);
 }
 
-void ff_scale_dev(const void* x, void* y, const double2* alpha, int nrhs, size_t n, bool accumulate, cudaStream_t st,
-                  const int* act) {
-    const size_t total = n * nrhs;
-    KTimer kt("ff_scale", (double)total * (accumulate ? 3 : 2) * 16, 0.0, st);
-    ff_scale_kernel<<<grid_for(total), kThreads, 0, st>>>((const float4*)x, (float4*)y, alpha, nrhs, n, accumulate,
-                                                          act);
+void ff_gram_column(const void* W, int m, size_t n, const void* w, const void* v, double2* dots, double2* G, double2* H,
+                    int ld, void* partial, unsigned* counters, cudaStream_t st) {
+    KTimer kt("gram_column_ff", (double)(m + 3) * n * 16, 16.0 * (m + 1) * n, st);
+    const GramOut go{G, H, ld, m};
+    if (m < 8) launch_dots<1, 2>(W, m + 1, nullptr, 0, n, w, v, dots, dots + m + 1, partial, counters, go, st);
+    else launch_dots<2, 2>(W, m + 1, nullptr, 0, n, w, v, dots, dots + m + 1, partial, counters, go, st);
 }
 
-void ff_axpby(double2 a, const void* x, double2 b, void* y, size_t n, cudaStream_t st) {
-    KTimer kt("ff_axpby", (double)n * 3 * 16, 0.0, st);
-    ff_axpby_kernel<<<grid_for(n), kThreads, 0, st>>>(a, (const float4*)x, b, (float4*)y, n);
+void ff_project(const void* A, int na, const double2* ca, const void* B, int nb, const double2* cb, void* w, size_t n,
+                cudaStream_t st) {
+    if (na + nb <= 0) return;
+    KTimer kt("project_ff", (double)(na + nb + 2) * n * 16, 8.0 * (na + nb) * n, st);
+    ff_project_kernel<<<(unsigned)((n + 127) / 128), 128, 0, st>>>((const float4*)A, na, ca, (const float4*)B, nb, cb,
+                                                                   (float4*)w, n);
 }
 
-void ff_gamma5(const void* x, void* y, size_t nsites, cudaStream_t st) {
-    const size_t total = nsites * 12;
-    KTimer kt("ff_gamma5", (double)total * 2 * 16, 0.0, st);
-    ff_gamma5_kernel<<<grid_for(total), kThreads, 0, st>>>((const float4*)x, (float4*)y, nsites);
+void ff_ritz(const void* V, const void* W, int m, size_t n, const double2* s, void* u, void* Qu, double2* r, double2* d,
+             void* partial, unsigned* counters, cudaStream_t st) {
+    {
+        KTimer kt("ritz_ff", (double)(2 * m + 2) * n * 16, 16.0 * m * n, st);
+        const unsigned grid = (unsigned)std::min<size_t>((n + 127) / 128, kFFParts);
+        ff_ritz_kernel<<<grid, 128, 0, st>>>((const float4*)V, (const float4*)W, m, n, s, (float4*)u, (float4*)Qu,
+                                             (float2*)partial, counters, d);
+    }
+    KTimer kt("residual_ff", (double)n * 64, 0.0, st);
+    const unsigned grid = (unsigned)std::min<size_t>((n + 255) / 256, (size_t)sm_count() * 4);
+    ff_residual_kernel<<<grid, 256, 0, st>>>((float4*)u, (const float4*)Qu, d, n, r, (float2*)partial, counters, d + 2);
+}
+
+void ff_scale_out(void* v, double a, double2* y, size_t n, cudaStream_t st) {
+    KTimer kt("ff_scale_out", (double)n * 48, 0.0, st);
+    ff_scale_out_kernel<<<grid_for(n), kThreads, 0, st>>>((float4*)v, a, y, n);
 }
 
 void ff_transform_inplace(void* A, int m, const double2* C, int p, size_t n, void* cf_scratch, cudaStream_t st) {

@@ -144,14 +144,24 @@ void blas_axpby(int prec, double2 a, const void* x, double2 b, void* y, size_t n
 constexpr int QCD_FF = 2;
 // FP64 <-> FF, FF -> FP32 (hi + lo rounded), FP32 -> FF
 void ff_convert(int prec_in, const void* x, int prec_out, void* y, size_t n, cudaStream_t st);
-void ff_multidot(const void* X, int nvec, size_t xstride_vec, const void* w, int nrhs, size_t n, double2* dots,
-                 double2* partial, unsigned* counters, cudaStream_t st, const int* act);
-void ff_multiaxpy(const void* X, int nvec, size_t xstride_vec, const double2* c, double sign, void* w, int nrhs,
-                  size_t n, cudaStream_t st, const int* act);
-void ff_scale_dev(const void* x, void* y, const double2* alpha, int nrhs, size_t n, bool accumulate, cudaStream_t st,
-                  const int* act);
-void ff_axpby(double2 a, const void* x, double2 b, void* y, size_t n, cudaStream_t st);
-void ff_gamma5(const void* x, void* y, size_t nsites, cudaStream_t st);
+// Vectors of a set are n entries apart.  partial: kFFParts * 16 bytes per dot;
+// counters (zero, left zero): one per vector.
+constexpr int kFFParts = 4096;
+// dots[i] = <A_i, y>, dots[na + i] = <B_i, y>
+void ff_dots(const void* A, int na, const void* B, int nb, size_t n, const void* y, double2* dots, void* partial,
+             unsigned* counters, cudaStream_t st);
+// column and row m of G = W^H W and H = W^H V from w = W_m and v = V_m (dots: 2 (m + 1) of scratch)
+void ff_gram_column(const void* W, int m, size_t n, const void* w, const void* v, double2* dots, double2* G, double2* H,
+                    int ld, void* partial, unsigned* counters, cudaStream_t st);
+// w -= sum_i ca_i A_i + sum_i cb_i B_i
+void ff_project(const void* A, int na, const double2* ca, const void* B, int nb, const double2* cb, void* w, size_t n,
+                cudaStream_t st);
+// u = V s / ||V s||, r = (W s - rho V s) / ||V s|| in FP64, d = (u^H u and Re
+// u^H Q u before the normalisation, r^H r); Qu is scratch
+void ff_ritz(const void* V, const void* W, int m, size_t n, const double2* s, void* u, void* Qu, double2* r, double2* d,
+             void* partial, unsigned* counters, cudaStream_t st);
+// v <- a v, y = v in FP64
+void ff_scale_out(void* v, double a, double2* y, size_t n, cudaStream_t st);
 // A[j] <- sum_i C[i + j m] A[i] (j < p <= m) in place; cf_scratch: m * p * 16 bytes
 void ff_transform_inplace(void* A, int m, const double2* C, int p, size_t n, void* cf_scratch, cudaStream_t st);
 // Householder deflation of the pair (A0, A1) by the reflector hw (m + 1 entries); wf_scratch (m + 1) * 16 bytes
