@@ -497,8 +497,7 @@ __global__ void coarse_apply_mrhs_kernel(Geom gc, int nc, const Z* __restrict__ 
     const int s = blockIdx.x;
     const int j0 = blockIdx.y * rc;
     const size_t vstride = (size_t)gc.V * nc;
-    if (threadIdx.x < 9) {
-        const int d = threadIdx.x;
+    for (int d = threadIdx.x; d < 9; d += blockDim.x) {   // small blocks: fewer than nine threads
         int c[4];
         site_coords(gc, s, c);
         int sn = s;
@@ -655,16 +654,16 @@ __global__ void __launch_bounds__(128) coarse_apply_bulk_kernel(Geom gc, int nc,
     const int tid = threadIdx.x;
     const size_t vstride = (size_t)gc.V * nc;
     const size_t stage = coarse_bulk_stage_bytes(nc);
-    if (tid < 9) {
+    for (int d = tid; d < 9; d += blockDim.x) {   // small blocks: fewer than nine threads
         int c[4];
         site_coords(gc, s, c);
         int sn = s;
-        if (tid > 0) {
-            const int mu = (tid - 1) & 3, step = tid <= 4 ? 1 : -1;
+        if (d > 0) {
+            const int mu = (d - 1) & 3, step = d <= 4 ? 1 : -1;
             c[mu] = (c[mu] + step + gc.L[mu]) % gc.L[mu];
             sn = site_index(gc, c);
         }
-        nbr[tid] = sn;
+        nbr[d] = sn;
     }
     if (tid == 0) {
         mbar_init(&bar[0], 1);
@@ -684,7 +683,7 @@ __global__ void __launch_bounds__(128) coarse_apply_bulk_kernel(Geom gc, int nc,
         __syncwarp();
         if (tid < 32) {
             if (tid == 0) bulk_g2s(buf, A + ((size_t)s * 9 + d) * nc * nc, ablk, &bar[d & 1]);
-            for (int j = tid; j < nr; j += 32)
+            for (int j = tid; j < nr; j += min(32, (int)blockDim.x))
                 bulk_g2s(buf + coarse_bulk_xoff(nc, j), x + (size_t)(j0 + j) * vstride + (size_t)nbr[d] * nc, vseg,
                          &bar[d & 1]);
         }
