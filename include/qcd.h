@@ -110,7 +110,7 @@ typedef struct qcd_params {
                                 that does not fit returns EINVAL. */
     int    coarse_tensor;    /* FP32 coarse-stencil applies of the level-1 operator:
                                 0 (default) on the FMA units, stencil blocks and vectors
-                                staged into shared memory by bulk asynchronous copies
+                                staged into shared memory by asynchronous copies
                                 (16-byte aligned vectors; plain loads otherwise); 1 on the
                                 tensor cores (mma.sync, 2 Nv a multiple of 8), TF32 inputs
                                 split in big + small parts (three products, FP32

@@ -562,9 +562,8 @@ __global__ void coarse_apply_mrhs_kernel(Geom gc, int nc, const Z* __restrict__ 
     }
 }
 
-// ---- asynchronous bulk copies (TMA engine) into shared memory, completion
-// tracked by an mbarrier.  Every wait is bounded in time: a wait that gives up
-// counts itself in g_wait_timeouts and the caller skips its work.
+// ---- mbarrier waits, bounded in time: a wait that gives up counts itself in
+// g_wait_timeouts and the caller skips its work.
 __device__ unsigned long long g_wait_timeouts;
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
@@ -572,16 +571,6 @@ __device__ __forceinline__ uint32_t smem_u32(const void* p) {
 }
 __device__ __forceinline__ void mbar_init(uint64_t* bar, unsigned count) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, unsigned bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
-}
-// global -> shared copy of `bytes` (multiple of 16; both addresses 16-byte aligned)
-__device__ __forceinline__ void bulk_g2s(void* dst, const void* src, unsigned bytes, uint64_t* bar) {
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                     smem_u32(dst)),
-                 "l"(src), "r"(bytes), "r"(smem_u32(bar))
-                 : "memory");
 }
 __device__ __forceinline__ bool mbar_try(uint64_t* bar, unsigned parity) {
     uint32_t ok;
@@ -605,7 +594,6 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, unsigned parity, long l
     }
     return true;
 }
-__device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
 // Self-test of the bounded wait: one warp waits on an mbarrier that nothing
 // arrives at, gives up after `limit` clocks, counts itself and returns.
@@ -619,134 +607,182 @@ __global__ void wait_probe_kernel(long long limit) {
     if (threadIdx.x == 0) mbar_wait(&bar, 0, limit);
 }
 
-// FP32 coarse stencil on up to kBulkR right-hand sides per CTA, one coarse
-// site per CTA.  The 9 stencil blocks A_d (nc x nc complex, contiguous) and
-// the matching neighbour vectors (nc complex per right-hand side) stream
-// through two shared-memory stages filled by bulk asynchronous copies, so
-// each block is read from HBM exactly once while the previous one is
-// multiplied.  Thread (row r, group q) accumulates row r of y for the 8
-// right-hand sides 8q .. 8q+7: per column one block entry and eight
-// broadcast vector entries feed 32 FMAs.
-constexpr int kBulkR = 16;
-constexpr int kBulkG = 8;   // right-hand sides per thread
-
-// stage: block A_d, then the vectors of right-hand sides 0..7, 16 bytes of
-// padding (the two thread groups' broadcast reads then fall in different
-// banks), then right-hand sides 8..15
-__host__ __device__ inline size_t coarse_bulk_stage_bytes(int nc) {
-    return sizeof(float2) * ((size_t)nc * nc + (size_t)kBulkR * nc) + 16;
+// FP32 coarse stencil, one CTA per (coarse site, 2 J right-hand sides), one warp
+// per direction.  A warp streams its block A_d and its neighbour's vectors in
+// stages of eight columns through a ring of its own (asynchronous copies of 16
+// bytes per lane, three stages), so no barrier of the CTA stands between the nine
+// streams and two CTAs keep up to 220 KB per SM in flight.  Lane (r, h) holds rows
+// r, r + 16, .. of y for J right-hand sides: per pair of columns 2 R + J loads from
+// shared memory feed 8 R J FMAs (one row and eight right-hand sides per thread, as
+// before, are bound by the shared-memory loads).  The nine partial results are
+// added through shared memory at the end.  Bound by the FMA pipe and the issue slots
+// at 16 right-hand sides and by HBM below about 6.  Nv = 24: 8^4 sites, 16
+// right-hand sides 280 -> 253 us (43 TFLOP/s); 8 x 4^3 sites, 4 right-hand sides
+// 33 -> 18 us, 1: 31 -> 16.5 us (86 MB: 5.2 TB/s).  Blocks by cp.async.bulk (one
+// copy per stage and an mbarrier) 262 us, fma.f32x2 302 us.
+constexpr int kStageCols = 8;     // columns per stage
+constexpr int kStages = 3;
+// one warp's stages: kStageCols columns of A_d and of the W vectors; the sums of the
+// result reuse them, rows of W + 2
+__host__ __device__ constexpr size_t coarse_stage_bytes(int nc, int W) {
+    return sizeof(float2) * (size_t)kStageCols * (nc + W);
 }
-__host__ __device__ inline size_t coarse_bulk_xoff(int nc, int j) {
-    return sizeof(float2) * ((size_t)nc * nc + (size_t)j * nc) + (j >= kBulkG ? 16 : 0);
+__host__ __device__ inline size_t coarse_ring_bytes(int nc, int W) {
+    const size_t ring = kStages * coarse_stage_bytes(nc, W), sums = sizeof(float2) * (size_t)nc * (W + 2);
+    return ring > sums ? ring : sums;
 }
-size_t coarse_bulk_smem(int nc) { return 2 * coarse_bulk_stage_bytes(nc); }
-
-__global__ void __launch_bounds__(128) coarse_apply_bulk_kernel(Geom gc, int nc, const float2* __restrict__ A,
-                                                                const float2* __restrict__ x,
-                                                                float2* __restrict__ y, int op, Shifts tau,
-                                                                int nrhs) {
-    extern __shared__ __align__(128) unsigned char bsm[];
-    __shared__ __align__(8) uint64_t bar[2];
-    __shared__ int nbr[9];
-    __shared__ int fail;
-    const int s = blockIdx.x, j0 = blockIdx.y * kBulkR;
-    const int nr = min(kBulkR, nrhs - j0);
-    const int tid = threadIdx.x;
-    const size_t vstride = (size_t)gc.V * nc;
-    const size_t stage = coarse_bulk_stage_bytes(nc);
-    for (int d = tid; d < 9; d += blockDim.x) {   // small blocks: fewer than nine threads
-        int c[4];
-        site_coords(gc, s, c);
-        int sn = s;
-        if (d > 0) {
-            const int mu = (d - 1) & 3, step = d <= 4 ? 1 : -1;
-            c[mu] = (c[mu] + step + gc.L[mu]) % gc.L[mu];
-            sn = site_index(gc, c);
-        }
-        nbr[d] = sn;
+template <int R, int J>
+__global__ void __launch_bounds__(288, 2) coarse_apply_staged_kernel(Geom gc, int nc, const float2* __restrict__ A,
+                                                                  const float2* __restrict__ x,
+                                                                  float2* __restrict__ y, int op, Shifts tau,
+                                                                  int nrhs) {
+    constexpr int W = 2 * J, RS = W + 2;   // right-hand sides per CTA; row stride of the sums (16 bytes of padding)
+    extern __shared__ __align__(16) unsigned char dsm[];
+    const int lane = threadIdx.x & 31, d = threadIdx.x >> 5;
+    const int s = blockIdx.x, j0 = blockIdx.y * W;
+    const size_t vstride = (size_t)gc.V * nc, wbytes = coarse_ring_bytes(nc, W);
+    unsigned char* ring = dsm + d * wbytes;
+    const size_t stage = coarse_stage_bytes(nc, W);
+    int c[4];
+    site_coords(gc, s, c);
+#pragma unroll
+    for (int mu = 0; mu < 4; ++mu) {   // no indexed array: c stays in registers
+        if (d == mu + 1) c[mu] = c[mu] + 1 == gc.L[mu] ? 0 : c[mu] + 1;
+        if (d == mu + 5) c[mu] = c[mu] == 0 ? gc.L[mu] - 1 : c[mu] - 1;
     }
-    if (tid == 0) {
-        mbar_init(&bar[0], 1);
-        mbar_init(&bar[1], 1);
-        fail = 0;
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    const int sn = site_index(gc, c);
+    // 16-byte pieces: the columns of A_d are contiguous, two columns of a vector each
+    const int live = min(W, nrhs - j0), nst = (nc + kStageCols - 1) / kStageCols;
+    constexpr int XP = (W * kStageCols / 2 + 31) / 32;   // pieces of the vectors per lane and stage
+    const float2* pa = A + ((size_t)s * 9 + d) * nc * nc + 2 * lane;
+    const float2* px[XP];
+#pragma unroll
+    for (int i = 0; i < XP; ++i) {
+        const int e = lane + 32 * i, j = min(e / (kStageCols / 2), live - 1);
+        px[i] = x + (size_t)(j0 + j) * vstride + (size_t)sn * nc + e % (kStageCols / 2) * 2;
+    }
+    int filled = 0;
+    unsigned char* fbuf = ring;
+    auto fill = [&]() {
+        if (filled < nst) {
+            const int cols = min(kStageCols, nc - filled * kStageCols), np = cols * nc / 2;
+            Piece<float, 2>* o = reinterpret_cast<Piece<float, 2>*>(fbuf) + lane;
+            const float2* src = pa;
+#pragma unroll 2
+            for (int e = lane; e < np; e += 32, o += 32, src += 64) async_piece<float, 2>(o, src, true);
+            pa += kStageCols * nc;
+            o = reinterpret_cast<Piece<float, 2>*>(fbuf) + kStageCols / 2 * nc + lane;
+#pragma unroll
+            for (int i = 0; i < XP; ++i) {
+                const int e = lane + 32 * i;
+                if (e < live * (kStageCols / 2) && e % (kStageCols / 2) * 2 < cols) async_piece<float, 2>(o + 32 * i, px[i], true);
+                px[i] += kStageCols;
+            }
+            ++filled;
+            fbuf = filled % kStages == 0 ? ring : fbuf + stage;
+        }
+        async_commit();
+    };
+#pragma unroll
+    for (int i = 0; i < kStages - 1; ++i) fill();
+    const int r0 = lane & 15, h = lane >> 4;
+    float2 acc[R][J];
+#pragma unroll
+    for (int q = 0; q < R; ++q)
+#pragma unroll
+        for (int k = 0; k < J; ++k) acc[q][k] = make_float2(0.f, 0.f);
+    const unsigned char* buf = ring;
+    for (int i = 0; i < nst; ++i) {
+        fill();
+        async_wait<kStages - 1>();
+        __syncwarp();
+        // rows past the last read the next column (after the last the vectors): not kept
+        const float2* ap = reinterpret_cast<const float2*>(buf) + r0;
+        const float2* Xs = reinterpret_cast<const float2*>(buf) + (size_t)kStageCols * nc + h * J * kStageCols;
+        auto two = [&](const float2* xc) {
+            float2 a0[R], a1[R];
+#pragma unroll
+            for (int q = 0; q < R; ++q) {
+                a0[q] = ap[16 * q];
+                a1[q] = ap[nc + 16 * q];
+            }
+            ap += 2 * nc;
+#pragma unroll
+            for (int k = 0; k < J; ++k) {
+                const float4 v = *reinterpret_cast<const float4*>(xc + k * kStageCols);
+#pragma unroll
+                for (int q = 0; q < R; ++q) cmac(acc[q][k], a0[q], make_float2(v.x, v.y));
+#pragma unroll
+                for (int q = 0; q < R; ++q) cmac(acc[q][k], a1[q], make_float2(v.z, v.w));
+            }
+        };
+        const int cols = nc - i * kStageCols;
+        if (cols >= kStageCols) {
+#pragma unroll
+            for (int col = 0; col < kStageCols; col += 2) two(Xs + col);
+        } else {
+            for (int col = 0; col < cols; col += 2) two(Xs + col);
+        }
+        buf = (i + 1) % kStages == 0 ? ring : buf + stage;
+        __syncwarp();   // stage read: filled again next
+    }
+#pragma unroll
+    for (int q = 0; q < R; ++q) {
+        const int row = r0 + 16 * q;
+        if (row < nc) {
+            float4* o = reinterpret_cast<float4*>(reinterpret_cast<float2*>(ring) + (size_t)row * RS + h * J);
+#pragma unroll
+            for (int k = 0; k < J; k += 2)
+                o[k / 2] = make_float4(acc[q][k].x, acc[q][k].y, acc[q][k + 1].x, acc[q][k + 1].y);
+        }
     }
     __syncthreads();
-    const unsigned ablk = (unsigned)(sizeof(float2) * nc * nc), vseg = (unsigned)(sizeof(float2) * nc);
-    // stage d: block A_d and the neighbour vectors x_j(nbr[d]), j < nr
-    auto issue = [&](int d) {
-        unsigned char* buf = bsm + (d & 1) * stage;
-        if (tid == 0) {
-            fence_async_smem();
-            mbar_expect_tx(&bar[d & 1], ablk + (unsigned)nr * vseg);
-        }
-        __syncwarp();
-        if (tid < 32) {
-            if (tid == 0) bulk_g2s(buf, A + ((size_t)s * 9 + d) * nc * nc, ablk, &bar[d & 1]);
-            for (int j = tid; j < nr; j += min(32, (int)blockDim.x))
-                bulk_g2s(buf + coarse_bulk_xoff(nc, j), x + (size_t)(j0 + j) * vstride + (size_t)nbr[d] * nc, vseg,
-                         &bar[d & 1]);
-        }
-    };
-    issue(0);
-    issue(1);
-    const int r = tid % nc, q = tid / nc;
-    const bool active = q * kBulkG < nr;
-    float2 acc[kBulkG], xself[kBulkG];
+    for (int e = threadIdx.x; e < nc * J; e += blockDim.x) {
+        const int row = e % nc, k = e / nc * 2;
+        float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-    for (int k = 0; k < kBulkG; ++k) { acc[k] = make_float2(0.f, 0.f); xself[k] = make_float2(0.f, 0.f); }
-    for (int d = 0; d < 9; ++d) {
-        const unsigned char* buf = bsm + (d & 1) * stage;
-        if (!mbar_wait(&bar[d & 1], (unsigned)((d >> 1) & 1))) fail = 1;
-        __syncthreads();
-        if (fail) {
-            // copies may still be in flight into this CTA's shared memory
-            // (stages d and d + 1): wait for them once more, bounded, then
-            // leave without writing y
-            if (tid == 0) {
-                mbar_wait(&bar[d & 1], (unsigned)((d >> 1) & 1));
-                if (d + 1 < 9) mbar_wait(&bar[(d + 1) & 1], (unsigned)(((d + 1) >> 1) & 1));
-            }
-            __syncthreads();
-            return;
+        for (int dd = 0; dd < 9; ++dd) {
+            const float4 v = *reinterpret_cast<const float4*>(dsm + dd * wbytes + sizeof(float2) * ((size_t)row * RS + k));
+            o.x += v.x;
+            o.y += v.y;
+            o.z += v.z;
+            o.w += v.w;
         }
-        const float2* As = reinterpret_cast<const float2*>(buf);
-        const float2* Xs = reinterpret_cast<const float2*>(buf + coarse_bulk_xoff(nc, q * kBulkG));
-        if (active) {
-            if (d == 0) {
+        const float sg = row < nc / 2 ? 1.f : -1.f;
 #pragma unroll
-                for (int k = 0; k < kBulkG; ++k) xself[k] = Xs[(size_t)k * nc + r];
-            }
-            // two columns per step: one 16-byte broadcast load per right-hand side
-#pragma unroll 2
-            for (int col = 0; col < nc; col += 2) {
-                const float2 a0 = As[(size_t)col * nc + r], a1 = As[(size_t)(col + 1) * nc + r];
-#pragma unroll
-                for (int k = 0; k < kBulkG; ++k) {
-                    const float4 xv = *reinterpret_cast<const float4*>(Xs + (size_t)k * nc + col);
-                    acc[k].x = fmaf(a0.x, xv.x, fmaf(-a0.y, xv.y, acc[k].x));
-                    acc[k].y = fmaf(a0.x, xv.y, fmaf(a0.y, xv.x, acc[k].y));
-                    acc[k].x = fmaf(a1.x, xv.z, fmaf(-a1.y, xv.w, acc[k].x));
-                    acc[k].y = fmaf(a1.x, xv.w, fmaf(a1.y, xv.z, acc[k].y));
-                }
-            }
+        for (int i = 0; i < 2; ++i) {
+            const int j = j0 + k + i;
+            if (j >= nrhs) break;
+            const size_t at = (size_t)j * vstride + (size_t)s * nc + row;
+            const float tj = (float)tau.t[j];
+            const float2 xv = __ldg(x + at);
+            float2 r = i ? make_float2(o.z, o.w) : make_float2(o.x, o.y);
+            if (op == QCD_OP_D) { r -= (tj * sg) * xv; }
+            else { r = sg * r; r -= tj * xv; }
+            y[at] = r;
         }
-        __syncthreads();   // stage d & 1 no longer read
-        if (d + 2 < 9) issue(d + 2);
     }
-    if (!active) return;
-    const float sg = r < nc / 2 ? 1.f : -1.f;
-#pragma unroll
-    for (int k = 0; k < kBulkG; ++k) {
-        const int j = j0 + q * kBulkG + k;
-        if (j >= nrhs) break;
-        const float tj = (float)tau.t[j];
-        float2 o = acc[k];
-        const float2 xv = xself[k];
-        if (op == QCD_OP_D) { o -= (tj * sg) * xv; }
-        else { o = sg * o; o -= tj * xv; }
-        y[(size_t)j * vstride + (size_t)s * nc + r] = o;
-    }
+}
+
+template <int R, int J>
+static void launch_coarse_staged(const Coarse& c, int op, int nrhs, const float2* x, float2* y, const Shifts& sh,
+                              cudaStream_t st) {
+    const size_t sm = 9 * coarse_ring_bytes(c.nc, 2 * J);
+    if (sm > 48 * 1024)
+        cudaFuncSetAttribute(coarse_apply_staged_kernel<R, J>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    coarse_apply_staged_kernel<R, J><<<dim3(c.gc.V, (nrhs + 2 * J - 1) / (2 * J)), 288, sm, st>>>(c.gc, c.nc, c.A32, x, y,
+                                                                                               op, sh, nrhs);
+}
+// J: the fewest chunks of at most 16, evenly filled (20 right-hand sides: two of 12,
+// 47 us against 65 with 16 + 4 at 8 x 4^3 sites, Nv = 20)
+template <int R>
+static void coarse_staged_rows(const Coarse& c, int op, int nrhs, const float2* x, float2* y, const Shifts& sh,
+                             cudaStream_t st) {
+    const int chunks = (nrhs + 15) / 16, j = (nrhs + 2 * chunks - 1) / (2 * chunks);
+    if (j <= 2) launch_coarse_staged<R, 2>(c, op, nrhs, x, y, sh, st);
+    else if (j <= 4) launch_coarse_staged<R, 4>(c, op, nrhs, x, y, sh, st);
+    else if (j <= 6) launch_coarse_staged<R, 6>(c, op, nrhs, x, y, sh, st);
+    else launch_coarse_staged<R, 8>(c, op, nrhs, x, y, sh, st);
 }
 
 // Tensor-core coarse stencil (FP32 data, 3xTF32 products): per coarse site
@@ -1731,22 +1767,23 @@ void coarse_apply(const Coarse& c, int prec, int op, int nrhs, const void* x, vo
     for (int j = 0; j < nrhs; ++j) sh.t[j] = tau ? tau[j] : 0.0;
     const double es = prec == QCD_FP64 ? 16.0 : 8.0;
     const bool tc = prec == QCD_FP32 && tensor && c.nc % 8 == 0 && c.nc <= 64;
-    // bulk-copy kernel: FP32, 16-byte aligned vectors, 2 nc threads
-    const bool bulk = prec == QCD_FP32 && !tc && c.nc <= 64 && ((uintptr_t)x & 15) == 0 &&
+    // staged kernel: FP32, 16-byte aligned vectors (faster than the general one at
+    // every size measured, Nv 2 .. 24, 1 .. 20 right-hand sides, 16 to 4096 sites)
+    const bool staged = prec == QCD_FP32 && !tc && c.nc <= 64 && ((uintptr_t)x & 15) == 0 &&
                       ((uintptr_t)c.A32 & 15) == 0;
-    const int rchunk = bulk ? kBulkR : (tc ? kTcR : kCoarseRC);
+    const int rchunk = tc ? kTcR : 16;
     KTimer kt(prec == QCD_FP64 ? "coarse_apply_f64"
-                               : (tc ? "coarse_apply_tc" : (bulk ? "coarse_apply_bulk" : "coarse_apply_f32")),
+                               : (tc ? "coarse_apply_tc" : (staged ? "coarse_apply_bulk" : "coarse_apply_f32")),
               es * ((double)c.gc.V * 9 * c.nc * c.nc * ((nrhs + rchunk - 1) / rchunk) +
                     2.0 * nrhs * c.gc.V * c.nc),
               8.0 * 9 * c.nc * c.nc * (double)c.gc.V * nrhs, st);
-    if (bulk) {
-        const size_t sm = coarse_bulk_smem(c.nc);
-        if (sm + 1024 > 48 * 1024)
-            cudaFuncSetAttribute(coarse_apply_bulk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-        const dim3 grid(c.gc.V, (nrhs + kBulkR - 1) / kBulkR);
-        coarse_apply_bulk_kernel<<<grid, 2 * c.nc, sm, st>>>(c.gc, c.nc, c.A32, (const float2*)x, (float2*)y, op, sh,
-                                                            nrhs);
+    if (staged) {
+        const int rows = (c.nc + 15) / 16;
+        const float2* xf = (const float2*)x;
+        if (rows == 1) coarse_staged_rows<1>(c, op, nrhs, xf, (float2*)y, sh, st);
+        else if (rows == 2) coarse_staged_rows<2>(c, op, nrhs, xf, (float2*)y, sh, st);
+        else if (rows == 3) coarse_staged_rows<3>(c, op, nrhs, xf, (float2*)y, sh, st);
+        else coarse_staged_rows<4>(c, op, nrhs, xf, (float2*)y, sh, st);
         return;
     }
     if (prec == QCD_FP32 && tensor && c.nc % 8 == 0 && c.nc <= 64) {
