@@ -175,6 +175,10 @@ int qcd_set_params(qcd_ctx* ctx, const qcd_params* p);
  * extent must be >= 2; a previous hierarchy is dropped.  EINVAL on bad dims. */
 int qcd_set_gauge(qcd_ctx* ctx, const double* U, const int dims[4], double m0, double csw);
 
+/* The same with U in DEVICE memory, complete on the context's stream or before
+ * the call. */
+int qcd_set_gauge_device(qcd_ctx* ctx, const double* U, const int dims[4], double m0, double csw);
+
 /* out = (Q - tau) in  (Eq. 1.1 with A = Q; Eq. 3.6).  in/out: device
  * complex128 fields of 12 * V elements; in == out returns EINVAL. */
 int qcd_apply_Q(qcd_ctx* ctx, const void* in, void* out, double tau);

@@ -11,10 +11,10 @@ of that bilinear form, summed over the batch, so that Re tr(grad^H dU)
 reproduces dL for every such dU (the Riemannian gradient on SU(3); moves off
 the group are not represented).
 
-Links enter the library through ``qcd_set_gauge`` (a host copy): a forward
-with ``links`` given loads them into the context, and the backward uses the
-field the context holds, so run the backward before the context gets another
-field.  The context must run on torch's current stream; spinors are
+Links enter the library through ``qcd_set_gauge_device`` (CUDA tensors) or
+``qcd_set_gauge`` (a host copy): a forward with ``links`` given loads them into
+the context, and the backward uses the field the context holds, so run the
+backward before the context gets another field.  The context must run on torch's current stream; spinors are
 contiguous complex128 CUDA tensors of nrhs * V * 12 entries.
 """
 import numpy as np
@@ -31,8 +31,17 @@ class ShiftedQ(torch.autograd.Function):
         if nrhs * 12 * V != psi.numel():
             raise ValueError("psi must hold a whole number of fields")
         if links is not None:
-            Uh = links.detach().to("cpu", torch.complex128).contiguous().numpy()
-            qctx.qcd_set_gauge(Uh, dims, m0, csw)
+            # links on the device are copied there (a stand-in context without
+            # that call, or a lazily conjugated view, takes the host copy)
+            on_device = links.is_cuda and not links.is_conj() and not links.is_neg() and links.numel() == 36 * V
+            device_call = getattr(qctx, "qcd_set_gauge_device", None) if on_device else None
+            if device_call is not None:
+                Ud = links.detach().to(torch.complex128).contiguous()
+                torch.cuda.current_stream(links.device).synchronize()
+                device_call(Ud, dims, m0, csw)
+            else:
+                Uh = links.detach().to("cpu", torch.complex128).contiguous().numpy()
+                qctx.qcd_set_gauge(Uh, dims, m0, csw)
         out = torch.empty_like(psi)
         from . import qcd
         qctx.qcd_apply(qcd.QCD_OP_Q, qcd.QCD_FP64, nrhs, psi, out, [tau] * nrhs)

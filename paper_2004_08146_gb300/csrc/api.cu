@@ -76,11 +76,16 @@ struct qcd_ctx {
     ~qcd_ctx() { release(); }
 
     void release() {
-        for (auto& kv : ws) if (kv.second.p) cudaFree(kv.second.p);
-        ws.clear();
         auto fr = [](void* q) { if (q) cudaFree(q); };
         fr(f.U64); fr(f.U32); fr(f.U32s); fr(f.A64); fr(f.A32); fr(f.A32s);
         f.U64 = nullptr; f.U32 = nullptr; f.U32s = nullptr; f.A64 = nullptr; f.A32 = nullptr; f.A32s = nullptr;
+        drop_gauge_state();
+    }
+    // everything made from the gauge field, and all workspaces
+    void drop_gauge_state() {
+        auto fr = [](void* q) { if (q) cudaFree(q); };
+        for (auto& kv : ws) if (kv.second.p) cudaFree(kv.second.p);
+        ws.clear();
         drop_mg();
         fr(sap.blocks_of_colour[0]); fr(sap.blocks_of_colour[1]);
         sap.blocks_of_colour[0] = sap.blocks_of_colour[1] = nullptr;
@@ -1461,7 +1466,7 @@ int qcd_set_params(qcd_ctx* ctx, const qcd_params* p) {
     });
 }
 
-int qcd_set_gauge(qcd_ctx* ctx, const double* U, const int dims[4], double m0, double csw) {
+static int set_gauge_from(qcd_ctx* ctx, const double* U, cudaMemcpyKind kind, const int dims[4], double m0, double csw) {
     return guarded(ctx, [&]() {
         if (!U || !dims) throw QcdError(QCD_EINVAL, "null gauge field or dims");
         long long V = 1;
@@ -1472,22 +1477,27 @@ int qcd_set_gauge(qcd_ctx* ctx, const double* U, const int dims[4], double m0, d
         if (V > (1ll << 28)) throw QcdError(QCD_EINVAL, "lattice too large");
         if (!std::isfinite(m0) || !std::isfinite(csw)) throw QcdError(QCD_EINVAL, "m0 and csw must be finite");
         CK(cudaStreamSynchronize(ctx->st));
-        ctx->release();
-        ctx->have_gauge = false;
         FineOp& f = ctx->f;
+        // a field on the same lattice reuses the buffers of the last one
+        const bool keep = f.U64 && f.U32 && f.A64 && f.A32 && f.U32s && f.A32s && std::equal(dims, dims + 4, f.g.L);
+        if (keep) ctx->drop_gauge_state();
+        else ctx->release();
+        ctx->have_gauge = false;
         for (int mu = 0; mu < 4; ++mu) f.g.L[mu] = dims[mu];
         f.g.V = (int)V;
         f.g.antiperiodic = ctx->p.antiperiodic_t;
         f.m0 = m0;
         f.csw = csw;
         const size_t nl = (size_t)V * 36;
-        CK(cudaMalloc(&f.U64, nl * sizeof(double2)));
-        CK(cudaMalloc(&f.U32, nl * sizeof(float2)));
-        CK(cudaMalloc(&f.A64, (size_t)V * 72 * sizeof(double)));
-        CK(cudaMalloc(&f.A32, (size_t)V * 72 * sizeof(float)));
-        CK(cudaMalloc(&f.U32s, nl * sizeof(float2)));
-        CK(cudaMalloc(&f.A32s, (size_t)V * 18 * sizeof(float4)));
-        CK(cudaMemcpyAsync(f.U64, U, nl * sizeof(double2), cudaMemcpyHostToDevice, ctx->st));
+        if (!keep) {
+            CK(cudaMalloc(&f.U64, nl * sizeof(double2)));
+            CK(cudaMalloc(&f.U32, nl * sizeof(float2)));
+            CK(cudaMalloc(&f.A64, (size_t)V * 72 * sizeof(double)));
+            CK(cudaMalloc(&f.A32, (size_t)V * 72 * sizeof(float)));
+            CK(cudaMalloc(&f.U32s, nl * sizeof(float2)));
+            CK(cudaMalloc(&f.A32s, (size_t)V * 18 * sizeof(float4)));
+        }
+        CK(cudaMemcpyAsync(f.U64, U, nl * sizeof(double2), kind, ctx->st));
         // the links must be SU(3) matrices (Sec. 2): finite and unitary
         const double dev = gauge_unitarity_deviation(f.U64, (size_t)V * 4, ctx->counters(), ctx->st);
         check_launch("gauge check");
@@ -1504,6 +1514,14 @@ int qcd_set_gauge(qcd_ctx* ctx, const double* U, const int dims[4], double m0, d
         ctx->have_gauge = true;
         return QCD_OK;
     });
+}
+
+int qcd_set_gauge(qcd_ctx* ctx, const double* U, const int dims[4], double m0, double csw) {
+    return set_gauge_from(ctx, U, cudaMemcpyHostToDevice, dims, m0, csw);
+}
+
+int qcd_set_gauge_device(qcd_ctx* ctx, const double* U, const int dims[4], double m0, double csw) {
+    return set_gauge_from(ctx, U, cudaMemcpyDeviceToDevice, dims, m0, csw);
 }
 
 int qcd_apply(qcd_ctx* ctx, int op, int prec, int nrhs, const void* in, void* out, const double* tau) {

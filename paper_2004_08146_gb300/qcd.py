@@ -97,6 +97,7 @@ _SIGS = {
     "qcd_last_error": (ctypes.c_char_p, [_P]),
     "qcd_set_params": (_I, [_P, ctypes.POINTER(qcd_params)]),
     "qcd_set_gauge": (_I, [_P, _DP, _IP, _D, _D]),
+    "qcd_set_gauge_device": (_I, [_P, _P, _IP, _D, _D]),
     "qcd_apply_Q": (_I, [_P, _P, _P, _D]),
     "qcd_apply": (_I, [_P, _I, _I, _I, _P, _P, _DP]),
     "qcd_mg_setup": (_I, [_P, _I, _IP]),
@@ -248,6 +249,18 @@ class Context:
         self.dims = tuple(int(x) for x in dims)
         self._U_keep = Uh
         return self._check(_lib.qcd_set_gauge(self.h, Uh.ctypes.data_as(_DP), d, float(m0), float(csw)))
+
+    def qcd_set_gauge_device(self, U, dims, m0, csw):
+        """qcd_set_gauge from a contiguous complex128 CUDA tensor of at least
+        prod(dims) * 36 entries, complete before the call."""
+        need = 36
+        for x in dims:
+            need *= max(int(x), 0)
+        if U.numel() < need or not U.is_contiguous() or U.element_size() != 16:
+            raise ValueError("links must be a contiguous complex128 tensor of prod(dims) * 36 entries")
+        d = (ctypes.c_int * 4)(*[int(x) for x in dims])
+        self.dims = tuple(int(x) for x in dims)
+        return self._check(_lib.qcd_set_gauge_device(self.h, _ptr(U), d, float(m0), float(csw)))
 
     def qcd_apply_Q(self, inp, out, tau=0.0):
         return self._check(_lib.qcd_apply_Q(self.h, _ptr(inp), _ptr(out), float(tau)))
