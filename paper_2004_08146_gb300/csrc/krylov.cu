@@ -130,6 +130,12 @@ __global__ void kry_finish_kernel(KryDev K) {
 // buffered by iteration parity, so zeroing the next iteration's buffer never
 // races with readers of the current one.  Every CTA performs the (tiny)
 // Givens updates itself on identical totals.
+// Bound by latency: per iteration two or three barriers, the gather of the
+// neighbour vectors and the serial bookkeeping.  Stencil blocks (in flight from the
+// start to the first apply) and neighbour vectors come by 16-byte asynchronous
+// copies; with loads of one entry through registers, a few in flight per thread,
+// the 16 x 8^3 hierarchy (512 sites, nc 16, 4 right-hand sides) took 39 us per solve
+// in two or three iterations and 148 in twelve, now 26 and 124.
 template <typename Z, typename R>
 struct CoarseArgs {
     Geom gc;
@@ -211,6 +217,16 @@ __host__ __device__ inline CoarseSmem coarse_smem(int nrhs, int maxit, int E, in
     return L;
 }
 
+// 16 bytes from global memory (through L2: other CTAs may have just written them) to
+// shared memory, in flight until the wait
+__device__ __forceinline__ void async16(void* dst, const void* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(static_cast<uint32_t>(__cvta_generic_to_shared(dst))),
+                 "l"(src)
+                 : "memory");
+}
+__device__ __forceinline__ void async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+__device__ __forceinline__ void async_wait_all() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
+
 template <typename Z, typename R>
 __global__ void __launch_bounds__(256) coarse_gmres_kernel(CoarseArgs<Z, R> a) {
     cg::grid_group grid = cg::this_grid();
@@ -245,8 +261,13 @@ __global__ void __launch_bounds__(256) coarse_gmres_kernel(CoarseArgs<Z, R> a) {
     const int s0 = blockIdx.x * a.sps;
     const int nsl = len / nc;                               // sites owned by this CTA
     if (a.a_smem) {
-        const Z* src = a.A + (size_t)s0 * 9 * nc * nc;
-        for (size_t t = threadIdx.x; t < (size_t)nsl * 9 * nc * nc; t += blockDim.x) As[t] = src[t];
+        // 16-byte copies in flight until the first operator apply (nc is even: blocks
+        // and vectors start on 16-byte boundaries)
+        const char* src = reinterpret_cast<const char*>(a.A + (size_t)s0 * 9 * nc * nc);
+        const size_t bytes = sizeof(Z) * (size_t)nsl * 9 * nc * nc;
+        for (size_t t = 16 * (size_t)threadIdx.x; t < bytes; t += 16 * (size_t)blockDim.x)
+            async16(reinterpret_cast<char*>(As) + t, src + t);
+        async_commit();
         for (int t = threadIdx.x; t < nsl * 9; t += blockDim.x) {
             const int sl = t / 9, d = t % 9;
             int c[4];
@@ -356,11 +377,18 @@ __global__ void __launch_bounds__(256) coarse_gmres_kernel(CoarseArgs<Z, R> a) {
         const Z* Vit = a.Vg + (size_t)par * nrhs * nco;
         if (a.a_smem) {
             // gather the 9 neighbour blocks of every owned site, then multiply from shared memory
-            for (int t = tid; t < nrhs * nsl * 9 * nc; t += blockDim.x) {
-                const int col = t % nc, d = (t / nc) % 9, sl = (t / (9 * nc)) % nsl, j = t / (9 * nc * nsl);
+            constexpr int E16 = 16 / sizeof(Z);   // entries per copy
+            const int pc = nc / E16, np = nsl * 9 * pc;
+            for (int j = 0; j < nrhs; ++j) {
                 if (!live[j]) continue;
-                xn[(((size_t)j * nsl + sl) * 9 + d) * nc + col] = Vit[(size_t)j * nco + (size_t)nbr[sl * 9 + d] * nc + col];
+                const Z* vj = Vit + (size_t)j * nco;
+                for (int t = tid; t < np; t += blockDim.x) {
+                    const int b = t / pc, q = (t - b * pc) * E16;
+                    async16(xn + ((size_t)j * nsl * 9 + b) * nc + q, vj + (size_t)nbr[b] * nc + q);
+                }
             }
+            async_commit();
+            async_wait_all();
             __syncthreads();
             // tpr consecutive threads share one row (idle threads otherwise)
             const int items = nrhs * len;
@@ -492,6 +520,7 @@ __global__ void __launch_bounds__(256) coarse_gmres_kernel(CoarseArgs<Z, R> a) {
         for (int j = tid; j < nrhs; j += blockDim.x) if (live[j] < 0) live[j] = 0;
         __syncthreads();
     }
+    async_wait_all();   // the staged blocks, when no iteration ran
     // triangular solve (CTA 0) and x = V y
     if (blockIdx.x == 0 && tid < nrhs) {
         const int j = tid, k = kd[j];
