@@ -365,7 +365,7 @@ DevGmresOut gmres_dev(qcd_ctx* ctx, int prec, size_t n, int nrhs, const OpFn& A,
     double2* h1 = (double2*)ctx->buf(tag + ".h1", (size_t)(maxit + 1) * nrhs * sizeof(double2));
     double2* h2 = (double2*)ctx->buf(tag + ".h2", (size_t)(maxit + 1) * nrhs * sizeof(double2));
     double2* nr = (double2*)ctx->buf(tag + ".nr", (size_t)nrhs * sizeof(double2));
-    double2* part = (double2*)ctx->buf(tag + ".part", (size_t)(maxit + 2) * nrhs * 64 * sizeof(double2));
+    double2* part = (double2*)ctx->buf(tag + ".part", (size_t)(maxit + 2) * nrhs * kKryParts * sizeof(double2));
     KryDev K = kry_layout(ctx->buf(tag + ".K", kry_bytes(nrhs, maxit)), nrhs, maxit, tol);
     blas_multidot(prec, b, 1, vs, b, nrhs, n, nr, part, ctx->dot_counters(nrhs), st);
     kry_init(K, nr, outer_act, st);
@@ -381,12 +381,7 @@ DevGmresOut gmres_dev(qcd_ctx* ctx, int prec, size_t n, int nrhs, const OpFn& A,
         } else {
             A(vj, w, K.active);
         }
-        blas_multidot(prec, Vk, it + 1, vs, w, nrhs, n, h1, part, ctx->dot_counters((size_t)(it + 1) * nrhs), st, K.active);
-        blas_multiaxpy(prec, Vk, it + 1, vs, h1, -1.0, w, nrhs, n, st, K.active);
-        blas_multidot(prec, Vk, it + 1, vs, w, nrhs, n, h2, part, ctx->dot_counters((size_t)(it + 1) * nrhs), st, K.active);
-        blas_multiaxpy(prec, Vk, it + 1, vs, h2, -1.0, w, nrhs, n, st, K.active);
-        blas_multidot(prec, w, 1, vs, w, nrhs, n, nr, part, ctx->dot_counters(nrhs), st, K.active);
-        kry_step(K, it, h1, h2, nr, st);
+        kry_arnoldi(K, prec, Vk, vs, n, it, w, h1, h2, part, ctx->dot_counters(nrhs), st);
         if (it + 1 < maxit) blas_scale_dev(prec, w, Vk + (size_t)(it + 1) * vs * eb, K.scale, nrhs, n, false, false, st,
                                            K.active);
         steps = it + 1;

@@ -31,11 +31,9 @@ __global__ void convert_kernel(const Zi* __restrict__ x, Zo* __restrict__ y, siz
 template <typename Z>
 __global__ void multidot_partial_kernel(const Z* __restrict__ X, size_t xstride_vec, const Z* __restrict__ w,
                                         int nrhs, size_t n, int nsplit, double2* __restrict__ partial,
-                                        unsigned* __restrict__ counters, double2* __restrict__ dots,
-                                        const int* __restrict__ act) {
+                                        unsigned* __restrict__ counters, double2* __restrict__ dots) {
     const int v = blockIdx.y;            // v = i * nrhs + j
     const int i = v / nrhs, j = v % nrhs;
-    if (act != nullptr && !act[j]) return;
     const Z* x = X + (size_t)i * xstride_vec + (size_t)j * n;
     const Z* y = w + (size_t)j * n;
     const size_t chunk = (n + nsplit - 1) / nsplit;
@@ -196,7 +194,7 @@ void blas_convert(int prec_in, const void* x, int prec_out, void* y, size_t n, c
         convert_kernel<float2, double2><<<grid_for(n), kThreads, 0, st>>>((const float2*)x, (double2*)y, n);
 }
 void blas_multidot(int prec, const void* X, int nvec, size_t xstride_vec, const void* w, int nrhs, size_t n,
-                   double2* dots, double2* partial, unsigned* counters, cudaStream_t st, const int* act) {
+                   double2* dots, double2* partial, unsigned* counters, cudaStream_t st) {
     if (nvec <= 0) return;
     // enough CTAs to fill the GPU (about 4 per SM), at least 2048 elements each
     int nsplit = 608 / (nvec * nrhs);
@@ -208,10 +206,10 @@ void blas_multidot(int prec, const void* X, int nvec, size_t xstride_vec, const 
               8.0 * nvec * nrhs * n, st);
     if (prec == QCD_FP64)
         multidot_partial_kernel<double2><<<grid, kThreads, 0, st>>>((const double2*)X, xstride_vec, (const double2*)w,
-                                                                   nrhs, n, nsplit, partial, counters, dots, act);
+                                                                   nrhs, n, nsplit, partial, counters, dots);
     else
         multidot_partial_kernel<float2><<<grid, kThreads, 0, st>>>((const float2*)X, xstride_vec, (const float2*)w,
-                                                                  nrhs, n, nsplit, partial, counters, dots, act);
+                                                                  nrhs, n, nsplit, partial, counters, dots);
 }
 void blas_multiaxpy(int prec, const void* X, int nvec, size_t xstride_vec, const double2* c, double sign, void* w,
                     int nrhs, size_t n, cudaStream_t st, const int* act) {

@@ -129,4 +129,26 @@ template <typename R> __device__ __forceinline__ R warp_sum(R v) {
     return v;
 }
 
+// Sum of N values per lane over the warp, halving what a lane holds at each
+// step: afterwards v[0 .. max(N / 32, 1)) are the sums of the values from
+// `base` on.
+template <int N, int O, typename R>
+__device__ __forceinline__ void scatter_sum(R* v, int lane, int& base) {
+    if constexpr (O > 0) {
+        constexpr int n = N > 1 ? N / 2 : 1;
+        if constexpr (N > 1) {
+            const bool up = lane & O;
+#pragma unroll
+            for (int k = 0; k < n; ++k) {
+                const R send = up ? v[k] : v[k + n], keep = up ? v[k + n] : v[k];
+                v[k] = keep + __shfl_xor_sync(0xffffffffu, send, O);
+            }
+            if (up) base += n;
+        } else {
+            v[0] += __shfl_xor_sync(0xffffffffu, v[0], O);
+        }
+        scatter_sum<n, O / 2>(v, lane, base);
+    }
+}
+
 }  // namespace qcd

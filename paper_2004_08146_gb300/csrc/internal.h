@@ -124,8 +124,7 @@ void blas_convert(int prec_in, const void* x, int prec_out, void* y, size_t n, c
 // unsigned that are zero on entry and are left zero (one launch: the last
 // CTA of each dot adds the partial sums).
 void blas_multidot(int prec, const void* X, int nvec, size_t xstride_vec, const void* w, int nrhs,
-                   size_t n, double2* dots, double2* partial, unsigned* counters, cudaStream_t st,
-                   const int* act = nullptr);
+                   size_t n, double2* dots, double2* partial, unsigned* counters, cudaStream_t st);
 // w[j] += sign * sum_i c[i*nrhs + j] X[i][j]
 void blas_multiaxpy(int prec, const void* X, int nvec, size_t xstride_vec, const double2* c, double sign,
                     void* w, int nrhs, size_t n, cudaStream_t st, const int* act = nullptr);
@@ -246,7 +245,14 @@ struct KryDev {
 size_t kry_bytes(int nrhs, int maxit);
 KryDev kry_layout(void* buf, int nrhs, int maxit, double tol);
 void kry_init(const KryDev& K, const double2* nrm, const int* outer_act, cudaStream_t st);
-void kry_step(const KryDev& K, int it, const double2* h1, const double2* h2, const double2* nrm, cudaStream_t st);
+// Arnoldi step `it` of the active right-hand sides: w (vs = n * nrhs entries) made
+// orthogonal to V_0 .. V_it by classical Gram-Schmidt applied twice (coefficients h1,
+// h2, [it + 1][nrhs]), then the Givens update; K.scale normalises w.  partial:
+// (maxit + 1) * nrhs * kKryParts * 16 bytes; counters (zero, left zero): one per
+// right-hand side.
+constexpr int kKryParts = 160;
+void kry_arnoldi(const KryDev& K, int prec, const void* V, size_t vs, size_t n, int it, void* w, double2* h1, double2* h2,
+                 void* partial, unsigned* counters, cudaStream_t st);
 void kry_finish(const KryDev& K, cudaStream_t st);
 // Whole batched GMRES on the coarse stencil in one cooperative launch;
 // returns 0 on success, < 0 when the cooperative launch is not possible.

@@ -85,40 +85,200 @@ __global__ void kry_init_kernel(KryDev K, const double2* __restrict__ nrm, const
     K.scale[j] = make_double2(on ? 1.0 / b : 0.0, 0.0);
 }
 
-__global__ void kry_step_kernel(KryDev K, int it, const double2* __restrict__ h1, const double2* __restrict__ h2,
-                                const double2* __restrict__ nrm) {
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= K.nrhs || !K.active[j]) return;
-    double2 h[kMaxKry + 1];
-    for (int i = 0; i <= it; ++i) h[i] = h1[i * K.nrhs + j] + h2[i * K.nrhs + j];
-    const double hn = sqrt(fmax(nrm[j].x, 0.0));
-    double* cs = K.cs + (size_t)j * K.maxit;
-    double2* sn = K.sn + (size_t)j * K.maxit;
-    double2* g = K.g + (size_t)j * (K.maxit + 1);
-    const double res = givens_column(h, hn, cs, sn, g, it);
-    double2* R = K.R + (size_t)j * K.maxit * K.maxit;
-    for (int i = 0; i <= it; ++i) R[(size_t)i * K.maxit + it] = h[i];
-    K.k[j] = it + 1;
-    K.scale[j] = make_double2(hn > 0 ? 1.0 / hn : 0.0, 0.0);
-    if (res <= K.tol * K.beta[j]) K.active[j] = 0;
-    K.resid[j] = K.beta[j] > 0 ? res / K.beta[j] : 0.0;
+// ------------------------------------------------------------------ Arnoldi step
+// One step of batched (F)GMRES in three launches (they were six): inner products
+// h1 = V^H w; w -= V h1 with h2 = V^H w of the result; w -= V h2 with ||w||^2 and the
+// Givens update.  CTA (x, j) owns a part of the entries of right-hand side j, and a
+// thread meets the same entries in both halves of a launch.  Bound by the reads of V
+// from L2; 16 inner products per pass over w (4 or 8 in the first steps), whose loads
+// overlap and whose sums share one halving reduction of the warp.  One wave of CTAs
+// (3 per SM with 16 products; 4 of them in two waves took 18 + 24 us).  16 x 8^3,
+// 4 right-hand sides, steps 1 to 20 with the launch records on: 75 -> 54 us (inner
+// products 15.6, with the first projection 18.3, second projection, norm and
+// rotation 20.3).
+template <typename Z, typename R>
+__device__ __forceinline__ Z kry_projected(const Z* __restrict__ V, size_t vs, int nv, const Z* cs, Z w, size_t e) {
+    Z acc;
+    acc.x = 0; acc.y = 0;
+    for (int i = 0; i < nv; i += 8) {
+        Z x[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            x[q].x = 0; x[q].y = 0;
+            if (i + q < nv) x[q] = __ldg(V + (size_t)(i + q) * vs + e);
+        }
+#pragma unroll
+        for (int q = 0; q < 8; ++q)
+            if (i + q < nv) cmac(acc, cs[i + q], x[q]);
+    }
+    w.x -= acc.x;
+    w.y -= acc.y;
+    return w;
 }
 
-__global__ void kry_finish_kernel(KryDev K) {
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= K.nrhs) return;
-    const int kd = K.k[j];
-    const double2* R = K.R + (size_t)j * K.maxit * K.maxit;
-    const double2* g = K.g + (size_t)j * (K.maxit + 1);
-    double2 y[kMaxKry];
-    for (int i = kd - 1; i >= 0; --i) {
-        double2 s = g[i];
-        for (int l = i + 1; l < kd; ++l) s -= R[(size_t)i * K.maxit + l] * y[l];
-        double2 d = R[(size_t)i * K.maxit + i];
-        double den = cabs2(d);
-        y[i] = den > 0 ? (1.0 / den) * cmulc(d, s) : make_double2(0, 0);
+// true in the CTA of right-hand side j that finishes last
+__device__ __forceinline__ bool kry_last(unsigned* counter) {
+    __shared__ bool last;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        last = atomicAdd(counter, 1u) == gridDim.x - 1;
     }
-    for (int i = 0; i < K.maxit; ++i) K.coef[(size_t)i * K.nrhs + j] = i < kd ? y[i] : make_double2(0, 0);
+    __syncthreads();
+    if (last) __threadfence();
+    return last;
+}
+
+// CTAs per SM that the registers of 2 G sums and G loads leave
+template <typename R, int G> __host__ __device__ constexpr int kry_ctas() { return sizeof(R) * G >= 64 ? 3 : 4; }
+template <typename Z, typename R, int G, bool kProject>
+__global__ void __launch_bounds__(256, kry_ctas<R, G>()) kry_dots_kernel(const Z* __restrict__ V, size_t vs, int nv, Z* w, size_t n,
+                                                       int nrhs, const double2* __restrict__ h,
+                                                       double* __restrict__ partial, unsigned* __restrict__ counters,
+                                                       double2* __restrict__ dots, const int* __restrict__ act) {
+    const int j = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, parts = gridDim.x;
+    if (!act[j]) return;
+    __shared__ Z cs[kMaxKry + 1];
+    __shared__ R red[8][2 * G];
+    const size_t lo = n * blockIdx.x / parts, hi = n * (blockIdx.x + 1) / parts;
+    const Z* Vj = V + (size_t)j * n;
+    Z* wj = w + (size_t)j * n;
+    if constexpr (kProject) {
+        for (int i = threadIdx.x; i < nv; i += blockDim.x) {
+            cs[i].x = (R)h[(size_t)i * nrhs + j].x;
+            cs[i].y = (R)h[(size_t)i * nrhs + j].y;
+        }
+        __syncthreads();
+        for (size_t e = lo + threadIdx.x; e < hi; e += blockDim.x)
+            wj[e] = kry_projected<Z, R>(Vj, vs, nv, cs, wj[e], e);
+    }
+    double* pj = partial + (size_t)j * nv * 2 * parts;
+    for (int i0 = 0; i0 < nv; i0 += G) {
+        R acc[2 * G];
+#pragma unroll
+        for (int q = 0; q < 2 * G; ++q) acc[q] = R(0);
+        for (size_t e = lo + threadIdx.x; e < hi; e += blockDim.x) {
+            const Z y = wj[e];
+            Z x[G];
+#pragma unroll
+            for (int q = 0; q < G; ++q) {
+                x[q].x = 0; x[q].y = 0;
+                if (i0 + q < nv) x[q] = __ldg(Vj + (size_t)(i0 + q) * vs + e);
+            }
+#pragma unroll
+            for (int q = 0; q < G; ++q) cdot(acc[2 * q], acc[2 * q + 1], x[q], y);
+        }
+        int base = 0;
+        scatter_sum<2 * G, 16>(acc, lane, base);
+        if ((lane & (32 / (2 * G) - 1)) == 0) red[warp][base] = acc[0];
+        __syncthreads();
+        // the sums of the warps in FP64, as everything across warps
+        if (threadIdx.x < 2 * G && i0 + threadIdx.x / 2 < nv) {
+            double s = 0.0;
+#pragma unroll
+            for (int k = 0; k < 8; ++k) s += (double)red[k][threadIdx.x];
+            pj[(size_t)(2 * i0 + threadIdx.x) * parts + blockIdx.x] = s;
+        }
+        __syncthreads();
+    }
+    if (!kry_last(&counters[j])) return;
+    for (int v = warp; v < nv; v += 8) {
+        double2 s = make_double2(0.0, 0.0);
+        for (int t = lane; t < parts; t += 32) {
+            s.x += __ldcg(pj + (size_t)(2 * v) * parts + t);
+            s.y += __ldcg(pj + (size_t)(2 * v + 1) * parts + t);
+        }
+        s.x = warp_sum(s.x);
+        s.y = warp_sum(s.y);
+        if (lane == 0) dots[(size_t)v * nrhs + j] = s;
+    }
+    if (threadIdx.x == 0) counters[j] = 0u;
+}
+
+// w -= V h2 and, in the CTA that finishes last, ||w|| and the Givens update
+template <typename Z, typename R>
+__global__ void __launch_bounds__(256) kry_step_kernel(KryDev K, int it, const Z* __restrict__ V, size_t vs, Z* w,
+                                                       size_t n, const double2* __restrict__ h1,
+                                                       const double2* __restrict__ h2, double* __restrict__ partial,
+                                                       unsigned* __restrict__ counters) {
+    const int j = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, parts = gridDim.x, nv = it + 1;
+    if (!K.active[j]) return;
+    __shared__ Z co[kMaxKry + 1];
+    __shared__ double red[8];
+    const size_t lo = n * blockIdx.x / parts, hi = n * (blockIdx.x + 1) / parts;
+    const Z* Vj = V + (size_t)j * n;
+    Z* wj = w + (size_t)j * n;
+    for (int i = threadIdx.x; i < nv; i += blockDim.x) {
+        co[i].x = (R)h2[(size_t)i * K.nrhs + j].x;
+        co[i].y = (R)h2[(size_t)i * K.nrhs + j].y;
+    }
+    __syncthreads();
+    R nn = 0;
+    for (size_t e = lo + threadIdx.x; e < hi; e += blockDim.x) {
+        const Z o = kry_projected<Z, R>(Vj, vs, nv, co, wj[e], e);
+        wj[e] = o;
+        nn += o.x * o.x + o.y * o.y;
+    }
+    nn = warp_sum(nn);
+    if (lane == 0) red[warp] = (double)nn;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double s = 0.0;
+        for (int k = 0; k < 8; ++k) s += red[k];
+        partial[(size_t)j * parts + blockIdx.x] = s;
+    }
+    if (!kry_last(&counters[j])) return;
+    // the column, the rotations so far and the norm in shared memory: one thread
+    // turns the column in a serial chain of FP64 operations
+    __shared__ double2 h[kMaxKry + 1], sn[kMaxKry];
+    __shared__ double cs[kMaxKry], norm2;
+    for (int i = threadIdx.x; i < nv; i += blockDim.x) h[i] = h1[(size_t)i * K.nrhs + j] + h2[(size_t)i * K.nrhs + j];
+    for (int i = threadIdx.x; i < it; i += blockDim.x) {
+        cs[i] = K.cs[(size_t)j * K.maxit + i];
+        sn[i] = K.sn[(size_t)j * K.maxit + i];
+    }
+    if (warp == 7) {
+        double s = 0.0;
+        for (int t = lane; t < parts; t += 32) s += __ldcg(partial + (size_t)j * parts + t);
+        s = warp_sum(s);
+        if (lane == 0) norm2 = s;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        const double hn = sqrt(fmax(norm2, 0.0)), beta = K.beta[j];
+        const double res = givens_column(h, hn, cs, sn, K.g + (size_t)j * (K.maxit + 1), it);
+        K.cs[(size_t)j * K.maxit + it] = cs[it];
+        K.sn[(size_t)j * K.maxit + it] = sn[it];
+        K.k[j] = it + 1;
+        K.scale[j] = make_double2(hn > 0 ? 1.0 / hn : 0.0, 0.0);
+        if (res <= K.tol * beta) K.active[j] = 0;
+        K.resid[j] = beta > 0 ? res / beta : 0.0;
+        counters[j] = 0u;
+    }
+    __syncthreads();
+    double2* Rj = K.R + (size_t)j * K.maxit * K.maxit;
+    for (int i = threadIdx.x; i <= it; i += blockDim.x) Rj[(size_t)i * K.maxit + it] = h[i];
+}
+
+// Triangular solve R y = g, one warp per right-hand side: each y_i is taken out of
+// the rows above at once (65 us with one thread per right-hand side and 20 steps).
+__global__ void __launch_bounds__(32) kry_finish_kernel(KryDev K) {
+    const int j = blockIdx.x, lane = threadIdx.x, kd = K.k[j];
+    const double2* R = K.R + (size_t)j * K.maxit * K.maxit;
+    __shared__ double2 y[kMaxKry];
+    for (int i = lane; i < kd; i += 32) y[i] = K.g[(size_t)j * (K.maxit + 1) + i];
+    __syncwarp();
+    for (int i = kd - 1; i >= 0; --i) {
+        const double2 d = R[(size_t)i * K.maxit + i];
+        const double den = cabs2(d);
+        const double2 v = den > 0 ? (1.0 / den) * cmulc(d, y[i]) : make_double2(0, 0);
+        __syncwarp();
+        if (lane == 0) y[i] = v;
+        for (int l = lane; l < i; l += 32) y[l] -= R[(size_t)l * K.maxit + i] * v;
+        __syncwarp();
+    }
+    for (int i = lane; i < K.maxit; i += 32)
+        K.coef[(size_t)i * K.nrhs + j] = i < kd ? y[i] : make_double2(0, 0);
 }
 
 // ------------------------------------------------------------------ coarse GMRES
@@ -584,15 +744,6 @@ void kry_init(const KryDev& K, const double2* nrm, const int* outer_act, cudaStr
     KTimer kt("kry_init", 0.0, 0.0, st);
     kry_init_kernel<<<1, 64, 0, st>>>(K, nrm, outer_act);
 }
-void kry_step(const KryDev& K, int it, const double2* h1, const double2* h2, const double2* nrm, cudaStream_t st) {
-    KTimer kt("kry_step", 0.0, 0.0, st);
-    kry_step_kernel<<<1, 64, 0, st>>>(K, it, h1, h2, nrm);
-}
-void kry_finish(const KryDev& K, cudaStream_t st) {
-    KTimer kt("kry_finish", 0.0, 0.0, st);
-    kry_finish_kernel<<<1, 64, 0, st>>>(K);
-}
-
 int coarse_gmres_grid() {
     static int nct = 0;
     if (nct == 0) {
@@ -603,6 +754,49 @@ int coarse_gmres_grid() {
     }
     return nct;
 }
+
+template <typename Z, typename R, int G, bool kProject>
+static void launch_kry_dots(const KryDev& K, const Z* V, size_t vs, size_t n, int nv, Z* w, const double2* h,
+                            double* partial, unsigned* counters, double2* dots, dim3 grid, cudaStream_t st) {
+    KTimer kt(std::is_same<R, double>::value ? (kProject ? "kry_project_f64" : "kry_dots_f64")
+                                             : (kProject ? "kry_project_f32" : "kry_dots_f32"),
+              (double)(nv + (kProject ? 2 : 1)) * K.nrhs * n * sizeof(Z), (kProject ? 16.0 : 8.0) * nv * K.nrhs * n, st);
+    kry_dots_kernel<Z, R, G, kProject><<<grid, 256, 0, st>>>(V, vs, nv, w, n, K.nrhs, h, partial, counters, dots, K.active);
+}
+// parts per right-hand side: one wave over all of them, at least 256 entries each
+static dim3 kry_grid(int nrhs, size_t n, int ctas) {
+    const size_t parts = std::max<size_t>(1, (size_t)ctas * coarse_gmres_grid() / nrhs);
+    return dim3((unsigned)std::min({parts, std::max<size_t>(1, n / 256), (size_t)kKryParts}), nrhs);
+}
+template <typename Z, typename R, int G>
+static void arnoldi_passes(const KryDev& K, const Z* V, size_t vs, size_t n, int nv, Z* w, double2* h1, double2* h2,
+                           double* partial, unsigned* counters, cudaStream_t st) {
+    const dim3 grid = kry_grid(K.nrhs, n, kry_ctas<R, G>());
+    launch_kry_dots<Z, R, G, false>(K, V, vs, n, nv, w, nullptr, partial, counters, h1, grid, st);
+    launch_kry_dots<Z, R, G, true>(K, V, vs, n, nv, w, h1, partial, counters, h2, grid, st);
+}
+template <typename Z, typename R, int GMAX>
+static void arnoldi(const KryDev& K, const Z* V, size_t vs, size_t n, int it, Z* w, double2* h1, double2* h2,
+                    double* partial, unsigned* counters, cudaStream_t st) {
+    const int nv = it + 1;
+    if (nv <= 4) arnoldi_passes<Z, R, 4>(K, V, vs, n, nv, w, h1, h2, partial, counters, st);
+    else if (nv <= 8 || GMAX == 8) arnoldi_passes<Z, R, 8>(K, V, vs, n, nv, w, h1, h2, partial, counters, st);
+    else arnoldi_passes<Z, R, GMAX>(K, V, vs, n, nv, w, h1, h2, partial, counters, st);
+    KTimer kt("kry_step", (double)(nv + 2) * K.nrhs * n * sizeof(Z), 8.0 * nv * K.nrhs * n, st);
+    kry_step_kernel<Z, R><<<kry_grid(K.nrhs, n, 4), 256, 0, st>>>(K, it, V, vs, w, n, h1, h2, partial, counters);
+}
+void kry_arnoldi(const KryDev& K, int prec, const void* V, size_t vs, size_t n, int it, void* w, double2* h1, double2* h2,
+                 void* partial, unsigned* counters, cudaStream_t st) {
+    if (prec == QCD_FP64)
+        arnoldi<double2, double, 8>(K, (const double2*)V, vs, n, it, (double2*)w, h1, h2, (double*)partial, counters, st);
+    else
+        arnoldi<float2, float, 16>(K, (const float2*)V, vs, n, it, (float2*)w, h1, h2, (double*)partial, counters, st);
+}
+void kry_finish(const KryDev& K, cudaStream_t st) {
+    KTimer kt("kry_finish", 0.0, 0.0, st);
+    kry_finish_kernel<<<K.nrhs, 32, 0, st>>>(K);
+}
+
 
 // Site-based partition: each CTA owns `sps` consecutive coarse sites.
 static void coarse_partition(const Coarse& c, int& sps, int& nblk) {

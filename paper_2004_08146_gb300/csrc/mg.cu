@@ -131,28 +131,6 @@ template <typename R, int E> __device__ __forceinline__ void async_piece(Piece<R
 __device__ __forceinline__ void async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N> __device__ __forceinline__ void async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
-// Sum of N values per lane over the warp, halving what a lane holds at each
-// step: afterwards v[0 .. max(N / 32, 1)) are the sums of the values from
-// `base` on.
-template <int N, int O, typename R>
-__device__ __forceinline__ void scatter_sum(R* v, int lane, int& base) {
-    if constexpr (O > 0) {
-        constexpr int n = N > 1 ? N / 2 : 1;
-        if constexpr (N > 1) {
-            const bool up = lane & O;
-#pragma unroll
-            for (int k = 0; k < n; ++k) {
-                const R send = up ? v[k] : v[k + n], keep = up ? v[k + n] : v[k];
-                v[k] = keep + __shfl_xor_sync(0xffffffffu, send, O);
-            }
-            if (up) base += n;
-        } else {
-            v[0] += __shfl_xor_sync(0xffffffffu, v[0], O);
-        }
-        scatter_sum<n, O / 2>(v, lane, base);
-    }
-}
-
 // x_c = P^H r: per (aggregate, chirality) the product of the nv x nloc rows of P
 // with the nloc x nrhs fine entries (nloc = 6 x aggregate sites).  A warp owns a
 // 4 x TJ tile of results, its lanes run along nloc in pieces of E entries (P rows
