@@ -1502,7 +1502,6 @@ static int set_gauge_from(qcd_ctx* ctx, const double* U, cudaMemcpyKind kind, co
                                                                 std::to_string(dev) + ")"
                                                           : "gauge links contain non-finite entries");
         }
-        blas_convert(QCD_FP64, f.U64, QCD_FP32, f.U32, nl, ctx->st);
         launch_clover_build(f, ctx->st);
         check_launch("set_gauge");
         CK(cudaStreamSynchronize(ctx->st));
