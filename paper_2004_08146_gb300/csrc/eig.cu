@@ -35,7 +35,9 @@ __device__ double block_reduce_sum(double v, double* red) {
 // and C (both FP64, leading dimension ld) and the FP32 eigenvectors Z of C
 // (column-major, ld).  Appending basis vectors leaves the leading m0 x m0
 // blocks of Li and C unchanged, so only rows m0..m-1 are computed, one row k
-// at a time by matrix-vector products (one warp per output entry):
+// at a time by matrix-vector products (eight lanes per output entry: bound by the
+// one FP64 pipe and latency, and a whole warp spends more on the sum over lanes than
+// on the products):
 //   l = conj(Li[0:k,0:k] G[0:k,k])           (row k of L left of the diagonal)
 //   L[k,k] = sqrt(G[k,k] - ||l||^2)
 //   Li[k,j] = -(1/L[k,k]) sum_{j<=q<k} l[q] Li[q,j],  Li[k,k] = 1/L[k,k]
@@ -64,26 +66,32 @@ __global__ void __launch_bounds__(kTE) harmonic_eig_inc_kernel(const double2* __
     __shared__ double2 rowv[kMaxBasis], rowt[kMaxBasis];
     __shared__ double lkk_s;
     extern __shared__ double2 shm[];
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarp = blockDim.x >> 5;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     double2* Li = state;                          // row-major: Li[i * ld + j] = Li_ij
     double2* C = state + (size_t)ld * ld;         // Hermitian, both triangles stored
     float2* Zg = reinterpret_cast<float2*>(state + (size_t)2 * ld * ld);   // column-major
     auto Gh = [&](int i, int j) { return 0.5 * (G[(size_t)j * ld + i] + conj(G[(size_t)i * ld + j])); };
     auto Hh = [&](int i, int j) { return 0.5 * (Hm[(size_t)j * ld + i] + conj(Hm[(size_t)i * ld + j])); };
-    auto wsum = [&](double2 v) {
-        for (int o = 16; o > 0; o >>= 1) {
+    const int sub = tid & 7, grp = tid >> 3, ngrp = blockDim.x >> 3;   // eight lanes per output
+    auto gsum = [&](double2 v) {
+        for (int o = 4; o > 0; o >>= 1) {
             v.x += __shfl_xor_sync(0xffffffffu, v.x, o);
             v.y += __shfl_xor_sync(0xffffffffu, v.y, o);
         }
         return v;
     };
+    // trips of a group over its outputs, the same for the whole CTA: every lane takes
+    // part in the sums
+    auto trips = [&](int cnt) { return (cnt + ngrp - 1) / ngrp; };
     for (int k = m0; k < m; ++k) {
         // l = conj(Li[0:k,0:k] G[0:k,k])
-        for (int i = warp; i < k; i += nwarp) {
+        for (int t = 0; t < trips(k); ++t) {
+            const int i = t * ngrp + grp;
             double2 acc = make_double2(0, 0);
-            for (int l = lane; l <= i; l += 32) acc += Li[(size_t)i * ld + l] * Gh(l, k);
-            acc = wsum(acc);
-            if (lane == 0) rowv[i] = conj(acc);
+            if (i < k)
+                for (int l = sub; l <= i; l += 8) cmac(acc, Li[(size_t)i * ld + l], Gh(l, k));
+            acc = gsum(acc);
+            if (sub == 0 && i < k) rowv[i] = conj(acc);
         }
         __syncthreads();
         if (warp == 0) {
@@ -99,11 +107,13 @@ __global__ void __launch_bounds__(kTE) harmonic_eig_inc_kernel(const double2* __
         __syncthreads();
         const double ilkk = 1.0 / lkk_s;
         // Li[k, j], j < k
-        for (int j = warp; j < k; j += nwarp) {
+        for (int t = 0; t < trips(k); ++t) {
+            const int j = t * ngrp + grp;
             double2 acc = make_double2(0, 0);
-            for (int l = j + lane; l < k; l += 32) acc += rowv[l] * Li[(size_t)l * ld + j];
-            acc = wsum(acc);
-            if (lane == 0) {
+            if (j < k)
+                for (int l = j + sub; l < k; l += 8) cmac(acc, rowv[l], Li[(size_t)l * ld + j]);
+            acc = gsum(acc);
+            if (sub == 0 && j < k) {
                 Li[(size_t)k * ld + j] = (-ilkk) * acc;
                 Li[(size_t)j * ld + k] = make_double2(0, 0);
             }
@@ -111,19 +121,23 @@ __global__ void __launch_bounds__(kTE) harmonic_eig_inc_kernel(const double2* __
         if (tid == 0) Li[(size_t)k * ld + k] = make_double2(ilkk, 0);
         __syncthreads();
         // t = Li[k,:] H
-        for (int b = warp; b <= k; b += nwarp) {
+        for (int t = 0; t < trips(k + 1); ++t) {
+            const int b = t * ngrp + grp;
             double2 acc = make_double2(0, 0);
-            for (int a = lane; a <= k; a += 32) acc += Li[(size_t)k * ld + a] * Hh(a, b);
-            acc = wsum(acc);
-            if (lane == 0) rowt[b] = acc;
+            if (b <= k)
+                for (int a = sub; a <= k; a += 8) cmac(acc, Li[(size_t)k * ld + a], Hh(a, b));
+            acc = gsum(acc);
+            if (sub == 0 && b <= k) rowt[b] = acc;
         }
         __syncthreads();
         // C[k, j] = t . conj(Li[j, :]), j <= k
-        for (int j = warp; j <= k; j += nwarp) {
+        for (int t = 0; t < trips(k + 1); ++t) {
+            const int j = t * ngrp + grp;
             double2 acc = make_double2(0, 0);
-            for (int b = lane; b <= j; b += 32) acc += rowt[b] * conj(Li[(size_t)j * ld + b]);
-            acc = wsum(acc);
-            if (lane == 0) {
+            if (j <= k)
+                for (int b = sub; b <= j; b += 8) cmacc(acc, Li[(size_t)j * ld + b], rowt[b]);
+            acc = gsum(acc);
+            if (sub == 0 && j <= k) {
                 if (j == k) acc.y = 0.0;
                 C[(size_t)j * ld + k] = acc;
                 C[(size_t)k * ld + j] = conj(acc);
