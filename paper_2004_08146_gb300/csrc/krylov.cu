@@ -13,6 +13,7 @@
 #include <cooperative_groups.h>
 
 #include <algorithm>
+#include <utility>
 #include "internal.h"
 
 namespace cg = cooperative_groups;
@@ -295,7 +296,9 @@ __global__ void __launch_bounds__(32) kry_finish_kernel(KryDev K) {
 // start to the first apply) and neighbour vectors come by 16-byte asynchronous
 // copies; with loads of one entry through registers, a few in flight per thread,
 // the 16 x 8^3 hierarchy (512 sites, nc 16, 4 right-hand sides) took 39 us per solve
-// in two or three iterations and 148 in twelve, now 26 and 124.
+// in two or three iterations and 148 in twelve, then 26 and 124.  The rotations run
+// between arriving at the end-of-iteration barrier and waiting, and the last
+// projection writes the next basis vector: 26 and 112.
 template <typename Z, typename R>
 struct CoarseArgs {
     Geom gc;
@@ -346,7 +349,7 @@ __device__ __forceinline__ void coarse_row(const CoarseArgs<Z, R>& a, const Z* x
     out = acc;
 }
 
-struct CoarseSmem { size_t As, xn, nbr, Vs, ws, hc, h1, hr, hcol, cs, sn, g, beta, after, live, kd, again, total; };
+struct CoarseSmem { size_t As, xn, nbr, Vs, ws, hr, hcol, cs, sn, g, beta, hn, live, kd, total; };
 // Shared-memory layout of one CTA.  sps = 0: no staged stencil blocks;
 // basis_in_smem = false: the Krylov basis and w chunks are in global memory.
 template <typename Z>
@@ -361,18 +364,15 @@ __host__ __device__ inline CoarseSmem coarse_smem(int nrhs, int maxit, int E, in
     L.nbr = o;  o = up(o + sizeof(int) * (size_t)sps * 9);
     L.Vs = o;   o = up(o + sizeof(Z) * (size_t)(maxit + 1) * nrhs * Eb);
     L.ws = o;   o = up(o + sizeof(Z) * (size_t)nrhs * Eb);
-    L.hc = o;   o = up(o + sizeof(Z) * (size_t)(maxit + 2) * nrhs);
-    L.h1 = o;   o = up(o + sizeof(Z) * (size_t)(maxit + 2) * nrhs);
     L.hr = o;   o = up(o + sizeof(Z) * (size_t)(maxit + 1) * nrhs);
     L.hcol = o; o = up(o + sizeof(Z) * (size_t)(maxit + 1) * nrhs);
     L.cs = o;   o = up(o + sizeof(Z) * (size_t)nrhs * maxit);
     L.sn = o;   o = up(o + sizeof(Z) * (size_t)nrhs * maxit);
     L.g = o;    o = up(o + sizeof(Z) * (size_t)nrhs * (maxit + 1));
     L.beta = o; o = up(o + sizeof(double) * nrhs);
-    L.after = o; o = up(o + sizeof(Z) * nrhs);
+    L.hn = o;   o = up(o + sizeof(Z) * nrhs);
     L.live = o; o = up(o + sizeof(int) * nrhs);
     L.kd = o;   o = up(o + sizeof(int) * nrhs);
-    L.again = o; o = up(o + sizeof(int) * 4);
     L.total = o;
     return L;
 }
@@ -386,6 +386,8 @@ __device__ __forceinline__ void async16(void* dst, const void* src) {
 }
 __device__ __forceinline__ void async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void async_wait_all() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
+
+template <typename Z> struct __align__(16) Pair { Z a, b; };
 
 template <typename Z, typename R>
 __global__ void __launch_bounds__(256) coarse_gmres_kernel(CoarseArgs<Z, R> a) {
@@ -402,8 +404,6 @@ __global__ void __launch_bounds__(256) coarse_gmres_kernel(CoarseArgs<Z, R> a) {
     Z* ws = gbasis ? a.wglob + (size_t)blockIdx.x * nrhs * E : reinterpret_cast<Z*>(sraw + LY.ws);
     // the serial per-iteration bookkeeping runs in the working precision R:
     // a dependent chain of FP64 operations is very slow on this part
-    Z* hc = reinterpret_cast<Z*>(sraw + LY.hc);          // coefficients of the current pass (+ norms)
-    Z* h1s = reinterpret_cast<Z*>(sraw + LY.h1);         // pass-1 coefficients, kept for the Hessenberg column
     Z* hr = reinterpret_cast<Z*>(sraw + LY.hr);               // current-pass coefficients in the working precision
     Z* hcol = reinterpret_cast<Z*>(sraw + LY.hcol);      // [nrhs][maxit+1] column under rotation
     R* cs = reinterpret_cast<R*>(sraw + LY.cs);
@@ -412,8 +412,7 @@ __global__ void __launch_bounds__(256) coarse_gmres_kernel(CoarseArgs<Z, R> a) {
     double* beta = reinterpret_cast<double*>(sraw + LY.beta);
     int* live = reinterpret_cast<int*>(sraw + LY.live);
     int* kd = reinterpret_cast<int*>(sraw + LY.kd);
-    R* after = reinterpret_cast<R*>(sraw + LY.after);   // [nrhs] ||w||^2 after pass 1
-    int* againf = reinterpret_cast<int*>(sraw + LY.again);
+    R* hn = reinterpret_cast<R*>(sraw + LY.hn);          // [nrhs] norm of the projected w
 
     const size_t nco = (size_t)a.gc.V * a.nc;
     const size_t lo = (size_t)blockIdx.x * E;
@@ -484,15 +483,40 @@ __global__ void __launch_bounds__(256) coarse_gmres_kernel(CoarseArgs<Z, R> a) {
                     }
         }
     };
-    // ws[j] -= sum_i hc[i][j] Vs_i[j]
-    auto project = [&](int ni) {
+    // put(j, e, ws[j][e] - sum_i hr[i][j] Vs_i[j][e])
+    auto project = [&](int ni, auto put) {
         for (int t = tid; t < nrhs * len; t += blockDim.x) {
             const int j = t / len, e = t % len;
             if (!live[j]) continue;
             Z acc = ws[(size_t)j * E + e];
-            for (int i = 0; i < ni; ++i) cmsub(acc, hr[i * nrhs + j], VS(i, j)[e]);
-            ws[(size_t)j * E + e] = acc;
+            const Z* v = VS(0, j) + e;
+#pragma unroll 4
+            for (int i = 0; i < ni; ++i, v += (size_t)nrhs * E) cmsub(acc, hr[i * nrhs + j], *v);
+            put(j, e, acc);
         }
+    };
+    // coefficients of a Gram-Schmidt pass from its totals (hr; added to hcol), one
+    // warp per right-hand side, and hn = ||w|| after it; 1 where another is needed
+    auto column = [&](int parity, int pass, int it) {
+        int again = 0;
+        for (int j = warp; j < nrhs; j += nw) {
+            if (!live[j]) continue;
+            const double2* tot = TOT(parity, pass);
+            R sq = 0;
+            for (int i = lane; i <= it; i += 32) {
+                const double2 v = tot[i * nrhs + j];
+                const Z c = mk<R>((R)v.x, (R)v.y);
+                Z* h = hcol + (size_t)j * (maxit + 1) + i;
+                hr[i * nrhs + j] = c;
+                *h = pass == 0 ? c : *h + c;
+                sq += c.x * c.x + c.y * c.y;
+            }
+            const R before = (R)tot[(maxit + 1) * nrhs + j].x;
+            const R rest = before - warp_sum(sq);
+            if (lane == 0) hn[j] = rest > R(0) ? sqrt(rest) : R(0);
+            again |= rest < R(0.1) * before;
+        }
+        return again;
     };
 
     // ---- load b, beta = ||b||
@@ -520,13 +544,12 @@ __global__ void __launch_bounds__(256) coarse_gmres_kernel(CoarseArgs<Z, R> a) {
         VS(0, j)[e] = v;
         a.Vg[(size_t)j * nco + lo + e] = v;
     }
-    int it = 0;
-    for (; it < maxit; ++it) {
+    grid.sync();
+    for (int it = 0; it < maxit; ++it) {
         int any = 0;
         for (int j = 0; j < nrhs; ++j) any |= live[j];
         if (!any) break;
         const int par = it & 1;
-        grid.sync();
         // zero the other parity's totals: every CTA has passed the barrier, so
         // nobody still reads them (they held the previous iteration's sums, or
         // beta in iteration 0), and the next atomics into them follow the
@@ -550,36 +573,50 @@ __global__ void __launch_bounds__(256) coarse_gmres_kernel(CoarseArgs<Z, R> a) {
             async_commit();
             async_wait_all();
             __syncthreads();
-            // tpr consecutive threads share one row (idle threads otherwise)
-            const int items = nrhs * len;
-            int tpr = 1;
-            while (tpr < 4 && items * tpr * 2 <= (int)blockDim.x) tpr *= 2;
-            const int span = (9 * nc + tpr - 1) / tpr;
-            for (int t0 = tid; t0 < ((items * tpr + 31) / 32) * 32; t0 += blockDim.x) {
-                const int item = t0 / tpr, sub = t0 % tpr;
-                const bool ok = item < items && live[item / len];
-                Z acc; acc.x = 0; acc.y = 0;
-                int j = 0, e = 0, sl = 0, r = 0;
-                if (ok) {
-                    j = item / len; e = item % len;
-                    sl = e / nc; r = e % nc;
-                    const Z* am = As + (size_t)sl * 9 * nc * nc + r;
-                    const Z* xs = xn + ((size_t)j * nsl + sl) * 9 * nc;
-                    const int d0 = sub * span, d1 = min(9 * nc, d0 + span);
-                    for (int dc = d0; dc < d1; ++dc) cmac(acc, am[(size_t)dc * nc], xs[dc]);
+            // Tiles of two rows by two right-hand sides, the columns dealt to four
+            // lanes: per column one load of two block entries and two of vector
+            // entries feed four products.  The eight tiles of a warp cover
+            // consecutive rows (conflict-free), and the sums over the four lanes
+            // leave one of the four results in each.
+            const int rp = len / 2, tiles = rp * ((nrhs + 1) / 2), g8 = 8 * warp + (lane & 7), sub = lane >> 3;
+            for (int t0 = 0; t0 < tiles; t0 += 8 * nw) {
+                const int t = min(t0 + g8, tiles - 1);
+                const int e = t % rp * 2, j = t / rp * 2, j1 = min(j + 1, nrhs - 1), sl = e / nc, r = e - sl * nc;
+                const Z* am = As + (size_t)sl * 9 * nc * nc + r;
+                const Z* x0 = xn + ((size_t)j * nsl + sl) * 9 * nc;
+                const Z* x1 = xn + ((size_t)j1 * nsl + sl) * 9 * nc;
+                Z acc[2][2];   // [rhs][row]
+#pragma unroll
+                for (int q = 0; q < 4; ++q) { acc[q >> 1][q & 1].x = 0; acc[q >> 1][q & 1].y = 0; }
+                const Pair<Z>* ap = reinterpret_cast<const Pair<Z>*>(am + (size_t)sub * nc);
+#pragma unroll 4
+                for (int dc = sub; dc < 9 * nc; dc += 4, ap += 2 * nc) {
+                    const Pair<Z> m = *ap;
+                    const Z u0 = x0[dc], u1 = x1[dc];
+                    cmac(acc[0][0], m.a, u0);
+                    cmac(acc[0][1], m.b, u0);
+                    cmac(acc[1][0], m.a, u1);
+                    cmac(acc[1][1], m.b, u1);
                 }
-                for (int o = tpr / 2; o > 0; o >>= 1) {
-                    acc.x += __shfl_xor_sync(0xffffffffu, acc.x, o);
-                    acc.y += __shfl_xor_sync(0xffffffffu, acc.y, o);
-                }
-                if (ok && sub == 0) {
-                    const Z* xs = xn + ((size_t)j * nsl + sl) * 9 * nc;
-                    const R sg = r < nc / 2 ? R(1) : R(-1);
-                    const R tj = (R)a.tau[j];
-                    const Z xv = xs[r];      // direction 0 is the site itself
-                    if (a.op == QCD_OP_D) { acc -= (tj * sg) * xv; }
-                    else { acc = sg * acc; acc -= tj * xv; }
-                    ws[(size_t)j * E + e] = acc;
+                const bool hi = sub & 2, odd = sub & 1;   // lane bits 16 and 8
+                Z k0 = hi ? acc[1][0] : acc[0][0], k1 = hi ? acc[1][1] : acc[0][1];
+                const Z g0 = hi ? acc[0][0] : acc[1][0], g1 = hi ? acc[0][1] : acc[1][1];
+                k0.x += __shfl_xor_sync(0xffffffffu, g0.x, 16);
+                k0.y += __shfl_xor_sync(0xffffffffu, g0.y, 16);
+                k1.x += __shfl_xor_sync(0xffffffffu, g1.x, 16);
+                k1.y += __shfl_xor_sync(0xffffffffu, g1.y, 16);
+                Z o = odd ? k1 : k0;
+                const Z gv = odd ? k0 : k1;
+                o.x += __shfl_xor_sync(0xffffffffu, gv.x, 8);
+                o.y += __shfl_xor_sync(0xffffffffu, gv.y, 8);
+                const int jo = j + (hi ? 1 : 0), eo = e + (odd ? 1 : 0), ro = r + (odd ? 1 : 0);
+                if (t0 + g8 < tiles && jo < nrhs && live[jo]) {
+                    const R sg = ro < nc / 2 ? R(1) : R(-1);
+                    const R tj = (R)a.tau[jo];
+                    const Z xv = (hi ? x1 : x0)[ro];      // direction 0 is the site itself
+                    if (a.op == QCD_OP_D) { o -= (tj * sg) * xv; }
+                    else { o = sg * o; o -= tj * xv; }
+                    ws[(size_t)jo * E + eo] = o;
                 }
             }
         } else {
@@ -599,85 +636,43 @@ __global__ void __launch_bounds__(256) coarse_gmres_kernel(CoarseArgs<Z, R> a) {
         // classical Gram-Schmidt, pass 1, with ||w||^2 before the projection
         dots(TOT(par, 0), it + 1, true, ws);
         grid.sync();
-        for (int t = tid; t < (it + 1) * nrhs; t += blockDim.x) {
-            const double2 v = TOT(par, 0)[t];
-            hc[t] = h1s[t] = hr[t] = mk<R>((R)v.x, (R)v.y);
-        }
-        if (tid == 0) againf[0] = 0;
-        __syncthreads();
         // second pass only if some right-hand side lost more than 90% of its
         // squared norm in the first (a Kahan-Parlett test, loosened for a
         // solve that only needs a 0.5 reduction); every CTA takes the same
-        // decision from the same totals
-        if (tid < nrhs) {
-            const int j = tid;
-            const R before = (R)TOT(par, 0)[(maxit + 1) * nrhs + j].x;
-            R proj = 0;
-            for (int i = 0; i <= it; ++i) proj += h1s[i * nrhs + j].x * h1s[i * nrhs + j].x + h1s[i * nrhs + j].y * h1s[i * nrhs + j].y;
-            after[j] = before - proj;
-            if (live[j] && before - proj < R(0.1) * before) atomicOr(againf, 1);
-        }
-        __syncthreads();
-        const int again = againf[0];
-        project(it + 1);
-        __syncthreads();
+        // decision from the same totals.  Without it ||w||^2 is by Pythagoras.
+        const bool again = __syncthreads_or(column(par, 0, it));
         if (again) {
+            project(it + 1, [&](int j, int e, Z v) { ws[(size_t)j * E + e] = v; });
+            __syncthreads();
             dots(TOT(par, 1), it + 1, true, ws);
             grid.sync();
-            for (int t = tid; t < (it + 1) * nrhs; t += blockDim.x) {
-                const double2 v = TOT(par, 1)[t];
-                hc[t] = hr[t] = mk<R>((R)v.x, (R)v.y);
-            }
-            for (int t = tid; t < nrhs; t += blockDim.x) {
-                const double2 v = TOT(par, 1)[(maxit + 1) * nrhs + t];
-                hc[(maxit + 1) * nrhs + t] = mk<R>((R)v.x, (R)v.y);
-            }
-            __syncthreads();
-            project(it + 1);
-        } else {
-            // no second pass: its coefficients are zero, ||w||^2 by Pythagoras
-            for (int t = tid; t < (it + 1) * nrhs; t += blockDim.x) hc[t] = mk<R>(R(0), R(0));
-            for (int j = tid; j < nrhs; j += blockDim.x) hc[(maxit + 1) * nrhs + j] = mk<R>(after[j], R(0));
+            column(par, 1, it);
             __syncthreads();
         }
-        if (tid < nrhs) {
-            const int j = tid;
-            if (live[j]) {
-                Z* h = hcol + (size_t)j * (maxit + 1);
-                R h2n = 0;
-                for (int i = 0; i <= it; ++i) {
-                    const Z p2 = hc[i * nrhs + j];
-                    h[i] = h1s[i * nrhs + j] + p2;
-                    h2n += p2.x * p2.x + p2.y * p2.y;
-                }
-                const R hn2 = hc[(maxit + 1) * nrhs + j].x - h2n;
-                const R hn = hn2 > R(0) ? sqrt(hn2) : R(0);
-                hc[(maxit + 1) * nrhs + j] = mk<R>(hn, R(0));
-                const double res = givens_column_t<R>(h, hn, cs + (size_t)j * maxit, sn + (size_t)j * maxit,
-                                                      g + (size_t)j * (maxit + 1), it);
-                if (blockIdx.x == 0) {
-                    Z* Rj = reinterpret_cast<Z*>(a.Rg) + (size_t)j * maxit * maxit;
-                    for (int i = 0; i <= it; ++i) Rj[(size_t)i * maxit + it] = h[i];
-                    a.resid[j] = beta[j] > 0 ? res / beta[j] : 0.0;
-                }
-                kd[j] = it + 1;
-                if (res <= a.tol * beta[j]) live[j] = -1;   // converged: finish this step, then stop
-            }
-        }
-        __syncthreads();
-        // v_{it+1} = w / hn
-        for (int t = tid; t < nrhs * len; t += blockDim.x) {
-            const int j = t / len, e = t % len;
-            if (kd[j] != it + 1) continue;
-            const R hn = hc[(maxit + 1) * nrhs + j].x;
-            const R ih = hn > R(0) ? R(1) / hn : R(0);
-            Z v = ws[(size_t)j * E + e];
+        // v_{it+1} = w / ||w||, w projected for the last time
+        project(it + 1, [&](int j, int e, Z v) {
+            const R ih = hn[j] > R(0) ? R(1) / hn[j] : R(0);
             v.x *= ih; v.y *= ih;
             VS(it + 1, j)[e] = v;
             a.Vg[((size_t)(par ^ 1) * nrhs + j) * nco + lo + e] = v;
-        }
+        });
+        // the rotations, a serial chain, while the other CTAs arrive
         __syncthreads();
-        for (int j = tid; j < nrhs; j += blockDim.x) if (live[j] < 0) live[j] = 0;
+        auto token = grid.barrier_arrive();
+        if (tid < nrhs && live[tid]) {
+            const int j = tid;
+            Z* h = hcol + (size_t)j * (maxit + 1);
+            const double res = givens_column_t<R>(h, hn[j], cs + (size_t)j * maxit, sn + (size_t)j * maxit,
+                                                  g + (size_t)j * (maxit + 1), it);
+            if (blockIdx.x == 0) {
+                Z* Rj = reinterpret_cast<Z*>(a.Rg) + (size_t)j * maxit * maxit;
+                for (int i = 0; i <= it; ++i) Rj[(size_t)i * maxit + it] = h[i];
+                a.resid[j] = beta[j] > 0 ? res / beta[j] : 0.0;
+            }
+            kd[j] = it + 1;
+            if (res <= a.tol * beta[j]) live[j] = 0;   // converged
+        }
+        grid.barrier_wait(std::move(token));
         __syncthreads();
     }
     async_wait_all();   // the staged blocks, when no iteration ran
