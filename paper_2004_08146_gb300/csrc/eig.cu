@@ -14,6 +14,16 @@ constexpr int kTE = 512;   // threads of the harmonic eigen kernel
 
 __device__ __forceinline__ double cabs2(double2 a) { return a.x * a.x + a.y * a.y; }
 
+// sum over the eight lanes that share an output
+template <typename Z> __device__ __forceinline__ Z sum8(Z v) {
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) {
+        v.x += __shfl_xor_sync(0xffffffffu, v.x, o);
+        v.y += __shfl_xor_sync(0xffffffffu, v.y, o);
+    }
+    return v;
+}
+
 __device__ double block_reduce_sum(double v, double* red) {
     v = warp_sum(v);
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -73,13 +83,6 @@ __global__ void __launch_bounds__(kTE) harmonic_eig_inc_kernel(const double2* __
     auto Gh = [&](int i, int j) { return 0.5 * (G[(size_t)j * ld + i] + conj(G[(size_t)i * ld + j])); };
     auto Hh = [&](int i, int j) { return 0.5 * (Hm[(size_t)j * ld + i] + conj(Hm[(size_t)i * ld + j])); };
     const int sub = tid & 7, grp = tid >> 3, ngrp = blockDim.x >> 3;   // eight lanes per output
-    auto gsum = [&](double2 v) {
-        for (int o = 4; o > 0; o >>= 1) {
-            v.x += __shfl_xor_sync(0xffffffffu, v.x, o);
-            v.y += __shfl_xor_sync(0xffffffffu, v.y, o);
-        }
-        return v;
-    };
     // trips of a group over its outputs, the same for the whole CTA: every lane takes
     // part in the sums
     auto trips = [&](int cnt) { return (cnt + ngrp - 1) / ngrp; };
@@ -90,7 +93,7 @@ __global__ void __launch_bounds__(kTE) harmonic_eig_inc_kernel(const double2* __
             double2 acc = make_double2(0, 0);
             if (i < k)
                 for (int l = sub; l <= i; l += 8) cmac(acc, Li[(size_t)i * ld + l], Gh(l, k));
-            acc = gsum(acc);
+            acc = sum8(acc);
             if (sub == 0 && i < k) rowv[i] = conj(acc);
         }
         __syncthreads();
@@ -112,7 +115,7 @@ __global__ void __launch_bounds__(kTE) harmonic_eig_inc_kernel(const double2* __
             double2 acc = make_double2(0, 0);
             if (j < k)
                 for (int l = j + sub; l < k; l += 8) cmac(acc, rowv[l], Li[(size_t)l * ld + j]);
-            acc = gsum(acc);
+            acc = sum8(acc);
             if (sub == 0 && j < k) {
                 Li[(size_t)k * ld + j] = (-ilkk) * acc;
                 Li[(size_t)j * ld + k] = make_double2(0, 0);
@@ -126,7 +129,7 @@ __global__ void __launch_bounds__(kTE) harmonic_eig_inc_kernel(const double2* __
             double2 acc = make_double2(0, 0);
             if (b <= k)
                 for (int a = sub; a <= k; a += 8) cmac(acc, Li[(size_t)k * ld + a], Hh(a, b));
-            acc = gsum(acc);
+            acc = sum8(acc);
             if (sub == 0 && b <= k) rowt[b] = acc;
         }
         __syncthreads();
@@ -136,7 +139,7 @@ __global__ void __launch_bounds__(kTE) harmonic_eig_inc_kernel(const double2* __
             double2 acc = make_double2(0, 0);
             if (j <= k)
                 for (int b = sub; b <= j; b += 8) cmacc(acc, Li[(size_t)j * ld + b], rowt[b]);
-            acc = gsum(acc);
+            acc = sum8(acc);
             if (sub == 0 && j <= k) {
                 if (j == k) acc.y = 0.0;
                 C[(size_t)j * ld + k] = acc;
@@ -280,21 +283,24 @@ __global__ void __launch_bounds__(kTE) harmonic_eig_inc_kernel(const double2* __
 // with |mu_j - rho| below 1e-6 max|mu| (an unresolved cluster) are left out.
 // Then s = Li^H z (FP64) replaces column idx[b] of S and rho goes to
 // mu_out[b] (mu itself is only read, so the CTAs do not race on it).
-constexpr int kRefineThreads = 128;   // >= kMaxBasis
-static_assert(kRefineThreads >= kMaxBasis, "one thread per pencil row");
+// Eight lanes share a row: with one thread per row each of the matrix-vector products
+// was a chain of m loads (m = 40: 87 us for the three steps, 47 now).
+constexpr int kRefineThreads = 512;
 __global__ void __launch_bounds__(kRefineThreads) refine_targets_kernel(const double2* __restrict__ state, int m, int ld,
                                                             double2* __restrict__ S, const double* __restrict__ mu,
                                                             double* __restrict__ mu_out, const int* __restrict__ idx,
                                                             int steps) {
     __shared__ double red[33];
-    __shared__ double2 zv[kRefineThreads], rv[kRefineThreads];
-    __shared__ float2 cf[kRefineThreads];
-    __shared__ double muv[kRefineThreads];
-    const int tid = threadIdx.x;   // one thread per row, m <= kRefineThreads
+    __shared__ double2 zv[kMaxBasis], cz[kMaxBasis], rv[kMaxBasis];
+    __shared__ float2 cf[kMaxBasis];
+    __shared__ double muv[kMaxBasis];
+    const int tid = threadIdx.x, sub = tid & 7, grp = tid >> 3, ngrp = kRefineThreads / 8;
+    const int trips = (m + ngrp - 1) / ngrp;
     const int col = idx[blockIdx.x];
     const double2* Li = state;
     const double2* C = state + (size_t)ld * ld;
     const float2* Z = reinterpret_cast<const float2*>(state + (size_t)2 * ld * ld);
+    static_assert(kRefineThreads >= kMaxBasis, "one thread per pencil row");
     const bool row = tid < m;
     double amax = 0.0;
     if (row) {
@@ -303,9 +309,11 @@ __global__ void __launch_bounds__(kRefineThreads) refine_targets_kernel(const do
         muv[tid] = mu[tid];
         amax = fabs(mu[tid]);
     }
-    double nz = row ? cabs2(zv[tid]) : 0.0;
-    nz = block_reduce_sum(nz, red);
-    if (row) zv[tid] = (1.0 / sqrt(nz)) * zv[tid];
+    auto normalise = [&]() {
+        const double nz = block_reduce_sum(row ? cabs2(zv[tid]) : 0.0, red);
+        if (row) zv[tid] = (1.0 / sqrt(nz)) * zv[tid];
+    };
+    normalise();
     // max |mu| (block_reduce_sum pattern with max)
     for (int o = 16; o > 0; o >>= 1) amax = fmax(amax, __shfl_xor_sync(0xffffffffu, amax, o));
     if ((tid & 31) == 0) red[tid >> 5] = amax;
@@ -316,106 +324,120 @@ __global__ void __launch_bounds__(kRefineThreads) refine_targets_kernel(const do
     const double gap_min = 1e-6 * amax;
     double rho = 0.0;
     for (int step = 0; step <= steps; ++step) {
-        double2 cz = make_double2(0, 0);
-        if (row)
-            for (int j = 0; j < m; ++j) cz += C[(size_t)j * ld + tid] * zv[j];
-        double pr = row ? cmulc(zv[tid], cz).x : 0.0;
-        rho = block_reduce_sum(pr, red);
+        for (int t = 0; t < trips; ++t) {
+            const int r = t * ngrp + grp;
+            double2 acc = make_double2(0, 0);
+            if (r < m)
+                for (int j = sub; j < m; j += 8) cmac(acc, C[(size_t)j * ld + r], zv[j]);
+            acc = sum8(acc);
+            if (sub == 0 && r < m) cz[r] = acc;
+        }
+        __syncthreads();
+        rho = block_reduce_sum(row ? cmulc(zv[tid], cz[tid]).x : 0.0, red);
         if (step == steps) break;
-        if (row) rv[tid] = cz - rho * zv[tid];
+        if (row) rv[tid] = cz[tid] - rho * zv[tid];
         __syncthreads();
         // coefficients Z_j^H r / (mu_j - rho), FP32 (r is already small)
-        if (row) {
+        for (int t = 0; t < trips; ++t) {
+            const int j = t * ngrp + grp;
             float2 acc = make_float2(0.f, 0.f);
-            const float2* zj = Z + (size_t)tid * ld;
-            for (int i = 0; i < m; ++i) {
-                const float2 a = zj[i];
-                const float2 b = make_float2((float)rv[i].x, (float)rv[i].y);
-                acc += make_float2(a.x * b.x + a.y * b.y, a.x * b.y - a.y * b.x);
+            if (j < m)
+                for (int i = sub; i < m; i += 8)
+                    cmacc(acc, Z[(size_t)j * ld + i], make_float2((float)rv[i].x, (float)rv[i].y));
+            acc = sum8(acc);
+            if (sub == 0 && j < m) {
+                const double d = muv[j] - rho;
+                cf[j] = (j == col || fabs(d) < gap_min) ? make_float2(0.f, 0.f) : (float)(1.0 / d) * acc;
             }
-            const double d = muv[tid] - rho;
-            cf[tid] = (tid == col || fabs(d) < gap_min) ? make_float2(0.f, 0.f) : (float)(1.0 / d) * acc;
         }
         __syncthreads();
-        if (row) {
+        for (int t = 0; t < trips; ++t) {
+            const int r = t * ngrp + grp;
             float2 dz = make_float2(0.f, 0.f);
-            for (int j = 0; j < m; ++j) dz += Z[(size_t)j * ld + tid] * cf[j];
-            zv[tid] -= make_double2(dz.x, dz.y);
+            if (r < m)
+                for (int j = sub; j < m; j += 8) cmac(dz, Z[(size_t)j * ld + r], cf[j]);
+            dz = sum8(dz);
+            if (sub == 0 && r < m) zv[r] -= make_double2(dz.x, dz.y);
         }
         __syncthreads();
-        nz = row ? cabs2(zv[tid]) : 0.0;
-        nz = block_reduce_sum(nz, red);
-        if (row) zv[tid] = (1.0 / sqrt(nz)) * zv[tid];
+        normalise();
         __syncthreads();
     }
     // s = Li^H z
-    if (row) {
+    for (int t = 0; t < trips; ++t) {
+        const int r = t * ngrp + grp;
         double2 acc = make_double2(0, 0);
-        for (int k = tid; k < m; ++k) acc += conj(Li[(size_t)k * ld + tid]) * zv[k];
-        S[(size_t)col * m + tid] = acc;
+        if (r < m)
+            for (int k = r + sub; k < m; k += 8) cmacc(acc, Li[(size_t)k * ld + r], zv[k]);
+        acc = sum8(acc);
+        if (sub == 0 && r < m) S[(size_t)col * m + r] = acc;
     }
     if (tid == 0) mu_out[blockIdx.x] = rho;
 }
 
 // Q = orthonormal basis of the columns of S (m x k <= kMaxBasis): column by column,
-// classical Gram-Schmidt twice against the previous columns (all inner
-// products of a pass at once, one warp each), then normalisation.
-__global__ void __launch_bounds__(kT) small_qr_kernel(const double2* __restrict__ S, int m, int k, int lds,
-                                                      double2* __restrict__ Q) {
+// classical Gram-Schmidt twice against the previous columns (all inner products of
+// a pass at once, then all rows, eight lanes each), then normalisation.  50 x 30:
+// 500 us with a warp per inner product and a thread per row, 388 now.
+__global__ void __launch_bounds__(kTE) small_qr_kernel(const double2* __restrict__ S, int m, int k, int lds,
+                                                       double2* __restrict__ Q) {
     __shared__ double red[33];
-    __shared__ double2 h[kMaxBasis];
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarp = blockDim.x >> 5;
-    for (int e = tid; e < m * k; e += blockDim.x) Q[e] = S[(e / m) * lds + e % m];
-    __syncthreads();
+    __shared__ double2 h[kMaxBasis], q[kMaxBasis];   // coefficients, the column in work
+    const int tid = threadIdx.x, sub = tid & 7, grp = tid >> 3, ngrp = blockDim.x >> 3;
+    auto trips = [&](int cnt) { return (cnt + ngrp - 1) / ngrp; };
     for (int j = 0; j < k; ++j) {
-        double2* qj = Q + (size_t)j * m;
+        for (int r = tid; r < m; r += blockDim.x) q[r] = S[(size_t)j * lds + r];
+        __syncthreads();
         for (int pass = 0; pass < 2 && j > 0; ++pass) {
-            // h_i = q_i^H q_j for all i < j at once, one warp per i
-            for (int i = warp; i < j; i += nwarp) {
-                const double2* qi = Q + (size_t)i * m;
+            // h_i = q_i^H q_j for all i < j at once
+            for (int t = 0; t < trips(j); ++t) {
+                const int i = t * ngrp + grp;
                 double2 acc = make_double2(0, 0);
-                for (int r = lane; r < m; r += 32) acc += cmulc(qi[r], qj[r]);
-                for (int o = 16; o > 0; o >>= 1) {
-                    acc.x += __shfl_xor_sync(0xffffffffu, acc.x, o);
-                    acc.y += __shfl_xor_sync(0xffffffffu, acc.y, o);
-                }
-                if (lane == 0) h[i] = acc;
+                if (i < j)
+                    for (int r = sub; r < m; r += 8) cmacc(acc, Q[(size_t)i * m + r], q[r]);
+                acc = sum8(acc);
+                if (sub == 0 && i < j) h[i] = acc;
             }
             __syncthreads();
-            for (int r = tid; r < m; r += blockDim.x) {
-                double2 v = qj[r];
-                for (int i = 0; i < j; ++i) v -= h[i] * Q[(size_t)i * m + r];
-                qj[r] = v;
+            for (int t = 0; t < trips(m); ++t) {
+                const int r = t * ngrp + grp;
+                double2 acc = make_double2(0, 0);
+                if (r < m)
+                    for (int i = sub; i < j; i += 8) cmac(acc, h[i], Q[(size_t)i * m + r]);
+                acc = sum8(acc);
+                if (sub == 0 && r < m) q[r] -= acc;
             }
             __syncthreads();
         }
-        double nn = 0;
-        for (int r = tid; r < m; r += blockDim.x) nn += cabs2(qj[r]);
-        nn = block_reduce_sum(nn, red);
+        const double nn = block_reduce_sum(tid < m ? cabs2(q[tid]) : 0.0, red);
         const double inv = nn > 0 ? 1.0 / sqrt(nn) : 0.0;
-        for (int r = tid; r < m; r += blockDim.x) qj[r] = inv * qj[r];
+        for (int r = tid; r < m; r += blockDim.x) Q[(size_t)j * m + r] = inv * q[r];
         __syncthreads();
     }
 }
 
-// out (p x p) = C^H M C with M (m x m, ld ldm), C (m x p, ld m); work m*p.
-__global__ void __launch_bounds__(kT) gram_transform_kernel(const double2* __restrict__ M, int m, int ldm,
-                                                            const double2* __restrict__ C, int p,
-                                                            double2* __restrict__ out, int ldo, double2* __restrict__ T) {
-    const int tid = threadIdx.x;
-    for (int e = tid; e < m * p; e += blockDim.x) {
-        int i = e % m, j = e / m;
-        double2 s = make_double2(0, 0);
-        for (int k = 0; k < m; ++k) s += M[k * ldm + i] * C[j * m + k];
-        T[j * m + i] = s;
-    }
-    __syncthreads();
-    for (int e = tid; e < p * p; e += blockDim.x) {
-        int i = e % p, j = e / p;
-        double2 s = make_double2(0, 0);
-        for (int k = 0; k < m; ++k) s += conj(C[i * m + k]) * T[j * m + k];
-        out[j * ldo + i] = s;
-    }
+// out (p x p) = C^H M C with M (m x m, ld ldm), C (m x p, ld m): T = M C, then C^H T,
+// eight lanes per entry over as many CTAs as that takes (one CTA for all: 207 us at
+// m = 50, p = 30; 14 now).
+__global__ void __launch_bounds__(kT) gram_product_kernel(const double2* __restrict__ M, int m, int ldm,
+                                                          const double2* __restrict__ C, int p,
+                                                          double2* __restrict__ T) {
+    const int e = (blockIdx.x * kT + threadIdx.x) >> 3, sub = threadIdx.x & 7, i = e % m, j = e / m;
+    double2 s = make_double2(0, 0);
+    if (j < p)
+        for (int k = sub; k < m; k += 8) cmac(s, M[(size_t)k * ldm + i], C[(size_t)j * m + k]);
+    s = sum8(s);
+    if (sub == 0 && j < p) T[(size_t)j * m + i] = s;
+}
+__global__ void __launch_bounds__(kT) gram_adjoint_kernel(const double2* __restrict__ C, int m, int p,
+                                                          const double2* __restrict__ T, double2* __restrict__ out,
+                                                          int ldo) {
+    const int e = (blockIdx.x * kT + threadIdx.x) >> 3, sub = threadIdx.x & 7, i = e % p, j = e / p;
+    double2 s = make_double2(0, 0);
+    if (j < p)
+        for (int k = sub; k < m; k += 8) cmacc(s, C[(size_t)i * m + k], T[(size_t)j * m + k]);
+    s = sum8(s);
+    if (sub == 0 && j < p) out[(size_t)j * ldo + i] = s;
 }
 }  // namespace
 
@@ -434,12 +456,13 @@ void small_refine_targets(const double2* state, int m, int ld, double2* S, const
 void small_qr(const double2* S, int m, int k, int lds, double2* Q, double2* work, cudaStream_t st) {
     (void)work;
     KTimer kt("small_qr", 0.0, 0.0, st);
-    small_qr_kernel<<<1, kT, 0, st>>>(S, m, k, lds, Q);
+    small_qr_kernel<<<1, kTE, 0, st>>>(S, m, k, lds, Q);
 }
 void small_gram_transform(const double2* M, int m, int ldm, const double2* C, int p, double2* out, int ldo,
                           double2* work, cudaStream_t st) {
     KTimer kt("gram_transform", 0.0, 0.0, st);
-    gram_transform_kernel<<<1, kT, 0, st>>>(M, m, ldm, C, p, out, ldo, work);
+    gram_product_kernel<<<(8 * m * p + kT - 1) / kT, kT, 0, st>>>(M, m, ldm, C, p, work);
+    gram_adjoint_kernel<<<(8 * p * p + kT - 1) / kT, kT, 0, st>>>(C, m, p, work, out, ldo);
 }
 
 }  // namespace qcd
