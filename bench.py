@@ -110,13 +110,12 @@ def max_over_ranks(value, device=None):
 # DRAM bytes per launch (dram__bytes_read.sum + dram__bytes_write.sum) from
 # one ncu capture of each kernel as it stands now, for the roofline's
 # "traffic"; a kernel that changes is taken out of this table until it is
-# captured again (the field is then null).  coarse_gmres_f32: two launches of
-# coarse_gmres_kernel<float2, float> in the 16 x 8^3 step (k = 4, 4 targets),
-# dram__bytes.sum.per_second x gpu__time_duration.sum = 9.808 and 9.820 MB
-# (profiles/coarse_gmres_f32_c2_16x8c3.md).  sap_block_f32: two launches of
-# sap_chi_kernel<float, float2> in the same step (four block solves per CTA),
-# 6.8831 and 6.8836 MB read, 0 written (profiles/sap_chi_f32_c2_16x8c3.md).
-NCU_TRAFFIC = {"coarse_gmres_f32": 9.814e6, "sap_block_f32": 6.8833e6}
+# captured again (the field is then null).  Two launches each in the 16 x 8^3
+# step (k = 4, 4 targets; profiles/case_kernels.md): coarse_gmres_f32
+# (coarse_gmres_kernel<float2, float>) 9.7997 and 9.7999 MB read; sap_block_f32
+# (sap_cube_kernel<float, float2>, up to four block solves per CTA) 8.8131 MB
+# read, nothing written.
+NCU_TRAFFIC = {"coarse_gmres_f32": 9.7998e6, "sap_block_f32": 8.8131e6}
 
 # Work model of the SAP block solves for the FP32-ALU roofline, per block
 # site and GMRES step j (0-based) of a block solve of k steps: the Dirichlet
