@@ -73,7 +73,7 @@ __global__ void __launch_bounds__(kTE) harmonic_eig_inc_kernel(const double2* __
     __shared__ double red[33];
     __shared__ int pp[kPairs], qq[kPairs];
     __shared__ float2 pj[kPairs][3];   // per pair: (c, s), e^{i phi}, unused
-    __shared__ double2 rowv[kMaxBasis], rowt[kMaxBasis];
+    __shared__ double2 rowv[kMaxBasis], rowt[kMaxBasis], colg[kMaxBasis];
     __shared__ double lkk_s;
     extern __shared__ double2 shm[];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -81,18 +81,28 @@ __global__ void __launch_bounds__(kTE) harmonic_eig_inc_kernel(const double2* __
     double2* C = state + (size_t)ld * ld;         // Hermitian, both triangles stored
     float2* Zg = reinterpret_cast<float2*>(state + (size_t)2 * ld * ld);   // column-major
     auto Gh = [&](int i, int j) { return 0.5 * (G[(size_t)j * ld + i] + conj(G[(size_t)i * ld + j])); };
-    auto Hh = [&](int i, int j) { return 0.5 * (Hm[(size_t)j * ld + i] + conj(Hm[(size_t)i * ld + j])); };
     const int sub = tid & 7, grp = tid >> 3, ngrp = blockDim.x >> 3;   // eight lanes per output
     // trips of a group over its outputs, the same for the whole CTA: every lane takes
     // part in the sums
     auto trips = [&](int cnt) { return (cnt + ngrp - 1) / ngrp; };
+    // the Hermitian part of H once, where the FP32 matrices live later (the same bytes),
+    // and of G's column a row ahead: formed in the products below it took as many FP64
+    // operations as they do
+    double2* Hs = shm;
+    for (int e = tid; e < m * m; e += blockDim.x) {
+        const int i = e % m, j = e / m;
+        Hs[e] = 0.5 * (Hm[(size_t)j * ld + i] + conj(Hm[(size_t)i * ld + j]));
+    }
+    if (m0 < m)
+        for (int l = tid; l <= m0; l += blockDim.x) colg[l] = Gh(l, m0);
+    __syncthreads();
     for (int k = m0; k < m; ++k) {
         // l = conj(Li[0:k,0:k] G[0:k,k])
         for (int t = 0; t < trips(k); ++t) {
             const int i = t * ngrp + grp;
             double2 acc = make_double2(0, 0);
             if (i < k)
-                for (int l = sub; l <= i; l += 8) cmac(acc, Li[(size_t)i * ld + l], Gh(l, k));
+                for (int l = sub; l <= i; l += 8) cmac(acc, Li[(size_t)i * ld + l], colg[l]);
             acc = sum8(acc);
             if (sub == 0 && i < k) rowv[i] = conj(acc);
         }
@@ -102,7 +112,7 @@ __global__ void __launch_bounds__(kTE) harmonic_eig_inc_kernel(const double2* __
             for (int i = lane; i < k; i += 32) nn += rowv[i].x * rowv[i].x + rowv[i].y * rowv[i].y;
             for (int o = 16; o > 0; o >>= 1) nn += __shfl_xor_sync(0xffffffffu, nn, o);
             if (lane == 0) {
-                double d = Gh(k, k).x - nn;
+                double d = colg[k].x - nn;
                 if (!(d > 0.0)) { status[0] = 1; d = 1e-300; }
                 lkk_s = sqrt(d);
             }
@@ -128,11 +138,13 @@ __global__ void __launch_bounds__(kTE) harmonic_eig_inc_kernel(const double2* __
             const int b = t * ngrp + grp;
             double2 acc = make_double2(0, 0);
             if (b <= k)
-                for (int a = sub; a <= k; a += 8) cmac(acc, Li[(size_t)k * ld + a], Hh(a, b));
+                for (int a = sub; a <= k; a += 8) cmac(acc, Li[(size_t)k * ld + a], Hs[b * m + a]);
             acc = sum8(acc);
             if (sub == 0 && b <= k) rowt[b] = acc;
         }
         __syncthreads();
+        if (k + 1 < m)
+            for (int l = tid; l <= k + 1; l += blockDim.x) colg[l] = Gh(l, k + 1);
         // C[k, j] = t . conj(Li[j, :]), j <= k
         for (int t = 0; t < trips(k + 1); ++t) {
             const int j = t * ngrp + grp;
