@@ -60,7 +60,9 @@ __device__ double block_reduce_sum(double v, double* red) {
 // eigenvectors: in the basis Z0 (+) I the matrix is diag(mu_prev) bordered by
 // Z0^H C[0:m0, m0:m] and C[m0:m, m0:m], which a few sweeps finish.  Each
 // round applies the disjoint rotations J of its pairs as 2x2 blocks
-// J_P^H A[P, Q] J_Q, one thread per block, so a round needs two barriers.
+// J_P^H A[P, Q] J_Q, one thread per block, so a round needs two barriers; two warps
+// find the next round's rotations, a chain of square roots and divisions, while the
+// others turn the eigenvectors.
 // The sweeps stop once the off-diagonal mass reaches the FP32 round-off
 // floor, 4 m^2 u^2 ||C||_F^2 (u = 2^-24), or stops decreasing.  Outputs mu
 // (eigenvalues of C, previous values read from mu when m0 > 0), S = Li^H Z
@@ -71,8 +73,9 @@ __global__ void __launch_bounds__(kTE) harmonic_eig_inc_kernel(const double2* __
                                                               double2* __restrict__ state, int* __restrict__ status) {
     constexpr int kPairs = kMaxBasis / 2 + 1;
     __shared__ double red[33];
-    __shared__ int pp[kPairs], qq[kPairs];
-    __shared__ float2 pj[kPairs][3];   // per pair: (c, s), e^{i phi}, unused
+    // per round (two of them): the pairs, (c, s) and e^{i phi}
+    __shared__ int pairs[2][kPairs][2];
+    __shared__ float2 angles[2][kPairs][2];
     __shared__ double2 rowv[kMaxBasis], rowt[kMaxBasis], colg[kMaxBasis];
     __shared__ double lkk_s;
     extern __shared__ double2 shm[];
@@ -200,6 +203,34 @@ __global__ void __launch_bounds__(kTE) harmonic_eig_inc_kernel(const double2* __
     fro = (float)block_reduce_sum((double)fro, red);
     const float floor_off = 4.0f * (float)(m * m) * 3.5527137e-15f * fro;   // 4 m^2 (2^-24)^2 ||C||^2
     float prev_off = 3.0e38f;
+    constexpr int kAngleT = 64;
+    static_assert(kPairs <= kAngleT, "one thread per pair");
+    // rotations of a round from A as it stands
+    auto rotations = [&](int rnd, int to) {
+        if (tid >= npair) return;
+        auto player = [&](int pos) { return pos == 0 ? 0 : ((rnd + pos - 1) % (mm - 1)) + 1; };
+        int p = player(tid), q = player(mm - 1 - tid);
+        if (p > q) { int t = p; p = q; q = t; }
+        float c = 1.f, sv = 0.f;
+        float2 ph = make_float2(1.f, 0.f);
+        if (q < m) {
+            const float2 b = Af[IDX(p, q)];
+            const float ab = sqrtf(b.x * b.x + b.y * b.y);
+            if (ab > 1e-30f) {
+                ph = make_float2(b.x / ab, b.y / ab);
+                const float zeta = (Af[IDX(q, q)].x - Af[IDX(p, p)].x) / (2.0f * ab);
+                const float t = (zeta >= 0 ? 1.0f : -1.0f) / (fabsf(zeta) + sqrtf(1.0f + zeta * zeta));
+                c = rsqrtf(1.0f + t * t);
+                sv = t * c;
+            }
+        }
+        pairs[to][tid][0] = p;
+        pairs[to][tid][1] = q;
+        angles[to][tid][0] = make_float2(c, sv);
+        angles[to][tid][1] = ph;
+    };
+    int buf = 0;
+    if (m > 1) rotations(0, 0);
     for (int sweep = 0; sweep < 40 && m > 1; ++sweep) {
         float off = 0.0f;
         for (int e = tid; e < m * m; e += blockDim.x)
@@ -207,33 +238,14 @@ __global__ void __launch_bounds__(kTE) harmonic_eig_inc_kernel(const double2* __
         off = (float)block_reduce_sum((double)off, red);
         if (off <= floor_off || off >= prev_off) break;
         prev_off = off;
-        for (int rnd = 0; rnd < mm - 1; ++rnd) {
-            if (tid < npair) {
-                auto player = [&](int pos) { return pos == 0 ? 0 : ((rnd + pos - 1) % (mm - 1)) + 1; };
-                int p = player(tid), q = player(mm - 1 - tid);
-                if (p > q) { int t = p; p = q; q = t; }
-                float c = 1.f, sv = 0.f;
-                float2 ph = make_float2(1.f, 0.f);
-                if (q < m) {
-                    const float2 b = Af[IDX(p, q)];
-                    const float ab = sqrtf(b.x * b.x + b.y * b.y);
-                    if (ab > 1e-30f) {
-                        ph = make_float2(b.x / ab, b.y / ab);
-                        const float zeta = (Af[IDX(q, q)].x - Af[IDX(p, p)].x) / (2.0f * ab);
-                        const float t = (zeta >= 0 ? 1.0f : -1.0f) / (fabsf(zeta) + sqrtf(1.0f + zeta * zeta));
-                        c = rsqrtf(1.0f + t * t);
-                        sv = t * c;
-                    }
-                }
-                pp[tid] = p; qq[tid] = q;
-                pj[tid][0] = make_float2(c, sv);
-                pj[tid][1] = ph;
-            }
-            __syncthreads();
+        for (int rnd = 0; rnd < mm - 1; ++rnd, buf ^= 1) {
+            __syncthreads();   // rotations of this round ready, Z of the last one done
+            const auto& pr = pairs[buf];
+            const auto& pj = angles[buf];
             // J = [[c, s], [-s conj(ph), c conj(ph)]] on columns (p, q); rows get J^H
             for (int e = tid; e < npair * npair; e += blockDim.x) {
                 const int P = e % npair, Q = e / npair;
-                const int p1 = pp[P], q1 = qq[P], p2 = pp[Q], q2 = qq[Q];
+                const int p1 = pr[P][0], q1 = pr[P][1], p2 = pr[Q][0], q2 = pr[Q][1];
                 const bool v1 = q1 < m, v2 = q2 < m;
                 const float2 cs1 = pj[P][0], e1 = pj[P][1], cs2 = pj[Q][0], e2 = pj[Q][1];
                 const float2 a00 = Af[IDX(p1, p2)];
@@ -250,19 +262,25 @@ __global__ void __launch_bounds__(kTE) harmonic_eig_inc_kernel(const double2* __
                 if (v1) Af[IDX(q1, p2)] = cs1.y * t00 + cs1.x * (e1 * t10);
                 if (v1 && v2) Af[IDX(q1, q2)] = cs1.y * t01 + cs1.x * (e1 * t11);
             }
-            for (int e = tid; e < npair * m; e += blockDim.x) {
-                const int r = e % m, Q = e / m;
-                const int p = pp[Q], q = qq[Q];
-                if (q >= m) continue;
-                const float2 cs = pj[Q][0], ph = pj[Q][1];
-                const float2 em = make_float2(ph.x, -ph.y);
-                const float2 zp = Zf[IDX(r, p)], zq = Zf[IDX(r, q)];
-                Zf[IDX(r, p)] = cs.x * zp - cs.y * (em * zq);
-                Zf[IDX(r, q)] = cs.y * zp + cs.x * (em * zq);
-            }
             __syncthreads();
+            // two warps find the next round's rotations while the others turn Z
+            if (tid < kAngleT) {
+                rotations(rnd + 1 < mm - 1 ? rnd + 1 : 0, buf ^ 1);
+            } else {
+                for (int e = tid - kAngleT; e < npair * m; e += kTE - kAngleT) {
+                    const int r = e % m, Q = e / m;
+                    const int p = pr[Q][0], q = pr[Q][1];
+                    if (q >= m) continue;
+                    const float2 cs = pj[Q][0], ph = pj[Q][1];
+                    const float2 em = make_float2(ph.x, -ph.y);
+                    const float2 zp = Zf[IDX(r, p)], zq = Zf[IDX(r, q)];
+                    Zf[IDX(r, p)] = cs.x * zp - cs.y * (em * zq);
+                    Zf[IDX(r, q)] = cs.y * zp + cs.x * (em * zq);
+                }
+            }
         }
     }
+    __syncthreads();
     for (int i = tid; i < m; i += blockDim.x) mu[i] = (double)Af[IDX(i, i)].x;
     for (int e = tid; e < m * m; e += blockDim.x) Zg[(size_t)(e / m) * ld + (e % m)] = Zf[e];
     __syncthreads();
