@@ -160,14 +160,15 @@ template <int N> __device__ __forceinline__ void async_wait() { asm volatile("cp
 // stage, through a ring of kRing stages of asynchronous copies (loading into
 // registers kept one stage, 18 KB per SM, in flight and ran at 1.6 TB/s).
 // 32 x 16^3, 4^4 aggregates, nv 20, 16 right-hand sides: 786 us with
-// one chunk of 8 per pass and one warp per vector -> 143 us (3.2 TB/s, 47 % of the
-// FMA pipe; prologue of a single resident CTA per SM not hidden).
+// one chunk of 8 per pass and one warp per vector -> 154 us (3.0 TB/s; prologue of a
+// single resident CTA per SM not hidden); 143 us with one chain of fused
+// multiply-adds per sum.
 template <typename R> constexpr int kTransferRhs = sizeof(R) == 4 ? 16 : 8;
 constexpr int kRestrictTI = 4;
-constexpr int kRing = 4, kStage = 64;
+constexpr int kRing = 4, kStage = 64;   // a stage: two pieces of a row per lane
 constexpr int kSiteTable = 1024;   // aggregates up to this size look their entries up
 template <typename R, int E, int TJ>
-__global__ void __launch_bounds__(TJ == 4 ? 640 : 512) restrict_tile_kernel(
+__global__ void __launch_bounds__(TJ == 4 && sizeof(R) == 4 ? 640 : 512) restrict_tile_kernel(
     Geom g, Blocking B, int nv, const cplx<R>* __restrict__ P, const cplx<R>* __restrict__ r, cplx<R>* __restrict__ xc,
     int nrhs, int ring, const int* __restrict__ act) {
     constexpr int TI = kRestrictTI;
@@ -227,19 +228,25 @@ __global__ void __launch_bounds__(TJ == 4 ? 640 : 512) restrict_tile_kernel(
         next = cur;
         const Pc* sp = stage + cur;
         cur = cur + slots == kRing * slots ? 0 : cur + slots;
+        // the products of a stage by themselves, then into the running sum, which so
+        // rounds once in 2 E products (in the chain of all of them it rounds twice in
+        // each; 4^4 aggregates: 1.0e-7 from the exact sum against 1.9e-7)
+        Pc a[2][TI];
 #pragma unroll
-        for (int h = 0; h < kStage; h += 32) {
-            Pc a[TI];
+        for (int q = 0; q < TI; ++q) {
+            a[0][q] = sp[ra[q]];
+            a[1][q] = sp[ra[q] + 32];
+        }
 #pragma unroll
-            for (int q = 0; q < TI; ++q) a[q] = sp[ra[q] + h];
+        for (int u = 0; u < TJ; ++u) {
+            const Pc b[2] = {sp[ru[u]], sp[ru[u] + 32]};
 #pragma unroll
-            for (int u = 0; u < TJ; ++u) {
-                const Pc b = sp[ru[u] + h];
+            for (int q = 0; q < TI; ++q) {
+                cplx<R> t = cmulc(a[0][q].at(0), b[0].at(0));
 #pragma unroll
-                for (int k = 0; k < E; ++k)
-#pragma unroll
-                    for (int q = 0; q < TI; ++q)
-                        cdot(acc[(q * TJ + u) * 2], acc[(q * TJ + u) * 2 + 1], a[q].at(k), b.at(k));
+                for (int k = 1; k < 2 * E; ++k) cmacc(t, a[k / E][q].at(k % E), b[k / E].at(k % E));
+                acc[(q * TJ + u) * 2] += t.x;
+                acc[(q * TJ + u) * 2 + 1] += t.y;
             }
         }
     }
@@ -265,11 +272,12 @@ __global__ void __launch_bounds__(TJ == 4 ? 640 : 512) restrict_tile_kernel(
 // L2.  P comes by asynchronous copies kAhead rows ahead into a ring that each
 // thread fills and reads for itself (no barrier).
 // 32 x 16^3, 4^4 aggregates, nv 20, 16 right-hand sides: 339 us ->
-// 145 us (3.1 TB/s, 46 % of the FMA pipe).
+// 153 us (3.0 TB/s) at five CTAs per SM; 145 us with one chain of fused multiply-adds
+// per sum, four or six CTAs 165 / 158 us.
 constexpr int kAhead = 8;
 constexpr int kProlongT = 96;   // whole warps and whole sites: both pieces lie at the same place of a site
 template <typename R, int E, int TJ>
-__global__ void __launch_bounds__(kProlongT) prolong_tile_kernel(Geom g, Blocking B, int nv,
+__global__ void __launch_bounds__(kProlongT, 5) prolong_tile_kernel(Geom g, Blocking B, int nv,
                                                                  const cplx<R>* __restrict__ P,
                                                                  const cplx<R>* __restrict__ xc, cplx<R>* __restrict__ x,
                                                                  int nrhs, int parts, const int* __restrict__ act) {
@@ -279,7 +287,7 @@ __global__ void __launch_bounds__(kProlongT) prolong_tile_kernel(Geom g, Blockin
     extern __shared__ __align__(16) unsigned char psm[];
     Pc* ring = reinterpret_cast<Pc*>(psm) + threadIdx.x;   // [kAhead][2][T]
     cplx<R>* cs = reinterpret_cast<cplx<R>*>(psm + sizeof(Pc) * kAhead * 2 * T);
-    const int nc = 2 * nv, nloc = B.bs * 6, half = nv * TJ + 2;
+    const int nc = 2 * nv, nloc = B.bs * 6, half = (nv + (nv & 1)) * TJ + 2;
     const int groups = (nrhs + TJ - 1) / TJ;
     const int j0 = (blockIdx.x % groups) * TJ, part = (blockIdx.x / groups) % parts, blk = blockIdx.x / groups / parts;
     const int l = 2 * part * kStep + threadIdx.x / kPer, w = threadIdx.x % kPer;
@@ -298,13 +306,14 @@ __global__ void __launch_bounds__(kProlongT) prolong_tile_kernel(Geom g, Blockin
         async_commit();
     };
 #pragma unroll
-    for (int i = 0; i < kAhead - 1; ++i) fill(i);
+    for (int i = 0; i < kAhead - 2; ++i) fill(i);
     for (int e = threadIdx.x; e < nc * TJ; e += T) {
         const int i = e % nc, u = e / nc;
         cplx<R> v = czero<R>();
         if (j0 + u < nrhs) v = xc[(size_t)(j0 + u) * B.nb * nc + (size_t)blk * nc + i];
         cs[(i / nv) * half + (i % nv) * TJ + u] = v;
     }
+    if ((nv & 1) && threadIdx.x < 2 * TJ) cs[threadIdx.x / TJ * half + nv * TJ + threadIdx.x % TJ] = czero<R>();
     __syncthreads();
     const cplx<R>* c = cs + chi * half;
     cplx<R> acc[2][TJ][E];
@@ -314,18 +323,28 @@ __global__ void __launch_bounds__(kProlongT) prolong_tile_kernel(Geom g, Blockin
         for (int u = 0; u < TJ; ++u)
 #pragma unroll
             for (int k = 0; k < E; ++k) acc[h][u][k] = czero<R>();
-    for (int i = 0; i < nv; ++i) {
-        async_wait<kAhead - 2>();
-        const Pc a0 = ring[(i % kAhead) * 2 * T], a1 = ring[((i % kAhead) * 2 + (two ? 1 : 0)) * T];
+    // two rows at a time, summed by themselves before they join the running sum (one
+    // chain over all rows: 1.14e-7 from the exact sum against 7.4e-8 at nv 20)
+    const int second = two ? T : 0;
+    for (int i = 0; i < nv; i += 2) {
+        async_wait<kAhead - 4>();
+        // past the last of an odd number: the same row again, times the zeros behind it
+        const bool pair = i + 1 < nv;
+        const Pc *r0 = ring + (i % kAhead) * 2 * T, *r1 = pair ? ring + ((i + 1) % kAhead) * 2 * T : r0;
+        const Pc a[2][2] = {{r0[0], r0[second]}, {r1[0], r1[second]}};   // [row][piece]
+        fill(i + kAhead - 2);
         fill(i + kAhead - 1);
 #pragma unroll
         for (int u = 0; u < TJ; ++u) {
-            const cplx<R> v = c[i * TJ + u];
+            const cplx<R> v = c[i * TJ + u], w = c[(i + 1) * TJ + u];
 #pragma unroll
-            for (int k = 0; k < E; ++k) {
-                cmac(acc[0][u][k], a0.at(k), v);
-                cmac(acc[1][u][k], a1.at(k), v);
-            }
+            for (int h = 0; h < 2; ++h)
+#pragma unroll
+                for (int k = 0; k < E; ++k) {
+                    cplx<R> t = a[0][h].at(k) * v;
+                    cmac(t, a[1][h].at(k), w);
+                    acc[h][u][k] += t;
+                }
         }
     }
 #pragma unroll
@@ -1714,7 +1733,7 @@ static void launch_prolong(const FineOp& f, const Coarse& c, int nrhs, const cpl
                            cudaStream_t st, const int* act) {
     const int parts = (c.B.bs * 12 / E + 2 * kProlongT - 1) / (2 * kProlongT);
     const unsigned grid = (unsigned)c.B.nb * parts * ((nrhs + TJ - 1) / TJ);
-    const size_t sm = sizeof(Piece<R, E>) * kAhead * 2 * kProlongT + 2 * (size_t)(c.nv * TJ + 2) * sizeof(cplx<R>);
+    const size_t sm = sizeof(Piece<R, E>) * kAhead * 2 * kProlongT + 2 * (size_t)((c.nv + (c.nv & 1)) * TJ + 2) * sizeof(cplx<R>);
     prolong_tile_kernel<R, E, TJ><<<grid, kProlongT, sm, st>>>(f.g, c.B, c.nv, P, (const cplx<R>*)xc, (cplx<R>*)x, nrhs,
                                                                parts, act);
 }
