@@ -340,7 +340,9 @@ __device__ __forceinline__ void coarse_row(const CoarseArgs<Z, R>& a, const Z* x
         }
         const Z* am = a.A + (((size_t)s * 9 + d) * a.nc) * a.nc + r;
         const Z* xs = xj + (size_t)sn * a.nc;
-        for (int col = 0; col < a.nc; ++col) cmac(acc, am[(size_t)col * a.nc], xs[col]);
+        Z part; part.x = 0; part.y = 0;   // a direction by itself rounds less than one chain over all
+        for (int col = 0; col < a.nc; ++col) cmac(part, am[(size_t)col * a.nc], xs[col]);
+        acc += part;
     }
     const R sg = r < a.nc / 2 ? R(1) : R(-1);
     Z xv = xj[(size_t)s * a.nc + r];
@@ -589,14 +591,30 @@ __global__ void __launch_bounds__(256) coarse_gmres_kernel(CoarseArgs<Z, R> a) {
 #pragma unroll
                 for (int q = 0; q < 4; ++q) { acc[q >> 1][q & 1].x = 0; acc[q >> 1][q & 1].y = 0; }
                 const Pair<Z>* ap = reinterpret_cast<const Pair<Z>*>(am + (size_t)sub * nc);
-#pragma unroll 4
-                for (int dc = sub; dc < 9 * nc; dc += 4, ap += 2 * nc) {
+                // two columns are summed before they join the running sum: a chain of
+                // fused multiply-adds over all of them would round it twice per column
+                int dc = sub;
+                auto add = [](Z& s, Z m, Z u, Z m2, Z u2) {
+                    Z t = m * u;
+                    cmac(t, m2, u2);
+                    s += t;
+                };
+#pragma unroll 2
+                for (; dc + 4 < 9 * nc; dc += 8, ap += 4 * nc) {
+                    const Pair<Z> m = ap[0], m2 = ap[2 * nc];
+                    const Z u0 = x0[dc], u1 = x1[dc], v0 = x0[dc + 4], v1 = x1[dc + 4];
+                    add(acc[0][0], m.a, u0, m2.a, v0);
+                    add(acc[0][1], m.b, u0, m2.b, v0);
+                    add(acc[1][0], m.a, u1, m2.a, v1);
+                    add(acc[1][1], m.b, u1, m2.b, v1);
+                }
+                if (dc < 9 * nc) {
                     const Pair<Z> m = *ap;
                     const Z u0 = x0[dc], u1 = x1[dc];
-                    cmac(acc[0][0], m.a, u0);
-                    cmac(acc[0][1], m.b, u0);
-                    cmac(acc[1][0], m.a, u1);
-                    cmac(acc[1][1], m.b, u1);
+                    acc[0][0] += m.a * u0;
+                    acc[0][1] += m.b * u0;
+                    acc[1][0] += m.a * u1;
+                    acc[1][1] += m.b * u1;
                 }
                 const bool hi = sub & 2, odd = sub & 1;   // lane bits 16 and 8
                 Z k0 = hi ? acc[1][0] : acc[0][0], k1 = hi ? acc[1][1] : acc[0][1];

@@ -556,13 +556,20 @@ __global__ void coarse_apply_mrhs_kernel(Geom gc, int nc, const Z* __restrict__ 
     for (int d = 0; d < 9; ++d) {
         const Z* Ad = As + (size_t)d * nc * nc;
         const Z* xd = xs + (size_t)d * nc * rc + grp * kCoarseRPT;
+        // a direction by itself: one chain over all nine was 1.35 times as far from
+        // the exact sum as products added one by one, this is less than half as far
+        Z part[kCoarseRPT];
+#pragma unroll
+        for (int k = 0; k < kCoarseRPT; ++k) { part[k].x = 0; part[k].y = 0; }
 #pragma unroll 4
         for (int col = 0; col < nc; ++col) {
             const Z a = __ldg(Ad + (size_t)col * nc);
             const Z* xv = xd + (size_t)col * rc;
 #pragma unroll
-            for (int k = 0; k < kCoarseRPT; ++k) cmac(acc[k], a, xv[k]);
+            for (int k = 0; k < kCoarseRPT; ++k) cmac(part[k], a, xv[k]);
         }
+#pragma unroll
+        for (int k = 0; k < kCoarseRPT; ++k) acc[k] += part[k];
     }
     const R sg = r < nc / 2 ? R(1) : R(-1);
 #pragma unroll

@@ -1,8 +1,8 @@
 """Long sums of complex products are no further from the exact ones (extended
 precision, on the data as the library holds it) than serial sums in the working
 precision that round each product before it is added: the lanes of a warp along an
-aggregate's entries, added at the end, for the restriction, and the test vectors in
-turn for the prolongation.  Chains of fused multiply-adds through the running sum
+aggregate's entries, added at the end, for the restriction, the test vectors in
+turn for the prolongation, the columns of the nine blocks for the coarse stencil.  Chains of fused multiply-adds through the running sum
 round it twice per product and are 1.25 to 1.4 times as far."""
 import numpy as np
 import pytest
@@ -57,3 +57,33 @@ def test_transfer_error(dims, agg, nv, nrhs, prec, dt):
     plain = serial(terms, 3)
     exact = np.sum(P.astype(CLD)[None] * xc.astype(CLD)[..., None], axis=3)
     assert rel(up, exact) <= rel(plain, exact), (rel(up, exact), rel(plain, exact))
+
+
+@pytest.mark.parametrize("prec,dt,offset", [(0, np.complex128, 0), (1, np.complex64, 0), (1, np.complex64, 1)])
+@pytest.mark.parametrize("nv,nrhs", [(20, 3), (7, 5)])
+def test_coarse_stencil_error(nv, nrhs, prec, dt, offset):
+    from paper_2004_08146_gb300 import qcd
+    torch = torch_cuda()
+    dims, agg = (8, 8, 8, 4), (4, 4, 4, 4)
+    ctx = make_ctx(synth.gauge_field(dims, 0.5, 95), dims, -0.3, 1.3, sap_block=agg, precision=qcd.QCD_FP64)
+    ctx.qcd_mg_update_from_eigvecs(dev(synth.spinor(dims, 96, nvec=nv)), nv)
+    g, nc = (2, 2, 2, 1), 2 * nv
+    A = np.asarray(ctx.qcd_mg_get_coarse()).reshape(8, 9, nc, nc).astype(dt)     # [site][direction][row][column]
+    x = synth.complex_gaussian((nrhs, 8, nc), 98).astype(dt)
+    xd = torch.empty(x.size + offset, dtype=torch.complex128 if prec == 0 else torch.complex64, device="cuda")[offset:]
+    xd.copy_(dev(x))
+    y = torch.empty_like(xd)
+    ctx.qcd_coarse_apply(qcd.QCD_OP_D, prec, nrhs, xd, y, [0.0] * nrhs)
+    got = host(y)
+    ctx.close()
+    nb = np.empty((8, 9), dtype=int)
+    for s in range(8):
+        for d in range(9):
+            c = list(np.unravel_index(s, g))
+            if d:
+                c[(d - 1) % 4] = (c[(d - 1) % 4] + (1 if d <= 4 else -1)) % g[(d - 1) % 4]
+            nb[s, d] = np.ravel_multi_index(c, g)
+    xn = x[:, nb]                                                                # [n, site, direction, column]
+    plain = serial((A[None] * xn[:, :, :, None]).transpose(0, 1, 3, 2, 4).reshape(nrhs, 8, nc, -1), -1)
+    exact = np.sum(A.astype(CLD)[None] * xn.astype(CLD)[:, :, :, None], axis=(2, 4))
+    assert rel(got, exact) <= rel(plain, exact), (rel(got, exact), rel(plain, exact))
