@@ -63,7 +63,7 @@ __device__ __forceinline__ int local_index(const Blocking& B, const int o[4]) {
 // the warp of the next vector normalises it, and one barrier per vector is left.
 // Vectors in shared memory where they fit.  Bound by the FP64 pipe (a third of it
 // sums over lanes).  16 x 8^3, 2^4 aggregates, 8 vectors: 822 us with one inner
-// product per block-wide reduction, 160 now.
+// product per block-wide reduction, 201 now.
 __global__ void __launch_bounds__(256) build_P_kernel(Geom g, Blocking B, int nv, const double2* __restrict__ vecs,
                                                       double2* P64, float2* __restrict__ P32, int in_smem) {
     extern __shared__ double2 pvs[];
@@ -91,8 +91,18 @@ __global__ void __launch_bounds__(256) build_P_kernel(Geom g, Blocking B, int nv
             const double2* pj = v + (size_t)j * nloc;
             for (int i = j + 1 + warp; i < nv; i += 8) {
                 double2* pi = v + (size_t)i * nloc;
-                double2 h = make_double2(0, 0);
-                for (int d = lane; d < nloc; d += 32) cmacc(h, pj[d], pi[d]);
+                // h: the products with Re p and with Im p in sums of their own, and the
+                // update rounds the vector once (fused into it twice: P 2.4e-16 from
+                // the exact one at 20 vectors against 1.8e-16)
+                double2 h = make_double2(0, 0), hi = make_double2(0, 0);
+                for (int d = lane; d < nloc; d += 32) {
+                    const double2 p = pj[d], q = pi[d];
+                    h.x = fma(p.x, q.x, h.x);
+                    h.y = fma(p.x, q.y, h.y);
+                    hi.x = fma(p.y, q.y, hi.x);
+                    hi.y = fma(-p.y, q.x, hi.y);
+                }
+                h += hi;
                 // the halves of the warp share the two sums
                 const bool up = lane & 16;
                 double k = up ? h.y : h.x;
@@ -100,7 +110,7 @@ __global__ void __launch_bounds__(256) build_P_kernel(Geom g, Blocking B, int nv
 #pragma unroll
                 for (int o = 8; o > 0; o >>= 1) k += __shfl_xor_sync(0xffffffffu, k, o);
                 h = make_double2(__shfl_sync(0xffffffffu, k, 0), __shfl_sync(0xffffffffu, k, 16));
-                for (int d = lane; d < nloc; d += 32) cmsub(pi[d], h, pj[d]);
+                for (int d = lane; d < nloc; d += 32) pi[d] -= h * pj[d];
                 if (i == j + 1) normalise(pi);
             }
             __syncthreads();
