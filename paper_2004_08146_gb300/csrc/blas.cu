@@ -108,7 +108,7 @@ __global__ void multiaxpy_kernel(const Z* __restrict__ X, int nvec, size_t xstri
             if (staged) ci = cs[i * nrhs + j];
             else { ci.x = (R)c[i * nrhs + j].x; ci.y = (R)c[i * nrhs + j].y; }
             if (ci.x == R(0) && ci.y == R(0)) continue;   // unused basis slots may hold stale data
-            cmac(acc, ci, X[(size_t)i * xstride_vec + (size_t)j * n + k]);
+            acc += ci * X[(size_t)i * xstride_vec + (size_t)j * n + k];
         }
         Z o = w[t];
         const R sg = (R)sign;

@@ -110,7 +110,7 @@ __device__ __forceinline__ Z kry_projected(const Z* __restrict__ V, size_t vs, i
         }
 #pragma unroll
         for (int q = 0; q < 8; ++q)
-            if (i + q < nv) cmac(acc, cs[i + q], x[q]);
+            if (i + q < nv) acc += cs[i + q] * x[q];
     }
     w.x -= acc.x;
     w.y -= acc.y;
@@ -493,7 +493,7 @@ __global__ void __launch_bounds__(256) coarse_gmres_kernel(CoarseArgs<Z, R> a) {
             Z acc = ws[(size_t)j * E + e];
             const Z* v = VS(0, j) + e;
 #pragma unroll 4
-            for (int i = 0; i < ni; ++i, v += (size_t)nrhs * E) cmsub(acc, hr[i * nrhs + j], *v);
+            for (int i = 0; i < ni; ++i, v += (size_t)nrhs * E) acc -= hr[i * nrhs + j] * *v;
             put(j, e, acc);
         }
     };
@@ -720,7 +720,7 @@ __global__ void __launch_bounds__(256) coarse_gmres_kernel(CoarseArgs<Z, R> a) {
         const int k = kd[j];
         const Z* y = reinterpret_cast<const Z*>(a.yv) + (size_t)j * maxit;
         Z o; o.x = 0; o.y = 0;
-        for (int i = 0; i < k; ++i) cmac(o, y[i], VS(i, j)[e]);
+        for (int i = 0; i < k; ++i) o += y[i] * VS(i, j)[e];
         a.x[(size_t)j * nco + lo + e] = o;
     }
 }

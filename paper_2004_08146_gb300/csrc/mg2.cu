@@ -131,7 +131,7 @@ __global__ void prolong2_kernel(Geom g1, Blocking B2, int nv1, int nv2, const Z*
         Z acc;
         acc.x = 0;
         acc.y = 0;
-        for (int i2 = 0; i2 < nv2; ++i2) cmac(acc, p[(size_t)i2 * nloc], c[i2]);
+        for (int i2 = 0; i2 < nv2; ++i2) acc += p[(size_t)i2 * nloc] * c[i2];
         const int l = d / nv1, i = d % nv1;
         x[(size_t)j * g1.V * nc1 + (size_t)block_fine_site(g1, B2, blk, l) * nc1 + chi * nv1 + i] = acc;
     }
@@ -185,7 +185,7 @@ __global__ void __launch_bounds__(kC2Threads) build_coarse2_kernel(Geom g1, Bloc
             if (t < nc1) {
                 const Z1* a = A1 + ((size_t)x * 9 + d1) * nc1 * nc1 + (size_t)chic * nv1 * nc1 + t;
                 double2 s = make_double2(0, 0);
-                for (int i = 0; i < nv1; ++i) cmac(s, cvt<double2>(a[(size_t)i * nc1]), sv[i]);
+                for (int i = 0; i < nv1; ++i) s += cvt<double2>(a[(size_t)i * nc1]) * sv[i];
                 h[t] = s;
             }
             __syncthreads();
@@ -193,7 +193,7 @@ __global__ void __launch_bounds__(kC2Threads) build_coarse2_kernel(Geom g1, Bloc
                 const int chi = t / nv2, j = t % nv2;
                 const double2* p = P2 + (((size_t)b2 * 2 + chi) * nv2 + j) * nloc + (size_t)l * nv1;
                 double2 s = make_double2(0, 0);
-                for (int i = 0; i < nv1; ++i) cmacc(s, p[i], h[chi * nv1 + i]);
+                for (int i = 0; i < nv1; ++i) s += conj(p[i]) * h[chi * nv1 + i];
                 acc[d2][t] += s;
             }
             __syncthreads();
