@@ -12,6 +12,7 @@
 // pipe.  Results of inner products are returned in FP64.
 #include <algorithm>
 
+#include "ffsum.cuh"
 #include "internal.h"
 
 namespace qcd {
@@ -20,20 +21,6 @@ namespace {
 
 constexpr int kThreads = 256;
 
-struct ffr {
-    float h, l;
-};
-
-__device__ __forceinline__ ffr two_sum(float a, float b) {
-    const float s = a + b;
-    const float bb = s - a;
-    const float e = (a - (s - bb)) + (b - bb);
-    return {s, e};
-}
-__device__ __forceinline__ ffr fast_two_sum(float a, float b) {   // |a| >= |b| or a == 0
-    const float s = a + b;
-    return {s, b - (s - a)};
-}
 __device__ __forceinline__ ffr two_prod(float a, float b) {
     const float p = a * b;
     return {p, fmaf(a, b, -p)};
@@ -61,11 +48,6 @@ struct acc_t {
     __device__ __forceinline__ void msub(float ah, float al, float bh, float bl) { mac(-ah, -al, bh, bl); }
     __device__ __forceinline__ ffr get() const { return fast_two_sum(h, l); }
 };
-
-__device__ __forceinline__ ffr ff_add(ffr a, ffr b) {
-    const ffr s = two_sum(a.h, b.h);
-    return fast_two_sum(s.h, s.l + a.l + b.l);
-}
 
 // ---- element access: float4 = (re.h, im.h, re.l, im.l)
 __device__ __forceinline__ float4 pack(ffr re, ffr im) { return make_float4(re.h, im.h, re.l, im.l); }
@@ -112,54 +94,30 @@ struct acc2_t {
     }
 };
 
-__device__ __forceinline__ ffr ff_warp_sum(ffr v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const ffr w{__shfl_xor_sync(0xffffffffu, v.h, o), __shfl_xor_sync(0xffffffffu, v.l, o)};
-        v = ff_add(v, w);
-    }
-    return v;
+// sums over the lanes of a warp, the same in all of them
+__device__ __forceinline__ void add_lane(sum3_t& t, int o) {
+    t.add(sum3_t(__shfl_xor_sync(0xffffffffu, t.a, o), __shfl_xor_sync(0xffffffffu, t.b, o),
+                 __shfl_xor_sync(0xffffffffu, t.c, o)));
 }
-// Sum of many double-floats: three floats that are exact sums of one another's
-// rounding errors, so the total is good to FP64 roundoff without the FP64 pipe
-// (2 additions per clock and SM).
-struct sum3_t {
-    float a = 0.f, b = 0.f, c = 0.f;
-    __device__ __forceinline__ void add(float h, float l) {
-        const ffr s = two_sum(a, h), t = two_sum(b, l), u = two_sum(t.h, s.l);
-        a = s.h;
-        b = u.h;
-        c += t.l + u.l;
-    }
-    __device__ __forceinline__ void add_lane(int o) {
-        const float h = __shfl_xor_sync(0xffffffffu, a, o), l = __shfl_xor_sync(0xffffffffu, b, o),
-                    m = __shfl_xor_sync(0xffffffffu, c, o);
-        add(h, l);
-        c += m;
-    }
-    __device__ __forceinline__ ffr get() const {
-        const ffr s = two_sum(a, b);
-        return fast_two_sum(s.h, s.l + c);
-    }
-    __device__ __forceinline__ double warp_sum() {   // the same in all lanes
+__device__ __forceinline__ sum3_t ff_warp_sum(sum3_t t) {
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) add_lane(o);
-        return (double)a + ((double)b + (double)c);
-    }
-};
+    for (int o = 16; o > 0; o >>= 1) add_lane(t, o);
+    return t;
+}
 // both sums of a complex number, (re, im) in lanes 0 and 16: the halves of the warp
 // share them first
-__device__ __forceinline__ ffr ff_warp_sum2(ffr re, ffr im, int lane) {
+__device__ __forceinline__ sum3_t ff_warp_sum2(ffr re, ffr im, int lane) {
     const bool up = lane & 16;
     const ffr k = up ? im : re, s = up ? re : im;
-    sum3_t t;
-    t.a = k.h;
-    t.b = k.l;
+    sum3_t t(k.h, k.l);
     t.add(__shfl_xor_sync(0xffffffffu, s.h, 16), __shfl_xor_sync(0xffffffffu, s.l, 16));
 #pragma unroll
-    for (int o = 8; o > 0; o >>= 1) t.add_lane(o);
-    return t.get();
+    for (int o = 8; o > 0; o >>= 1) add_lane(t, o);
+    return t;
 }
+// a partial sum in memory: 16 bytes
+__device__ __forceinline__ float4 pack3(const sum3_t& t) { return make_float4(t.a, t.b, t.c, 0.f); }
+__device__ __forceinline__ sum3_t unpack3(const float4& v) { return sum3_t(v.x, v.y, v.z); }
 
 // Dot products of up to two vectors y with the na vectors of set A and the nb of
 // set B (Gram-Schmidt against [V X]; the Gram columns W^H W_m, W^H V_m).  A warp
@@ -179,9 +137,9 @@ template <int Q, int NY>
 __global__ void __launch_bounds__(256, 4) ff_dots_kernel(const float4* __restrict__ A, int na, const float4* __restrict__ B,
                                                       int nb, size_t n, const float4* __restrict__ y0,
                                                       const float4* __restrict__ y1,
-                                                      float2* __restrict__ partial, unsigned* __restrict__ counters,
+                                                      float4* __restrict__ partial, unsigned* __restrict__ counters,
                                                       double2* __restrict__ d0, double2* __restrict__ d1, GramOut go) {
-    __shared__ float2 red[8][2 * NY * Q];   // re and im of each sum
+    __shared__ float4 red[8][2 * NY * Q];   // re and im of each sum
     __shared__ bool last;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nv = na + nb, v0 = blockIdx.y * Q;
     const int part = blockIdx.x * 8 + warp, parts = gridDim.x * 8;
@@ -232,17 +190,16 @@ __global__ void __launch_bounds__(256, 4) ff_dots_kernel(const float4* __restric
     for (int k = 0; k < NY; ++k)
 #pragma unroll
         for (int q = 0; q < Q; ++q) {
-            const ffr r = ff_warp_sum2(acc[k][q].re.get(), acc[k][q].im.get(), lane);
-            if ((lane & 15) == 0) red[warp][2 * (k * Q + q) + (lane >> 4)] = make_float2(r.h, r.l);
+            const sum3_t r = ff_warp_sum2(acc[k][q].re.get(), acc[k][q].im.get(), lane);
+            if ((lane & 15) == 0) red[warp][2 * (k * Q + q) + (lane >> 4)] = pack3(r);
         }
     __syncthreads();
     if (warp == 0) {
         if (lane < 2 * NY * Q) {
             sum3_t t;
 #pragma unroll
-            for (int w = 0; w < 8; ++w) t.add(red[w][lane].x, red[w][lane].y);
-            const ffr r = t.get();
-            partial[((size_t)blockIdx.y * 2 * NY * Q + lane) * gridDim.x + blockIdx.x] = make_float2(r.h, r.l);
+            for (int w = 0; w < 8; ++w) t.add(unpack3(red[w][lane]));
+            partial[((size_t)blockIdx.y * 2 * NY * Q + lane) * gridDim.x + blockIdx.x] = pack3(t);
             __threadfence();
         }
         __syncwarp();
@@ -255,12 +212,11 @@ __global__ void __launch_bounds__(256, 4) ff_dots_kernel(const float4* __restric
     if (warp < NY * Q && v < nv) {
         sum3_t re, im;
         for (unsigned t = lane; t < gridDim.x; t += 32) {
-            const float2* p = partial + ((size_t)blockIdx.y * 2 * NY * Q + 2 * warp) * gridDim.x + t;
-            const float2 x = __ldcg(p), y = __ldcg(p + gridDim.x);
-            re.add(x.x, x.y);
-            im.add(y.x, y.y);
+            const float4* p = partial + ((size_t)blockIdx.y * 2 * NY * Q + 2 * warp) * gridDim.x + t;
+            re.add(unpack3(__ldcg(p)));
+            im.add(unpack3(__ldcg(p + gridDim.x)));
         }
-        const double2 d = make_double2(re.warp_sum(), im.warp_sum());
+        const double2 d = make_double2(ff_warp_sum(re).value(), ff_warp_sum(im).value());
         if (lane == 0) {
             (k == 0 ? d0 : d1)[v] = d;
             // new column and row of G = W^H W and H = W^H V (Hermitian)
@@ -328,25 +284,24 @@ __global__ void __launch_bounds__(128, 6) ff_project_kernel(const float4* __rest
     if (in) w[k] = pack(acc.re.get(), acc.im.get());
 }
 
-// Double-float sums of NV values over all threads of the grid, NV <= 2: one
+// Sums of NV double-float values over all threads of the grid, NV <= 2: one
 // partial per CTA, the last CTA adds them; FP64 results in out[v].x.
 template <int NV>
-__device__ __forceinline__ void ff_grid_sum(ffr (&v)[NV], float2* partial, unsigned* counter, double2* out) {
-    __shared__ float2 red[NV][32];
+__device__ __forceinline__ void ff_grid_sum(ffr (&v)[NV], float4* partial, unsigned* counter, double2* out) {
+    __shared__ float4 red[NV][32];
     __shared__ bool last;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
 #pragma unroll
     for (int q = 0; q < NV; ++q) {
-        const ffr r = ff_warp_sum(v[q]);
-        if (lane == 0) red[q][warp] = make_float2(r.h, r.l);
+        const sum3_t r = ff_warp_sum(sum3_t(v[q].h, v[q].l));
+        if (lane == 0) red[q][warp] = pack3(r);
     }
     __syncthreads();
     if (warp == 0) {
 #pragma unroll
         for (int q = 0; q < NV; ++q) {
-            const float2 r = lane < nw ? red[q][lane] : make_float2(0.f, 0.f);
-            const ffr s = ff_warp_sum(ffr{r.x, r.y});
-            if (lane == 0) partial[(size_t)q * gridDim.x + blockIdx.x] = make_float2(s.h, s.l);
+            const sum3_t s = ff_warp_sum(lane < nw ? unpack3(red[q][lane]) : sum3_t());
+            if (lane == 0) partial[(size_t)q * gridDim.x + blockIdx.x] = pack3(s);
         }
     }
     if (threadIdx.x == 0) {
@@ -360,11 +315,8 @@ __device__ __forceinline__ void ff_grid_sum(ffr (&v)[NV], float2* partial, unsig
     for (int q = 0; q < NV; ++q) {
         if (warp != q) continue;   // NV <= warps of the CTA
         sum3_t a;
-        for (unsigned t = lane; t < gridDim.x; t += 32) {
-            const float2 r = __ldcg(&partial[(size_t)q * gridDim.x + t]);
-            a.add(r.x, r.y);
-        }
-        const double s = a.warp_sum();
+        for (unsigned t = lane; t < gridDim.x; t += 32) a.add(unpack3(__ldcg(&partial[(size_t)q * gridDim.x + t])));
+        const double s = ff_warp_sum(a).value();
         if (lane == 0) out[q] = make_double2(s, 0.0);
     }
     if (threadIdx.x == 0) *counter = 0u;
@@ -375,7 +327,7 @@ __device__ __forceinline__ void ff_grid_sum(ffr (&v)[NV], float2* partial, unsig
 __global__ void __launch_bounds__(128, 6) ff_ritz_kernel(const float4* __restrict__ V, const float4* __restrict__ W,
                                                          int m, size_t n, const double2* __restrict__ s,
                                                          float4* __restrict__ u, float4* __restrict__ Qu,
-                                                         float2* __restrict__ partial, unsigned* __restrict__ counter,
+                                                         float4* __restrict__ partial, unsigned* __restrict__ counter,
                                                          double2* __restrict__ d) {
     __shared__ float4 cs[kFFCoef];
     acc_t uu, uq;
@@ -403,7 +355,7 @@ __global__ void __launch_bounds__(128, 6) ff_ritz_kernel(const float4* __restric
 // FP64 (rho the Rayleigh quotient), u <- u / ||u||, and rr = r^H r.
 __global__ void __launch_bounds__(256) ff_residual_kernel(float4* __restrict__ u, const float4* __restrict__ Qu,
                                                           const double2* __restrict__ d, size_t n,
-                                                          double2* __restrict__ r, float2* __restrict__ partial,
+                                                          double2* __restrict__ r, float4* __restrict__ partial,
                                                           unsigned* __restrict__ counter, double2* __restrict__ rr) {
     __shared__ float4 cf;   // iu and -rho iu
     if (threadIdx.x == 0) {
@@ -567,7 +519,7 @@ static void launch_dots(const void* A, int na, const void* B, int nb, size_t n, 
     size_t gx = std::max(1, 4 * sm_count() / sets);
     gx = std::min({gx, std::max<size_t>(1, n / 512), (size_t)kFFParts});
     ff_dots_kernel<Q, NY><<<dim3((unsigned)gx, sets), 256, 0, st>>>(
-        (const float4*)A, na, (const float4*)B, nb, n, (const float4*)y0, (const float4*)y1, (float2*)partial,
+        (const float4*)A, na, (const float4*)B, nb, n, (const float4*)y0, (const float4*)y1, (float4*)partial,
         counters, d0, d1, go);
 }
 
@@ -604,11 +556,11 @@ void ff_ritz(const void* V, const void* W, int m, size_t n, const double2* s, vo
         KTimer kt("ritz_ff", (double)(2 * m + 2) * n * 16, 16.0 * m * n, st);
         const unsigned grid = (unsigned)std::min<size_t>((n + 127) / 128, kFFParts);
         ff_ritz_kernel<<<grid, 128, 0, st>>>((const float4*)V, (const float4*)W, m, n, s, (float4*)u, (float4*)Qu,
-                                             (float2*)partial, counters, d);
+                                             (float4*)partial, counters, d);
     }
     KTimer kt("residual_ff", (double)n * 64, 0.0, st);
     const unsigned grid = (unsigned)std::min<size_t>((n + 255) / 256, (size_t)sm_count() * 4);
-    ff_residual_kernel<<<grid, 256, 0, st>>>((float4*)u, (const float4*)Qu, d, n, r, (float2*)partial, counters, d + 2);
+    ff_residual_kernel<<<grid, 256, 0, st>>>((float4*)u, (const float4*)Qu, d, n, r, (float4*)partial, counters, d + 2);
 }
 
 void ff_scale_out(void* v, double a, double2* y, size_t n, cudaStream_t st) {

@@ -1,5 +1,5 @@
 // Host entry points over the host/device arithmetic of the library's headers.
-#include "common.cuh"
+#include "ffsum.cuh"
 
 using namespace qcd;
 
@@ -13,4 +13,28 @@ extern "C" void host_cdot(const float* a, const float* b, int n, int terms, floa
         out[2 * k] = re;
         out[2 * k + 1] = im;
     }
+}
+
+// n double-floats (h, l) summed as the Davidson kernels do: 32 lanes, 8 warps, CTAs.
+// keep = 0 rounds every partial sum to a double-float between the stages.
+extern "C" double host_stage_sum(const float* hl, int ctas, int keep) {
+    auto stage = [&](const sum3_t& t) {
+        if (keep) return t;
+        const ffr s = two_sum(t.a, t.b), r = fast_two_sum(s.h, s.l + t.c);
+        return sum3_t(r.h, r.l);
+    };
+    sum3_t total;
+    for (int c = 0; c < ctas; ++c) {
+        sum3_t cta;
+        for (int w = 0; w < 8; ++w) {
+            sum3_t warp;
+            for (int l = 0; l < 32; ++l) {
+                const float* p = hl + 2 * ((c * 8 + w) * 32 + l);
+                warp.add(p[0], p[1]);
+            }
+            cta.add(stage(warp));
+        }
+        total.add(stage(cta));
+    }
+    return total.value();
 }

@@ -42,3 +42,21 @@ def test_inner_products_round_the_running_sum_once(lib):
     exact = np.sum(ca.astype(np.complex128).conj() * cb.astype(np.complex128), axis=1)
     err = [np.linalg.norm(v - exact) / np.linalg.norm(exact) for v in (out[:, 0] + 1j * out[:, 1], plain)]
     assert err[0] <= 1.03 * err[1], err
+
+
+def test_double_float_sums_keep_fp64(lib):
+    """Partial sums of double-floats passed from stage to stage with all three parts
+    stay within a rounding of FP64 (2^-53) of the sum of the absolute values; rounded
+    to double-floats in between they do not (2^-49 of it and less, rms)."""
+    lib.host_stage_sum.restype = ctypes.c_double
+    rng = np.random.default_rng(5)
+    worst = [0.0, 0.0]
+    for _ in range(20):
+        v = rng.standard_normal((12, 8, 32)) ** 2          # a squared norm: no cancellation
+        h = v.astype(np.float32)
+        hl = np.stack([h, (v - h).astype(np.float32)], axis=-1)
+        exact = np.sum(hl.astype(np.longdouble))
+        for keep in (0, 1):
+            d = abs(np.longdouble(lib.host_stage_sum(ptr(np.ascontiguousarray(hl)), 12, keep)) - exact)
+            worst[keep] = max(worst[keep], float(d / exact))
+    assert worst[1] <= 2.0 ** -53 < worst[0], worst
