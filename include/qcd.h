@@ -306,7 +306,11 @@ int qcd_bilinear_force(qcd_ctx* ctx, int nvec, const void* G, const void* Psi, i
  * field F, DEVICE complex128 [site][mu][3][3]): the link gradient of a batch.
  * The field is linear in the outer products of psi_k and g_k, which are summed
  * first, so the cost is close to that of one field.  nvec = 0 leaves F alone;
- * otherwise as qcd_bilinear_force. */
+ * otherwise as qcd_bilinear_force.
+ * The force calls with c_sw != 0 keep a workspace in the context, 4320 bytes per
+ * site up to 300,000 sites and 1440 above, less (1440, 720) where there is not
+ * memory for that; it is given back when another allocation of the context would
+ * fail and when another field is loaded. */
 int qcd_bilinear_force_sum(qcd_ctx* ctx, int nvec, const void* G, const void* Psi, int grad, void* F);
 
 /* Local coherence lc(v) = ||Pi v|| / ||v|| (Sec. 3, the local coherence

@@ -120,19 +120,48 @@ struct qcd_ctx {
         if (it->second.p) cudaFree(it->second.p);
         ws.erase(it);
     }
+    // cudaMalloc that gives back the link force's scratch, which no other call uses, if
+    // that is in the way
+    cudaError_t dev_malloc(void** q, size_t bytes) {
+        cudaError_t e = cudaMalloc(q, bytes);
+        if (e == cudaErrorMemoryAllocation && ws.count("force")) {
+            drop_buf("force");
+            e = cudaMalloc(q, bytes);
+        }
+        cudaGetLastError();   // a failure is reported by the return value alone
+        return e;
+    }
     void* buf(const std::string& name, size_t bytes) {
         DevBuf& b = ws[name];
         if (b.bytes < bytes) {
             if (b.p) CK(cudaFree(b.p));
             b.p = nullptr;
             b.bytes = 0;
-            if (cudaMalloc(&b.p, bytes) != cudaSuccess) {
+            if (dev_malloc(&b.p, bytes) != cudaSuccess) {
                 cudaGetLastError();
                 throw QcdError(QCD_ENOMEM, "device allocation of " + std::to_string(bytes) + " bytes for " + name);
             }
             b.bytes = bytes;
         }
         return b.p;
+    }
+    // scratch of the link force in the largest form that there is memory for; the
+    // caller has all its other buffers by then
+    void* force_buf(int& form) {
+        for (form = 0;; ++form) {
+            const size_t need = force_scratch(f, form);
+            auto it = ws.find("force");
+            if (it != ws.end() && it->second.bytes >= need) return it->second.p;
+            drop_buf("force");
+            void* q = nullptr;
+            if (need == 0 || cudaMalloc(&q, need) == cudaSuccess) {
+                ws["force"] = DevBuf{q, need};
+                return q;
+            }
+            cudaGetLastError();
+            if (form == 2)
+                throw QcdError(QCD_ENOMEM, "device allocation of " + std::to_string(need) + " bytes for the link force");
+        }
     }
     // completion counters for dot products, zero between launches
     unsigned* dot_counters(size_t n) {
@@ -144,7 +173,7 @@ struct qcd_ctx {
             }
             md_cnt = nullptr;
             md_cnt_n = 0;
-            if (cudaMalloc(&md_cnt, n * sizeof(unsigned)) != cudaSuccess) {
+            if (dev_malloc((void**)&md_cnt, n * sizeof(unsigned)) != cudaSuccess) {
                 cudaGetLastError();
                 throw QcdError(QCD_ENOMEM, "device allocation of dot-product counters");
             }
@@ -450,7 +479,7 @@ void ensure_sap(qcd_ctx* ctx) {
         lists[(c0 + c1 + c2 + c3) % 2].push_back(b);
     }
     for (int c = 0; c < 2; ++c) {
-        CK(cudaMalloc(&ctx->sap.blocks_of_colour[c], lists[c].size() * sizeof(int)));
+        CK(ctx->dev_malloc((void**)&ctx->sap.blocks_of_colour[c], lists[c].size() * sizeof(int)));
         CK(cudaMemcpy(ctx->sap.blocks_of_colour[c], lists[c].data(), lists[c].size() * sizeof(int), cudaMemcpyHostToDevice));
         ctx->sap.ncol[c] = (int)lists[c].size();
     }
@@ -690,10 +719,10 @@ void build_level2(qcd_ctx* ctx, const double2* V, int nvec) {
         c2.gc.antiperiodic = 0;
         const size_t np = (size_t)B2.nb * 2 * nv2 * B2.bs * c.nv;
         const size_t na = (size_t)B2.nb * 9 * c2.nc * c2.nc;
-        CK(cudaMalloc(&c2.P64, np * sizeof(double2)));
-        CK(cudaMalloc(&c2.P32, np * sizeof(float2)));
-        CK(cudaMalloc(&c2.A64, na * sizeof(double2)));
-        CK(cudaMalloc(&c2.A32, na * sizeof(float2)));
+        CK(ctx->dev_malloc((void**)&c2.P64, np * sizeof(double2)));
+        CK(ctx->dev_malloc((void**)&c2.P32, np * sizeof(float2)));
+        CK(ctx->dev_malloc((void**)&c2.A64, na * sizeof(double2)));
+        CK(ctx->dev_malloc((void**)&c2.A32, na * sizeof(float2)));
         ctx->c2_nv1 = c.nv;
     }
     // an FP64 context builds level 2 from the FP64 level-1 operator; a
@@ -728,10 +757,10 @@ void build_from_vectors(qcd_ctx* ctx, const double2* V, int nvec, const int bloc
         c.gc.antiperiodic = 0;
         size_t np = (size_t)B.nb * 2 * nvec * B.bs * 6;
         size_t na = (size_t)B.nb * 9 * c.nc * c.nc;
-        CK(cudaMalloc(&c.P64, np * sizeof(double2)));
-        CK(cudaMalloc(&c.P32, np * sizeof(float2)));
-        CK(cudaMalloc(&c.A64, na * sizeof(double2)));
-        CK(cudaMalloc(&c.A32, na * sizeof(float2)));
+        CK(ctx->dev_malloc((void**)&c.P64, np * sizeof(double2)));
+        CK(ctx->dev_malloc((void**)&c.P32, np * sizeof(float2)));
+        CK(ctx->dev_malloc((void**)&c.A64, na * sizeof(double2)));
+        CK(ctx->dev_malloc((void**)&c.A32, na * sizeof(float2)));
     }
     mg_build_P(ctx->f, c, V, nvec, ctx->st);
     // a mixed-precision context runs its cycles in FP32: build only that
@@ -749,7 +778,7 @@ void mg_setup_impl(qcd_ctx* ctx, int Nv, const int block[4]) {
     const int prec = ctx->p.precision == QCD_FP64 ? QCD_FP64 : QCD_FP32;
     if (ctx->test_vectors) CK(cudaFree(ctx->test_vectors));
     ctx->test_vectors = nullptr;
-    CK(cudaMalloc(&ctx->test_vectors, (size_t)Nv * n * sizeof(double2)));
+    CK(ctx->dev_malloc((void**)&ctx->test_vectors, (size_t)Nv * n * sizeof(double2)));
     ctx->n_test = Nv;
     double2* W = ctx->test_vectors;
     blas_gaussian(W, (size_t)Nv * n, ctx->p.seed, 0x5e7000000000ull, ctx->st);
@@ -1559,7 +1588,7 @@ int qcd_mg_update_from_eigvecs(qcd_ctx* ctx, const void* V, int nvec) {
         build_from_vectors(ctx, (const double2*)V, nvec, b);
         if (ctx->n_test != nvec || !ctx->test_vectors) {
             if (ctx->test_vectors) CK(cudaFree(ctx->test_vectors));
-            CK(cudaMalloc(&ctx->test_vectors, (size_t)nvec * ctx->nfine() * sizeof(double2)));
+            CK(ctx->dev_malloc((void**)&ctx->test_vectors, (size_t)nvec * ctx->nfine() * sizeof(double2)));
             ctx->n_test = nvec;
         }
         CK(cudaMemcpyAsync(ctx->test_vectors, V, (size_t)nvec * ctx->nfine() * sizeof(double2),
@@ -1662,13 +1691,15 @@ int qcd_eig_force(qcd_ctx* ctx, int nvec, const void* V, void* F) {
         check_align(F, "F");
         const FineOp& f = ctx->f;
         const size_t n = ctx->nfine(), nl = (size_t)f.g.V * 36;
-        void* scratch = ctx->buf("force", force_scratch(f));
         double2* nrm = (double2*)ctx->buf("force.nrm", sizeof(double2));
         double2* part = (double2*)ctx->buf("force.part", (size_t)64 * sizeof(double2));
+        ctx->dot_counters(1);
+        int form;
+        void* scratch = ctx->force_buf(form);
         for (int j = 0; j < nvec; ++j) {
             const double2* v = (const double2*)V + (size_t)j * n;
             blas_multidot(QCD_FP64, v, 1, n, v, 1, n, nrm, part, ctx->dot_counters(1), ctx->st);
-            bilinear_force(f, 1, v, v, nrm, 0, scratch, (double2*)F + (size_t)j * nl, ctx->st);
+            bilinear_force(f, 1, v, v, nrm, 0, scratch, form, (double2*)F + (size_t)j * nl, ctx->st);
         }
         check_launch("eig force");
         return QCD_OK;
@@ -1687,10 +1718,11 @@ static int bilinear_force_call(qcd_ctx* ctx, int nvec, const void* G, const void
         check_align(F, "F");
         const FineOp& f = ctx->f;
         const size_t n = ctx->nfine(), nl = (size_t)f.g.V * 36;
-        void* scratch = ctx->buf("force", force_scratch(f));
+        int form;
+        void* scratch = ctx->force_buf(form);
         for (int j = 0; j < (sum ? 1 : nvec); ++j)
             bilinear_force(f, sum ? nvec : 1, (const double2*)G + (size_t)j * n, (const double2*)Psi + (size_t)j * n,
-                           nullptr, grad, scratch, (double2*)F + (size_t)j * nl, ctx->st);
+                           nullptr, grad, scratch, form, (double2*)F + (size_t)j * nl, ctx->st);
         check_launch("bilinear force");
         return QCD_OK;
     });

@@ -314,8 +314,9 @@ __device__ __forceinline__ double2 shfl2(double2 v, int o) {
 // and sigma^chi_{jk} = -eps_jkl sigma_l, and Gamma5 g changes sign with chi, so
 // plane (0, k) is T^0_k + T^1_k and plane (j, k) is -eps_jkl (T^0_l - T^1_l): sums
 // and differences between lanes.
+// only >= 0: that plane alone, [site][3][3].
 __global__ void __launch_bounds__(128) clover_insertion_kernel(const double2* __restrict__ psi,
-                                                               const double2* __restrict__ gv, int nvec, Geom g,
+                                                               const double2* __restrict__ gv, int nvec, Geom g, int only,
                                                                double2* __restrict__ Bt) {
     const unsigned tid = blockIdx.x * blockDim.x + threadIdx.x;
     const bool live = (int)(tid >> 3) < g.V;
@@ -362,7 +363,8 @@ __global__ void __launch_bounds__(128) clover_insertion_kernel(const double2* __
     if (!live || (i && j)) return;
     const int plane = chi ? 6 - k : k - 1;
     const bool minus = chi && k != 2;   // -eps: planes (1,2), (2,3) minus, (1,3) plus
-    double2* o = Bt + ((size_t)s * 6 + plane) * 9;
+    if (only >= 0 && plane != only) return;
+    double2* o = Bt + (only >= 0 ? (size_t)s : (size_t)s * 6 + plane) * 9;
 #pragma unroll
     for (int a = 0; a < 3; ++a)
 #pragma unroll
@@ -476,7 +478,7 @@ __global__ void __launch_bounds__(128) hop_force_kernel(const double2* __restric
 // d][site][3][3].
 __global__ void __launch_bounds__(128) plaquette_force_kernel(const double2* __restrict__ U,
                                                               const double2* __restrict__ Bt, Geom g, int plane0,
-                                                              double2* __restrict__ W4) {
+                                                              int only, double2* __restrict__ W4) {
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= g.V) return;
     const int pl = plane0 + blockIdx.y;
@@ -485,7 +487,7 @@ __global__ void __launch_bounds__(128) plaquette_force_kernel(const double2* __r
     site_coords(g, s, x);
     const int s1 = shifted(g, x, mu, 1, nu, 0), s3 = shifted(g, x, mu, 0, nu, 1), s2 = shifted(g, x, mu, 1, nu, 1);
     auto link = [&](int site, int d) { return m3_load(U + ((size_t)site * 4 + d) * 9); };
-    auto ins = [&](int site) { return m3_load(Bt + ((size_t)site * 6 + pl) * 9); };
+    auto ins = [&](int site) { return m3_load(Bt + (only >= 0 ? (size_t)site : (size_t)site * 6 + pl) * 9); };
     double2* out = W4 + (size_t)blockIdx.y * 4 * g.V * 9 + (size_t)s * 9;
     const size_t step = (size_t)g.V * 9;
     M3<double> E, D, X, Y;
@@ -576,36 +578,42 @@ __global__ void __launch_bounds__(128) link_force_kernel(const double2* __restri
         for (int b = 0; b < 3; ++b) F[e * 9 + a * 3 + b] = inv * (grad ? mul_ipow(H.e[a][b], 1) : H.e[a][b]);
 }
 
-// planes handled per launch: all six while their terms (3456 bytes per site)
-// stay below 1 GB, one at a time on larger lattices
-static int force_planes(const FineOp& f) { return f.csw == 0.0 ? 0 : (f.g.V <= 300000 ? 6 : 1); }
-size_t force_scratch(const FineOp& f) {
-    return f.csw == 0.0 ? 0 : ((size_t)54 + 36 * force_planes(f)) * f.g.V * sizeof(double2);
+// Planes handled per launch: all six while their terms (3456 bytes per site) stay
+// below 1 GB, one at a time on larger lattices and where memory is short (form 1),
+// and there the insertions plane by plane too (form 2: 720 bytes per site against
+// 1440 and 4320; six insertion passes instead of one).  The terms of a link are added
+// in the same order in all forms: the same bits.
+size_t force_scratch(const FineOp& f, int form) {
+    if (f.csw == 0.0) return 0;
+    const size_t per = form == 0 && f.g.V <= 300000 ? 54 + 6 * 36 : (form < 2 ? 54 + 36 : 9 + 36);
+    return per * f.g.V * sizeof(double2);
 }
 
 void bilinear_force(const FineOp& f, int nvec, const double2* gv, const double2* psi, const double2* nrm, int grad,
-                    void* scratch, double2* F, cudaStream_t st) {
+                    void* scratch, int form, double2* F, cudaStream_t st) {
     double2* Bt = (double2*)scratch;
-    double2* W4 = Bt + (size_t)f.g.V * 54;
+    double2* W4 = Bt + (size_t)f.g.V * (form < 2 ? 54 : 9);
     const unsigned sites = (f.g.V + 127) / 128, links = (unsigned)(((size_t)f.g.V * 4 + 127) / 128);
     {
         KTimer kt("hop_force", 0.0, 0.0, st);
         hop_force_kernel<<<dim3(sites, 4), 128, 0, st>>>(f.U64, psi, gv, nvec, f.g, F);
     }
-    const int np = force_planes(f);
-    if (np == 0) {
+    if (f.csw == 0.0) {
         KTimer kt("link_force", 0.0, 0.0, st);
         link_force_kernel<<<links, 128, 0, st>>>(f.U64, nullptr, nrm, f.g, 0.0, 0, 0, 1, grad, F);
         return;
     }
-    {
-        KTimer kt("clover_insertion", 0.0, 0.0, st);
-        clover_insertion_kernel<<<(unsigned)(((size_t)f.g.V * 8 + 127) / 128), 128, 0, st>>>(psi, gv, nvec, f.g, Bt);
-    }
+    const int np = form == 0 && f.g.V <= 300000 ? 6 : 1;
     for (int p0 = 0; p0 < 6; p0 += np) {
+        const int only = form < 2 ? -1 : p0;
+        if (p0 == 0 || only >= 0) {
+            KTimer kt("clover_insertion", 0.0, 0.0, st);
+            clover_insertion_kernel<<<(unsigned)(((size_t)f.g.V * 8 + 127) / 128), 128, 0, st>>>(psi, gv, nvec, f.g, only,
+                                                                                                 Bt);
+        }
         {
             KTimer kt("plaquette_force", 0.0, 0.0, st);
-            plaquette_force_kernel<<<dim3(sites, np), 128, 0, st>>>(f.U64, Bt, f.g, p0, W4);
+            plaquette_force_kernel<<<dim3(sites, np), 128, 0, st>>>(f.U64, Bt, f.g, p0, only, W4);
         }
         KTimer kt("link_force", 0.0, 0.0, st);
         link_force_kernel<<<links, 128, 0, st>>>(f.U64, W4, nrm, f.g, f.csw, p0, np, p0 + np >= 6, grad, F);

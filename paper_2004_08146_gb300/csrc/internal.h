@@ -104,10 +104,11 @@ void apply_tangent(const FineOp& f, const double2* dU, const double* dA, int nrh
                    cudaStream_t st);
 // Force of sum_k Re <gv_k, Q' psi_k> per link (F [V][4][9], traceless
 // Hermitian; nvec consecutive fields each), or with grad = 1 the link gradient
-// i F U; nrm (device, may be null) divides.  scratch: force_scratch bytes.
-size_t force_scratch(const FineOp& f);
+// i F U; nrm (device, may be null) divides.  scratch: force_scratch bytes of the form
+// (0 .. 2, ever fewer).
+size_t force_scratch(const FineOp& f, int form);
 void bilinear_force(const FineOp& f, int nvec, const double2* gv, const double2* psi, const double2* nrm, int grad,
-                    void* scratch, double2* F, cudaStream_t st);
+                    void* scratch, int form, double2* F, cudaStream_t st);
 void apply_op(const FineOp& f, int prec, int op, int nrhs, const void* in, void* out,
               const double* tau, cudaStream_t st, const int* act = nullptr);
 void residual_op(const FineOp& f, int prec, int op, int nrhs, const void* b, const void* x, void* r,
