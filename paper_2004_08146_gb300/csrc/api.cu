@@ -1001,7 +1001,7 @@ struct GD {
         Gt = B("Gt", (size_t)mcap * mcap); Hmt = B("Hmt", (size_t)mcap * mcap);
         S = B("S", (size_t)mcap * mcap); work = B("work", (size_t)(6 + block) * mcap * mcap); C = B("C", (size_t)mcap * mcap);
         dots = B("dots", (size_t)4 * (mcap + kcap + 8));
-        part = B("part", (size_t)(2 * mcap + kcap + 8) * kFFParts);
+        part = (double2*)ctx->buf("gd.part", ff_part_bytes(mcap + kcap));
         u = B("u", n); Qu = B("Qu", n); R = B("R", (size_t)block * n); T = B("T", (size_t)block * n);
         tmp = B("tmp", n); tmp2 = B("tmp2", n);
         ffc = B("ffc", (size_t)mcap * mcap); ffw = B("ffw", (size_t)mcap + 1);

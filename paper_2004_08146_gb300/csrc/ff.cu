@@ -510,6 +510,13 @@ void ff_convert(int prec_in, const void* x, int prec_out, void* y, size_t n, cud
         ff_from_fp32_kernel<<<grid_for(n), kThreads, 0, st>>>((const float2*)x, (float4*)y, n);
 }
 
+// A partial sum is 16 bytes.  launch_dots: at most 16 sums (8 complex) per set of
+// vectors and CTA, one wave of CTAs or one CTA per set; ff_ritz: two per CTA.
+constexpr int kRitzCtas = 4096;
+size_t ff_part_bytes(int nvec) {
+    return sizeof(float4) * (size_t)std::max(16 * std::max(4 * sm_count(), nvec), 2 * kRitzCtas);
+}
+
 // CTAs: one wave over all sets of vectors, at least 64 entries per warp
 template <int Q, int NY>
 static void launch_dots(const void* A, int na, const void* B, int nb, size_t n, const void* y0, const void* y1,
@@ -517,7 +524,7 @@ static void launch_dots(const void* A, int na, const void* B, int nb, size_t n, 
     static_assert(Q * NY <= 8, "one warp per sum");
     const int sets = (na + nb + Q - 1) / Q;
     size_t gx = std::max(1, 4 * sm_count() / sets);
-    gx = std::min({gx, std::max<size_t>(1, n / 512), (size_t)kFFParts});
+    gx = std::min(gx, std::max<size_t>(1, n / 512));
     ff_dots_kernel<Q, NY><<<dim3((unsigned)gx, sets), 256, 0, st>>>(
         (const float4*)A, na, (const float4*)B, nb, n, (const float4*)y0, (const float4*)y1, (float4*)partial,
         counters, d0, d1, go);
@@ -554,7 +561,7 @@ void ff_ritz(const void* V, const void* W, int m, size_t n, const double2* s, vo
              void* partial, unsigned* counters, cudaStream_t st) {
     {
         KTimer kt("ritz_ff", (double)(2 * m + 2) * n * 16, 16.0 * m * n, st);
-        const unsigned grid = (unsigned)std::min<size_t>((n + 127) / 128, kFFParts);
+        const unsigned grid = (unsigned)std::min<size_t>((n + 127) / 128, kRitzCtas);
         ff_ritz_kernel<<<grid, 128, 0, st>>>((const float4*)V, (const float4*)W, m, n, s, (float4*)u, (float4*)Qu,
                                              (float4*)partial, counters, d);
     }

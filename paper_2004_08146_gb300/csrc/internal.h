@@ -144,9 +144,9 @@ void blas_axpby(int prec, double2 a, const void* x, double2 b, void* y, size_t n
 constexpr int QCD_FF = 2;
 // FP64 <-> FF, FF -> FP32 (hi + lo rounded), FP32 -> FF
 void ff_convert(int prec_in, const void* x, int prec_out, void* y, size_t n, cudaStream_t st);
-// Vectors of a set are n entries apart.  partial: kFFParts * 16 bytes per dot;
-// counters (zero, left zero): one per vector.
-constexpr int kFFParts = 4096;
+// Vectors of a set are n entries apart.  partial: ff_part_bytes(nvec) for up to nvec
+// vectors in both sets; counters (zero, left zero): one per vector.
+size_t ff_part_bytes(int nvec);
 // dots[i] = <A_i, y>, dots[na + i] = <B_i, y>
 void ff_dots(const void* A, int na, const void* B, int nb, size_t n, const void* y, double2* dots, void* partial,
              unsigned* counters, cudaStream_t st);
