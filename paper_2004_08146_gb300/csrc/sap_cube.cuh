@@ -242,11 +242,11 @@ __device__ __forceinline__ void cube_diag(int op, R t, int chi, const R (&a)[36]
     }
 }
 
-// 1 / sqrt(v) to working accuracy (0 for v = 0): the hardware estimate with
-// one Newton step in FP32
+// 1 / sqrt(v) to working accuracy (0 for v = 0 and for infinity): the hardware
+// estimate with one Newton step in FP32
 __device__ __forceinline__ float inv_sqrt(float v) {
     const float r = rsqrtf(v);
-    return v > 0.f ? r * fmaf(-0.5f * v * r, r, 1.5f) : 0.f;
+    return v > 0.f && r > 0.f ? r * fmaf(-0.5f * v * r, r, 1.5f) : 0.f;
 }
 __device__ __forceinline__ double inv_sqrt(double v) { return v > 0.0 ? rsqrt(v) : 0.0; }
 
@@ -404,8 +404,10 @@ sap_cube_kernel(Geom g, Blocking B, const cplx<R>* __restrict__ U, const R* __re
 #pragma unroll
     for (int k = 0; k < 6; ++k) nn += w[k].x * w[k].x + w[k].y * w[k].y;
     nn = warp_sum(nn);
-    const R ib = inv_sqrt(nn), beta = nn * ib;
-    if (!(beta > R(0))) return;
+    if (!(nn > R(0))) return;
+    // an infinite norm: vectors of zeros where the entries are finite (no correction),
+    // of NaN where they are not, so that x shows it
+    const R ib = inv_sqrt(nn), beta = ib > R(0) ? nn * ib : R(1);
     const R thr = cube_threshold<R>(tol, beta);
     __syncwarp();   // x of the neighbours is read
     {
