@@ -737,7 +737,10 @@ __global__ void __launch_bounds__(128) wilson_clover_f64_kernel(
             if (a == c && sp == p) m = make_double2(__ldg(Ab + i), 0.0);
             else m = __ldg(reinterpret_cast<const double2*>(Ab + herm_off(lo, hi)));
             m.y = flip(m.y, i > k ? kSign : 0);
-            cmac(acc, m, psi[c]);
+            // the real diagonal: nothing times its zero (not NaN for an infinite psi)
+            const double2 v = psi[c], z = a == c && sp == p ? make_double2(0.0, 0.0) : v;
+            acc.x = fma(-m.y, z.y, fma(m.x, v.x, acc.x));
+            acc.y = fma(m.y, z.x, fma(m.x, v.y, acc.y));
         }
         r[a] = sg < 0 ? -acc : acc;
     }
