@@ -256,8 +256,10 @@ class Context:
         need = 36
         for x in dims:
             need *= max(int(x), 0)
-        if U.numel() < need or not U.is_contiguous() or U.element_size() != 16:
-            raise ValueError("links must be a contiguous complex128 tensor of prod(dims) * 36 entries")
+        # a lazily conjugated or negated view is contiguous too, but its memory is not it
+        if (U.numel() < need or not U.is_contiguous() or U.element_size() != 16 or not U.is_cuda
+                or U.is_conj() or U.is_neg()):
+            raise ValueError("links must be a contiguous complex128 CUDA tensor of prod(dims) * 36 entries")
         d = (ctypes.c_int * 4)(*[int(x) for x in dims])
         self.dims = tuple(int(x) for x in dims)
         return self._check(_lib.qcd_set_gauge_device(self.h, _ptr(U), d, float(m0), float(csw)))
