@@ -1029,11 +1029,14 @@ void launch_clover_build(const FineOp& f, cudaStream_t st) {
 
 static void launch_f64(const FineOp& f, const double2* U, const double* A, int op, int nrhs, const double2* in,
                        double2* out, const double2* b, const Shifts& sh, const int* act, cudaStream_t st) {
-    // One thread per site once a single field gives each FP64 pipe (four per SM)
-    // more than three warps; eight lanes per site below.  Measured, eight lanes
-    // against one: 8^4 16.6 / 45.4 us, 16 x 8^3 27 / 45, 16^4 156 / 166, 32 x 16^3
-    // 307 / 289, 8 fields of 16^4 1206 / 1088.  The line depends on the lattice
-    // only, so a field's result does not depend on the batch it is in.
+    // One thread per site (8 % fewer operations) from the lattice where batches of any
+    // size gain more than a single field loses; eight lanes per site below.  The line
+    // depends on the lattice only, so a field's result does not depend on the batch it
+    // is in.  Measured, eight lanes / one thread, 1, 2 and 8 fields (us):
+    //   8^4 16.9 / 45.8, 27 / 46, 85 / 85        12^4 56 / 85, 107 / 126, 390 / 365
+    //   16^3 x 8 85 / 85, 157 / 166, 607 / 565   16^3 x 15 151 / 166, 290 / 287, 1133 / 1043
+    //   16^4 157 / 167, 308 / 288, 1206 / 1088   32 x 16^3 308 / 290, 607 / 570, 2403 / 2166
+    // Batches of four and more lose up to 9 % to one thread between 12^4 and the line.
     if (f.g.V >= 65536) {
         const dim3 grid((f.g.V + 127) / 128, nrhs);
         wilson_clover_f64_site_kernel<<<grid, 128, 0, st>>>(out, in, b, U, A, f.g, op, sh, (size_t)f.g.V * 12, act);
@@ -1066,8 +1069,9 @@ static void launch_dirac(const FineOp& f, int prec, int op, int nrhs, const void
     const unsigned grid = (unsigned)((f.g.V + 127) / 128) * (unsigned)((nrhs + nr - 1) / nr);
     auto kern = nr == 2 ? (w32 ? wilson_clover_soa_kernel<2, true> : wilson_clover_soa_kernel<2, false>)
                         : (w32 ? wilson_clover_soa_kernel<1, true> : wilson_clover_soa_kernel<1, false>);
-    // a single right-hand side far past L2: 168 registers, more loads in flight
-    // per thread (64 x 32^3 280 us against 288; 32 x 16^3 23.7 against 22.5)
+    // a single right-hand side far past L2: 168 registers, more loads in flight per
+    // thread (2^21 sites 281 us against 291, 2^20 146 / 152, 2^19 76.5 / 78.6, 2^18 43.5 /
+    // 45.0; 2^17, in L2, 25.0 / 23.3): the line lies inside what was faster
     if (nr == 1 && w32 && f.g.V >= (1 << 20)) kern = wilson_clover_soa_kernel<1, true, 3>;
     kern<<<grid, 128, 0, st>>>((float2*)out, (const float2*)in, (const float2*)b, f.U32s, f.A32s, f.g, op, sh,
                                (size_t)f.g.V * 12, act, nrhs, tb);

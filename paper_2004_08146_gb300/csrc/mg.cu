@@ -302,7 +302,10 @@ __global__ void __launch_bounds__(kProlongT, 5) prolong_tile_kernel(Geom g, Bloc
     const int j0 = (blockIdx.x % groups) * TJ, part = (blockIdx.x / groups) % parts, blk = blockIdx.x / groups / parts;
     const int l = 2 * part * kStep + threadIdx.x / kPer, w = threadIdx.x % kPer;
     const int chi = w / (kPer / 2), s = (w % (kPer / 2)) * E;
-    const bool two = B.bs > kStep;   // otherwise the second piece repeats the first and is not stored
+    // aggregates that one piece per thread covers: the second repeats the first and is
+    // multiplied for nothing (16 sites, 16 x 8^3, 4 right-hand sides: 9 us, launch and
+    // latency, not arithmetic)
+    const bool two = B.bs > kStep;
     const cplx<R>* p = P + ((size_t)blk * 2 + chi) * nv * nloc + s;
     auto fill = [&](int i) {
         if (i < nv)
@@ -1754,7 +1757,9 @@ static void launch_prolong(const FineOp& f, const Coarse& c, int nrhs, const cpl
                                                                parts, act);
 }
 
-// tiles as wide as the right-hand sides fill, at most TJ
+// Tiles as wide as the right-hand sides fill, at most TJ.  Four wide while the warps of
+// 16 right-hand sides (ceil(nv / 4) x 4) fit the 640 threads of that launch bound, nv
+// <= 20; eight wide, with half the warps, beyond.
 template <typename R, int E, int TJ>
 static void restrict_width(const FineOp& f, const Coarse& c, int nrhs, const cplx<R>* P, const void* r, void* xc,
                            cudaStream_t st, const int* act) {
