@@ -112,10 +112,10 @@ def max_over_ranks(value, device=None):
 # "traffic"; a kernel that changes is taken out of this table until it is
 # captured again (the field is then null).  Two launches each in the 16 x 8^3
 # step (k = 4, 4 targets; profiles/case_kernels.md): coarse_gmres_f32
-# (coarse_gmres_kernel<float2, float>) 9.7997 and 9.7999 MB read; sap_block_f32
-# (sap_cube_kernel<float, float2>, up to four block solves per CTA) 8.8131 MB
-# read, nothing written.
-NCU_TRAFFIC = {"coarse_gmres_f32": 9.7998e6, "sap_block_f32": 8.8131e6}
+# (coarse_gmres_kernel<float2, float>) 9.7987 and 9.7984 MB read; sap_block_f32
+# (sap_cube_kernel<float, float2>, up to four block solves per CTA) 8.8136 and
+# 8.8131 MB read, nothing written.
+NCU_TRAFFIC = {"coarse_gmres_f32": 9.7985e6, "sap_block_f32": 8.8133e6}
 
 # Work model of the SAP block solves for the FP32-ALU roofline, per block
 # site and GMRES step j (0-based) of a block solve of k steps: the Dirichlet
