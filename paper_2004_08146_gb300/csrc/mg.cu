@@ -173,21 +173,26 @@ template <int N> __device__ __forceinline__ void async_wait() { asm volatile("cp
 // one chunk of 8 per pass and one warp per vector -> 154 us (3.0 TB/s; prologue of a
 // single resident CTA per SM not hidden); 143 us with one chain of fused
 // multiply-adds per sum.
-template <typename R> constexpr int kTransferRhs = sizeof(R) == 4 ? 16 : 8;
-constexpr int kRestrictTI = 4;
+// FP64 is bound by its pipe (2 operations per clock and SM, a quarter of them for each
+// quarter of the warps): smaller tiles without rows of padding, at least four warps
+// where there is work for them, and the terms with Re P and with Im P in sums of their
+// own, which costs registers instead of operations.
+template <typename R> constexpr int kTransferRhs = sizeof(R) == 4 ? 16 : 4;
+template <typename R, int TI, int TJ> constexpr int kRestrictThreads =
+    sizeof(R) == 4 ? (TJ == 4 ? 640 : 512) : (TI * TJ <= 2 ? 1024 : (TI * TJ == 4 ? 768 : 512));
 constexpr int kRing = 4, kStage = 64;   // a stage: two pieces of a row per lane
 constexpr int kSiteTable = 1024;   // aggregates up to this size look their entries up
-template <typename R, int E, int TJ>
-__global__ void __launch_bounds__(TJ == 4 && sizeof(R) == 4 ? 640 : 512) restrict_tile_kernel(
+template <typename R, int E, int TI, int TJ>
+__global__ void __launch_bounds__(kRestrictThreads<R, TI, TJ>) restrict_tile_kernel(
     Geom g, Blocking B, int nv, const cplx<R>* __restrict__ P, const cplx<R>* __restrict__ r, cplx<R>* __restrict__ xc,
-    int nrhs, int ring, const int* __restrict__ act) {
-    constexpr int TI = kRestrictTI;
+    int nrhs, int chunk, int ring, const int* __restrict__ act) {
+    constexpr bool kTwo = sizeof(R) == 8;
     using Pc = Piece<R, E>;
     extern __shared__ __align__(16) unsigned char rsm[];
     const int nc = 2 * nv, nloc = B.bs * 6, np = nloc / E;
     const bool table = B.bs <= kSiteTable;
     const int blk = blockIdx.x >> 1, chi = blockIdx.x & 1;
-    const int jc = blockIdx.y * kTransferRhs<R>, nr = min(nrhs - jc, kTransferRhs<R>), rows = nv + nr;
+    const int jc = blockIdx.y * chunk, nr = min(nrhs - jc, chunk), rows = nv + nr;
     Pc* stage = reinterpret_cast<Pc*>(rsm);                                       // [ring][rows][kStage]
     int* entry = reinterpret_cast<int*>(stage + (size_t)ring * rows * kStage);    // fine entry of a piece
     auto entry_of = [&](int e) { return block_fine_site(g, B, blk, e * E / 6) * 12 + e * E % 6 + 6 * chi; };
@@ -221,9 +226,13 @@ __global__ void __launch_bounds__(TJ == 4 && sizeof(R) == 4 ? 640 : 512) restric
     for (int st = 0; st < kRing - 1; ++st) fill(st, st * slots);
     const int nit = (nv + TI - 1) / TI;
     const int i0 = (warp % nit) * TI, j0 = (warp / nit) * TJ;
-    R acc[TI * TJ * 2];
+    const bool idle = j0 >= nr;   // the last chunk may need fewer warps
+    R acc[TI * TJ * 2], acc2[kTwo ? TI * TJ * 2 : 1];
 #pragma unroll
-    for (int q = 0; q < TI * TJ * 2; ++q) acc[q] = R(0);
+    for (int q = 0; q < TI * TJ * 2; ++q) {
+        acc[q] = R(0);
+        if constexpr (kTwo) acc2[q] = R(0);
+    }
     // rows past the last are read like the last and not written
     int ra[TI], ru[TJ];
 #pragma unroll
@@ -238,9 +247,10 @@ __global__ void __launch_bounds__(TJ == 4 && sizeof(R) == 4 ? 640 : 512) restric
         next = cur;
         const Pc* sp = stage + cur;
         cur = cur + slots == kRing * slots ? 0 : cur + slots;
-        // the products of a stage by themselves, then into the running sum, which so
-        // rounds once in 2 E products (in the chain of all of them it rounds twice in
-        // each; 4^4 aggregates: 1.0e-7 from the exact sum against 1.9e-7)
+        if (idle) continue;
+        // FP32: the products of a stage by themselves, then into the running sum, which
+        // so rounds once in 2 E products (in the chain of all of them it rounds twice in
+        // each; 4^4 aggregates: 1.1e-7 from the exact sum against 1.9e-7)
         Pc a[2][TI];
 #pragma unroll
         for (int q = 0; q < TI; ++q) {
@@ -252,14 +262,33 @@ __global__ void __launch_bounds__(TJ == 4 && sizeof(R) == 4 ? 640 : 512) restric
             const Pc b[2] = {sp[ru[u]], sp[ru[u] + 32]};
 #pragma unroll
             for (int q = 0; q < TI; ++q) {
-                cplx<R> t = cmulc(a[0][q].at(0), b[0].at(0));
+                R &re = acc[(q * TJ + u) * 2], &im = acc[(q * TJ + u) * 2 + 1];
+                if constexpr (kTwo) {
+                    R &re2 = acc2[(q * TJ + u) * 2], &im2 = acc2[(q * TJ + u) * 2 + 1];
 #pragma unroll
-                for (int k = 1; k < 2 * E; ++k) cmacc(t, a[k / E][q].at(k % E), b[k / E].at(k % E));
-                acc[(q * TJ + u) * 2] += t.x;
-                acc[(q * TJ + u) * 2 + 1] += t.y;
+                    for (int h = 0; h < 2; ++h) {
+                        const cplx<R> m = a[h][q].at(0), v = b[h].at(0);
+                        re = fma(m.x, v.x, re);
+                        im = fma(m.x, v.y, im);
+                        re2 = fma(m.y, v.y, re2);
+                        im2 = fma(m.y, v.x, im2);
+                    }
+                } else {
+                    cplx<R> t = cmulc(a[0][q].at(0), b[0].at(0));
+#pragma unroll
+                    for (int k = 1; k < 2 * E; ++k) cmacc(t, a[k / E][q].at(k % E), b[k / E].at(k % E));
+                    re += t.x;
+                    im += t.y;
+                }
             }
         }
     }
+    if constexpr (kTwo)
+#pragma unroll
+        for (int q = 0; q < TI * TJ * 2; q += 2) {
+            acc[q] += acc2[q];
+            acc[q + 1] -= acc2[q + 1];
+        }
     constexpr int N = TI * TJ * 2, keep = N / 32 > 1 ? N / 32 : 1, dup = N < 32 ? 32 / N : 1;
     int base = 0;
     scatter_sum<N, 16>(acc, lane, base);
@@ -283,7 +312,8 @@ __global__ void __launch_bounds__(TJ == 4 && sizeof(R) == 4 ? 640 : 512) restric
 // thread fills and reads for itself (no barrier).
 // 32 x 16^3, 4^4 aggregates, nv 20, 16 right-hand sides: 339 us ->
 // 153 us (3.0 TB/s) at five CTAs per SM; 145 us with one chain of fused multiply-adds
-// per sum, four or six CTAs 165 / 158 us.
+// per sum, four or six CTAs 165 / 158 us.  FP64 takes one piece per thread and at most
+// two right-hand sides: what counts there are the operations on padding.
 constexpr int kAhead = 8;
 constexpr int kProlongT = 96;   // whole warps and whole sites: both pieces lie at the same place of a site
 template <typename R, int E, int TJ>
@@ -291,30 +321,32 @@ __global__ void __launch_bounds__(kProlongT, 5) prolong_tile_kernel(Geom g, Bloc
                                                                  const cplx<R>* __restrict__ P,
                                                                  const cplx<R>* __restrict__ xc, cplx<R>* __restrict__ x,
                                                                  int nrhs, int parts, const int* __restrict__ act) {
+    constexpr bool kTwo = sizeof(R) == 8;
+    constexpr int NP = kTwo ? 1 : 2;   // pieces of a thread
     constexpr int kPer = 12 / E, T = kProlongT, kStep = T / kPer;   // pieces per site, sites between the two pieces
     static_assert(T % kPer == 0 && T % 32 == 0, "CTA of whole warps and whole sites");
     using Pc = Piece<R, E>;
     extern __shared__ __align__(16) unsigned char psm[];
-    Pc* ring = reinterpret_cast<Pc*>(psm) + threadIdx.x;   // [kAhead][2][T]
-    cplx<R>* cs = reinterpret_cast<cplx<R>*>(psm + sizeof(Pc) * kAhead * 2 * T);
+    Pc* ring = reinterpret_cast<Pc*>(psm) + threadIdx.x;   // [kAhead][NP][T]
+    cplx<R>* cs = reinterpret_cast<cplx<R>*>(psm + sizeof(Pc) * kAhead * NP * T);
     const int nc = 2 * nv, nloc = B.bs * 6, half = (nv + (nv & 1)) * TJ + 2;
     const int groups = (nrhs + TJ - 1) / TJ;
     const int j0 = (blockIdx.x % groups) * TJ, part = (blockIdx.x / groups) % parts, blk = blockIdx.x / groups / parts;
-    const int l = 2 * part * kStep + threadIdx.x / kPer, w = threadIdx.x % kPer;
+    const int l = NP * part * kStep + threadIdx.x / kPer, w = threadIdx.x % kPer;
     const int chi = w / (kPer / 2), s = (w % (kPer / 2)) * E;
     // aggregates that one piece per thread covers: the second repeats the first and is
     // multiplied for nothing (16 sites, 16 x 8^3, 4 right-hand sides: 9 us, launch and
     // latency, not arithmetic)
-    const bool two = B.bs > kStep;
+    const bool two = NP == 2 && B.bs > kStep;
     const cplx<R>* p = P + ((size_t)blk * 2 + chi) * nv * nloc + s;
     auto fill = [&](int i) {
         if (i < nv)
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
+            for (int h = 0; h < NP; ++h) {
                 const int lh = l + h * kStep;
                 const bool in = lh < B.bs;
                 if (h == 0 || two)
-                    async_piece<R, E>(ring + ((i % kAhead) * 2 + h) * T, p + (size_t)i * nloc + (in ? lh * 6 : 0), in);
+                    async_piece<R, E>(ring + ((i % kAhead) * NP + h) * T, p + (size_t)i * nloc + (in ? lh * 6 : 0), in);
             }
         async_commit();
     };
@@ -329,39 +361,56 @@ __global__ void __launch_bounds__(kProlongT, 5) prolong_tile_kernel(Geom g, Bloc
     if ((nv & 1) && threadIdx.x < 2 * TJ) cs[threadIdx.x / TJ * half + nv * TJ + threadIdx.x % TJ] = czero<R>();
     __syncthreads();
     const cplx<R>* c = cs + chi * half;
-    cplx<R> acc[2][TJ][E];
+    cplx<R> acc[NP][TJ][E], acc2[kTwo ? TJ : 1];
 #pragma unroll
-    for (int h = 0; h < 2; ++h)
+    for (int u = 0; u < TJ; ++u) {
+        if constexpr (kTwo) acc2[u] = czero<R>();
 #pragma unroll
-        for (int u = 0; u < TJ; ++u)
+        for (int h = 0; h < NP; ++h)
 #pragma unroll
             for (int k = 0; k < E; ++k) acc[h][u][k] = czero<R>();
-    // two rows at a time, summed by themselves before they join the running sum (one
-    // chain over all rows: 1.14e-7 from the exact sum against 7.4e-8 at nv 20)
+    }
+    // FP32: two rows at a time, summed by themselves before they join the running sum
+    // (one chain over all rows: 1.14e-7 from the exact sum against 7.4e-8 at nv 20)
     const int second = two ? T : 0;
     for (int i = 0; i < nv; i += 2) {
         async_wait<kAhead - 4>();
         // past the last of an odd number: the same row again, times the zeros behind it
         const bool pair = i + 1 < nv;
-        const Pc *r0 = ring + (i % kAhead) * 2 * T, *r1 = pair ? ring + ((i + 1) % kAhead) * 2 * T : r0;
+        const Pc *r0 = ring + (i % kAhead) * NP * T, *r1 = pair ? ring + ((i + 1) % kAhead) * NP * T : r0;
         const Pc a[2][2] = {{r0[0], r0[second]}, {r1[0], r1[second]}};   // [row][piece]
         fill(i + kAhead - 2);
         fill(i + kAhead - 1);
 #pragma unroll
         for (int u = 0; u < TJ; ++u) {
             const cplx<R> v = c[i * TJ + u], w = c[(i + 1) * TJ + u];
+            if constexpr (kTwo) {
+                cplx<R>&s1 = acc[0][u][0], &s2 = acc2[u];
 #pragma unroll
-            for (int h = 0; h < 2; ++h)
-#pragma unroll
-                for (int k = 0; k < E; ++k) {
-                    cplx<R> t = a[0][h].at(k) * v;
-                    cmac(t, a[1][h].at(k), w);
-                    acc[h][u][k] += t;
+                for (int q = 0; q < 2; ++q) {
+                    const cplx<R> m = a[q][0].at(0), z = q ? w : v;
+                    s1.x = fma(m.x, z.x, s1.x);
+                    s1.y = fma(m.x, z.y, s1.y);
+                    s2.x = fma(m.y, z.y, s2.x);
+                    s2.y = fma(m.y, z.x, s2.y);
                 }
+            } else {
+#pragma unroll
+                for (int h = 0; h < 2; ++h)
+#pragma unroll
+                    for (int k = 0; k < E; ++k) {
+                        cplx<R> t = a[0][h].at(k) * v;
+                        cmac(t, a[1][h].at(k), w);
+                        acc[h][u][k] += t;
+                    }
+            }
         }
     }
+    if constexpr (kTwo)
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
+        for (int u = 0; u < TJ; ++u) acc[0][u][0] = mk<R>(acc[0][u][0].x - acc2[u].x, acc[0][u][0].y + acc2[u].y);
+#pragma unroll
+    for (int h = 0; h < NP; ++h) {
         const int lh = l + h * kStep;
         if (lh >= B.bs) continue;
         cplx<R>* o = x + (size_t)block_fine_site(g, B, blk, lh) * 12 + 6 * chi + s;
@@ -1733,46 +1782,61 @@ void mg_build_coarse(const FineOp& f, Coarse& c, cudaStream_t st, bool fp32_only
     c.a64_stale = false;
 }
 
-template <typename R, int E, int TJ>
-static void launch_restrict(const FineOp& f, const Coarse& c, int nrhs, const cplx<R>* P, const void* r, void* xc,
-                            cudaStream_t st, const int* act) {
-    const int chunk = std::min(nrhs, kTransferRhs<R>);
-    const int warps = (c.nv + kRestrictTI - 1) / kRestrictTI * ((chunk + TJ - 1) / TJ);
-    const dim3 grid(c.B.nb * 2, (nrhs + kTransferRhs<R> - 1) / kTransferRhs<R>);
+template <typename R, int E, int TI, int TJ>
+static void launch_restrict(const FineOp& f, const Coarse& c, int nrhs, int chunk, const cplx<R>* P, const void* r,
+                            void* xc, cudaStream_t st, const int* act) {
+    const int warps = (c.nv + TI - 1) / TI * ((chunk + TJ - 1) / TJ);
+    const dim3 grid(c.B.nb * 2, (nrhs + chunk - 1) / chunk);
     const int ring = std::min(kRing, (c.B.bs * 6 / E + kStage - 1) / kStage);   // no more stages than there are
     const size_t sm = (size_t)ring * (c.nv + chunk) * kStage * sizeof(Piece<R, E>) +
                       (c.B.bs <= kSiteTable ? c.B.bs * 6 / E * sizeof(int) : 0);
-    if (sm > 48 * 1024)
-        cudaFuncSetAttribute(restrict_tile_kernel<R, E, TJ>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    restrict_tile_kernel<R, E, TJ><<<grid, 32 * warps, sm, st>>>(f.g, c.B, c.nv, P, (const cplx<R>*)r, (cplx<R>*)xc, nrhs,
-                                                                 ring, act);
+    auto kern = restrict_tile_kernel<R, E, TI, TJ>;
+    if (sm > 48 * 1024) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    kern<<<grid, 32 * warps, sm, st>>>(f.g, c.B, c.nv, P, (const cplx<R>*)r, (cplx<R>*)xc, nrhs, chunk, ring, act);
 }
 template <typename R, int E, int TJ>
 static void launch_prolong(const FineOp& f, const Coarse& c, int nrhs, const cplx<R>* P, const void* xc, void* x,
                            cudaStream_t st, const int* act) {
-    const int parts = (c.B.bs * 12 / E + 2 * kProlongT - 1) / (2 * kProlongT);
+    constexpr int per = (sizeof(R) == 8 ? 1 : 2) * kProlongT;   // pieces per CTA
+    const int parts = (c.B.bs * 12 / E + per - 1) / per;
     const unsigned grid = (unsigned)c.B.nb * parts * ((nrhs + TJ - 1) / TJ);
-    const size_t sm = sizeof(Piece<R, E>) * kAhead * 2 * kProlongT + 2 * (size_t)((c.nv + (c.nv & 1)) * TJ + 2) * sizeof(cplx<R>);
+    const size_t sm = sizeof(Piece<R, E>) * kAhead * per + 2 * (size_t)((c.nv + (c.nv & 1)) * TJ + 2) * sizeof(cplx<R>);
     prolong_tile_kernel<R, E, TJ><<<grid, kProlongT, sm, st>>>(f.g, c.B, c.nv, P, (const cplx<R>*)xc, (cplx<R>*)x, nrhs,
                                                                parts, act);
 }
 
-// Tiles as wide as the right-hand sides fill, at most TJ.  Four wide while the warps of
-// 16 right-hand sides (ceil(nv / 4) x 4) fit the 640 threads of that launch bound, nv
-// <= 20; eight wide, with half the warps, beyond.
-template <typename R, int E, int TJ>
-static void restrict_width(const FineOp& f, const Coarse& c, int nrhs, const cplx<R>* P, const void* r, void* xc,
-                           cudaStream_t st, const int* act) {
+// FP32 tiles as wide as the right-hand sides fill, at most TJ.  Four wide while the
+// warps of 16 right-hand sides (ceil(nv / 4) x 4) fit the 640 threads of that launch
+// bound, nv <= 20; eight wide, with half the warps, beyond.
+template <int E, int TJ>
+static void restrict_width(const FineOp& f, const Coarse& c, int nrhs, const void* r, void* xc, cudaStream_t st,
+                           const int* act) {
     if constexpr (TJ > 1)
-        if (2 * nrhs <= TJ || (TJ == 8 && c.nv <= 20)) return restrict_width<R, E, TJ / 2>(f, c, nrhs, P, r, xc, st, act);
-    launch_restrict<R, E, TJ>(f, c, nrhs, P, r, xc, st, act);
+        if (2 * nrhs <= TJ || (TJ == 8 && c.nv <= 20)) return restrict_width<E, TJ / 2>(f, c, nrhs, r, xc, st, act);
+    launch_restrict<float, E, 4, TJ>(f, c, nrhs, std::min(nrhs, kTransferRhs<float>), c.P32, r, xc, st, act);
 }
-template <typename R, int E, int TJ>
-static void prolong_width(const FineOp& f, const Coarse& c, int nrhs, const cplx<R>* P, const void* xc, void* x,
-                          cudaStream_t st, const int* act) {
+template <int E, int TJ>
+static void prolong_width(const FineOp& f, const Coarse& c, int nrhs, const void* xc, void* x, cudaStream_t st,
+                          const int* act) {
     if constexpr (TJ > 1)
-        if (2 * nrhs <= TJ) return prolong_width<R, E, TJ / 2>(f, c, nrhs, P, xc, x, st, act);
-    launch_prolong<R, E, TJ>(f, c, nrhs, P, xc, x, st, act);
+        if (2 * nrhs <= TJ) return prolong_width<E, TJ / 2>(f, c, nrhs, xc, x, st, act);
+    launch_prolong<float, E, TJ>(f, c, nrhs, c.P32, xc, x, st, act);
+}
+// FP64: fewer right-hand sides per CTA until two waves of CTAs are there, then the
+// smallest tile whose warps fit its launch bound.  With 4 x 4 tiles and chunks of eight
+// (restriction) or four right-hand sides and two pieces per thread (prolongation) five
+// vectors and three right-hand sides took 140 us on 16 x 8^3 with 4^4 aggregates (one
+// warp per vector before: 72) and 18 us on 12 x 6^3 with 3^4 (12); now 27 and 9.  16^4,
+// 4^4 aggregates, nv 20, 8 right-hand sides: 943 and 845 us.
+static void restrict_f64(const FineOp& f, const Coarse& c, int nrhs, const void* r, void* xc, cudaStream_t st,
+                         const int* act) {
+    int chunk = std::min(nrhs, kTransferRhs<double>);
+    while (chunk > 1 && 2 * c.B.nb * ((nrhs + chunk - 1) / chunk) < 2 * coarse_gmres_grid()) chunk = (chunk + 1) / 2;
+    const int nv = c.nv;
+    if (nv * chunk <= 32) launch_restrict<double, 1, 1, 1>(f, c, nrhs, chunk, c.P64, r, xc, st, act);
+    else if ((nv + 1) / 2 * chunk <= 32) launch_restrict<double, 1, 2, 1>(f, c, nrhs, chunk, c.P64, r, xc, st, act);
+    else if ((nv + 3) / 4 * chunk <= 24) launch_restrict<double, 1, 4, 1>(f, c, nrhs, chunk, c.P64, r, xc, st, act);
+    else launch_restrict<double, 1, 4, 2>(f, c, nrhs, chunk, c.P64, r, xc, st, act);
 }
 
 void mg_restrict(const FineOp& f, const Coarse& c, int prec, int nrhs, const void* r, void* xc, cudaStream_t st,
@@ -1783,9 +1847,9 @@ void mg_restrict(const FineOp& f, const Coarse& c, int prec, int nrhs, const voi
     KTimer kt(prec == QCD_FP64 ? "restrict_f64" : "restrict_f32",
               es * (nfine * c.nv * ((nrhs + per - 1) / per) + nrhs * (nfine + (double)c.gc.V * c.nc)),
               8.0 * nfine * c.nv * nrhs, st);
-    if (prec == QCD_FP64) restrict_width<double, 1, 4>(f, c, nrhs, c.P64, r, xc, st, act);
-    else if ((uintptr_t)r & 15) restrict_width<float, 1, 8>(f, c, nrhs, c.P32, r, xc, st, act);
-    else restrict_width<float, 2, 8>(f, c, nrhs, c.P32, r, xc, st, act);
+    if (prec == QCD_FP64) restrict_f64(f, c, nrhs, r, xc, st, act);
+    else if ((uintptr_t)r & 15) restrict_width<1, 8>(f, c, nrhs, r, xc, st, act);
+    else restrict_width<2, 8>(f, c, nrhs, r, xc, st, act);
 }
 
 void mg_prolong(const FineOp& f, const Coarse& c, int prec, int nrhs, const void* xc, void* x, cudaStream_t st,
@@ -1796,9 +1860,10 @@ void mg_prolong(const FineOp& f, const Coarse& c, int prec, int nrhs, const void
     KTimer kt(prec == QCD_FP64 ? "prolong_f64" : "prolong_f32",
               es * (nfine * c.nv * ((nrhs + per - 1) / per) + nrhs * (nfine + (double)c.gc.V * c.nc)),
               8.0 * nfine * c.nv * nrhs, st);
-    if (prec == QCD_FP64) prolong_width<double, 1, 4>(f, c, nrhs, c.P64, xc, x, st, act);
-    else if ((uintptr_t)x & 15) prolong_width<float, 1, 8>(f, c, nrhs, c.P32, xc, x, st, act);
-    else prolong_width<float, 2, 8>(f, c, nrhs, c.P32, xc, x, st, act);
+    if (prec == QCD_FP64 && nrhs % 2) launch_prolong<double, 1, 1>(f, c, nrhs, c.P64, xc, x, st, act);
+    else if (prec == QCD_FP64) launch_prolong<double, 1, 2>(f, c, nrhs, c.P64, xc, x, st, act);
+    else if ((uintptr_t)x & 15) prolong_width<1, 8>(f, c, nrhs, xc, x, st, act);
+    else prolong_width<2, 8>(f, c, nrhs, xc, x, st, act);
 }
 
 void coarse_apply(const Coarse& c, int prec, int op, int nrhs, const void* x, void* y, const double* tau,
