@@ -128,7 +128,7 @@ struct qcd_ctx {
             drop_buf("force");
             e = cudaMalloc(q, bytes);
         }
-        cudaGetLastError();   // a failure is reported by the return value alone
+        if (e != cudaSuccess) cudaGetLastError();   // the return value reports it; a pending launch error stays
         return e;
     }
     void* buf(const std::string& name, size_t bytes) {
