@@ -123,12 +123,16 @@ struct qcd_ctx {
     // cudaMalloc that gives back the link force's scratch, which no other call uses, if
     // that is in the way
     cudaError_t dev_malloc(void** q, size_t bytes) {
+        // failures are reported by the return value; a launch error that is still pending
+        // stays after a success
         cudaError_t e = cudaMalloc(q, bytes);
+        if (e == cudaSuccess) return e;
+        cudaGetLastError();
         if (e == cudaErrorMemoryAllocation && ws.count("force")) {
             drop_buf("force");
             e = cudaMalloc(q, bytes);
+            if (e != cudaSuccess) cudaGetLastError();
         }
-        if (e != cudaSuccess) cudaGetLastError();   // the return value reports it; a pending launch error stays
         return e;
     }
     void* buf(const std::string& name, size_t bytes) {

@@ -54,3 +54,4 @@ def test_force_in_little_memory():
         torch.cuda.empty_cache()
     assert torch.equal(F, F0)
     ctx.close()
+    make_ctx(U, DIMS, -0.3, 1.5).close()               # no error of the refused allocations is left
